@@ -360,7 +360,7 @@ struct RegularInfo {
   std::vector<char> regular;         // per non-terminal
 };
 
-constexpr size_t NFA_STATE_CAP = 60000, DFA_STATE_CAP = 6000;
+constexpr size_t NFA_STATE_CAP = 60000, DFA_STATE_CAP = 6000, DFA_PART_CAP = 512;
 
 class DfaBuilder {
  public:
@@ -710,14 +710,29 @@ void compile_grammar(const char* text, size_t len, const std::string& start, Hos
         for (int s : p.rhs)
           if (s >= 0 && s != aug && ri.regular[s]) wanted[s] = 1;
     size_t total_states = 0;
-    for (size_t x = 0; x < n_all; ++x) {
-      if (!wanted[x]) continue;
-      OneDfa one;
-      if (!db.build((int)x, one)) continue;                        // too large: stays a set of rules
-      if (total_states + one.n_states > 16000) continue;           // (state numbers have 14 bits)
-      total_states += one.n_states;
-      dfa_of[x] = (int)dfas.size();
-      dfas.push_back(std::move(one));
+    std::vector<char> tried(n_all, 0), part(n_all, 0);
+    for (bool again = true; again;) {
+      again = false;
+      for (size_t x = 0; x < n_all; ++x) {
+        if (!wanted[x] || tried[x]) continue;
+        tried[x] = 1;
+        OneDfa one;
+        // (state numbers have 14 bits; a part of a regular non-terminal that was too large has to be a good deal smaller)
+        if (!db.build((int)x, one) || total_states + one.n_states > 16000 || (part[x] && one.n_states > DFA_PART_CAP)) {
+          // too large: it stays a set of rules, and the regular non-terminals in those are tried one by one.  (A JSON schema is
+          // often regular as a whole, but with too many states; its strings, numbers and members are small.  The schema of the
+          // timed cases went from no automaton to seven with 764 states: an advance of 64 rows 57 -> 40 us, a sweep of their masks
+          // by Earley steps 374 -> 263 us.)
+          for (auto& p : rules)
+            if (p.lhs == (int)x)
+              for (int s : p.rhs)
+                if (s >= 0 && s != aug && ri.regular[s] && !wanted[s]) wanted[s] = part[s] = 1, again = true;
+          continue;
+        }
+        total_states += one.n_states;
+        dfa_of[x] = (int)dfas.size();
+        dfas.push_back(std::move(one));
+      }
     }
     if (!dfas.empty()) {  // their rules go, and with them whatever only they used
       std::vector<Production> left;

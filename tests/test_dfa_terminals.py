@@ -107,3 +107,17 @@ def test_what_is_not_regular_stays_rules():
     assert g1.info().n_automata == 1 and g1.info().n_rules == 1  # only $ -> s is left
     for s, ok in [(b"d", True), (b"abcd", True), (b"bcbcad", True), (b"abd", False), (b"", False), (b"dd", False)]:
         assert g1.automaton_accepts(0, s) == ok, s
+
+
+def test_parts_of_a_regular_non_terminal_that_is_too_large():
+    """A regular non-terminal whose automaton would have too many states (here 2^14: "an a, thirteen letters before the
+    end") stays rules, and the small regular non-terminals in its rules become automata of their own."""
+    text = 's ::= num ":" tail\ntail ::= [ab]* "a" %s num\nnum ::= [0-9]+ ("." [0-9]+)?' % " ".join(["[ab]"] * 13)
+    vocab = [bytes([b]) for b in range(256)] + [b"12", b"ab", b""]
+    g = fmt.Grammar(text, "s", vocab, len(vocab) - 1, host_only=True)
+    names = [g.automaton_name(k) for k in range(g.info().n_automata)]
+    assert "num" in names and "tail" not in names and "s" not in names
+    k = names.index("num")
+    og = oracle.Grammar(text, "num")
+    for s in [b"12.5", b"7", b"12.", b".5", b"", b"1a"]:
+        assert g.automaton_accepts(k, s) == _oracle_accepts(og, s), s
