@@ -113,6 +113,7 @@ struct fmt_state {
   int32_t* result_dev = nullptr;
   uint8_t* query_dev = nullptr;  // scratch for fmt_state_query
   int sweep_grid = 1;
+  bool swept = false;         // the tables of the grid-wide sweep are there
   uint32_t next_gen = 1;      // generations handed to the fills: two per fill, 1 .. 65534
   size_t device_bytes = 0;    // what fmt_state_create allocated
   // The device sets this host-mapped word when the state cache has no room for a new entry; the next
@@ -141,8 +142,8 @@ static cudaError_t next_generations(fmt_state* s, cudaStream_t st) {
   StateDev& d = s->dev;
   cudaError_t e = cudaSuccess;
   if (s->next_gen + 1u > 65534u) {
-    e = cudaMemsetAsync(d.au.hash, 0, (size_t)d.B * (d.au.hash_mask + 1u) * 4, st);
-    if (e == cudaSuccess) e = cudaMemsetAsync(d.au.req, 0, (size_t)d.au.req_cap * 8, st);
+    if (s->swept) e = cudaMemsetAsync(d.au.hash, 0, (size_t)d.B * (d.au.hash_mask + 1u) * 4, st);
+    if (e == cudaSuccess && s->swept) e = cudaMemsetAsync(d.au.req, 0, (size_t)d.au.req_cap * 8, st);
     if (e == cudaSuccess && d.rt.on) e = cudaMemsetAsync(d.cx.ctab, 0, (size_t)d.B * CT_SLOTS * 8, st);
     if (e == cudaSuccess && d.rt.on) e = cudaMemsetAsync(d.cx.req2, 0, (size_t)d.cx.req2_cap * 16, st);
     s->next_gen = 1;
@@ -183,6 +184,7 @@ fmt_status fmt_compile(const char* ebnf, size_t ebnf_len, const char* start_rule
     build_trie(vocab_bytes ? vocab_bytes : &none, vocab_offsets, V, eos_token_id, g->host);
     if (eos_token_id >= 0 && vocab_offsets[eos_token_id + 1] != vocab_offsets[eos_token_id])
       throw CompileError{FMT_ERR_INVALID_ARG, "the EOS token must have no bytes"};
+    if (!(opt && opt->host_only)) build_grammar_automaton(g->host);
   } catch (const CompileError& e) {
     delete g;
     return fail((fmt_status)e.code, e.msg);
@@ -238,6 +240,19 @@ fmt_status fmt_compile(const char* ebnf, size_t ebnf_len, const char* start_rule
     UP(child_off);
     UP(tok_off);
     UP(tok_ids);
+    if (h.ga_on) {
+      d.ga_on = 1, d.ga_acc_mask = h.ga_acc_mask;
+      UP(ga_root);
+      UP(ga_trans);
+      UP(ga_acc);
+      UP(ga_node);
+      UP(ga_tok);
+      d.ga_lvl2 = h.ga_lvl2, d.ga_lvl3 = h.ga_lvl3;
+      UP(ga_wide);
+      UP(ga_wide_rec);
+      UP(ga_wide_mask);
+      UP(ga_wide_exit);
+    }
     UP(vocab_off);
     UP(vocab_bytes);
 #undef UP
@@ -354,6 +369,35 @@ fmt_status fmt_grammar_copy_table(const fmt_grammar* g, int which, void* out, si
   return FMT_OK;
 }
 
+// The tables of the grid-wide sweep; its capacities (au.cap, au.rec_words, au.hash_mask, au.items_cap) are set.
+static cudaError_t alloc_sweep(fmt_state* s) {
+  StateDev& d = s->dev;
+  AutoDev& au = d.au;
+  const GrammarDev& G = s->g->dev;
+  sweep_layout(G, &au.smem_bytes, &au.tables_in_smem);
+  int per_sm = 0, sms = 0, dev = 0;
+  cudaError_t e = sweep_blocks_per_sm(&per_sm, au.smem_bytes);
+  if (e == cudaSuccess) e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (e == cudaSuccess && per_sm < 1) e = cudaErrorInvalidConfiguration;  // the sweep kernel does not fit on this device
+  s->sweep_grid = std::max(1, per_sm * sms);
+  const size_t big_words = (size_t)s->sweep_grid * sweep_warps() * ((size_t)d.big_arena_items + d.big_hset_slots);
+  au.st_stride = (G.T + 63u) & ~63u;
+  au.req_cap = 1u << 20;
+#define AL(ptr, count, fill) if (e == cudaSuccess) e = s->bufs.alloc((size_t)(count), &(ptr), (fill))
+  AL(d.big_scratch, big_words, 0xFF);
+  AL(au.recs, (size_t)d.B * au.cap * au.rec_words, 0);
+  AL(au.hash, (size_t)d.B * (au.hash_mask + 1u), 0);
+  AL(au.items, au.items_cap, 0);
+  AL(au.n_states, d.B, 0);
+  AL(au.st, (size_t)d.B * au.st_stride, 0xFF);
+  AL(au.req, au.req_cap, 0);
+  AL(au.job_info, d.B, 0);
+#undef AL
+  if (e == cudaSuccess) s->swept = true;
+  return e;
+}
+
 fmt_status fmt_state_create(const fmt_grammar* g, uint32_t batch, const fmt_state_options* opt, void* stream,
                             fmt_state** out) {
   if (!out) return fail(FMT_ERR_INVALID_ARG, "out is NULL");
@@ -416,18 +460,19 @@ fmt_status fmt_state_create(const fmt_grammar* g, uint32_t batch, const fmt_stat
   rt.tr_cap = 256u << 20;
   rt.pend_cap = 4096;
 
-  sweep_layout(g->dev, &au.smem_bytes, &au.tables_in_smem);
   cudaError_t e = configure_kernels();
-  int per_sm = 0, sms = 0, dev = 0;
-  if (e == cudaSuccess) e = sweep_blocks_per_sm(&per_sm, au.smem_bytes);
+  int sms = 0, dev = 0;
   if (e == cudaSuccess) e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  if (e == cudaSuccess && per_sm < 1) {
-    delete s;
-    return fail(FMT_ERR_CUDA, "the sweep kernel does not fit on this device");
+  // Rows are filled by the grammar's automaton if it has one.  A state that asks for the cache of
+  // context-independent entries, limits the sets of a sweep or the polls of a wait is swept by the grid.
+  AutoFillDev& af = d.af;
+  af.on = (g->dev.ga_on && !rt.on && !(opt && opt->sweep_states) && !d.poll_limit_shift) ? 1u : 0u;
+  if (af.on) {
+    af.stack_cap = 128u << 10;
+    af.ctx_cap = 4096, af.pool_cap = 64u << 10, af.big_cap = 64u << 10;
+    automaton_fill_layout(g->dev, batch, 2u * (uint32_t)std::max(1, sms), af);
   }
-  s->sweep_grid = std::max(1, per_sm * sms);
-  const size_t big_words = (size_t)s->sweep_grid * sweep_warps() * ((size_t)d.big_arena_items + d.big_hset_slots);
 #define AL(ptr, count, fill) if (e == cudaSuccess) e = s->bufs.alloc((size_t)(count), &(ptr), (fill))
   AL(d.arena, d.pool_base + d.pool_words * (two_gens ? 2 : 1), 0);
   AL(d.row_chart, batch, 0);
@@ -454,16 +499,12 @@ fmt_status fmt_state_create(const fmt_grammar* g, uint32_t batch, const fmt_stat
   AL(d.tr_val, trn, 0x80);
   AL(d.jobs, batch, 0);
   AL(d.counters, CNT_TOTAL, 0);
-  AL(d.big_scratch, big_words, 0xFF);
-  AL(au.recs, (size_t)batch * au.cap * au.rec_words, 0);
-  AL(au.hash, (size_t)batch * hs, 0);
-  AL(au.items, au.items_cap, 0);
-  AL(au.n_states, batch, 0);
-  au.st_stride = (g->dev.T + 63u) & ~63u;
-  AL(au.st, (size_t)batch * au.st_stride, 0xFF);
-  au.req_cap = 1u << 20;
-  AL(au.req, au.req_cap, 0);
-  AL(au.job_info, batch, 0);
+  if (af.on) {
+    AL(af.stack, (size_t)af.grid * af.stack_cap, 0);
+    AL(af.scratch, (size_t)af.grid * af.scratch_words, 0);
+  } else if (e == cudaSuccess) {
+    e = alloc_sweep(s);
+  }
   AL(rt.n_roots, 4, 0);
   AL(rt.tops, TOP_N, 0);
   AL(rt.counters, CNT_TOTAL, 0);
@@ -682,6 +723,14 @@ fmt_status fmt_state_ci_cache_clear(fmt_state* s, void* stream) {
 
 fmt_status fmt_state_set_wait_limit(fmt_state* s, uint32_t log2_polls) {
   if (!s) return fail(FMT_ERR_INVALID_ARG, "NULL state");
+  // (the fill by the grammar's automaton has no waits: with a limit the rows are swept by the grid, whose waits it bounds)
+  if (log2_polls && !s->swept) {
+    cudaError_t e = alloc_sweep(s);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(nullptr);  // (the tables are cleared there)
+    if (e != cudaSuccess) return cuda_fail(e, "fmt_state_set_wait_limit");
+    s->device_bytes = s->bufs.bytes;
+  }
+  s->dev.af.on = s->dev.af.stack && !log2_polls ? 1u : 0u;
   s->dev.poll_limit_shift = std::min(log2_polls, 30u);
   return FMT_OK;
 }

@@ -1006,7 +1006,8 @@ void launch_fill(const GrammarDev& G, const StateDev& S, int sweep_grid, cudaStr
   if (!S.rt.on) {
     // without the cache of context-independent entries every row is swept from its chart's last set
     if (before_sweep) cudaEventRecord(before_sweep, st);
-    launch_sweep(G, S, sweep_grid, st);
+    if (S.af.on) launch_automaton_fill(G, S, st);
+    else launch_sweep(G, S, sweep_grid, st);
     if (after_sweep) cudaEventRecord(after_sweep, st);
     launch_publish(S, st);
     return;

@@ -35,6 +35,18 @@ struct GrammarDev {
   const uint32_t* child_off;     // [T+1] children of node n are nodes child_off[n] .. child_off[n+1]-1
   const uint32_t* tok_off;       // [T+1] tokens whose bytes end at node n (duplicates included)
   const uint32_t* tok_ids;
+  // the grammar automaton over the vocabulary (see host_tables.h), if the grammar has one
+  uint32_t ga_on, ga_acc_mask;
+  const uint32_t* ga_root;       // [D]
+  const uint32_t* ga_trans;      // [sets][n_eq]
+  const uint32_t* ga_acc;        // [ga_acc_mask + 1][2]
+  const uint32_t* ga_node;       // [nodes][4]
+  const uint32_t* ga_tok;
+  uint32_t ga_lvl2, ga_lvl3;
+  const uint32_t* ga_wide;       // [D]
+  const uint32_t* ga_wide_rec;   // [entries][4]
+  const uint32_t* ga_wide_mask;  // [entries][Wm]
+  const uint32_t* ga_wide_exit;  // [][2]
   const uint32_t* vocab_off;     // [V+1]
   const uint8_t* vocab_bytes;
 };
@@ -232,6 +244,19 @@ struct CtxDev {
   uint32_t req2_cap;
 };
 
+// What the fill by the grammar automaton needs (automaton_fill.cu): per thread block a stack of threads and the
+// contexts of the row it works on.
+struct AutoFillDev {
+  uint32_t on;               // rows are filled by the automaton
+  uint32_t grid, parts;      // thread blocks, and how many of them share a row (a cluster)
+  uint32_t smem_bytes;
+  uint4* stack;              // [grid][stack_cap] first child, children, code, context
+  uint32_t stack_cap;
+  uint32_t* scratch;         // [grid][scratch_words]
+  uint32_t scratch_words;
+  uint32_t ctx_cap, pool_cap, big_cap;  // contexts per row, words for their lists, items of the largest expansion (powers of two)
+};
+
 struct StateDev {
   uint32_t B;
   uint32_t ctx_mode;          // 1: this is the view of a root sweep (see RootDev)
@@ -267,7 +292,8 @@ struct StateDev {
   uint32_t* counters;         // [CNT_TOTAL]
   uint32_t* big_scratch;      // per-warp large scratch areas of the trie walk
   uint32_t big_arena_items, big_hset_slots;
-  AutoDev au;
+  AutoFillDev af;
+  AutoDev au;   // the grid-wide sweep: of entries of the context-independent cache, and of rows whose grammar has no automaton
   RootDev rt;
   CtxDev cx;
 };

@@ -1,0 +1,417 @@
+// The grammar automaton: what a token's bytes do to ONE unfinished Earley item, worked out at compile time.
+//
+// Earley's steps are linear in the kernel of a set (its scanned and completed items): the sets reached from a kernel
+// by some bytes are the unions of what is reached from its items taken one by one.  From one item (d, o) - dotted rule d,
+// begun in set o - everything that happens inside a token depends on d alone, except where the rule of d is completed
+// and o has to be asked who waited for it.  So the sets reached from {(d, here)} along byte strings, with the origin o left
+// open, can be hash-consed and their transitions tabulated once for a grammar and a vocabulary (Section 4.3 of the paper
+// keeps a context-independent part of the masks in the same spirit); a fill then walks the vocabulary trie by table look-ups
+// and runs Earley completions only where a rule of the chart ends (automaton_fill.cu).
+//
+// Which transitions are needed follows from the vocabulary: the trie is walked once with the codes of all items that a
+// kernel can hold, and where a rule of non-terminal A ends inside a token the walk goes on, from that node, with every item that
+// completing A can yield in any chart of the grammar.
+#include <algorithm>
+#include <cstring>
+#include <unordered_map>
+#include <utility>
+
+#include "host_tables.h"
+
+namespace fmt {
+namespace {
+
+using u32 = uint32_t;
+using u64 = uint64_t;
+
+// limits; a grammar beyond them has no automaton and its fills run the Earley steps themselves
+constexpr u32 GA_MAX_SETS = 1u << 18;
+constexpr u64 GA_MAX_TRANS = 32u << 20;   // table entries (4 bytes each)
+constexpr u64 GA_MAX_WALK = 60u << 20;    // look-ups of the walk over the trie (about half a second)
+constexpr size_t GA_MAX_WIDE = 32u << 20;  // words of the masks and lists of wide items
+constexpr size_t GA_WIDE_NODES = 1024;    // an item is wide from so many trie nodes on
+constexpr size_t GA_MAX_ITEMS = 1024;     // items of one set, predicted ones included: alternations of thousands of literals
+                                          // would be scanned again for every set that predicts them
+
+struct VecHash {
+  size_t operator()(const std::vector<u64>& v) const {
+    u64 h = 0x9E3779B97F4A7C15ull;
+    for (u64 x : v) {
+      h = (h ^ x) * 0xD6E8FEB86659FD93ull;
+      h ^= h >> 32;
+    }
+    return (size_t)h;
+  }
+};
+
+class Builder {
+ public:
+  explicit Builder(HostTables& h) : h_(h), n_eq_(h.n_eq) {
+    for (int b = 255; b >= 0; --b) rep_[h.eq_of_byte[b]] = (uint8_t)b;
+  }
+
+  bool run() {
+    roots();
+    class_trie();
+    follow();
+    std::vector<u32> first;
+    for (u32 d = 0; d < h_.D; ++d)
+      if (h_.ga_root[d] != GA_DEAD) first.push_back(h_.ga_root[d]);
+    dedupe(first, 0);
+    arena_ = first;
+    if (!too_big_) walk(0, 0, arena_.size());
+    if (too_big_) return false;
+    wide_roots();
+    finish_tables();
+    return true;
+  }
+
+ private:
+  struct Set {
+    std::vector<u64> kernel;                  // origin << 32 | dotted rule; origin 0 = open, u + 1 = set u
+    std::vector<u64> scan;                    // kernel and predicted items before a terminal or inside an automaton
+    std::vector<std::pair<u32, u64>> wait;    // post-dot non-terminal -> the item with the dot moved over it
+    u32 lhs = 0;                              // whose rule the open origin belongs to
+    bool expanded = false;
+  };
+
+  HostTables& h_;
+  const u32 n_eq_;
+  uint8_t rep_[256];
+  std::vector<Set> sets_;
+  std::unordered_map<std::vector<u64>, u32, VecHash> ids_;
+  std::vector<u32> trans_;
+  std::unordered_map<u32, u32> accept_;
+  std::vector<u64> cur_;
+  std::vector<u32> arena_;
+  std::vector<std::vector<u32>> follow_;      // per non-terminal: codes of the items that completing it can yield
+  u64 walked_ = 0;
+  bool too_big_ = false;
+
+  const u32* node(u32 n) const { return &h_.ga_node[(size_t)n * 4]; }
+  u32 kind(u32 d) const { return h_.info[d] >> INFO_KIND_SHIFT; }
+  u32 arg(u32 d) const { return h_.info[d] & INFO_ARG_MASK; }
+
+  u32 lhs_of(u32 code) const {
+    if (!(code & GA_ITEM)) return sets_[code].lhs;
+    const u32 org = (code >> 14) & 0xFFFFu;
+    return org ? sets_[org - 1].lhs : h_.lhs[h_.dfa_first + (code & 0x3FFFu)];
+  }
+
+  // The code of the set with this kernel (ascending).  A kernel of one item inside an automaton is its own code.
+  u32 intern(std::vector<u64>& k) {
+    if (k.empty()) return GA_NONE;
+    const u64 org = k[0] >> 32;
+    if (k.size() == 1 && kind((u32)k[0]) == KIND_DFA && org < 0xFFFFu)
+      return GA_ITEM | (u32)(org << 14) | arg((u32)k[0]);
+    const auto it = ids_.find(k);
+    if (it != ids_.end()) return it->second;
+    const u32 id = (u32)sets_.size();
+    if (id + 1 >= GA_MAX_SETS || (u64)(id + 1) * n_eq_ > GA_MAX_TRANS) {
+      too_big_ = true;
+      return GA_NONE;
+    }
+    ids_.emplace(k, id);
+    sets_.emplace_back();
+    sets_[id].kernel = k;
+    sets_[id].lhs = org ? sets_[org - 1].lhs : h_.lhs[(u32)k[0]];
+    trans_.resize((size_t)(id + 1) * n_eq_, GA_UNKNOWN);
+    return id;
+  }
+
+  void expand(u32 s) {
+    if (sets_[s].expanded) return;
+    Set& set = sets_[s];
+    set.expanded = true;
+    std::vector<u32> nts(h_.Nw, 0u);
+    auto put = [&](u64 it) {
+      const u32 d = (u32)it;
+      if (kind(d) == KIND_NT) set.wait.push_back({arg(d), it + 1});
+      else if (kind(d) != KIND_END) set.scan.push_back(it);
+    };
+    for (u64 it : set.kernel) {
+      put(it);
+      if (kind((u32)it) == KIND_NT)
+        for (u32 w = 0; w < h_.Nw; ++w) nts[w] |= h_.nt_closure[(size_t)arg((u32)it) * h_.Nw + w];
+    }
+    for (u32 w = 0; w < h_.Nw; ++w)
+      for (u32 bits = nts[w]; bits; bits &= bits - 1) {
+        const u32 z = w * 32 + (u32)__builtin_ctz(bits);
+        for (u32 k = h_.direct_off[z]; k < h_.direct_off[z + 1]; ++k) put((u64)(s + 1) << 32 | h_.direct_items[k]);
+      }
+    std::sort(set.wait.begin(), set.wait.end());
+    if (set.scan.size() + set.wait.size() > GA_MAX_ITEMS) too_big_ = true;
+  }
+
+  void add(u64 it) {
+    for (u32 j = 0; j <= h_.skip[(u32)it]; ++j)
+      if (std::find(cur_.begin(), cur_.end(), it + j) == cur_.end()) cur_.push_back(it + j);
+  }
+
+  // Complete (Section 3.2) over cur_, then the set's code; GA_EXIT when the open origin has to be asked.
+  u32 complete() {
+    if (cur_.empty()) return GA_DEAD;
+    bool exits = false;
+    std::vector<u64> k;
+    for (size_t i = 0; i < cur_.size() && !too_big_; ++i) {
+      const u64 it = cur_[i];
+      if (kind((u32)it) != KIND_END) {
+        k.push_back(it);
+        continue;
+      }
+      const u32 org = (u32)(it >> 32);
+      if (org == 0) {
+        exits = true;
+        continue;
+      }
+      expand(org - 1);
+      const auto& w = sets_[org - 1].wait;
+      for (auto lo = std::lower_bound(w.begin(), w.end(), std::make_pair(arg((u32)it), (u64)0)); lo != w.end() && lo->first == arg((u32)it); ++lo)
+        add(lo->second);
+    }
+    std::sort(k.begin(), k.end());
+    return intern(k) | (exits ? GA_EXIT : 0u);
+  }
+
+  u32 next(u32 code, u32 e) {
+    ++walked_;
+    if (code & GA_ITEM) {
+      const u32 org = (code >> 14) & 0xFFFFu, g = code & 0x3FFFu;
+      const u32 t = h_.dfa_trans[(size_t)g * n_eq_ + e];
+      if (t == 0xFFFFu || !(t & 0xC000u)) return GA_DEAD;
+      if (!(t & 0x8000u)) return GA_ITEM | (org << 14) | (t & 0x3FFFu);
+      if (org == 0) return GA_EXIT | ((t & 0x4000u) ? (GA_ITEM | (t & 0x3FFFu)) : GA_NONE);
+      const u32 key = org << 16 | t;
+      const auto it = accept_.find(key);
+      if (it != accept_.end()) return it->second;
+      cur_.clear();
+      if (t & 0x4000u) cur_.push_back((u64)org << 32 | (h_.dfa_first + (t & 0x3FFFu)));
+      cur_.push_back((u64)org << 32 | h_.dfa_done[t & 0x3FFFu]);
+      const u32 r = complete();
+      accept_.emplace(key, r);
+      return r;
+    }
+    const size_t slot = (size_t)code * n_eq_ + e;
+    if (trans_[slot] != GA_UNKNOWN) return trans_[slot];
+    expand(code);
+    cur_.clear();
+    const u32 b = rep_[e];
+    for (u64 it : sets_[code].scan) {
+      const u32 d = (u32)it, a = arg(d);
+      if (kind(d) == KIND_TERM) {
+        if ((h_.class_bits[(size_t)a * 8 + (b >> 5)] >> (b & 31)) & 1u) add(it + 1);
+      } else {
+        const u32 t = h_.dfa_trans[(size_t)a * n_eq_ + e];
+        if (t == 0xFFFFu) continue;
+        if (t & 0x4000u) add((it & ~0xFFFFFFFFull) | (h_.dfa_first + (t & 0x3FFFu)));
+        if (t & 0x8000u) add((it & ~0xFFFFFFFFull) | h_.dfa_done[a]);
+      }
+    }
+    const u32 r = complete();
+    trans_[slot] = r;
+    return r;
+  }
+
+  // ga_root[d]: the code of the kernel {(d, open)}, nullable non-terminals skipped, for every item a kernel can hold
+  void roots() {
+    h_.ga_root.assign(h_.D, GA_DEAD);
+    for (u32 d = 0; d < h_.D && !too_big_; ++d) {
+      if (kind(d) == KIND_END) continue;
+      if (kind(d) == KIND_DFA) {
+        h_.ga_root[d] = GA_ITEM | arg(d);
+        continue;
+      }
+      const bool begins_rule = d != ITEM_START && (kind(d - 1) == KIND_END || d == 0);
+      if (begins_rule) continue;
+      std::vector<u64> k;
+      for (u32 j = 0; j <= h_.skip[d]; ++j)
+        if (kind(d + j) != KIND_END) k.push_back(d + j);
+      h_.ga_root[d] = intern(k);
+    }
+  }
+
+  // follow_[A]: what completing A yields, whoever waits for it
+  void follow() {
+    const u32 N = h_.N;
+    std::vector<std::vector<u32>> up(N);  // A -> non-terminals completed with it (its rule may end right after A)
+    std::vector<std::vector<u32>> own(N);
+    for (u32 d = 0; d < h_.D; ++d) {
+      if (kind(d) != KIND_NT) continue;
+      const u32 a = arg(d), skip = h_.skip[d + 1];
+      if (kind(d + 1) != KIND_END) own[a].push_back(h_.ga_root[d + 1]);
+      if (kind(d + 1 + skip) == KIND_END) up[a].push_back(h_.lhs[d]);
+    }
+    follow_.assign(N, {});
+    for (u32 a = 0; a < N; ++a) {
+      std::vector<char> seen(N, 0);
+      std::vector<u32> work{a};
+      seen[a] = 1;
+      while (!work.empty()) {
+        const u32 x = work.back();
+        work.pop_back();
+        follow_[a].insert(follow_[a].end(), own[x].begin(), own[x].end());
+        for (u32 y : up[x])
+          if (!seen[y]) seen[y] = 1, work.push_back(y);
+      }
+      dedupe(follow_[a], 0);
+    }
+  }
+
+  static void dedupe(std::vector<u32>& v, size_t from) {
+    std::sort(v.begin() + from, v.end());
+    v.erase(std::unique(v.begin() + from, v.end()), v.end());
+  }
+
+  // The vocabulary trie over byte classes: bytes that no terminal tells apart share a node.  Nodes are numbered breadth
+  // first, so the children of a node are consecutive; the tokens that end at a node are listed together.
+  void class_trie() {
+    std::vector<u32> node(h_.T, 0);  // byte trie -> preliminary number
+    size_t cap = 1024;
+    while (cap < (size_t)h_.T * 2) cap <<= 1;
+    std::vector<u64> key(cap, 0);
+    std::vector<u32> val(cap), child(1, 0), sibling(1, 0);
+    std::vector<uint8_t> eq(1, 0);
+    for (u32 v = 1; v < h_.T; ++v) {
+      const u32 p = node[h_.parent[v]], e = h_.eq_of_byte[h_.node_byte[v]];
+      const u64 k = ((u64)p << 8 | e) + 1;
+      size_t s = (size_t)(k * 0x9E3779B97F4A7C15ull >> 32) & (cap - 1);
+      while (key[s] && key[s] != k) s = (s + 1) & (cap - 1);
+      if (!key[s]) {
+        key[s] = k, val[s] = (u32)eq.size();
+        eq.push_back((uint8_t)e), child.push_back(0), sibling.push_back(child[p]);
+        child[p] = val[s];
+      }
+      node[v] = val[s];
+    }
+    const u32 n = (u32)eq.size();
+    std::vector<u32> order(1, 0), number(n, 0), depth(1, 0);
+    order.reserve(n);
+    h_.ga_node.assign((size_t)n * 4, 0u);
+    h_.ga_lvl2 = h_.ga_lvl3 = n;
+    for (u32 i = 0; i < (u32)order.size(); ++i) {
+      u32* r = &h_.ga_node[(size_t)i * 4];
+      r[0] = (u32)order.size();
+      u32 kids = 0;
+      for (u32 c = child[order[i]]; c; c = sibling[c], ++kids) number[c] = (u32)order.size(), order.push_back(c), depth.push_back(depth[i] + 1);
+      r[1] = kids << 8 | eq[order[i]];
+      if (depth[i] == 2) h_.ga_lvl2 = std::min(h_.ga_lvl2, i);
+      if (depth[i] == 3) h_.ga_lvl3 = std::min(h_.ga_lvl3, i);
+    }
+    std::vector<u32> count(n + 1, 0);  // tokens by node
+    for (u32 v = 0; v < h_.T; ++v) count[number[node[v]] + 1] += h_.tok_off[v + 1] - h_.tok_off[v];
+    for (u32 i = 0; i < n; ++i) count[i + 1] += count[i];
+    h_.ga_tok.assign(std::max<u32>(count[n], 1), 0);
+    std::vector<u32> at(count.begin(), count.end() - 1);
+    for (u32 v = 0; v < h_.T; ++v)
+      for (u32 k = h_.tok_off[v]; k < h_.tok_off[v + 1]; ++k) h_.ga_tok[at[number[node[v]]]++] = h_.tok_ids[k];
+    for (u32 i = 0; i < n; ++i) {  // a single token is named in the node itself
+      u32* r = &h_.ga_node[(size_t)i * 4];
+      r[3] = count[i + 1] - count[i];
+      r[2] = r[3] == 1 ? h_.ga_tok[count[i]] : count[i];
+    }
+  }
+
+  // All children of trie node v with the codes arena_[lo, hi) at v.
+  void walk(u32 v, size_t lo, size_t hi) {
+    const u32 first = node(v)[0], end = first + (node(v)[1] >> 8);
+    for (u32 c = first; c < end && !too_big_; ++c) {
+      const size_t base = arena_.size();
+      const u32 e = node(c)[1] & 0xFFu, kids = node(c)[1] >> 8;
+      for (size_t i = lo; i < hi; ++i) {
+        const u32 code = arena_[i], r = next(code, e);
+        if (r == GA_DEAD || kids == 0) continue;
+        if ((r & ~GA_EXIT) != GA_NONE) arena_.push_back(r & ~GA_EXIT);
+        if (r & GA_EXIT) {
+          const auto& f = follow_[lhs_of(code)];
+          arena_.insert(arena_.end(), f.begin(), f.end());
+        }
+      }
+      if (walked_ > GA_MAX_WALK) too_big_ = true;
+      dedupe(arena_, base);
+      if (arena_.size() > base) walk(c, base, arena_.size());
+      arena_.resize(base);
+    }
+  }
+
+  // Items from which a large part of the vocabulary can follow (inside a string, mostly): the tokens that are valid whatever
+  // the chart holds, and the nodes where the chart has to be asked, are kept as a mask and a list.
+  void wide_roots() {
+    h_.ga_wide.assign(h_.D, GA_DEAD);
+    h_.ga_wide_rec.clear(), h_.ga_wide_mask.clear(), h_.ga_wide_exit.clear();
+    walked_ = 0;
+    std::unordered_map<u32, u32> known;  // items with one code share an entry
+    std::vector<u32> alive, mask(h_.Wm);
+    std::vector<std::pair<u32, u32>> work;  // (node, code)
+    std::vector<u32> exits;
+    for (u32 d = 0; d < h_.D; ++d) {
+      if (h_.ga_root[d] == GA_DEAD) continue;
+      const auto it = known.find(h_.ga_root[d]);
+      if (it != known.end()) {
+        h_.ga_wide[d] = it->second;
+        continue;
+      }
+      if (walked_ > GA_MAX_WALK || h_.ga_wide_mask.size() + h_.ga_wide_exit.size() > GA_MAX_WIDE) break;
+      alive.clear(), exits.clear();
+      work.assign(1, {0u, h_.ga_root[d]});
+      while (!work.empty()) {
+        const auto [v, code] = work.back();
+        work.pop_back();
+        const u32 first = node(v)[0], end = first + (node(v)[1] >> 8);
+        for (u32 c = first; c < end; ++c) {
+          const u32 r = next(code, node(c)[1] & 0xFFu);
+          if (r == GA_DEAD) continue;
+          alive.push_back(c);
+          if ((node(c)[1] >> 8) == 0u) continue;
+          if ((r & ~GA_EXIT) != GA_NONE) work.push_back({c, r & ~GA_EXIT});
+          if (r & GA_EXIT) exits.push_back(c);
+        }
+      }
+      u32 id = GA_DEAD;
+      if (alive.size() >= GA_WIDE_NODES) {
+        id = (u32)h_.ga_wide_rec.size() / 4;
+        std::sort(exits.begin(), exits.end());
+        h_.ga_wide_rec.insert(h_.ga_wide_rec.end(), {id, (u32)h_.ga_wide_exit.size() / 2, (u32)exits.size(), 0u});
+        std::fill(mask.begin(), mask.end(), 0u);
+        for (u32 c : alive) {
+          if (node(c)[3] == 1) mask[node(c)[2] >> 5] |= 1u << (node(c)[2] & 31);
+          else
+            for (u32 k = 0; k < node(c)[3]; ++k) mask[h_.ga_tok[node(c)[2] + k] >> 5] |= 1u << (h_.ga_tok[node(c)[2] + k] & 31);
+        }
+        h_.ga_wide_mask.insert(h_.ga_wide_mask.end(), mask.begin(), mask.end());
+        for (u32 c : exits) h_.ga_wide_exit.push_back(node(c)[0]), h_.ga_wide_exit.push_back(node(c)[1] >> 8);
+      }
+      h_.ga_wide[d] = id;
+      known.emplace(h_.ga_root[d], id);
+    }
+  }
+
+  void finish_tables() {
+    h_.ga_sets = (u32)sets_.size();
+    if (trans_.empty()) trans_.push_back(GA_UNKNOWN);
+    h_.ga_trans.swap(trans_);
+    u32 cap = 16;
+    while (cap < accept_.size() * 4) cap <<= 1;
+    h_.ga_acc_mask = cap - 1;
+    h_.ga_acc.assign((size_t)cap * 2, 0u);
+    for (const auto& kv : accept_) {
+      u32 s = ga_hash(kv.first) & h_.ga_acc_mask;
+      while (h_.ga_acc[2 * s]) s = (s + 1) & h_.ga_acc_mask;
+      h_.ga_acc[2 * s] = kv.first, h_.ga_acc[2 * s + 1] = kv.second;
+    }
+  }
+};
+
+}  // namespace
+
+void build_grammar_automaton(HostTables& h) {
+  h.ga_on = false;
+  if (h.D > 65535 || h.T >= (1u << 24)) return;
+  Builder b(h);
+  h.ga_on = b.run();
+  if (!h.ga_on) {
+    h.ga_root.clear();
+    h.ga_sets = 0;
+  }
+}
+
+}  // namespace fmt

@@ -23,6 +23,20 @@ constexpr uint32_t ITEM_ACCEPT = 1;  // $ -> start .
 constexpr uint32_t MAX_TOKEN_BYTES = 32;
 constexpr uint32_t MAX_NONTERMINALS = 4096;
 
+// Codes of the grammar automaton: the number of a set, or GA_ITEM | (set + 1, or 0 for the open origin) << 14 | state
+// for a kernel that is one item inside an automaton of a regular non-terminal; with GA_EXIT where a rule begun in the open
+// origin is completed.  GA_NONE: nothing is left but completed items.
+constexpr uint32_t GA_DEAD = 0xFFFFFFFFu, GA_UNKNOWN = 0xFFFFFFFEu, GA_ITEM = 1u << 31, GA_EXIT = 1u << 30, GA_NONE = GA_EXIT - 1u;
+#ifdef __CUDACC__
+__host__ __device__
+#endif
+inline uint32_t ga_hash(uint32_t key) {
+  key ^= key >> 15;
+  key *= 0x2C1B3C6Du;
+  key ^= key >> 12;
+  return key;
+}
+
 struct CompileError {
   int code;
   std::string msg;
@@ -65,6 +79,21 @@ struct HostTables {
   std::vector<uint32_t> tok_ids;
   std::vector<uint32_t> lvl_off;    // [depth+2] nodes of depth L are lvl_off[L]..lvl_off[L+1]-1
   std::vector<uint32_t> tok_node;   // [V] node where the token's bytes end, 0xFFFFFFFF for empty tokens
+  // ---- the grammar automaton over this vocabulary (grammar_automaton.cpp), if it stays within its limits
+  bool ga_on = false;
+  uint32_t ga_sets = 0, ga_acc_mask = 0;
+  std::vector<uint32_t> ga_root;   // [D] code of the kernel {(d, open)}
+  std::vector<uint32_t> ga_trans;  // [ga_sets][n_eq] code
+  std::vector<uint32_t> ga_acc;    // [ga_acc_mask + 1][2] hash: set + 1 << 16 | automaton transition -> code
+  // the vocabulary trie over byte classes, breadth first
+  std::vector<uint32_t> ga_node;   // [nodes][4] first child, children << 8 | byte class, the token (or where in ga_tok they begin), tokens
+  std::vector<uint32_t> ga_tok;    // token ids by node
+  uint32_t ga_lvl2 = 0, ga_lvl3 = 0;  // first nodes of depth 2 and 3
+  // wide items: what follows from them alone
+  std::vector<uint32_t> ga_wide;       // [D] entry or GA_DEAD
+  std::vector<uint32_t> ga_wide_rec;   // [entries][4] mask row, first exit, exits
+  std::vector<uint32_t> ga_wide_mask;  // [entries][Wm] tokens that are valid whatever the chart holds
+  std::vector<uint32_t> ga_wide_exit;  // [][2] nodes (first child, children) at which the item's rule ends
   std::vector<uint32_t> vocab_off;  // [V+1] byte offsets (32-bit) into vocab_bytes
   std::vector<uint8_t> vocab_bytes;
 };
@@ -74,6 +103,8 @@ std::string json_schema_to_ebnf(const char* schema, size_t len);
 
 // Both throw CompileError.
 void compile_grammar(const char* text, size_t len, const std::string& start, HostTables& out, bool dfa_terminals = true);
+// After the two above: the automaton of the grammar over the vocabulary; h.ga_on says whether there is one.
+void build_grammar_automaton(HostTables& h);
 void build_trie(const uint8_t* bytes, const uint64_t* offs, uint32_t V, int32_t eos, HostTables& out);
 
 }  // namespace fmt

@@ -996,6 +996,7 @@ cudaError_t configure_kernels() {
   if ((e = opt_in_smem((const void*)advance_kernel, (size_t)ADV_WARPS * ADV_WARP_WORDS * 4 + HOT_TABLE_BYTES)) != cudaSuccess) return e;
   if ((e = opt_in_smem((const void*)forced_kernel, (size_t)ADV_WARPS * ADV_WARP_WORDS * 4 + HOT_TABLE_BYTES)) != cudaSuccess) return e;
   if ((e = opt_in_smem((const void*)sweep_kernel, SWEEP_SMEM_LIMIT)) != cudaSuccess) return e;
+  if ((e = configure_automaton_fill()) != cudaSuccess) return e;
   return configure_walk_kernels();
 }
 

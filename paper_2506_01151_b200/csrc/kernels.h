@@ -13,6 +13,11 @@ cudaError_t sweep_blocks_per_sm(int* out, uint32_t smem_bytes);
 void sweep_layout(const GrammarDev& G, uint32_t* smem_bytes, uint32_t* tables_in_smem);
 int sweep_warps();
 
+// the fill by the grammar automaton (automaton_fill.cu); the layout sets what follows from the grammar and the capacities in A
+void automaton_fill_layout(const GrammarDev& G, uint32_t rows, uint32_t max_blocks, AutoFillDev& A);
+cudaError_t configure_automaton_fill();
+void launch_automaton_fill(const GrammarDev& G, const StateDev& S, cudaStream_t st);
+
 void launch_init(const GrammarDev& G, const StateDev& S, int32_t* result_dev, cudaStream_t st);
 void launch_intern_init(const StateDev& S, int32_t* init_state_dev, cudaStream_t st);
 void launch_reset(const StateDev& S, const uint32_t* rows_dev, uint32_t n, const int32_t* init_state_dev, cudaStream_t st);

@@ -48,6 +48,12 @@ constexpr size_t NA_ST_ENTRIES = 8u << 20;
 constexpr size_t NA_OFF_ST = NA_OFF_ITEMS + NA_ITEM_WORDS;
 constexpr size_t NA_OFF_REQ = NA_OFF_ST + NA_ST_ENTRIES / 2;       // 8-byte aligned: all sizes above are even
 constexpr size_t NA_WORDS = NA_OFF_REQ + 2 * (size_t)NA_REQ_CAP;
+// the fill by the grammar's automaton uses the same array: per thread block a stack of threads and the contexts of a row
+constexpr uint32_t NA_FILL_BLOCKS = 64, NA_STACK = 16u << 10;
+constexpr uint32_t NA_CTX = 1024, NA_POOL = 16u << 10, NA_LARGE = 8u << 10;
+constexpr uint32_t NA_FILL_SCRATCH = 7u * NA_CTX + NA_POOL + NA_LARGE / 4u + NA_LARGE / 2u + NA_LARGE;
+constexpr size_t NA_OFF_FILL = NA_HEADER_WORDS + 4 * (size_t)NA_FILL_BLOCKS * NA_STACK;
+static_assert(NA_OFF_FILL + (size_t)NA_FILL_BLOCKS * NA_FILL_SCRATCH <= NA_WORDS, "the fill's tables do not fit");
 static_assert(CNT_TOTAL <= NA_OFF_JOBS, "the counters overlap the job list");
 static_assert(NA_OFF_JOBINFO + 4 * NA_MAX <= NA_HEADER_WORDS, "header too small");
 static_assert((NA_OFF_JOBINFO % 4) == 0, "job records must be 16-byte aligned");
@@ -83,6 +89,7 @@ __global__ void noalloc_prepare_kernel(GrammarDev G, StateDev S, uint32_t* scrat
     S.row_flags[r] = 0u;
   }
   for (size_t i = tid; i < (size_t)n * G.Wm; i += nth) mask[i] = 0u;
+  if (S.af.on) return;
   for (size_t i = tid; i < (size_t)NA_MAX * NA_HASH_SLOTS; i += nth) S.au.hash[i] = 0u;
   for (size_t i = tid; i < NA_REQ_CAP; i += nth) S.au.req[i] = 0ull;  // no stale tags: every call is generation 1
   uint32_t* big = S.big_scratch;
@@ -213,11 +220,21 @@ extern "C" fmt_status fmt_fill_mask_noalloc(const fmt_grammar* g, const uint32_t
   S.au.req_cap = NA_REQ_CAP;
   S.au.job_info = reinterpret_cast<uint4*>(scratch + NA_OFF_JOBINFO);
   sweep_layout(*G, &S.au.smem_bytes, &S.au.tables_in_smem);
+  if (G->ga_on) {
+    AutoFillDev& A = S.af;
+    A.on = 1;
+    A.stack = reinterpret_cast<uint4*>(scratch + NA_HEADER_WORDS);
+    A.stack_cap = NA_STACK;
+    A.scratch = scratch + NA_OFF_FILL;
+    A.ctx_cap = NA_CTX, A.pool_cap = NA_POOL, A.big_cap = NA_LARGE;
+    automaton_fill_layout(*G, n, NA_FILL_BLOCKS, A);
+  }
   cudaStream_t st = (cudaStream_t)stream;
   noalloc_prepare_kernel<<<256, 256, 0, st>>>(*G, S, scratch, charts_dev, off, n, mask_dev);
   noalloc_validate_kernel<<<n, 256, 0, st>>>(*G, scratch, charts_dev, off, n);
   noalloc_jobs_kernel<<<1, 32, 0, st>>>(S, scratch, n);
-  launch_sweep(*G, S, (int)NA_GRID, st);
+  if (S.af.on) launch_automaton_fill(*G, S, st);
+  else launch_sweep(*G, S, (int)NA_GRID, st);
   noalloc_finish_kernel<<<n, 128, 0, st>>>(*G, S, scratch, n, mask_dev, status_dev);
   e = cudaGetLastError();
   if (e != cudaSuccess) return fail(FMT_ERR_CUDA, cudaGetErrorString(e));

@@ -1,0 +1,106 @@
+"""The fill by the grammar's automaton (fmt_compile tabulates what a token does to one Earley item) at the sizes where it
+takes another path: rows per thread block, large vocabularies, many tokens at one trie node, long expansions, and grammars
+without an automaton.  Masks are exact: they are compared with the oracle's bit by bit."""
+import numpy as np
+import pytest
+
+import oracle
+import workloads
+
+pytestmark = pytest.mark.gpu
+
+
+def _run(text, start, vocab, prefixes, batch=None, check=None, **options):
+    """Rows with these prefixes (taken in turn up to `batch`); the masks of the rows `check` against the oracle's."""
+    import torch
+
+    import paper_2506_01151_b200 as fmt
+
+    eos = len(vocab) - 1
+    g = fmt.Grammar(text, start, vocab, eos)
+    batch = batch or len(prefixes)
+    st = fmt.State(g, batch, cache=False, **options)
+    longest = max(len(p) for p in prefixes)
+    for i in range(longest):
+        t = [prefixes[b % len(prefixes)][i] if i < len(prefixes[b % len(prefixes)]) else -1 for b in range(batch)]
+        st.advance(torch.tensor(t, dtype=torch.int32, device="cuda"))
+    mask = torch.full((batch, g.mask_words), -1, dtype=torch.int32, device="cuda")
+    st.fill_mask(mask)
+    got = mask.cpu().numpy().view(np.uint32)
+    og, ov = oracle.Grammar(text, start), oracle.Vocab(vocab, eos)
+    want = []
+    for p in prefixes:
+        s = oracle.Sequence_(og)
+        assert s.advance(bytes(p)) or not p
+        want.append(s.mask(ov))
+    for b in range(batch) if check is None else check:
+        assert np.array_equal(got[b], want[b % len(want)]), b
+    stats = st.stats()
+    assert stats["capacity_errors"] == 0 and stats["fills_aborted"] == 0
+    return stats
+
+
+JSON_PREFIXES = [list(x) for x in (b"", b'{"a": "x', b"[1, 2", b'{"k": tr', b"[[[", b'[{"a":[1.5e', b'{"a\\', b'["b", nul', b" ", b'{"q":{"r":[] ')]
+
+
+@pytest.mark.parametrize("batch", [1, 2, 19, 37, 74, 75, 148, 297, 700])
+def test_rows_of_every_share_of_the_grid(batch):
+    """One row may be shared by up to eight thread blocks, or a block may take several rows in turn."""
+    w = workloads.build(2, V=3000, batch=1, steps=1)
+    _run(w.ebnf, w.start, w.vocab, JSON_PREFIXES, batch=batch)
+
+
+@pytest.mark.parametrize("size", [258, 6144 * 32, 6144 * 32 + 1])
+def test_masks_in_and_out_of_shared_memory(size):
+    """Rows of more than 6144 mask words are collected in global memory.  Thousands of tokens end at one node of the trie over
+    byte classes (words no terminal tells apart), duplicates among them."""
+    rng = np.random.default_rng(3)
+    letters = b"ghijkmopqvwxyzGHIJ"
+    vocab = [bytes([b]) for b in range(256)]
+    while len(vocab) < size - 1:
+        n = int(rng.integers(1, 7))
+        vocab.append(bytes(letters[i] for i in rng.integers(0, len(letters), n)) + (b'"' if rng.random() < 0.1 else b""))
+    w = workloads.build(2, V=300, batch=1, steps=1)
+    _run(w.ebnf, w.start, vocab + [b""], JSON_PREFIXES, batch=12)
+
+
+@pytest.mark.parametrize("n", [1, 2, 31, 32])
+def test_tokens_up_to_the_longest(n):
+    vocab = [bytes([b]) for b in range(256)] + [b"["] * 2 + [b"[" * n, b"]" * n, (b"[]," * 11)[:n], b'"' + b"a" * (n - 1), b"a" * (n - 1) + b'"', b""]
+    w = workloads.build(2, V=300, batch=1, steps=1)
+    prefixes = [b"", b"[" * 5, b"[" * 40, b'["', b"[[1"]
+    _run(w.ebnf, w.start, vocab, [list(p) for p in prefixes])
+
+
+@pytest.mark.parametrize("n", [4, 60, 150])
+def test_contexts_of_many_origins(n):
+    """In an ambiguous grammar the rules that may end inside a token were begun in as many sets as there are letters; from some
+    fifty on an expansion leaves shared memory."""
+    text = 's ::= "<" e ">"\ne ::= e e | e "+" e | "(" e ")" | "a" | "b"'
+    vocab = [bytes([b]) for b in range(256)] + [b"ab", b"a+b", b"a>", b"b)", b")+", b"ab+a(b)a>", b"+a>", b">a", b"(((a", b""]
+    rng = np.random.default_rng(n)
+    prefix = b"<" + bytes(b"ab"[i] for i in rng.integers(0, 2, n))
+    _run(text, "s", vocab, [list(prefix), list(prefix + b"("), list(b"<(" + prefix[1:] + b")+")], chart_words=1 << 20)
+
+
+def test_left_recursion_nullables_and_shared_prefixes():
+    text = ('s ::= x\nx ::= x y | x z | ""\ny ::= w "a" w | "(" x ")"\nz ::= w "a" w | w "b" x "b"\nw ::= n n\nn ::= "_" | ""')
+    vocab = [bytes([b]) for b in range(256)] + [b"aa", b"_a", b"a_a_", b"(a", b")a)", b"bab", b"__", b"_" * 5, b"((__a", b""]
+    _run(text, "s", vocab, [list(p) for p in (b"", b"a", b"a_", b"(a_", b"bab", b"((b_", b"baaaab(a)")])
+
+
+def test_grammar_without_an_automaton():
+    """Alternations of more than a thousand literals have none: their rows are swept by Earley steps."""
+    names = sorted({"k%06d" % (i * 7919 % 999983) for i in range(1200)})
+    text = 's ::= "[" name ( "," name )* "]"\nname ::= ' + " | ".join('"%s"' % x for x in names)
+    vocab = [bytes([b]) for b in range(256)] + [b"[k", b"k0", b"k1", names[5].encode(), (names[3] + ",").encode(), b""]
+    s = _run(text, "s", vocab, [list(b"[k"), list(b"[" + names[9].encode()), list(b"")])
+    assert s["walk_states"] > 0
+
+
+def test_no_automaton_for_states_that_ask_for_earley_steps():
+    """sweep_states limits the Earley sets of a sweep: a state that sets it runs the steps, and gives the same masks."""
+    w = workloads.build(2, V=3000, batch=1, steps=1)
+    a = _run(w.ebnf, w.start, w.vocab, JSON_PREFIXES)
+    b = _run(w.ebnf, w.start, w.vocab, JSON_PREFIXES, sweep_states=4096)
+    assert a["walk_states"] < b["walk_states"]
