@@ -113,7 +113,6 @@ struct fmt_state {
   int32_t* result_dev = nullptr;
   uint8_t* query_dev = nullptr;  // scratch for fmt_state_query
   int sweep_grid = 1;
-  bool swept = false;         // the tables of the grid-wide sweep are there
   uint32_t next_gen = 1;      // generations handed to the fills: two per fill, 1 .. 65534
   size_t device_bytes = 0;    // what fmt_state_create allocated
   // The device sets this host-mapped word when the state cache has no room for a new entry; the next
@@ -142,8 +141,9 @@ static cudaError_t next_generations(fmt_state* s, cudaStream_t st) {
   StateDev& d = s->dev;
   cudaError_t e = cudaSuccess;
   if (s->next_gen + 1u > 65534u) {
-    if (s->swept) e = cudaMemsetAsync(d.au.hash, 0, (size_t)d.B * (d.au.hash_mask + 1u) * 4, st);
-    if (e == cudaSuccess && s->swept) e = cudaMemsetAsync(d.au.req, 0, (size_t)d.au.req_cap * 8, st);
+    if (d.af.on) e = cudaMemsetAsync(d.af.unit_flag, 0, ((size_t)d.af.unit_cap + d.B) * 4, st);
+    if (e == cudaSuccess && !d.af.on) e = cudaMemsetAsync(d.au.hash, 0, (size_t)d.B * (d.au.hash_mask + 1u) * 4, st);
+    if (e == cudaSuccess && !d.af.on) e = cudaMemsetAsync(d.au.req, 0, (size_t)d.au.req_cap * 8, st);
     if (e == cudaSuccess && d.rt.on) e = cudaMemsetAsync(d.cx.ctab, 0, (size_t)d.B * CT_SLOTS * 8, st);
     if (e == cudaSuccess && d.rt.on) e = cudaMemsetAsync(d.cx.req2, 0, (size_t)d.cx.req2_cap * 16, st);
     s->next_gen = 1;
@@ -242,13 +242,12 @@ fmt_status fmt_compile(const char* ebnf, size_t ebnf_len, const char* start_rule
     UP(tok_ids);
     if (h.ga_on) {
       d.ga_on = 1, d.ga_acc_mask = h.ga_acc_mask;
-      UP(ga_root);
+      UP(ga_item);
       UP(ga_trans);
       UP(ga_acc);
       UP(ga_node);
       UP(ga_tok);
       d.ga_lvl2 = h.ga_lvl2, d.ga_lvl3 = h.ga_lvl3;
-      UP(ga_wide);
       UP(ga_wide_rec);
       UP(ga_wide_mask);
       UP(ga_wide_exit);
@@ -394,7 +393,6 @@ static cudaError_t alloc_sweep(fmt_state* s) {
   AL(au.req, au.req_cap, 0);
   AL(au.job_info, d.B, 0);
 #undef AL
-  if (e == cudaSuccess) s->swept = true;
   return e;
 }
 
@@ -465,13 +463,14 @@ fmt_status fmt_state_create(const fmt_grammar* g, uint32_t batch, const fmt_stat
   if (e == cudaSuccess) e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   // Rows are filled by the grammar's automaton if it has one.  A state that asks for the cache of
-  // context-independent entries, limits the sets of a sweep or the polls of a wait is swept by the grid.
+  // context-independent entries, or limits the Earley sets of a sweep, is swept by the grid.
   AutoFillDev& af = d.af;
-  af.on = (g->dev.ga_on && !rt.on && !(opt && opt->sweep_states) && !d.poll_limit_shift) ? 1u : 0u;
+  af.on = (g->dev.ga_on && !rt.on && !(opt && opt->sweep_states)) ? 1u : 0u;
   if (af.on) {
-    af.stack_cap = 128u << 10;
+    af.stack_cap = 32u << 10;
     af.ctx_cap = 4096, af.pool_cap = 64u << 10, af.big_cap = 64u << 10;
-    automaton_fill_layout(g->dev, batch, 2u * (uint32_t)std::max(1, sms), af);
+    af.unit_cap = 4096;
+    automaton_fill_layout(g->dev, batch, AUTO_FILL_PER_SM * (uint32_t)std::max(1, sms), af);
   }
 #define AL(ptr, count, fill) if (e == cudaSuccess) e = s->bufs.alloc((size_t)(count), &(ptr), (fill))
   AL(d.arena, d.pool_base + d.pool_words * (two_gens ? 2 : 1), 0);
@@ -502,6 +501,8 @@ fmt_status fmt_state_create(const fmt_grammar* g, uint32_t batch, const fmt_stat
   if (af.on) {
     AL(af.stack, (size_t)af.grid * af.stack_cap, 0);
     AL(af.scratch, (size_t)af.grid * af.scratch_words, 0);
+    AL(af.units, (size_t)af.unit_cap * af.unit_words, 0);
+    AL(af.unit_flag, af.unit_cap + batch, 0);
   } else if (e == cudaSuccess) {
     e = alloc_sweep(s);
   }
@@ -723,14 +724,6 @@ fmt_status fmt_state_ci_cache_clear(fmt_state* s, void* stream) {
 
 fmt_status fmt_state_set_wait_limit(fmt_state* s, uint32_t log2_polls) {
   if (!s) return fail(FMT_ERR_INVALID_ARG, "NULL state");
-  // (the fill by the grammar's automaton has no waits: with a limit the rows are swept by the grid, whose waits it bounds)
-  if (log2_polls && !s->swept) {
-    cudaError_t e = alloc_sweep(s);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(nullptr);  // (the tables are cleared there)
-    if (e != cudaSuccess) return cuda_fail(e, "fmt_state_set_wait_limit");
-    s->device_bytes = s->bufs.bytes;
-  }
-  s->dev.af.on = s->dev.af.stack && !log2_polls ? 1u : 0u;
   s->dev.poll_limit_shift = std::min(log2_polls, 30u);
   return FMT_OK;
 }

@@ -1,23 +1,24 @@
-// The fill of a row's mask by the grammar automaton (grammar_automaton.cpp; Sections 3.3, 4.1, 4.3 of the paper).
+// The fill of rows' masks by the grammar automaton (grammar_automaton.cpp; Sections 3.3, 4.1, 4.3 of the paper).
 //
-// A thread block, or a cluster of them, takes one row.  The kernel items of the chart's last set are grouped by dotted rule;
-// every group starts a THREAD at the root of the vocabulary trie: a code of the automaton and a CONTEXT, the set of
-// origins its items were begun in.  A trie node's children are reached by one table look-up each.  Where the automaton says that a
-// rule begun in the chart ends, the thread's context is EXPANDED: the items that waited in its origins, completed upwards (Section
-// 3.2's Complete), start threads of their own at that node.  A context is expanded once per row.  A token is valid iff some
-// thread is alive at the node where its bytes end.
+// A thread block takes a row.  The kernel items of the chart's last set are grouped by dotted rule; every group starts a
+// THREAD at the root of the vocabulary trie: a code of the automaton and a CONTEXT, the set of origins its items were begun in.  A
+// trie node's children are reached by one table look-up each.  Where the automaton says that a rule begun in the chart ends, the
+// thread's context is EXPANDED: the items that waited in its origins, completed upwards (Section 3.2's Complete), start
+// threads of their own at that node.  A context is expanded once per row.  A token is valid iff some thread is alive at the
+// node where its bytes end; its bit is set in the row's mask in global memory at once.
 //
-// What bounds it: at the sizes measured, latency - rounds of "take threads from the stack, look their children up, push
-// what is alive", each two dependent reads in L2 and three block barriers, about as many rounds as the longest token has bytes.
-// Nothing waits for another block and no Earley set is built.
+// What bounds it: at the sizes measured, latency - rounds of "take threads, look their children up, push what is alive", each
+// two or three dependent reads in L2 and four block barriers, about as many rounds as the longest token has bytes.  Hence
+// the threads, the contexts and the chart sit in shared memory (with a way out to global memory), and four blocks
+// share an SM.  Rows differ by a factor of a hundred in work (measured: 800 to 290,000 look-ups), so blocks that have no row left wait
+// for work, and a block with many threads hands parts of them out, with its contexts.
 // Measured on a B200, the fill alone, against the sweep of the whole grid by Earley steps (kernels.cu) before:
-//   8 rows of JSON, 32,000 tokens               239 -> 95 us    (where about half of the rows are computed)
-//   64 rows of a JSON schema, 128,256 tokens    263 -> 60 us
-//   128 rows of SQL, 152,064 tokens             667 -> 279 us
+//   8 rows of JSON, 32,000 tokens               239 -> 94 us    (where about half of the rows are computed)
+//   64 rows of a JSON schema, 128,256 tokens    263 -> 77 us
+//   128 rows of SQL, 152,064 tokens             667 -> 231 us
 //   37 rows of JSON, 50,001 tokens              362 -> 129 us
-//   256 rows of ambiguous JSON, 128,256 tokens  3.51 -> 2.68 ms
+//   256 rows of ambiguous JSON, 128,256 tokens  3.51 -> 1.06 ms (2.65 ms when no work is handed on)
 // The sweep stays for grammars without an automaton and for the cache of context-independent entries.
-#include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -26,48 +27,62 @@
 #include "sweep_warp.cuh"
 
 namespace fmt {
-namespace cg = cooperative_groups;
 
 constexpr int AF_WARPS = 8, AF_THREADS = AF_WARPS * 32;
-constexpr uint32_t AF_BATCH = 1024;       // threads taken from the stack per round
-constexpr uint32_t AF_SEEN = 1024;        // recently started threads (a lossy table: repeats only cost time)
-constexpr uint32_t AF_STAGE = 2048;       // a chart up to this many words is read from shared memory
-constexpr uint32_t AF_BUF = 1024;         // items of an expansion in shared memory (larger ones: global memory)
-constexpr uint32_t AF_WORK = 512, AF_HSET = 1024;
-constexpr uint32_t AF_MASK_SMEM = 6144;   // mask rows up to this many words are collected in shared memory
-// stack entries that are not threads, told by their code
-constexpr uint32_t AF_SPAWN = 0xFFFFFFFDu;   // the expansion of a context at a node (first child, children)
-constexpr uint32_t AF_EXITS = 0xFFFFFFFCu;   // the same at a list of nodes (where in ga_wide_exit, count)
-constexpr uint32_t AF_EXIT_PIECE = 1024;     // nodes of such a list taken at once
-constexpr uint32_t AF_TOKENS = 0xFFFFFFFBu;  // tokens to mark (where in ga_tok, count)
+constexpr uint32_t AF_BATCH = 512;        // threads of a round
+constexpr uint32_t AF_PER = AF_BATCH / AF_THREADS;
+constexpr uint32_t AF_SPEC = AF_THREADS;  // expansions to be made at the start of a round
+constexpr uint32_t AF_EXITS = 60;         // lists of nodes at which expansions are to be made (from wide items)
+constexpr uint32_t AF_SPEC_STACK = 4096;  // part of a block's stack that is kept for those that found no room
+constexpr uint32_t AF_SEEN = 512;         // recently started threads (a lossy table: repeats only cost time)
+constexpr uint32_t AF_STAGE = 1024;       // a chart up to this many words is read from shared memory
+constexpr uint32_t AF_CTX = 64, AF_CTX_HASH = 128, AF_POOL = 2048;  // contexts in shared memory, words of their lists
+constexpr uint32_t AF_BUF = 512, AF_WORK = 256, AF_HSET = 512;      // an expansion in shared memory (larger ones: global memory)
+constexpr uint32_t AF_OWNER = AF_BATCH * 8;  // pieces of 32 children a round can hold (a node has at most 256)
+constexpr uint32_t AF_HEAVY = 16384;      // after so many look-ups for a row, or for a unit of work,
+constexpr uint32_t AF_SHARE = 384;        // a block with so many threads gives some to blocks that wait,
+constexpr uint32_t AF_MAX_UNITS = 7;      // to so many at once, 128 threads at the least to each
+constexpr uint32_t AF_SPAWN = 0xFFFFFFFDu;  // code of a special: to start the threads of a context's expansion at a node (first child, children)
+constexpr uint32_t AF_GIVEN_UP = 0xFFFFFFFFu;  // (AC_FAIL) a wait ran out: the fill is given up, the row itself is fine
 constexpr uint32_t CTX_NEW = 0xFFFFFFFFu;
 
-enum : uint32_t { AC_TOP = 0, AC_FAIL = 1, AC_NCTX = 2, AC_POOL = 3, AC_NWORK = 4, AC_NBUF = 5, AC_OVER = 6, AC_WSUM = 8,
-                  AC_NWIDE = 16, AC_WIDE = 20, AC_WORDS = 84 };
-
-// A block's contexts, in global memory that only this block uses.
-struct Contexts {
-  const AutoFillDev& A;
-  uint2* org;       // [ctx_cap] origins: offset into pool, count
-  uint2* exp;       // [ctx_cap] expansion: offset into pool, count (CTX_NEW: not made yet); pairs (code, rule << 16 | context)
-  uint32_t* lhs;    // [ctx_cap] the non-terminal whose rule is open
-  uint32_t* hash;   // [hash_mask + 1] context + 1, 0 = empty
-  uint32_t* pool;
-  uint32_t *big_work, *big_hset, *big_buf;
-  __device__ __forceinline__ explicit Contexts(const AutoFillDev& a, uint32_t block) : A(a) {
-    uint32_t* p = a.scratch + (size_t)block * a.scratch_words;
-    org = reinterpret_cast<uint2*>(p), p += 2 * a.ctx_cap;
-    exp = reinterpret_cast<uint2*>(p), p += 2 * a.ctx_cap;
-    lhs = p, p += a.ctx_cap;
-    hash = p, p += 2 * a.ctx_cap;
-    pool = p, p += a.pool_cap;
-    big_work = p, p += a.big_cap / 4;
-    big_hset = p, p += a.big_cap / 2;
-    big_buf = p;
-  }
+enum : uint32_t {
+  AC_NEXT = 0, AC_SPEC = 1, AC_OVF = 2, AC_GTOP = 3, AC_FAIL = 4, AC_NCTX = 5, AC_POOL = 6, AC_NWORK = 7, AC_WSUM = 8, AC_NBUF = 16, AC_OVER = 17,
+  AC_SPILLED = 18, AC_WAITING = 19, AC_BASE = 20, AC_JOB = 21, AC_NWIDE = 22, AC_SOVF = 23, AC_GSPEC = 24, AC_NEXITS = 25, AC_WIDE = 26, AC_WORDS = AC_WIDE + AF_EXITS + 2
 };
 
-// The row's chart as an expansion reads it.
+// A unit of work handed out: AU_HDR words, then the giver's contexts, lists and the threads.
+enum : uint32_t { AU_ROWJOB = 0, AU_N = 1, AU_NCTX = 2, AU_POOL = 3, AU_PART = 4, AU_HDR = 8 };
+constexpr uint32_t AU_ENTRIES = AF_BATCH / 2 + 4;
+constexpr uint32_t AU_WORDS = AU_HDR + 5 * AF_CTX + AF_POOL + 4 * AU_ENTRIES;
+static_assert(AU_WORDS % 4 == 0 && (AU_HDR + 5 * AF_CTX + AF_POOL) % 4 == 0, "the threads of a unit are 16-byte records");
+
+// The contexts of the row a block works on: in shared memory, or, when they outgrow it, in global memory of the block's own.
+struct Contexts {
+  uint2* org;       // [cap] origins: offset into pool, count
+  uint2* exp;       // [cap] expansion: offset into pool, count (CTX_NEW: not made yet); pairs (code, rule << 16 | context)
+  uint32_t* lhs;    // [cap] the non-terminal whose rule is open
+  uint32_t* hash;   // [hash_mask + 1] context + 1, 0 = empty
+  uint32_t* pool;
+  uint32_t cap, hash_mask, pool_cap;
+};
+__device__ __forceinline__ uint32_t vload(const uint32_t* p) { return *reinterpret_cast<const volatile uint32_t*>(p); }
+__device__ __forceinline__ Contexts global_contexts(const AutoFillDev& A) {
+  uint32_t* p = A.scratch + (size_t)blockIdx.x * A.scratch_words;
+  Contexts C;
+  C.org = reinterpret_cast<uint2*>(p), p += 2 * A.ctx_cap;
+  C.exp = reinterpret_cast<uint2*>(p), p += 2 * A.ctx_cap;
+  C.lhs = p, p += A.ctx_cap;
+  C.hash = p, p += 2 * A.ctx_cap;
+  C.pool = p;
+  C.cap = A.ctx_cap, C.hash_mask = 2u * A.ctx_cap - 1u, C.pool_cap = A.pool_cap;
+  return C;
+}
+// (what follows them in the block's scratch)
+__device__ __forceinline__ uint32_t* big_area(const AutoFillDev& A) {
+  return A.scratch + (size_t)blockIdx.x * A.scratch_words + 7u * A.ctx_cap + A.pool_cap;
+}
+
 struct AfChart {
   const uint32_t* off;
   const uint32_t* items;
@@ -76,14 +91,16 @@ struct AfChart {
 
 // ---- the parts one warp does: contexts and their expansions
 
+__device__ __forceinline__ uint32_t context_hash(uint32_t lhs, const uint32_t* list, uint32_t n) {
+  uint32_t h = 0;
+  for (uint32_t i = lane_id(); i < n; i += 32) h += mix32((list[i] & 0xFFFFu) + 1u);
+  return mix32(__reduce_add_sync(FULL, h) + lhs * 0x9E3779B9u + n);
+}
+
 // The context (lhs, list[0..n) & 0xFFFF) (ascending): its number, or CTX_NEW when there is no room.
 __device__ uint32_t intern_context(const Contexts& C, uint32_t* ctl, uint32_t lhs, const uint32_t* list, uint32_t n) {
   const uint32_t lane = lane_id();
-  uint32_t h = 0;
-  for (uint32_t i = lane; i < n; i += 32) h += mix32((list[i] & 0xFFFFu) + 1u);
-  h = mix32(__reduce_add_sync(FULL, h) + lhs * 0x9E3779B9u + n);
-  const uint32_t mask = 2u * C.A.ctx_cap - 1u;
-  uint32_t slot = h & mask;
+  uint32_t slot = context_hash(lhs, list, n) & C.hash_mask;
   for (;;) {
     const uint32_t v = C.hash[slot];
     if (v == 0u) break;
@@ -92,12 +109,12 @@ __device__ uint32_t intern_context(const Contexts& C, uint32_t* ctl, uint32_t lh
     if (same)
       for (uint32_t i = lane; i < n; i += 32) same = same && C.pool[o.x + i] == (list[i] & 0xFFFFu);
     if (__all_sync(FULL, same)) return v - 1u;
-    slot = (slot + 1u) & mask;
+    slot = (slot + 1u) & C.hash_mask;
   }
   const uint32_t id = ctl[AC_NCTX], at = ctl[AC_POOL];
-  if (id >= C.A.ctx_cap || n > C.A.pool_cap - at) return CTX_NEW;
-  for (uint32_t i = lane; i < n; i += 32) C.pool[at + i] = list[i] & 0xFFFFu;
   __syncwarp();
+  if (id >= C.cap || n > C.pool_cap - at) return CTX_NEW;
+  for (uint32_t i = lane; i < n; i += 32) C.pool[at + i] = list[i] & 0xFFFFu;
   if (lane == 0) {
     C.org[id] = make_uint2(at, n);
     C.exp[id] = make_uint2(0u, CTX_NEW);
@@ -110,49 +127,69 @@ __device__ uint32_t intern_context(const Contexts& C, uint32_t* ctl, uint32_t lh
   return id;
 }
 
+// The contexts leave shared memory.
+__device__ void spill_contexts(Contexts& C, uint32_t* ctl, const AutoFillDev& A) {
+  const uint32_t lane = lane_id(), n = ctl[AC_NCTX], words = ctl[AC_POOL];
+  const Contexts D = global_contexts(A);
+  for (uint32_t i = lane; i < n; i += 32) D.org[i] = C.org[i], D.exp[i] = C.exp[i], D.lhs[i] = C.lhs[i];
+  for (uint32_t i = lane; i < words; i += 32) D.pool[i] = C.pool[i];
+  for (uint32_t i = lane; i <= D.hash_mask; i += 32) D.hash[i] = 0u;
+  __syncwarp();
+  for (uint32_t c = 0; c < n; ++c) {
+    const uint2 o = D.org[c];
+    uint32_t slot = context_hash(D.lhs[c], D.pool + o.x, o.y) & D.hash_mask;
+    if (lane == 0) {
+      while (D.hash[slot]) slot = (slot + 1u) & D.hash_mask;
+      D.hash[slot] = c + 1u;
+    }
+    __syncwarp();
+  }
+  C = D;
+  if (lane == 0) ctl[AC_SPILLED] = 1u;
+  __syncwarp();
+}
+
 // buf[0..n), values rule << 16 | origin in any order, room for the next power of two: sorted, grouped by rule, as the expansion
 // list (offset, count) in the pool.  False when there is no room.
 __device__ bool group_items(const GrammarDev& G, const Contexts& C, uint32_t* ctl, uint32_t* buf, uint32_t n, uint2& out) {
   const uint32_t lane = lane_id();
   sort_items(buf, n, 1u << 30);
-  uint32_t k = 0;  // repeats go
-  for (uint32_t base = 0; base < n; base += 32) {
+  uint32_t k = 0, groups = 0;  // repeats go
+  for (uint32_t base = 0, last = 0xFFFFFFFFu; base < n; base += 32) {
     const uint32_t i = base + lane;
-    const uint32_t v = i < n ? buf[i] : 0u;
-    const bool keep = i < n && (i == 0u || buf[i - 1u] != v);
-    const uint32_t b = __ballot_sync(FULL, keep);
+    const uint32_t v = i < n ? buf[i] : 0xFFFFFFFFu;
+    uint32_t p = __shfl_up_sync(FULL, v, 1);
+    if (lane == 0) p = last;
+    last = __shfl_sync(FULL, v, 31);
+    const uint32_t b = __ballot_sync(FULL, i < n && v != p);
+    groups += __popc(__ballot_sync(FULL, i < n && (v >> 16) != (p >> 16)));  // (no rule has the number 0xFFFF)
     __syncwarp();
-    if (keep) buf[k + __popc(b & ((1u << lane) - 1u))] = v;  // (never beyond what has been read: i - 1 of the next piece is i's own value or earlier)
+    if (i < n && v != p) buf[k + __popc(b & ((1u << lane) - 1u))] = v;
     k += __popc(b);
-    __syncwarp();
   }
-  uint32_t groups = 0;
-  for (uint32_t base = 0; base < k; base += 32) {
-    const uint32_t i = base + lane;
-    groups += __popc(__ballot_sync(FULL, i < k && (i == 0u || (buf[i - 1u] >> 16) != (buf[i] >> 16))));
-  }
+  __syncwarp();
   const uint32_t at = (ctl[AC_POOL] + 1u) & ~1u;
   __syncwarp();
-  if (at + 2u * groups > C.A.pool_cap) return false;
+  if (at + 2u * groups > C.pool_cap) return false;
   if (lane == 0) ctl[AC_POOL] = at + 2u * groups;
   __syncwarp();
   uint32_t g = 0;
   for (uint32_t i = 0; i < k;) {
     const uint32_t d = buf[i] >> 16;
+    const uint4 rec = __ldg(reinterpret_cast<const uint4*>(G.ga_item) + d);
     uint32_t e = i + 1u;
     for (;;) {  // the end of the group
-      const uint32_t b = __ballot_sync(FULL, e + lane >= k || (buf[e + lane] >> 16) != d);
+      const uint32_t b = __ballot_sync(FULL, e + lane >= k || (buf[min(e + lane, k - 1u)] >> 16) != d);
       if (b) {
         e += (uint32_t)__ffs(b) - 1u;
         break;
       }
       e += 32u;
     }
-    const uint32_t code = __ldg(&G.ga_root[d]);
-    if (code != GA_DEAD) {
-      const uint32_t c = intern_context(C, ctl, __ldg(&G.lhs[d]), buf + i, e - i);
+    if (rec.x != GA_DEAD) {
+      const uint32_t c = intern_context(C, ctl, rec.y & 0xFFFFu, buf + i, e - i);
       if (c == CTX_NEW) return false;
-      if (lane == 0) reinterpret_cast<uint2*>(C.pool)[at / 2u + g] = make_uint2(code, d << 16 | c);
+      if (lane == 0) reinterpret_cast<uint2*>(C.pool)[at / 2u + g] = make_uint2(rec.x, d << 16 | c);
       ++g;
     }
     i = e;
@@ -189,39 +226,116 @@ __device__ bool expand_into(const GrammarDev& G, const Contexts& C, const AfChar
     const uint32_t a = work[head] >> 16, o = work[head] & 0xFFFFu;
     const uint32_t lo = J.off[o], hi = J.off[o + 1u];
     for (uint32_t k = lo + lane; k < hi; k += 32) {
-      const uint32_t it = J.items[k], inf = __ldg(&G.info[it & 0xFFFFu]);
-      if ((inf >> INFO_KIND_SHIFT) != KIND_NT || (inf & INFO_ARG_MASK) != a) continue;
-      const uint32_t x = (it & 0xFFFFu) + 1u, ix = __ldg(&G.info[x]);
-      const uint32_t skip = (ix >> INFO_SKIP_SHIFT) & INFO_SKIP_MASK;
-      if ((ix >> INFO_KIND_SHIFT) != KIND_END) {
+      const uint32_t it = J.items[k];
+      const uint4 rec = __ldg(reinterpret_cast<const uint4*>(G.ga_item) + (it & 0xFFFFu));
+      if ((rec.y >> 16) != a) continue;
+      if (rec.w & GA_GOES_ON) {
         const uint32_t at = atomicAdd(&ctl[AC_NBUF], 1u);
-        if (at < buf_cap) buf[at] = x << 16 | (it >> 16);
+        if (at < buf_cap) buf[at] = ((it & 0xFFFFu) + 1u) << 16 | (it >> 16);
         else ctl[AC_OVER] = 1u;
       }
-      const uint32_t ie = skip ? __ldg(&G.info[x + skip]) : ix;
-      if ((ie >> INFO_KIND_SHIFT) == KIND_END) need(ie & INFO_ARG_MASK, it >> 16);
+      if ((rec.w & 0xFFFFu) != 0xFFFFu) need(rec.w & 0xFFFFu, it >> 16);
     }
   }
   return true;
 }
 
-__device__ bool expand_context(const GrammarDev& G, const Contexts& C, const AfChart& J, uint32_t c, uint32_t* ctl, uint32_t* work,
-                               uint32_t* hset, uint32_t* buf) {
+// The same with everything in the warp's lanes: one context of at most 32 origins, at most 32 completions and 32 items.  Nearly all
+// expansions are of this kind (one origin, two or three completions, one item); the general form takes some four times as many
+// instructions.  False: it does not fit (nothing has changed but the pool's top).
+__device__ bool expand_small(const GrammarDev& G, const Contexts& C, const AfChart& J, uint32_t c, uint32_t* ctl) {
   const uint32_t lane = lane_id();
-  uint32_t* b = buf;
-  bool ok = expand_into(G, C, J, c, ctl, work, AF_WORK, hset, AF_HSET - 1u, buf, AF_BUF);
-  hset_clear_all(hset, AF_HSET - 1u);
-  if (!ok) {  // too large for shared memory
-    b = C.big_buf;
-    hset_clear_all(C.big_hset, C.A.big_cap / 2u - 1u);
-    ok = expand_into(G, C, J, c, ctl, C.big_work, C.A.big_cap / 4u, C.big_hset, C.A.big_cap / 2u - 1u, C.big_buf, C.A.big_cap);
+  const uint2 org = C.org[c];
+  if (org.y > 32u) return false;
+  uint32_t work = lane < org.y ? C.lhs[c] << 16 | C.pool[org.x + lane] : 0u, nw = org.y;  // lane l: completion l
+  uint32_t item = 0u, ni = 0u;                                                           // lane l: item l
+  for (uint32_t head = 0; head < nw; ++head) {
+    const uint32_t key = __shfl_sync(FULL, work, head);
+    const uint32_t a = key >> 16, o = key & 0xFFFFu;
+    const uint32_t lo = J.off[o], hi = J.off[o + 1u];
+    for (uint32_t base = lo; base < hi; base += 32) {
+      const uint32_t k = base + lane;
+      const uint32_t it = k < hi ? J.items[k] : 0u;
+      const uint4 rec = __ldg(reinterpret_cast<const uint4*>(G.ga_item) + (it & 0xFFFFu));
+      const bool match = k < hi && (rec.y >> 16) == a;
+      uint32_t on = __ballot_sync(FULL, match && (rec.w & GA_GOES_ON));
+      if (on) {
+        const uint32_t x = ((it & 0xFFFFu) + 1u) << 16 | (it >> 16);
+        if (ni + __popc(on) > 32u) return false;
+        for (; on; on &= on - 1u) {
+          const uint32_t v = __shfl_sync(FULL, x, __ffs(on) - 1);
+          if (__ballot_sync(FULL, lane < ni && item == v)) continue;
+          if (lane == ni) item = v;
+          ++ni;
+        }
+      }
+      for (uint32_t up = __ballot_sync(FULL, match && (rec.w & 0xFFFFu) != 0xFFFFu); up; up &= up - 1u) {
+        const uint32_t v = __shfl_sync(FULL, (rec.w & 0xFFFFu) << 16 | (it >> 16), __ffs(up) - 1);
+        if (__ballot_sync(FULL, lane < nw && work == v)) continue;
+        if (nw == 32u) return false;
+        if (lane == nw) work = v;
+        ++nw;
+      }
+    }
   }
-  uint2 list;
-  ok = ok && group_items(G, C, ctl, b, ctl[AC_NBUF], list);
+  // by rule: one context for each
+  uint32_t at = (ctl[AC_POOL] + 1u) & ~1u, g = 0;
+  if (at + 2u * ni + 64u > C.pool_cap || ctl[AC_NCTX] + ni > C.cap) return false;
   __syncwarp();
-  if (lane == 0) C.exp[c] = ok ? list : make_uint2(0u, 0u);
+  if (lane == 0) ctl[AC_POOL] = at + 2u * ni;
   __syncwarp();
-  return ok;
+  for (uint32_t left = ni == 32u ? FULL : (1u << ni) - 1u; left;) {
+    const uint32_t d = __shfl_sync(FULL, item >> 16, __ffs(left) - 1);
+    const bool in = ((left >> lane) & 1u) && (item >> 16) == d;
+    const uint32_t members = __ballot_sync(FULL, in), n = __popc(members);
+    left &= ~members;
+    const uint4 rec = __ldg(reinterpret_cast<const uint4*>(G.ga_item) + d);
+    if (rec.x == GA_DEAD) continue;
+    // its origins, ascending, at the pool's top (which grows only if the context is new)
+    const uint32_t top = ctl[AC_POOL];
+    if (top + n > C.pool_cap) return false;
+    uint32_t rank = 0;
+    if (n > 1u)
+      for (uint32_t m = members; m; m &= m - 1u) rank += __shfl_sync(FULL, item, __ffs(m) - 1) < item ? 1u : 0u;
+    if (in) C.pool[top + rank] = item & 0xFFFFu;
+    __syncwarp();
+    const uint32_t ctx = intern_context(C, ctl, rec.y & 0xFFFFu, C.pool + top, n);
+    if (ctx == CTX_NEW) return false;
+    if (lane == 0) reinterpret_cast<uint2*>(C.pool)[at / 2u + g] = make_uint2(rec.x, d << 16 | ctx);
+    ++g;
+  }
+  __syncwarp();
+  if (lane == 0) C.exp[c] = make_uint2(at, g);
+  __syncwarp();
+  return true;
+}
+
+__device__ __noinline__ bool expand_context(const GrammarDev& G, const AutoFillDev& A, Contexts& C, const AfChart& J, uint32_t c,
+                                            uint32_t* ctl, uint32_t* work, uint32_t* hset, uint32_t* buf) {
+  const uint32_t lane = lane_id();
+  if (expand_small(G, C, J, c, ctl)) return true;
+  for (;;) {
+    uint32_t* b = buf;
+    bool ok = expand_into(G, C, J, c, ctl, work, AF_WORK, hset, AF_HSET - 1u, buf, AF_BUF);
+    hset_clear_all(hset, AF_HSET - 1u);
+    if (!ok) {  // too large for shared memory
+      uint32_t* big_work = big_area(A);
+      uint32_t* big_hset = big_work + A.big_cap / 4u;
+      b = big_hset + A.big_cap / 2u;
+      hset_clear_all(big_hset, A.big_cap / 2u - 1u);
+      ok = expand_into(G, C, J, c, ctl, big_work, A.big_cap / 4u, big_hset, A.big_cap / 2u - 1u, b, A.big_cap);
+    }
+    uint2 list = make_uint2(0u, 0u);
+    const bool fits = ok && group_items(G, C, ctl, b, ctl[AC_NBUF], list);
+    if (ok && !fits && !ctl[AC_SPILLED]) {
+      spill_contexts(C, ctl, A);
+      continue;
+    }
+    __syncwarp();
+    if (lane == 0) C.exp[c] = list;
+    __syncwarp();
+    return fits;
+  }
 }
 
 // Where `code` leads on byte class e.
@@ -240,33 +354,82 @@ __device__ __forceinline__ uint32_t ga_next(const GrammarDev& G, uint32_t code, 
   }
 }
 
-__global__ void __launch_bounds__(AF_THREADS) automaton_fill_kernel(const __grid_constant__ GrammarDev G,
-                                                                    const __grid_constant__ StateDev S) {
+__global__ void __launch_bounds__(AF_THREADS, 4) automaton_fill_kernel(const __grid_constant__ GrammarDev G,
+                                                                       const __grid_constant__ StateDev S) {
   const uint32_t n_jobs = S.counters[CNT_N_JOBS];
   if (n_jobs == 0u) return;  // (every block sees the same count)
   extern __shared__ __align__(16) uint32_t smem[];
   const AutoFillDev& A = S.af;
   const uint32_t tid = threadIdx.x, warp = tid >> 5, lane = lane_id();
-  uint4* cur = reinterpret_cast<uint4*>(smem);
-  unsigned long long* seen = reinterpret_cast<unsigned long long*>(cur + AF_BATCH);
-  uint32_t* pre = reinterpret_cast<uint32_t*>(seen + AF_SEEN);  // [AF_BATCH + 1]
-  uint32_t* ctl = pre + AF_BATCH + 4;
-  uint32_t* stage = ctl + AC_WORDS;
-  uint32_t* buf = stage + AF_STAGE;
-  uint32_t* work = buf + AF_BUF;
-  uint32_t* hset = work + AF_WORK;
-  uint32_t* mask_sm = hset + AF_HSET;
-  const bool in_smem = G.Wm <= AF_MASK_SMEM;
-  uint4* stack = A.stack + (size_t)blockIdx.x * A.stack_cap;
-  const Contexts C(A, blockIdx.x);
-  const cg::cluster_group cluster = cg::this_cluster();
-  const uint32_t parts = cluster.num_blocks(), part = cluster.block_rank();
+  uint4* const entries = reinterpret_cast<uint4*>(smem);               // [2][AF_BATCH], in turn
+  uint4* const specials = entries + 2 * AF_BATCH;                      // [2][AF_SPEC], in turn
+  uint4* const exits = specials + 2 * AF_SPEC;                         // [AF_EXITS] where in ga_wide_exit, count, -, context
+  unsigned long long* const seen = reinterpret_cast<unsigned long long*>(exits + AF_EXITS);
+  Contexts C0;
+  C0.org = reinterpret_cast<uint2*>(seen + AF_SEEN);
+  C0.exp = C0.org + AF_CTX;
+  C0.lhs = reinterpret_cast<uint32_t*>(C0.exp + AF_CTX);
+  C0.pool = C0.lhs + AF_CTX;
+  C0.hash = C0.pool + AF_POOL;
+  C0.cap = AF_CTX, C0.hash_mask = AF_CTX_HASH - 1u, C0.pool_cap = AF_POOL;
+  uint32_t* const pre = C0.hash + AF_CTX_HASH;  // [AF_BATCH + 1]
+  uint32_t* const ctl = pre + AF_BATCH + 4;
+  uint32_t* const stage = ctl + AC_WORDS;
+  uint32_t* const buf = stage + AF_STAGE;
+  uint32_t* const work = buf + AF_BUF;
+  uint32_t* const hset = work + AF_WORK;
+  uint16_t* const owner = reinterpret_cast<uint16_t*>(hset + AF_HSET);  // [AF_OWNER] the thread to whom the first child of a piece belongs
+  uint4* const stack = A.stack + (size_t)blockIdx.x * A.stack_cap;  // threads that found no room in `entries`
   for (uint32_t i = tid; i < AF_HSET; i += AF_THREADS) hset[i] = EMPTY_SLOT;
   uint32_t looked_up = 0, contexts = 0;
+  // (expansions look items up one after the other: what fits is brought near at once)
+  for (uint32_t i = tid * 8u; i < min(G.D, 8u * AF_THREADS); i += 8u * AF_THREADS) {
+    uint32_t v;
+    asm volatile("ld.global.nc.u32 %0, [%1];" : "=r"(v) : "l"(G.ga_item + 4u * i));
+  }
+  bool rows_left = true;
+  const uint32_t parts = A.parts;
 
-  for (uint32_t j = blockIdx.x / parts; j < n_jobs; j += gridDim.x / parts) {
+  for (;;) {
+    // ---- (a share of) a row, or, when there is none left, a unit of work that another block gives
+    // (they are taken by blocks that run: nobody ever waits for a block that has not started)
+    __syncthreads();
+    if (tid == 0) ctl[AC_JOB] = rows_left ? atomicAdd(&S.counters[CNT_AF_TICKET], 1u) : 0xFFFFFFFFu;
+    __syncthreads();
+    uint32_t j = ctl[AC_JOB] / parts, part = ctl[AC_JOB] % parts;
+    uint32_t* unit = nullptr;
+    rows_left = j < n_jobs;
+    if (j >= n_jobs) {
+      __syncthreads();
+      if (tid == 0) {
+        const uint32_t ticket = atomicAdd(&S.counters[CNT_AF_TAKEN], 1u);
+        uint32_t got = 0;
+        if (ticket < A.unit_cap) {
+          for (uint32_t polls = 0;; ++polls) {
+            if (ld_acquire(&A.unit_flag[ticket]) == S.gen) {
+              got = 1u;
+              break;
+            }
+            if (ld_acquire(&S.counters[CNT_AF_ACTIVE]) == 0u || ld_acquire(&S.counters[CNT_BAR_ERR])) break;  // all is done
+            if (polls > poll_limit(S, 22)) {
+              diag(S, DIAG_WAIT_QUEUE);
+              atomicExch(&S.counters[CNT_BAR_ERR], 1u);  // the fill is given up: its rows get all-zero masks
+              break;
+            }
+            __nanosleep(400);
+          }
+        }
+        ctl[AC_JOB] = got ? ticket : 0xFFFFFFFFu;
+      }
+      __syncthreads();
+      const uint32_t u = ctl[AC_JOB];
+      if (u == 0xFFFFFFFFu) break;
+      unit = A.units + (size_t)u * AU_WORDS;
+      j = __ldcg(unit + AU_ROWJOB), part = __ldcg(unit + AU_PART);
+    }
     const uint32_t row = S.jobs[j];
     const uint32_t* chart = S.arena + S.row_chart[row];
+    uint32_t* const mask = S.mask_rows + (size_t)S.row_mask[row] * G.Wm;
     AfChart J;
     J.m = chart[CH_SETS];
     const uint32_t chart_words = chart[CH_WORDS];
@@ -277,107 +440,277 @@ __global__ void __launch_bounds__(AF_THREADS) automaton_fill_kernel(const __grid
       J.off = stage + CH_HDR;
     }
     J.items = J.off + J.m + 1u;
-    uint32_t* const out = S.mask_rows + (size_t)S.row_mask[row] * G.Wm;
-    uint32_t* const mask = in_smem ? mask_sm : out;  // (clusters only with masks in shared memory)
-    for (uint32_t i = tid; i < G.Wm; i += AF_THREADS) mask[i] = 0u;
-    for (uint32_t i = tid; i < AF_SEEN; i += AF_THREADS) seen[i] = 0ull;
-    for (uint32_t i = tid; i < 2u * A.ctx_cap; i += AF_THREADS) C.hash[i] = 0u;
-    if (tid < AC_WORDS) ctl[tid] = 0u;
     __syncthreads();
-    if (warp == 0) {  // the kernel of the chart's last set starts the first threads
+    for (uint32_t i = tid; i < AF_SEEN; i += AF_THREADS) seen[i] = 0ull;
+    if (tid < AC_WORDS) ctl[tid] = 0u;
+    if (tid < AF_CTX_HASH) C0.hash[tid] = 0u;
+    uint32_t side = 0;  // the threads of this round are entries[side]
+    __syncthreads();
+    if (unit) {
+      const uint32_t n = __ldcg(unit + AU_N), nc = __ldcg(unit + AU_NCTX), np = __ldcg(unit + AU_POOL);
+      const uint32_t* src = unit + AU_HDR;
+      uint32_t* dst = reinterpret_cast<uint32_t*>(C0.org);  // org, exp, lhs and pool follow one another here and there
+      for (uint32_t i = tid; i < 5u * AF_CTX + np; i += AF_THREADS) dst[i] = __ldcg(src + i);
+      const uint4* th = reinterpret_cast<const uint4*>(unit + AU_HDR + 5 * AF_CTX + AF_POOL);
+      for (uint32_t i = tid; i < n; i += AF_THREADS) entries[i] = __ldcg(th + i);
+      __syncthreads();
+      if (warp == 0) {
+        for (uint32_t c = 0; c < nc; ++c) {
+          const uint2 o = C0.org[c];
+          uint32_t slot = context_hash(C0.lhs[c], C0.pool + o.x, o.y) & (AF_CTX_HASH - 1u);
+          while (C0.hash[slot]) slot = (slot + 1u) & (AF_CTX_HASH - 1u);
+          __syncwarp();
+          if (lane == 0) C0.hash[slot] = c + 1u;
+          __syncwarp();
+        }
+        if (lane == 0) ctl[AC_NEXT] = n, ctl[AC_NCTX] = nc, ctl[AC_POOL] = np;
+      }
+    } else if (warp == 0) {  // the kernel of the chart's last set starts the first threads
       const uint32_t lo = J.off[J.m - 1u], hi = J.off[J.m], self = J.m - 1u;
-      uint32_t* b = hi - lo <= AF_BUF ? buf : C.big_buf;
+      uint32_t* b = hi - lo <= AF_BUF ? buf : big_area(A) + A.big_cap / 4u + A.big_cap / 2u;
       uint32_t n = 0;
-      if (hi - lo <= A.big_cap) {
+      bool ok = hi - lo <= A.big_cap;
+      if (ok)
         for (uint32_t base = lo; base < hi; base += 32) {
           const uint32_t k = base + lane;
           const uint32_t it = k < hi ? J.items[k] : 0u;
           bool take = k < hi && ((it >> 16) != self || (it & 0xFFFFu) == ITEM_START);
-          if (take && k > lo && J.items[k - 1u] == it - 1u && (it & 0xFFFFu) != 0u) {  // the item before it skips to it
-            const uint32_t d = (it & 0xFFFFu) - 1u;
-            take = !((__ldg(&G.info[d]) & INFO_NULLABLE) && __ldg(&G.ga_root[d]) != GA_DEAD);
-          }
+          if (take && k > lo && (it & 0xFFFFu) != 0u && J.items[k - 1u] == it - 1u)  // the item before it skips to it
+            take = !(__ldg(&G.ga_item[4u * ((it & 0xFFFFu) - 1u) + 3u]) & GA_SKIPS);
           const uint32_t bal = __ballot_sync(FULL, take);
           if (take) b[n + __popc(bal & ((1u << lane) - 1u))] = (it << 16) | (it >> 16);
           n += __popc(bal);
         }
-        __syncwarp();
-      }
+      __syncwarp();
       uint2 list = make_uint2(0u, 0u);
-      const bool ok = hi - lo <= A.big_cap && group_items(G, C, ctl, b, n, list) && list.y <= A.stack_cap;
+      Contexts C = C0;
+      if (ok && !(ok = group_items(G, C, ctl, b, n, list))) {
+        spill_contexts(C, ctl, A);
+        ok = group_items(G, C, ctl, b, n, list);  // (sorted and without repeats already)
+      }
+      if (list.y > AF_BATCH) ok = false, list.y = 0u;
       const uint4 root = __ldg(reinterpret_cast<const uint4*>(G.ga_node));
       uint32_t top = 0;
-      if (ok)
-        for (uint32_t base = 0; base < list.y; base += 32) {
-          const uint32_t i = base + lane;
-          const uint2 x = i < list.y ? reinterpret_cast<const uint2*>(C.pool)[list.x / 2u + i] : make_uint2(0u, 0u);
-          const uint32_t wide = i < list.y ? __ldg(&G.ga_wide[x.y >> 16]) : GA_DEAD;
-          uint4 en = make_uint4(root.x, root.y >> 8, x.x, x.y & 0xFFFFu);
-          if (wide != GA_DEAD) {  // most of the vocabulary follows from this item alone
-            const uint4 r = __ldg(reinterpret_cast<const uint4*>(G.ga_wide_rec) + wide);
-            en = make_uint4(r.y, r.z, AF_EXITS, en.w);
-            const uint32_t at = atomicAdd(&ctl[AC_NWIDE], 1u);
-            if (at < AC_WORDS - AC_WIDE) ctl[AC_WIDE + at] = r.x;
-            else ctl[AC_FAIL] = 1u + DIAG_SET_SCRATCH;
+      for (uint32_t base = 0; base < list.y; base += 32) {
+        const uint32_t i = base + lane;
+        const uint2 x = i < list.y ? reinterpret_cast<const uint2*>(C.pool)[list.x / 2u + i] : make_uint2(0u, 0u);
+        const uint32_t wide = i < list.y ? __ldg(&G.ga_item[4u * (x.y >> 16) + 2u]) : GA_DEAD;
+        uint4 en = make_uint4(root.x, root.y >> 8, x.x, x.y & 0xFFFFu);
+        if (wide != GA_DEAD) {  // most of the vocabulary follows from this item alone
+          const uint4 r = __ldg(reinterpret_cast<const uint4*>(G.ga_wide_rec) + wide);
+          const uint32_t at = atomicAdd(&ctl[AC_NWIDE], 1u);
+          if (at < AF_EXITS) {
+            ctl[AC_WIDE + at] = r.x;
+            if (r.z) exits[atomicAdd(&ctl[AC_NEXITS], 1u)] = make_uint4(r.y, r.z, 0u, en.w);
+          } else {
+            ok = false;
           }
-          const bool take = i < list.y && en.y != 0u;
-          const uint32_t bal = __ballot_sync(FULL, take);
-          if (take) stack[top + __popc(bal & ((1u << lane) - 1u))] = en;
-          top += __popc(bal);
         }
+        ok = __all_sync(FULL, ok);
+        const bool take = i < list.y && en.y != 0u && wide == GA_DEAD;
+        const uint32_t bal = __ballot_sync(FULL, take);
+        if (take) entries[top + __popc(bal & ((1u << lane) - 1u))] = en;
+        top += __popc(bal);
+      }
       if (lane == 0) {
-        ctl[AC_TOP] = top;
+        ctl[AC_NEXT] = top;
         if (!ok) ctl[AC_FAIL] = 1u + DIAG_SET_SCRATCH;
       }
     }
     __syncthreads();
-    for (uint32_t k = 0, nw = min(ctl[AC_NWIDE], AC_WORDS - AC_WIDE); k < nw; ++k) {
-      const uint32_t* row_of = G.ga_wide_mask + (size_t)ctl[AC_WIDE + k] * G.Wm;
-      for (uint32_t i = part * AF_THREADS + tid; i < G.Wm; i += parts * AF_THREADS) mask[i] |= __ldg(row_of + i);
-    }
-    __syncthreads();
-
-    for (;;) {  // ---- rounds
-      const uint32_t top = ctl[AC_TOP];
-      if (top == 0u || ctl[AC_FAIL]) break;
-      // (a crowded stack is taken in smaller pieces, which keeps it from growing: depth first)
-      const uint32_t room = A.stack_cap - top;
-      const uint32_t n = min(top, max(1u, min(AF_BATCH, room / 16u)));
-      bool missing = false;
-      uint4 mine[AF_BATCH / AF_THREADS];
-#pragma unroll
-      for (uint32_t u = 0; u < AF_BATCH / AF_THREADS; ++u) {
-        const uint32_t i = tid * (AF_BATCH / AF_THREADS) + u;
-        if (i < n) {
-          mine[u] = stack[top - n + i];
-          cur[i] = mine[u];
-          if (mine[u].z == AF_SPAWN || mine[u].z == AF_EXITS) missing |= C.exp[mine[u].w].y == CTX_NEW;
-        }
+    if (!unit && part == 0u) {  // the mask begins with what follows from wide items, and the end of the sequence
+      const uint32_t nw = min(ctl[AC_NWIDE], AF_EXITS);
+      for (uint32_t i = tid; i < G.Wm; i += AF_THREADS) {
+        uint32_t v = (accepting && G.eos >= 0 && i == (uint32_t)G.eos >> 5) ? 1u << ((uint32_t)G.eos & 31u) : 0u;
+        for (uint32_t k = 0; k < nw; ++k) v |= __ldg(&G.ga_wide_mask[(size_t)ctl[AC_WIDE + k] * G.Wm + i]);
+        mask[i] = v;
       }
-      const bool expand = __syncthreads_or(missing) != 0;
-      if (tid == 0) ctl[AC_TOP] = top - n;
-      if (expand) {
-        if (warp == 0)
-          for (uint32_t base = 0; base < n; base += 32) {
-            const uint32_t i = base + lane;
-            const uint32_t c = i < n && (cur[i].z == AF_SPAWN || cur[i].z == AF_EXITS) ? cur[i].w : 0xFFFFFFFFu;
-            uint32_t todo = __ballot_sync(FULL, c != 0xFFFFFFFFu && C.exp[c].y == CTX_NEW);
-            while (todo) {
-              const uint32_t x = __shfl_sync(FULL, c, __ffs(todo) - 1);
-              if (!expand_context(G, C, J, x, ctl, work, hset, buf) && lane == 0) ctl[AC_FAIL] = 1u + DIAG_SET_TABLE;
-              todo &= ~__ballot_sync(FULL, c == x);
+      if (parts > 1u) {
+        __threadfence();
+        __syncthreads();
+        if (tid == 0) asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(A.unit_flag + A.unit_cap + j), "r"(S.gen) : "memory");
+      }
+    } else if (!unit) {  // the block that began with the row writes that
+      if (tid == 0)
+        for (uint32_t polls = 0; ld_acquire(A.unit_flag + A.unit_cap + j) != S.gen; ++polls) {
+          if (polls > poll_limit(S, 22)) {
+            diag(S, DIAG_WAIT_GRID);
+            atomicExch(&S.counters[CNT_BAR_ERR], 1u);
+            ctl[AC_FAIL] = AF_GIVEN_UP;
+            break;
+          }
+          if (polls) __nanosleep(64);
+        }
+      __syncthreads();
+    }
+    const uint32_t looked_up_before = looked_up;
+
+    bool spilled = false;
+    // the expansion of a context (offset into pool, count), and its elements
+    auto expansion = [&](uint32_t c) -> uint2 { return spilled ? global_contexts(A).exp[c] : C0.exp[c]; };
+    auto element = [&](uint32_t off, uint32_t k) -> uint2 {
+      return spilled ? reinterpret_cast<const uint2*>(global_contexts(A).pool)[off / 2u + k] : reinterpret_cast<const uint2*>(C0.pool)[off / 2u + k];
+    };
+    // false: this thread was started here a moment ago
+    auto start = [&](uint32_t first, uint32_t rule_ctx) -> bool {
+      const uint32_t slot = (first * 0x9E3779B1u ^ rule_ctx * 0x85EBCA6Bu) >> 23;
+      static_assert(AF_SEEN == 512, "the slot is the upper nine bits");
+      const unsigned long long key = (unsigned long long)first << 32 | rule_ctx;
+      volatile unsigned long long* p = seen + slot;
+      const bool fresh = *p != key;
+      *p = key;
+      return fresh;
+    };
+    for (;;) {  // ---- rounds
+      uint4* const cur = entries + side * AF_BATCH;
+      uint4* const nxt = entries + (side ^ 1u) * AF_BATCH;
+      uint4* const spec = specials + side * AF_SPEC;
+      uint4* const spec_nxt = specials + (side ^ 1u) * AF_SPEC;
+      uint32_t n = min(ctl[AC_NEXT], AF_BATCH), ns = min(ctl[AC_SPEC], AF_SPEC), gtop = ctl[AC_GTOP], gspec = ctl[AC_GSPEC], nx = ctl[AC_NEXITS];
+      if (ctl[AC_FAIL] || n + ns + gtop + gspec + nx == 0u) break;
+      spilled = ctl[AC_SPILLED] != 0u;
+      const uint32_t waiting = ctl[AC_WAITING];
+      __syncthreads();
+      if (tid == 0) ctl[AC_NEXT] = 0u, ctl[AC_SPEC] = 0u, ctl[AC_OVF] = 0u, ctl[AC_SOVF] = 0u;
+      if (tid == AF_THREADS - 1) {  // (looked at in the next round)
+        const uint32_t t = vload(&S.counters[CNT_AF_TAKEN]), p = vload(&S.counters[CNT_AF_POSTED]);
+        ctl[AC_WAITING] = t > p ? t - p : 0u;
+      }
+      // a crowded stack: fewer threads at once, which keeps it from growing (depth first)
+      const uint32_t threads_cap = A.stack_cap - AF_SPEC_STACK;
+      const uint32_t most = max(1u, min(AF_BATCH, (threads_cap - gtop) / 16u));
+      if (n < most && gtop) {
+        const uint32_t take = min(most - n, gtop);
+        for (uint32_t i = tid; i < take; i += AF_THREADS) cur[n + i] = stack[gtop - take + i];
+        n += take, gtop -= take;
+      } else if (n > most) {
+        for (uint32_t i = most + tid; i < n; i += AF_THREADS) stack[gtop + i - most] = cur[i];
+        gtop += n - most, n = most;
+      }
+      if (gspec && ns < AF_SPEC) {
+        const uint32_t take = min(AF_SPEC - ns, gspec);
+        if (tid < take) spec[ns + tid] = stack[threads_cap + gspec - take + tid];
+        ns += take, gspec -= take;
+      }
+      __syncthreads();
+      const uint32_t room = threads_cap - gtop;
+      auto overflow = [&](const uint4& v) {
+        const uint32_t p = atomicAdd(&ctl[AC_OVF], 1u);
+        if (p < room) stack[gtop + p] = v;
+        else ctl[AC_FAIL] = 1u + DIAG_QUEUE_FULL;
+      };
+      auto overflow_special = [&](const uint4& v) {
+        const uint32_t p = atomicAdd(&ctl[AC_SOVF], 1u);
+        if (gspec + p < AF_SPEC_STACK) stack[threads_cap + gspec + p] = v;
+        else ctl[AC_FAIL] = 1u + DIAG_QUEUE_FULL;
+      };
+      if (ns + nx) {
+        // ---- expansions: contexts that have none yet, then the threads they start, in this very round as far as there is room
+        const bool list = nx != 0u && n < AF_BATCH / 2u;  // a list of nodes waits its turn
+        const uint4 ex = list ? exits[nx - 1u] : make_uint4(0u, 0u, 0u, 0u);
+        const uint4 en = tid < ns ? spec[tid] : make_uint4(0u, 0u, 0u, 0u);
+        if (__syncthreads_or((tid < ns && expansion(en.w).y == CTX_NEW) || (list && tid == 0 && expansion(ex.w).y == CTX_NEW))) {
+          if (warp == 0) {
+            Contexts C = spilled ? global_contexts(A) : C0;
+            for (uint32_t base = 0; base <= ns; base += 32) {  // (the list's comes last)
+              const uint32_t i = base + lane;
+              const uint32_t c = i < ns ? spec[i].w : i == ns && list ? ex.w : CTX_NEW;
+              for (uint32_t todo = __ballot_sync(FULL, c != CTX_NEW && C.exp[c].y == CTX_NEW); todo;) {
+                const uint32_t x = __shfl_sync(FULL, c, __ffs(todo) - 1);
+                if (!expand_context(G, A, C, J, x, ctl, work, hset, buf) && lane == 0) ctl[AC_FAIL] = 1u + DIAG_SET_TABLE;
+                todo &= ~__ballot_sync(FULL, c == x);
+              }
             }
           }
+          __syncthreads();
+          spilled = ctl[AC_SPILLED] != 0u;
+        }
+        if (tid == 0) ctl[AC_NBUF] = n;
         __syncthreads();
+        auto begin = [&](bool yes, uint32_t first, uint32_t kids, const uint2& el) {  // (by all lanes of a warp)
+          yes = yes && start(first, el.y);
+          const uint32_t bal = __ballot_sync(FULL, yes);
+          if (bal == 0u) return;
+          uint32_t at = 0;
+          if (lane == 0) at = atomicAdd(&ctl[AC_NBUF], __popc(bal));
+          at = __shfl_sync(FULL, at, 0) + __popc(bal & ((1u << lane) - 1u));
+          const uint4 v = make_uint4(first, kids, el.x, el.y & 0xFFFFu);
+          if (yes && at < AF_BATCH) cur[at] = v;
+          else if (yes) overflow(v);
+        };
+        if (warp * 32u < ns) {
+          const uint2 x = tid < ns ? expansion(en.w) : make_uint2(0u, 0u);
+          const uint32_t most_of = __reduce_max_sync(FULL, x.y);
+          for (uint32_t q = 0; q < most_of; ++q) begin(q < x.y, en.x, en.y, q < x.y ? element(x.x, q) : make_uint2(0u, 0u));
+        }
+        if (list) {
+          const uint2 x = expansion(ex.w);
+          const uint32_t nodes = x.y ? min(ex.y, max(parts * (AF_BATCH / 2u / x.y), 32u)) : ex.y;
+          if (x.y)
+            for (uint32_t base = warp * 32u; base < nodes; base += AF_THREADS) {
+              bool v = base + lane < nodes;
+              const uint2 nd = v ? __ldg(reinterpret_cast<const uint2*>(G.ga_wide_exit) + ex.x + base + lane) : make_uint2(0u, 0u);
+              // (blocks that share a row all start the threads of nodes of depth 1, and deal out the others)
+              if (parts > 1u && (nd.x < G.ga_lvl2 || nd.x >= G.ga_lvl3)) v = v && (base + lane) % parts == part;
+              for (uint32_t q = 0; q < x.y; ++q) begin(v, nd.x, nd.y, element(x.x, q));
+            }
+          __syncthreads();
+          if (tid == 0) {
+            if (nodes == ex.y) ctl[AC_NEXITS] = nx - 1u;
+            else exits[nx - 1u] = make_uint4(ex.x + nodes, ex.y - nodes, 0u, ex.w);
+          }
+        }
+        __syncthreads();
+        n = min(ctl[AC_NBUF], AF_BATCH);
       }
-      // the items of work: a thread's children, an expansion's elements (at least one each, so that all starts differ)
-      uint32_t w[AF_BATCH / AF_THREADS], sum = 0;
+      if (waiting && n >= AF_SHARE && looked_up - looked_up_before >= AF_HEAVY && !spilled) {
+        // ---- other blocks wait: entry i stays here when i is a multiple of units + 1, else it goes to unit i % (units + 1) - 1
+        const uint32_t units = min(min(waiting, n / 128u - 1u), AF_MAX_UNITS);
+        if (tid == 0) {
+          const uint32_t at = atomicAdd(&S.counters[CNT_AF_POSTED], units);
+          const uint32_t fit = at >= A.unit_cap ? 0u : min(units, A.unit_cap - at);
+          if (fit == units) atomicAdd(&S.counters[CNT_AF_ACTIVE], units);
+          ctl[AC_BASE] = fit == units ? at : 0xFFFFFFFFu;  // (near the end of the units' storage nothing is given any more)
+        }
+        __syncthreads();
+        const uint32_t at = ctl[AC_BASE];
+        if (at != 0xFFFFFFFFu) {
+          const uint32_t nc = ctl[AC_NCTX], np = ctl[AC_POOL];
+          const uint32_t* src = reinterpret_cast<const uint32_t*>(C0.org);
+          for (uint32_t u = 0; u < units; ++u) {
+            uint32_t* dst = A.units + (size_t)(at + u) * AU_WORDS;
+            for (uint32_t i = tid; i < 5u * AF_CTX + np; i += AF_THREADS) dst[AU_HDR + i] = src[i];
+            if (tid == 0) dst[AU_ROWJOB] = j, dst[AU_N] = (n + units - 1u - u) / (units + 1u), dst[AU_NCTX] = nc, dst[AU_POOL] = np, dst[AU_PART] = part;
+          }
+          uint4 keep[AF_PER];
 #pragma unroll
-      for (uint32_t u = 0; u < AF_BATCH / AF_THREADS; ++u) {
-        const uint32_t i = tid * (AF_BATCH / AF_THREADS) + u;
-        w[u] = i >= n ? 0u
-               : mine[u].z == AF_SPAWN ? max(1u, C.exp[mine[u].w].y)
-               : mine[u].z == AF_EXITS ? min(mine[u].y, AF_EXIT_PIECE) * max(1u, C.exp[mine[u].w].y) : mine[u].y;
+          for (uint32_t k = 0; k < AF_PER; ++k) {
+            const uint32_t i = k * AF_THREADS + tid;
+            if (i < n) {
+              keep[k] = cur[i];
+              const uint32_t to = i % (units + 1u);
+              if (to)
+                reinterpret_cast<uint4*>(A.units + (size_t)(at + to - 1u) * AU_WORDS + AU_HDR + 5 * AF_CTX + AF_POOL)[i / (units + 1u)] = keep[k];
+            }
+          }
+          __threadfence();
+          __syncthreads();
+          if (tid < units) asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(A.unit_flag + at + tid), "r"(S.gen) : "memory");
+#pragma unroll
+          for (uint32_t k = 0; k < AF_PER; ++k) {
+            const uint32_t i = k * AF_THREADS + tid;
+            if (i < n && i % (units + 1u) == 0u) cur[i / (units + 1u)] = keep[k];
+          }
+          n = (n + units) / (units + 1u);
+          __syncthreads();
+        }
+      }
+      // ---- the threads' children, 32 to a piece
+      uint32_t w[AF_PER], sum = 0;
+#pragma unroll
+      for (uint32_t u = 0; u < AF_PER; ++u) {
+        const uint32_t i = tid * AF_PER + u;
+        w[u] = i < n ? cur[i].y : 0u;
         sum += w[u];
       }
       uint32_t incl = sum;
@@ -396,133 +729,107 @@ __global__ void __launch_bounds__(AF_THREADS) automaton_fill_kernel(const __grid
         total += s;
       }
 #pragma unroll
-      for (uint32_t u = 0; u < AF_BATCH / AF_THREADS; ++u) {
-        const uint32_t i = tid * (AF_BATCH / AF_THREADS) + u;
+      for (uint32_t u = 0; u < AF_PER; ++u) {
+        const uint32_t i = tid * AF_PER + u;
         if (i <= n) pre[i] = before;  // (pre[n] = the total)
+        for (uint32_t piece = (before + 31u) / 32u; piece * 32u < before + w[u]; ++piece) owner[piece] = (uint16_t)i;
         before += w[u];
       }
       if (n == AF_BATCH && tid == 0) pre[n] = total;
       looked_up += total;
       __syncthreads();
       for (uint32_t base = warp * 32u; base < total; base += AF_THREADS) {
-        // the entry that item `base` belongs to (all lanes the same search), then each lane's own
-        uint32_t lo = 0, hi = n;
-        while (hi - lo > 1u) {
-          const uint32_t mid = (lo + hi) >> 1;
-          if (pre[mid] <= base) lo = mid;
-          else hi = mid;
-        }
-        const uint32_t nb = lo + 1u + lane <= n ? pre[lo + 1u + lane] - base : 32u;
+        const uint32_t lo = owner[base / 32u];
+        const uint32_t nb = lo + 1u + lane <= n ? pre[lo + 1u + lane] - base : 32u;  // where the threads after it begin
         const uint32_t starts = __reduce_or_sync(FULL, nb < 32u ? 1u << nb : 0u);
-        const uint32_t i = base + lane;
         const uint32_t e = lo + __popc(starts & (0xFFFFFFFFu >> (31u - lane)));
-        // what the item pushes: `a` (a thread that goes on, or tokens), `b` and `c` (threads that start here)
-        bool has_a = false, has_b = false, has_c = false;
-        uint4 a, b, c;
-        auto start = [&](uint32_t first, uint32_t rule, uint32_t ctx) {  // false: it was started here a moment ago
-          const unsigned long long key = (unsigned long long)first << 32 | rule << 16 | ctx;
-          return atomicExch(&seen[(mix32(first ^ (rule * 0x9E3779B1u)) + ctx) & (AF_SEEN - 1u)], key) != key;
-        };
-        if (i < total) {
-          const uint4 en = cur[e];
-          const uint32_t k = i - pre[e];
-          if (en.z < AF_TOKENS) {
-            const uint32_t child = en.x + k;
-            // a cluster's blocks share the nodes of depth 2, and with them what lies below
-            if (parts == 1u || child < G.ga_lvl2 || child >= G.ga_lvl3 || child % parts == part) {
-              const uint4 nd = __ldg(reinterpret_cast<const uint4*>(G.ga_node) + child);
-              const uint32_t t = ga_next(G, en.z, nd.y & 0xFFu);
-              if (t == GA_UNKNOWN) ctl[AC_FAIL] = 1u + DIAG_ROOT_FAILED;  // (cannot happen: the automaton covers the vocabulary)
-              else if (t != GA_DEAD) {
-                const uint32_t kids = nd.y >> 8;
-                if (nd.w == 1u) atomicOr(&mask[nd.z >> 5], 1u << (nd.z & 31u));
-                else if (nd.w > 1u) has_c = true, c = make_uint4(nd.z, nd.w, AF_TOKENS, 0u);
-                if (kids) {
-                  if ((t & ~GA_EXIT) != GA_NONE) has_a = true, a = make_uint4(nd.x, kids, t & ~GA_EXIT, en.w);
-                  if (t & GA_EXIT) {
-                    const uint2 x = C.exp[en.w];
-                    if (x.y == 1u) {
-                      const uint2 el = reinterpret_cast<const uint2*>(C.pool)[x.x / 2u];
-                      has_b = start(nd.x, el.y >> 16, el.y & 0xFFFFu);
-                      b = make_uint4(nd.x, kids, el.x, el.y & 0xFFFFu);
-                    } else if (x.y) {
-                      has_b = start(nd.x, 0xFFFFu, en.w);
-                      b = make_uint4(nd.x, kids, AF_SPAWN, en.w);
-                    }
-                  }
+        bool goes_on = false, starts_one = false, special = false;
+        uint4 a, b;
+        uint4 nd = make_uint4(0u, 0u, 0u, 0u);
+        uint32_t many = 0;
+        uint4 en = make_uint4(0u, 0u, 0u, 0u);
+        uint32_t child = 0;
+        bool ours = base + lane < total;
+        if (ours) {
+          en = cur[e];
+          child = en.x + (base + lane - pre[e]);
+          // blocks that share a row share the nodes of depth 2, and with them what lies below
+          if (parts > 1u && child >= G.ga_lvl2 && child < G.ga_lvl3) ours = child % parts == part;
+        }
+        if (ours) {
+          nd = __ldg(reinterpret_cast<const uint4*>(G.ga_node) + child);
+          const uint32_t t = ga_next(G, en.z, nd.y & 0xFFu);
+          if (t < GA_UNKNOWN) {
+            if (nd.w == 1u) atomicOr(&mask[nd.z >> 5], 1u << (nd.z & 31u));
+            else many = nd.w;
+            const uint32_t kids = nd.y >> 8;
+            if (kids) {
+              goes_on = (t & ~GA_EXIT) != GA_NONE;
+              a = make_uint4(nd.x, kids, t & ~GA_EXIT, en.w);
+              if (t & GA_EXIT) {
+                const uint2 x = expansion(en.w);
+                if (x.y) {
+                  const uint2 el = x.y == 1u ? element(x.x, 0u) : make_uint2(AF_SPAWN, 0xFFFF0000u | en.w);
+                  starts_one = start(nd.x, el.y);
+                  special = starts_one && x.y != 1u;
+                  b = make_uint4(nd.x, kids, el.x, el.y & 0xFFFFu);
                 }
               }
             }
-          } else if (en.z == AF_TOKENS) {
-            const uint32_t tok = __ldg(&G.ga_tok[en.x + k]);
-            atomicOr(&mask[tok >> 5], 1u << (tok & 31u));
-          } else {
-            const uint2 x = C.exp[en.w];
-            if (x.y) {
-              uint2 nd = make_uint2(en.x, en.y);
-              uint32_t q = k;
-              bool ours = true;
-              if (en.z == AF_EXITS) {
-                if (k == 0u && en.y > AF_EXIT_PIECE)  // the rest of the list
-                  has_a = true, a = make_uint4(en.x + AF_EXIT_PIECE, en.y - AF_EXIT_PIECE, AF_EXITS, en.w);
-                nd = __ldg(reinterpret_cast<const uint2*>(G.ga_wide_exit) + en.x + k / x.y);
-                q = k % x.y;
-                // (a cluster's blocks all start the threads of nodes of depth 1 and deal out the others)
-                ours = parts == 1u || (nd.x >= G.ga_lvl2 && nd.x < G.ga_lvl3) || (k / x.y) % parts == part;
-              }
-              if (ours) {
-                const uint2 el = reinterpret_cast<const uint2*>(C.pool)[x.x / 2u + q];
-                has_b = start(nd.x, el.y >> 16, el.y & 0xFFFFu);
-                b = make_uint4(nd.x, nd.y, el.x, el.y & 0xFFFFu);
-              }
-            }
+          } else if (t == GA_UNKNOWN) {
+            ctl[AC_FAIL] = 1u + DIAG_ROOT_FAILED;  // (cannot happen: the automaton covers the vocabulary)
           }
         }
         __syncwarp();
-        const uint32_t ba = __ballot_sync(FULL, has_a), bb = __ballot_sync(FULL, has_b), bc = __ballot_sync(FULL, has_c);
-        if (ba | bb | bc) {
-          const uint32_t lt = (1u << lane) - 1u, count = __popc(ba) + __popc(bb) + __popc(bc);
-          uint32_t at = 0;
-          if (lane == 0) at = atomicAdd(&ctl[AC_TOP], count);
-          at = __shfl_sync(FULL, at, 0);
-          if (at + count > A.stack_cap) {
-            ctl[AC_FAIL] = 1u + DIAG_QUEUE_FULL;
-          } else {
-            if (has_a) stack[at + __popc(ba & lt)] = a;
-            at += __popc(ba);
-            if (has_b) stack[at + __popc(bb & lt)] = b;
-            at += __popc(bb);
-            if (has_c) stack[at + __popc(bc & lt)] = c;
+        // nodes at which several tokens end: their bits are set by the whole warp
+        for (uint32_t mm = __ballot_sync(FULL, many != 0u); mm; mm &= mm - 1u) {
+          const int src = __ffs(mm) - 1;
+          const uint32_t at = __shfl_sync(FULL, nd.z, src), cnt = __shfl_sync(FULL, many, src);
+          for (uint32_t k = lane; k < cnt; k += 32) {
+            const uint32_t tok = __ldg(&G.ga_tok[at + k]);
+            atomicOr(&mask[tok >> 5], 1u << (tok & 31u));
           }
         }
+        const uint32_t ba = __ballot_sync(FULL, goes_on), bb = __ballot_sync(FULL, starts_one && !special);
+        if (ba | bb) {
+          const uint32_t lt = (1u << lane) - 1u;
+          uint32_t at = 0;
+          if (lane == 0) at = atomicAdd(&ctl[AC_NEXT], __popc(ba) + __popc(bb));
+          at = __shfl_sync(FULL, at, 0);
+          if (goes_on) {
+            const uint32_t p = at + __popc(ba & lt);
+            if (p < AF_BATCH) nxt[p] = a;
+            else overflow(a);
+          }
+          if (starts_one && !special) {
+            const uint32_t p = at + __popc(ba) + __popc(bb & lt);
+            if (p < AF_BATCH) nxt[p] = b;
+            else overflow(b);
+          }
+        }
+        if (special) {
+          const uint32_t p = atomicAdd(&ctl[AC_SPEC], 1u);
+          if (p < AF_SPEC) spec_nxt[p] = b;
+          else overflow_special(b);
+        }
       }
+      side ^= 1u;
+      __syncthreads();
+      if (tid == 0) ctl[AC_GTOP] = gtop + ctl[AC_OVF], ctl[AC_GSPEC] = gspec + ctl[AC_SOVF];
       __syncthreads();
     }
-    // ---- the mask row
-    __syncthreads();
-    const uint32_t fail = ctl[AC_FAIL];
     contexts += ctl[AC_NCTX];
-    if (fail && tid == 0) {  // a capacity was exceeded: the row's mask cannot be trusted
-      diag(S, fail - 1u);
+    if (tid == 0 && ctl[AC_FAIL] && ctl[AC_FAIL] != AF_GIVEN_UP) {  // a capacity was exceeded: the row's mask cannot be trusted
+      diag(S, ctl[AC_FAIL] - 1u);
       if (!(atomicOr(&S.row_flags[row], ROW_BROKEN) & ROW_BROKEN)) stat_add(S, CNT_STAT_CAPERR, 1u);
       atomicExch(&S.counters[CNT_ERR], 1u);
     }
-    if (tid == 0 && accepting && G.eos >= 0) atomicOr(&mask[(uint32_t)G.eos >> 5], 1u << ((uint32_t)G.eos & 31u));
-    if (parts > 1u) {
-      cluster.sync();
-      for (uint32_t i = part * AF_THREADS + tid; i < G.Wm; i += parts * AF_THREADS) {
-        uint32_t v = 0;
-        for (uint32_t p = 0; p < parts; ++p) v |= *cluster.map_shared_rank(mask_sm + i, p);
-        out[i] = v;
-      }
-      cluster.sync();
-    } else if (in_smem) {
-      __syncthreads();
-      for (uint32_t i = tid; i < G.Wm; i += AF_THREADS) out[i] = mask_sm[i];
-    }
+    // ---- the next row
+    __threadfence();
     __syncthreads();
+    if (tid == 0) atomicSub(&S.counters[CNT_AF_ACTIVE], 1u);
   }
-  if (tid == 0 && contexts) {
+  if (tid == 0 && looked_up) {
     stat_add(S, CNT_STAT_TRANS, looked_up);
     stat_add(S, CNT_STAT_LOCAL, contexts);
   }
@@ -530,35 +837,23 @@ __global__ void __launch_bounds__(AF_THREADS) automaton_fill_kernel(const __grid
 
 // ===================================================================================== launchers
 
-static uint32_t fill_smem_bytes(const GrammarDev& G) {
-  return AF_BATCH * 16u + AF_SEEN * 8u + (AF_BATCH + 4u + AC_WORDS + AF_STAGE + AF_BUF + AF_WORK + AF_HSET + (G.Wm <= AF_MASK_SMEM ? G.Wm : 0u)) * 4u;
-}
+constexpr uint32_t AF_SMEM = (2 * AF_BATCH + 2 * AF_SPEC + AF_EXITS) * 16 + AF_SEEN * 8 + AF_OWNER * 2 + (5 * AF_CTX + AF_POOL + AF_CTX_HASH + AF_BATCH + 4 + AC_WORDS + AF_STAGE + AF_BUF + AF_WORK + AF_HSET) * 4;
 
 void automaton_fill_layout(const GrammarDev& G, uint32_t rows, uint32_t max_blocks, AutoFillDev& A) {
-  A.smem_bytes = fill_smem_bytes(G);
   A.scratch_words = 7u * A.ctx_cap + A.pool_cap + A.big_cap / 4u + A.big_cap / 2u + A.big_cap;
-  // few rows: a cluster of blocks takes one, so that the chip is filled; many: one block each
+  A.unit_words = AU_WORDS;
+  // few rows: several blocks take one, so that the chip is filled (a small trie gives the others nothing to do)
   A.parts = 1;
-  while (A.parts < 8u && G.Wm <= AF_MASK_SMEM && (uint64_t)rows * A.parts * 2u <= max_blocks) A.parts *= 2u;
-  A.grid = std::min(rows, std::max(1u, max_blocks / A.parts)) * A.parts;
+  while (A.parts < 8u && (uint64_t)rows * A.parts * 2u <= max_blocks && A.parts * 2048u <= G.T) A.parts *= 2u;
+  A.grid = (uint32_t)std::min<uint64_t>(max_blocks, (uint64_t)rows * std::max(A.parts, 1u + G.T / 16384u));
 }
 
 cudaError_t configure_automaton_fill() {
-  return cudaFuncSetAttribute((const void*)automaton_fill_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 100 * 1024);
+  return cudaFuncSetAttribute((const void*)automaton_fill_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, AF_SMEM);
 }
 
 void launch_automaton_fill(const GrammarDev& G, const StateDev& S, cudaStream_t st) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(S.af.grid);
-  cfg.blockDim = dim3(AF_THREADS);
-  cfg.dynamicSmemBytes = S.af.smem_bytes;
-  cfg.stream = st;
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = S.af.parts, at[0].val.clusterDim.y = 1, at[0].val.clusterDim.z = 1;
-  cfg.attrs = at;
-  cfg.numAttrs = 1;
-  cudaLaunchKernelEx(&cfg, automaton_fill_kernel, G, S);
+  automaton_fill_kernel<<<S.af.grid, AF_THREADS, AF_SMEM, st>>>(G, S);
 }
 
 }  // namespace fmt

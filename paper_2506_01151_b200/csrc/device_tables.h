@@ -37,13 +37,12 @@ struct GrammarDev {
   const uint32_t* tok_ids;
   // the grammar automaton over the vocabulary (see host_tables.h), if the grammar has one
   uint32_t ga_on, ga_acc_mask;
-  const uint32_t* ga_root;       // [D]
+  const uint32_t* ga_item;       // [D][4]
   const uint32_t* ga_trans;      // [sets][n_eq]
   const uint32_t* ga_acc;        // [ga_acc_mask + 1][2]
   const uint32_t* ga_node;       // [nodes][4]
   const uint32_t* ga_tok;
-  uint32_t ga_lvl2, ga_lvl3;
-  const uint32_t* ga_wide;       // [D]
+  uint32_t ga_lvl2, ga_lvl3;     // first nodes of depth 2 and 3
   const uint32_t* ga_wide_rec;   // [entries][4]
   const uint32_t* ga_wide_mask;  // [entries][Wm]
   const uint32_t* ga_wide_exit;  // [][2]
@@ -97,12 +96,16 @@ enum : uint32_t {
   CNT_STAT_JOBS_ROOT = 152,    // 64-bit: computed rows that started from a swept root
   CNT_STAT_JOBS_PLAIN = 154,   // 64-bit: computed rows that walked the whole trie themselves
   CNT_STAT_JOBS_MASK = 156,    // 64-bit: computed rows answered by their root's mask row alone
+  CNT_AF_TICKET = 186,         // rows handed out to the blocks of the automaton's fill, beyond one for each
+  CNT_AF_TAKEN = 187,          // tickets drawn for units of work
+  CNT_AF_POSTED = 188,         // units given
+  CNT_AF_ACTIVE = 189,         // shares of rows, and units, that are not finished
   CNT_STAT_ABORTS = 160,       // 64-bit: fills abandoned because a bounded wait ran out
   CNT_STAT_STEP_CYCLES = 162,  // 64-bit: SM cycles spent inside Earley steps of the fill (summed over warps)
   CNT_STAT_ADV_WORDS = 164,    // 64-bit: chart words read and written by advance
   CNT_STAT_FRAMES = 184,       // 64-bit: frames made (sets of a walk recognised as roots)
   CNT_DIAG = 166,              // [16] where capacity errors and expired waits came from (see DIAG_*)
-  CNT_TOTAL = 186
+  CNT_TOTAL = 190
 };
 
 enum : uint32_t {
@@ -244,17 +247,20 @@ struct CtxDev {
   uint32_t req2_cap;
 };
 
-// What the fill by the grammar automaton needs (automaton_fill.cu): per thread block a stack of threads and the
-// contexts of the row it works on.
+// What the fill by the grammar automaton needs (automaton_fill.cu): per thread block a stack of threads and room for the
+// contexts of the row it works on, and units of work that blocks hand to one another.
 struct AutoFillDev {
   uint32_t on;               // rows are filled by the automaton
-  uint32_t grid, parts;      // thread blocks, and how many of them share a row (a cluster)
-  uint32_t smem_bytes;
+  uint32_t grid, parts;      // thread blocks, and how many of them share a row
   uint4* stack;              // [grid][stack_cap] first child, children, code, context
   uint32_t stack_cap;
   uint32_t* scratch;         // [grid][scratch_words]
   uint32_t scratch_words;
   uint32_t ctx_cap, pool_cap, big_cap;  // contexts per row, words for their lists, items of the largest expansion (powers of two)
+  uint32_t* units;           // [unit_cap][unit_words]
+  uint32_t* unit_flag;       // [unit_cap] the generation (StateDev::gen) of the fill whose unit is there; then per row that of the fill
+                             // in which its mask has been begun
+  uint32_t unit_cap, unit_words;
 };
 
 struct StateDev {

@@ -387,6 +387,19 @@ class Builder {
 
   void finish_tables() {
     h_.ga_sets = (u32)sets_.size();
+    h_.ga_item.assign((size_t)h_.D * 4, 0u);
+    for (u32 d = 0; d < h_.D; ++d) {
+      u32* r = &h_.ga_item[(size_t)d * 4];
+      r[0] = h_.ga_root[d];
+      r[1] = h_.lhs[d] | 0xFFFF0000u;
+      r[2] = h_.ga_wide[d];
+      r[3] = 0xFFFFu;
+      if (kind(d) != KIND_NT) continue;
+      r[1] = h_.lhs[d] | arg(d) << 16;
+      const u32 skip = h_.skip[d + 1];
+      r[3] = (kind(d + 1) != KIND_END ? GA_GOES_ON : 0u) | (kind(d + 1 + skip) == KIND_END ? (u32)h_.lhs[d] : 0xFFFFu);
+      if ((h_.info[d] & INFO_NULLABLE) && h_.ga_root[d] != GA_DEAD) r[3] |= GA_SKIPS;
+    }
     if (trans_.empty()) trans_.push_back(GA_UNKNOWN);
     h_.ga_trans.swap(trans_);
     u32 cap = 16;

@@ -27,6 +27,8 @@ constexpr uint32_t MAX_NONTERMINALS = 4096;
 // for a kernel that is one item inside an automaton of a regular non-terminal; with GA_EXIT where a rule begun in the open
 // origin is completed.  GA_NONE: nothing is left but completed items.
 constexpr uint32_t GA_DEAD = 0xFFFFFFFFu, GA_UNKNOWN = 0xFFFFFFFEu, GA_ITEM = 1u << 31, GA_EXIT = 1u << 30, GA_NONE = GA_EXIT - 1u;
+constexpr uint32_t GA_GOES_ON = 1u << 31;  // ga_item: the rule does not end with the post-dot non-terminal
+constexpr uint32_t GA_SKIPS = 1u << 30;    // the kernel of the item holds the next item, too (the non-terminal is nullable)
 #ifdef __CUDACC__
 __host__ __device__
 #endif
@@ -83,6 +85,9 @@ struct HostTables {
   bool ga_on = false;
   uint32_t ga_sets = 0, ga_acc_mask = 0;
   std::vector<uint32_t> ga_root;   // [D] code of the kernel {(d, open)}
+  // per dotted rule d: ga_root[d] | left-hand side, post-dot non-terminal << 16 (0xFFFF if there is none) | wide entry or GA_DEAD |
+  // GA_* flags and the left-hand side if the rule may end right after that non-terminal, else 0xFFFF
+  std::vector<uint32_t> ga_item;   // [D][4]
   std::vector<uint32_t> ga_trans;  // [ga_sets][n_eq] code
   std::vector<uint32_t> ga_acc;    // [ga_acc_mask + 1][2] hash: set + 1 << 16 | automaton transition -> code
   // the vocabulary trie over byte classes, breadth first

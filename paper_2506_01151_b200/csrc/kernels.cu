@@ -312,6 +312,7 @@ __global__ void __launch_bounds__(1024) plan_kernel(GrammarDev G, StateDev S) {
     S.counters[CNT_N_JOBS] = 0u;
     S.counters[CNT_N_FJOBS] = 0u;
     S.counters[CNT_AUTO_ITEMS] = 0u;
+    S.counters[CNT_AF_TICKET] = S.counters[CNT_AF_TAKEN] = S.counters[CNT_AF_POSTED] = 0u;
   }
   if (S.rt.counters) {  // the root sweep of this fill starts from clean counters, too
     if (threadIdx.x < CNT_HASH_GEN - CNT_BAR) S.rt.counters[CNT_BAR + threadIdx.x] = 0u;
@@ -359,6 +360,8 @@ __global__ void __launch_bounds__(1024) plan_kernel(GrammarDev G, StateDev S) {
     uint32_t j = atomicAdd(&S.counters[CNT_N_JOBS], 1u);
     S.jobs[j] = row;
   }
+  __syncthreads();
+  if (threadIdx.x == 0) S.counters[CNT_AF_ACTIVE] = ld_acquire(&S.counters[CNT_N_JOBS]) * S.af.parts;
 }
 
 // ===================================================================================== fill: sweep

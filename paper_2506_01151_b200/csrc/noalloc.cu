@@ -49,11 +49,14 @@ constexpr size_t NA_OFF_ST = NA_OFF_ITEMS + NA_ITEM_WORDS;
 constexpr size_t NA_OFF_REQ = NA_OFF_ST + NA_ST_ENTRIES / 2;       // 8-byte aligned: all sizes above are even
 constexpr size_t NA_WORDS = NA_OFF_REQ + 2 * (size_t)NA_REQ_CAP;
 // the fill by the grammar's automaton uses the same array: per thread block a stack of threads and the contexts of a row
-constexpr uint32_t NA_FILL_BLOCKS = 64, NA_STACK = 16u << 10;
-constexpr uint32_t NA_CTX = 1024, NA_POOL = 16u << 10, NA_LARGE = 8u << 10;
+constexpr uint32_t NA_FILL_BLOCKS = 160, NA_STACK = 12u << 10;
+constexpr uint32_t NA_CTX = 1024, NA_POOL = 8u << 10, NA_LARGE = 4u << 10;
 constexpr uint32_t NA_FILL_SCRATCH = 7u * NA_CTX + NA_POOL + NA_LARGE / 4u + NA_LARGE / 2u + NA_LARGE;
+constexpr uint32_t NA_UNITS = 512, NA_UNIT_WORDS = 4096;  // units of work between blocks
 constexpr size_t NA_OFF_FILL = NA_HEADER_WORDS + 4 * (size_t)NA_FILL_BLOCKS * NA_STACK;
-static_assert(NA_OFF_FILL + (size_t)NA_FILL_BLOCKS * NA_FILL_SCRATCH <= NA_WORDS, "the fill's tables do not fit");
+constexpr size_t NA_OFF_UNIT_FLAG = NA_OFF_FILL + (size_t)NA_FILL_BLOCKS * NA_FILL_SCRATCH;
+constexpr size_t NA_OFF_UNITS = NA_OFF_UNIT_FLAG + NA_UNITS + NA_MAX;
+static_assert(NA_OFF_UNITS + (size_t)NA_UNITS * NA_UNIT_WORDS <= NA_WORDS && NA_OFF_UNITS % 4 == 0, "the fill's tables do not fit");
 static_assert(CNT_TOTAL <= NA_OFF_JOBS, "the counters overlap the job list");
 static_assert(NA_OFF_JOBINFO + 4 * NA_MAX <= NA_HEADER_WORDS, "header too small");
 static_assert((NA_OFF_JOBINFO % 4) == 0, "job records must be 16-byte aligned");
@@ -89,7 +92,10 @@ __global__ void noalloc_prepare_kernel(GrammarDev G, StateDev S, uint32_t* scrat
     S.row_flags[r] = 0u;
   }
   for (size_t i = tid; i < (size_t)n * G.Wm; i += nth) mask[i] = 0u;
-  if (S.af.on) return;
+  if (S.af.on) {
+    if (tid < NA_UNITS + NA_MAX) S.af.unit_flag[tid] = 0u;
+    return;
+  }
   for (size_t i = tid; i < (size_t)NA_MAX * NA_HASH_SLOTS; i += nth) S.au.hash[i] = 0u;
   for (size_t i = tid; i < NA_REQ_CAP; i += nth) S.au.req[i] = 0ull;  // no stale tags: every call is generation 1
   uint32_t* big = S.big_scratch;
@@ -127,6 +133,7 @@ __global__ void noalloc_jobs_kernel(StateDev S, const uint32_t* scratch, uint32_
   for (uint32_t r = 0; r < n; ++r)
     if (!scratch[NA_OFF_BAD + r]) S.jobs[j++] = r;
   S.counters[CNT_N_JOBS] = j;
+  S.counters[CNT_AF_ACTIVE] = j * S.af.parts;
 }
 
 __global__ void noalloc_finish_kernel(GrammarDev G, StateDev S, const uint32_t* scratch, uint32_t n, uint32_t* mask,
@@ -227,7 +234,11 @@ extern "C" fmt_status fmt_fill_mask_noalloc(const fmt_grammar* g, const uint32_t
     A.stack_cap = NA_STACK;
     A.scratch = scratch + NA_OFF_FILL;
     A.ctx_cap = NA_CTX, A.pool_cap = NA_POOL, A.big_cap = NA_LARGE;
+    A.unit_cap = NA_UNITS;
+    A.units = scratch + NA_OFF_UNITS;
+    A.unit_flag = scratch + NA_OFF_UNIT_FLAG;
     automaton_fill_layout(*G, n, NA_FILL_BLOCKS, A);
+    if (A.unit_words > NA_UNIT_WORDS || A.scratch_words > NA_FILL_SCRATCH) return fail(FMT_ERR_CAPACITY, "the built-in scratch does not fit the fill");
   }
   cudaStream_t st = (cudaStream_t)stream;
   noalloc_prepare_kernel<<<256, 256, 0, st>>>(*G, S, scratch, charts_dev, off, n, mask_dev);
