@@ -163,6 +163,103 @@ struct TokenView {
   }
 };
 
+// Scan and Complete (Section 3.2) for sets that outgrow a warp's lanes - an ambiguous grammar's, of a hundred items and more
+// out of as many origins.  What is in the set, and which (non-terminal, origin) have been completed, are bits in
+// shared memory, and the waiting items of all sets that a wave of completions asks are dealt out to the lanes together:
+// 58,000 cycles a byte in an ambiguous segment of sixty letters with a hash and one set asked after the other, now 15,000.  Returns the number of items in
+// s.w.cur, GEN_FULL when they outgrow it; the bits must fit (gen_fits).
+constexpr uint32_t GEN_FULL = 0xffffffffu;
+__device__ __forceinline__ bool gen_fits(const GrammarDev& G, uint32_t index) {
+  return G.D * (index + 1u) <= ADV_HSET * 32u && G.N * (index + 1u) <= ADV_PAIRS * 32u;
+}
+__device__ uint32_t gen_scan_complete(const GrammarDev& G, const AdvScratch& s, const TokenView& view, const uint32_t* set,
+                                      uint32_t len, uint32_t byte, uint32_t index) {
+  const uint32_t lane = lane_id(), lt = (1u << lane) - 1u, row = index + 1u;
+  uint32_t* const in_set = s.w.hset;   // [D][row] bits
+  uint32_t* const done = s.pairs;      // [N][row] bits
+  const uint32_t set_words = (G.D * row + 31u) / 32u, done_words = (G.N * row + 31u) / 32u;
+  __syncwarp();
+  for (uint32_t i = lane; i < set_words; i += 32) in_set[i] = 0u;
+  for (uint32_t i = lane; i < done_words; i += 32) done[i] = 0u;
+  __syncwarp();
+  uint32_t n = 0;
+  auto add = [&](bool v, uint32_t key) {  // by all lanes; the items reached over nullable non-terminals come along
+    const uint32_t more = v ? (G.info[key & 0xFFFFu] >> INFO_SKIP_SHIFT) & INFO_SKIP_MASK : 0u;
+    for (uint32_t j = 0;; ++j) {
+      bool fresh = false;
+      if (v && j <= more) {
+        const uint32_t at = ((key & 0xFFFFu) + j) * row + (key >> 16), bit = 1u << (at & 31u);
+        fresh = !(in_set[at >> 5] & bit) && !(atomicOr(&in_set[at >> 5], bit) & bit);
+      }
+      const uint32_t b = __ballot_sync(FULL, fresh);
+      if (fresh && n + __popc(b & lt) < s.w.cur_cap) s.w.cur[n + __popc(b & lt)] = key + j;
+      n += __popc(b);
+      if (!__any_sync(FULL, v && j < more)) break;
+    }
+  };
+  for (uint32_t base = 0; base < len; base += 32) {
+    const bool v = base + lane < len;
+    const uint32_t it = v ? set[base + lane] : 0u;
+    const Scanned sc = scan_item(G, it, v ? G.info[it & 0xFFFFu] : (KIND_NT << INFO_KIND_SHIFT), byte);
+    if (__any_sync(FULL, sc.has_a)) add(sc.has_a, sc.a);
+    if (__any_sync(FULL, sc.has_b)) add(sc.has_b, sc.b);
+  }
+  uint2* const ask = reinterpret_cast<uint2*>(s.live);  // per completion of a wave: where its set's items begin
+  uint32_t* const want = s.live + 64;                   // its non-terminal and origin
+  uint32_t* const from = s.live + 96;                   // its first place among the items dealt out
+  for (uint32_t head = 0; head < min(n, s.w.cur_cap);) {
+    __syncwarp();
+    const bool have = head + lane < n && head + lane < s.w.cur_cap;
+    const uint32_t until = n;
+    const uint32_t it = have ? s.w.cur[head + lane] : 0u;
+    const uint32_t inf = have ? G.info[it & 0xFFFFu] : 0u, kind = inf >> INFO_KIND_SHIFT, a = inf & INFO_ARG_MASK;
+    if (have && kind == KIND_NT) atomicOr(&s.w.nt[a >> 5], 1u << (a & 31u));
+    if (have && kind == KIND_END && (it & 0xFFFFu) == ITEM_ACCEPT) s.w.ctr[W_ACCEPT] = 1u;
+    bool asks = have && kind == KIND_END && (it >> 16) != index && (it & 0xFFFFu) != ITEM_ACCEPT;
+    if (asks) {
+      const uint32_t at = a * row + (it >> 16), bit = 1u << (at & 31u);
+      asks = !(atomicOr(&done[at >> 5], bit) & bit);
+    }
+    const uint32_t* sp = nullptr;
+    uint32_t sl = 0;
+    if (asks) view(it >> 16, sp, sl);
+    asks = sl != 0u;
+    uint32_t incl = sl;
+    for (int d = 1; d < 32; d <<= 1) {
+      const uint32_t t = __shfl_up_sync(FULL, incl, d);
+      if ((int)lane >= d) incl += t;
+    }
+    const uint32_t total = __shfl_sync(FULL, incl, 31), ab = __ballot_sync(FULL, asks), r = __popc(ab & lt);
+    if (asks) {
+      ask[r] = make_uint2((uint32_t)(uintptr_t)sp, (uint32_t)((uintptr_t)sp >> 32));
+      want[r] = a;
+      from[r] = incl - sl;
+    }
+    __syncwarp();
+    const uint32_t my_start = lane < (uint32_t)__popc(ab) ? from[lane] : 0xFFFFFFFFu;
+    for (uint32_t base = 0; base < total; base += 32) {
+      const uint32_t before = __popc(__ballot_sync(FULL, my_start <= base));  // completions that begin up to here
+      const uint32_t starts = __reduce_or_sync(FULL, my_start > base && my_start - base < 32u ? 1u << (my_start - base) : 0u);
+      const uint32_t q = before - 1u + __popc(starts & (0xFFFFFFFFu >> (31u - lane)));
+      bool match = false;
+      uint32_t wi = 0;
+      if (base + lane < total) {
+        const uint2 p = ask[q];
+        const uint32_t* items = reinterpret_cast<const uint32_t*>((uintptr_t)p.x | ((uintptr_t)p.y << 32));
+        wi = items[base + lane - from[q]];
+        const uint32_t winf = G.info[wi & 0xFFFFu];
+        match = (winf >> INFO_KIND_SHIFT) == KIND_NT && (winf & INFO_ARG_MASK) == want[q];
+      }
+      if (__any_sync(FULL, match)) add(match, wi + 1u);
+    }
+    head = min(head + 32u, until);  // (items added by this wave begin at `until`)
+  }
+  __syncwarp();
+  for (uint32_t i = lane; i < set_words; i += 32) in_set[i] = EMPTY_SLOT;
+  __syncwarp();
+  return n <= s.w.cur_cap ? n : GEN_FULL;
+}
+
 // All bytes of one token.  Returns 1 (dst holds the new chart), 0 (some byte cannot follow: dst
 // is garbage), -1 (a capacity limit was hit) or -2 (the arena for the token's sets is too small:
 // the caller may retry with a larger one).  src and dst must not overlap.  `arena` (arena_cap
@@ -221,9 +318,32 @@ __device__ int token_step(const GrammarDev& G, AdvScratch& s, const uint32_t* sr
     __syncwarp();
     const uint32_t index = m - 1 + L;
     uint32_t n;
-    // sets of up to 32 scanned and completed items (nearly all) are built in lanes ...
+    if (prev_len == 1u && !forced_out) {
+      // one item inside a literal or an automaton that moves on and completes nothing: the new set is that one item, and
+      // there is nothing to predict (inside strings and names: half of the steps and more)
+      const uint32_t it = prev[0], inf = G.info[it & 0xFFFFu], kind = inf >> INFO_KIND_SHIFT;
+      uint32_t to = 0;
+      if (kind == KIND_DFA) {
+        const uint32_t t = __ldg(&G.dfa_trans[(size_t)(inf & INFO_ARG_MASK) * G.n_eq + G.eq_of_byte[byte]]);
+        if (t != 0xFFFFu && (t & 0xC000u) == 0x4000u) to = (it & 0xFFFF0000u) | (G.dfa_first + (t & 0x3FFFu));
+      } else if (kind == KIND_TERM && class_has(G, inf & INFO_ARG_MASK, byte)) {
+        const uint32_t next = G.info[(it & 0xFFFFu) + 1u] >> INFO_KIND_SHIFT;
+        if (next == KIND_TERM || next == KIND_DFA) to = it + 1u;
+      }
+      if (to) {
+        prev = arena + top;
+        __syncwarp();
+        if (lane == 0) arena[top] = to, lvl_off[L + 1] = top + 1u;
+        ++top;
+        accepting = false;
+        __syncwarp();
+        continue;
+      }
+    }
+    // sets of up to 32 scanned and completed items (nearly all) are built in lanes; what comes from a set of more than 32 items
+    // seldom is one (trying it all the same cost an advance of 32 ambiguous rows 90 us, not trying 80) ...
     uint32_t mine;
-    const uint32_t ns = (prev_len <= 96u) ? small_scan_complete(G, s.w, view, prev, prev_len, byte, index,
+    const uint32_t ns = (prev_len <= (gen_fits(G, index) ? 32u : 96u)) ? small_scan_complete(G, s.w, view, prev, prev_len, byte, index,
                                                                  [](uint32_t it) { return it; }, mine, accepting)
                                            : SMALL_OVERFLOW;
     if (ns == 0) return forced_out ? (int)(L - 1) : 0;
@@ -233,7 +353,20 @@ __device__ int token_step(const GrammarDev& G, AdvScratch& s, const uint32_t* sr
       predict_into_cur(G, s.w, index);
       if (s.w.ctr[W_OVERFLOW]) return forced_out ? (int)(L - 1) : -2;
       n = min(s.w.ctr[W_NCUR], s.w.cur_cap);
-    } else {  // ... larger ones with the uniqueness hash
+    } else if (gen_fits(G, index)) {  // ... larger ones with a bit for every item there can be
+      n = gen_scan_complete(G, s, view, prev, prev_len, byte, index);
+      if (n == GEN_FULL) {
+        clear_nt(G, s.w);
+        return forced_out ? (int)(L - 1) : -2;
+      }
+      if (n == 0) return forced_out ? (int)(L - 1) : 0;
+      accepting = s.w.ctr[W_ACCEPT] != 0u;
+      n = drop_completed(G, s.w, n);
+      if (lane == 0) s.w.ctr[W_NCUR] = n;
+      predict_into_cur(G, s.w, index);
+      if (s.w.ctr[W_OVERFLOW]) return forced_out ? (int)(L - 1) : -2;
+      n = min(s.w.ctr[W_NCUR], s.w.cur_cap);
+    } else {  // ... and where that is too many, with the uniqueness hash
       n = scan_into_cur(G, s.w, prev, prev_len, byte);
       if (s.w.ctr[W_OVERFLOW]) {
         hset_clear_all(s.w.hset, s.w.hset_mask);
@@ -269,87 +402,180 @@ __device__ int token_step(const GrammarDev& G, AdvScratch& s, const uint32_t* sr
   if (n_bits > ADV_MAX_ITEMS) return -1;
   for (uint32_t i = lane; i < (n_bits + 31) / 32; i += 32) s.live[i] = 0u;
   __syncwarp();
-  for (uint32_t i = lane; i < n_last; i += 32) {
-    uint32_t it = arena[last_at + i];
-    if ((it >> 16) < last) push_need(s, it >> 16, __ldg(&G.lhs[it & 0xFFFFu]));
-  }
-  // needs are served a wave at a time: a need whose set is short is served by its own lane, the
-  // needs of long sets (alternations of many literals predicted at once) by the whole warp in turn
-  constexpr uint32_t NEED_SHORT = 8;
-  for (uint32_t head = 0;;) {
-    __syncwarp();
-    const uint32_t np = min(s.w.ctr[W_NPAIRS], ADV_PAIRS);
-    __syncwarp();
-    if (head >= np) break;
-    const uint32_t mine = head + lane;
-    uint32_t o = 0, A = 0, sl = 0, base = 0;
-    const uint32_t* sp = nullptr;
-    if (mine < np) {
-      const uint32_t key = s.pairs[mine];
-      o = key >> 16, A = key & 0xFFFFu;
-      view(o, sp, sl);
-      base = view.bit_base(o, n_items);
+  // ---- the needs, "somebody may complete a non-terminal begun in this set".  An item begun in a set lies in that set or
+  // in a later one, so one pass over the sets from the last to the first finds them all: per set a bit for every non-terminal;
+  // with a non-terminal come at once those whose prediction pulls it in (nt_up), which settles the items begun in the set itself.  One
+  // pass over a set's items per set: with a list of (set, non-terminal) pairs served one after the other Compact
+  // took 31,000 cycles for a JSON chart of 12 sets and 280,000 for an ambiguous one of 60, now 8,500 and 90,000.
+  const uint32_t M = last;  // earlier sets: 0..last-1
+  if (M * G.Nw <= ADV_HSET) {
+    uint32_t* need = s.w.hset;  // [M][Nw]
+    const uint32_t Nw = G.Nw;
+    for (uint32_t i = lane; i < M * Nw; i += 32) need[i] = 0u;
+    for (uint32_t k = lane; k < M; k += 32) s.sets[k] = 0u;
+    // below[k]: the earliest set in which an item of the source chart's sets after k begins.  Where it is not before k, everything
+    // before k is held by k's items alone, and as the source chart is pruned, all of it is needed if they all are:
+    // the way down a deep nesting ends at the first such set.  (Not for sets so long that finding out would cost more.)
+    uint32_t* below = s.pairs;
+    {
+      uint32_t longest = 0, carry = 0xFFFFFFFFu;
+      for (uint32_t k = lane; k < m; k += 32) longest = max(longest, soff[k + 1] - soff[k]);
+      const bool worth = __reduce_max_sync(FULL, longest) <= 16u && m <= ADV_PAIRS;
+      for (uint32_t end = m; end;) {
+        const uint32_t k = end - 1u - lane;
+        uint32_t lowest = 0xFFFFFFFFu;
+        if (k < end && worth)
+          for (uint32_t i = soff[k]; i < soff[k + 1]; ++i) lowest = min(lowest, sitems[i] >> 16);
+        for (int d = 1; d < 32; d <<= 1) {  // (lane l: over the sets end-1 .. end-1-l)
+          const uint32_t t = __shfl_up_sync(FULL, lowest, d);
+          if ((int)lane >= d) lowest = min(lowest, t);
+        }
+        uint32_t above = __shfl_up_sync(FULL, lowest, 1);
+        if (lane == 0) above = 0xFFFFFFFFu;
+        if (k < end && k < ADV_PAIRS) below[k] = worth ? min(above, carry) : 0u;
+        carry = min(carry, __shfl_sync(FULL, lowest, 31));
+        end -= min(end, 32u);
+      }
     }
-    auto serve = [&](const uint32_t* set, uint32_t k, uint32_t bit_base, uint32_t want) {
-      const uint32_t wi = set[k];
-      const uint32_t inf = G.info[wi & 0xFFFFu];
-      if ((inf >> INFO_KIND_SHIFT) == KIND_NT && (inf & INFO_ARG_MASK) == want) {
-        const uint32_t pos = bit_base + k;
-        const uint32_t bit = 1u << (pos & 31u);
-        const uint32_t old = atomicOr(&s.live[pos >> 5], bit);
-        if (!(old & bit)) push_need(s, wi >> 16, __ldg(&G.lhs[wi & 0xFFFFu]));
+    __syncwarp();
+    uint32_t first_asked = 0xFFFFFFFFu;  // (each lane: the earliest set it has asked)
+    auto ask = [&](uint32_t o, uint32_t A) {
+      first_asked = min(first_asked, o);
+      for (uint32_t w = 0; w < Nw; ++w) {
+        const uint32_t bits = G.nt_up[A * Nw + w];
+        if (bits) atomicOr(&need[o * Nw + w], bits);
       }
     };
-    if (sl <= NEED_SHORT)
-      for (uint32_t k = 0; k < sl; ++k) serve(sp, k, base, A);
-    uint32_t longs = __ballot_sync(FULL, sl > NEED_SHORT);
-    while (longs) {
-      const int src = __ffs(longs) - 1;
-      longs &= longs - 1;
-      const uint32_t so = __shfl_sync(FULL, o, src), sA = __shfl_sync(FULL, A, src);
-      const uint32_t* lp;
-      uint32_t ll;
-      view(so, lp, ll);
-      const uint32_t lbase = view.bit_base(so, n_items);
-      for (uint32_t k = lane; k < ll; k += 32) serve(lp, k, lbase, sA);
+    for (uint32_t i = lane; i < n_last; i += 32) {
+      const uint32_t it = arena[last_at + i];
+      if ((it >> 16) < last) ask(it >> 16, G.lhs[it & 0xFFFFu]);
     }
-    head = min(head + 32u, np);
-  }
-  const uint32_t n_pairs = min(s.w.ctr[W_NPAIRS], ADV_PAIRS);
-  __syncwarp();
-  if (n_pairs * 8u > s.w.hset_mask) {
-    hset_clear_all(s.w.hset, s.w.hset_mask);  // the hash held (set, non-terminal) pairs
-  } else {
-    for (uint32_t i = lane; i < n_pairs; i += 32) {
-      const uint32_t key = s.pairs[i];
-      uint32_t hh = mix32(key) & s.w.hset_mask;
-      for (uint32_t probe = 0; probe <= s.w.hset_mask; ++probe) {
-        if (s.w.hset[hh] == key) {
-          s.w.hset[hh] = EMPTY_SLOT;
-          break;
-        }
-        hh = (hh + 1) & s.w.hset_mask;
+    for (uint32_t end = M; end;) {  // sets 0 .. end-1 are left: the last of them that is asked for
+      __syncwarp();
+      const uint32_t k = end - 1u - lane;  // (wraps around for lanes beyond set 0)
+      bool asked = false;
+      if (k < end)
+        for (uint32_t w = 0; w < Nw; ++w) asked = asked || need[k * Nw + w] != 0u;
+      const uint32_t bal = __ballot_sync(FULL, asked);
+      if (bal == 0u) {
+        end -= min(end, 32u);
+        continue;
+      }
+      const uint32_t o = end - (uint32_t)__ffs(bal);
+      end = o;
+      const bool sole = __reduce_min_sync(FULL, first_asked) == o;  // nothing before it has been asked yet
+      const uint32_t* sp;
+      uint32_t sl;
+      view(o, sp, sl);
+      const uint32_t first_bit = view.bit_base(o, n_items);
+      uint32_t live = 0;
+      for (uint32_t base = 0; base < sl; base += 32) {
+        const uint32_t it = base + lane < sl ? sp[base + lane] : 0u;
+        const uint32_t inf = G.info[it & 0xFFFFu], A = inf & INFO_ARG_MASK;
+        const bool keep = base + lane < sl && (inf >> INFO_KIND_SHIFT) == KIND_NT && ((need[o * Nw + (A >> 5)] >> (A & 31u)) & 1u);
+        const uint32_t kb = __ballot_sync(FULL, keep);
+        if (kb == 0u) continue;
+        live += __popc(kb);
+        if (keep && (it >> 16) != o) ask(it >> 16, G.lhs[it & 0xFFFFu]);
+        const uint32_t at = first_bit + base, sh = at & 31u;
+        if (lane == 0) s.live[at >> 5] |= kb << sh;
+        if (lane == 1 && sh && (kb >> (32u - sh))) s.live[(at >> 5) + 1u] |= kb >> (32u - sh);
+        __syncwarp();
+      }
+      if (lane == 0) s.sets[o] = live;
+      if (sole && live == sl && o < m && o < ADV_PAIRS && below[o] >= o) {  // the rest stays as it is
+        const uint32_t bits = soff[o];
+        __syncwarp();
+        for (uint32_t k = lane; k < o; k += 32) s.sets[k] = soff[k + 1] - soff[k];
+        for (uint32_t i = lane; i < (bits + 31u) / 32u; i += 32) s.live[i] |= (i + 1u) * 32u <= bits ? FULL : (1u << (bits & 31u)) - 1u;
+        break;
       }
     }
     __syncwarp();
+    for (uint32_t i = lane; i < M * Nw; i += 32) need[i] = EMPTY_SLOT;
+    __syncwarp();
+  } else {
+    for (uint32_t i = lane; i < n_last; i += 32) {
+      uint32_t it = arena[last_at + i];
+      if ((it >> 16) < last) push_need(s, it >> 16, G.lhs[it & 0xFFFFu]);
+    }
+    // needs are served a wave at a time: a need whose set is short is served by its own lane, the
+    // needs of long sets (alternations of many literals predicted at once) by the whole warp in turn
+    constexpr uint32_t NEED_SHORT = 8;
+    for (uint32_t head = 0;;) {
+      __syncwarp();
+      const uint32_t np = min(s.w.ctr[W_NPAIRS], ADV_PAIRS);
+      __syncwarp();
+      if (head >= np) break;
+      const uint32_t mine = head + lane;
+      uint32_t o = 0, A = 0, sl = 0, base = 0;
+      const uint32_t* sp = nullptr;
+      if (mine < np) {
+        const uint32_t key = s.pairs[mine];
+        o = key >> 16, A = key & 0xFFFFu;
+        view(o, sp, sl);
+        base = view.bit_base(o, n_items);
+      }
+      auto serve = [&](const uint32_t* set, uint32_t k, uint32_t bit_base, uint32_t want) {
+        const uint32_t wi = set[k];
+        const uint32_t inf = G.info[wi & 0xFFFFu];
+        if ((inf >> INFO_KIND_SHIFT) == KIND_NT && (inf & INFO_ARG_MASK) == want) {
+          const uint32_t pos = bit_base + k;
+          const uint32_t bit = 1u << (pos & 31u);
+          const uint32_t old = atomicOr(&s.live[pos >> 5], bit);
+          if (!(old & bit)) push_need(s, wi >> 16, G.lhs[wi & 0xFFFFu]);
+        }
+      };
+      if (sl <= NEED_SHORT)
+        for (uint32_t k = 0; k < sl; ++k) serve(sp, k, base, A);
+      uint32_t longs = __ballot_sync(FULL, sl > NEED_SHORT);
+      while (longs) {
+        const int src = __ffs(longs) - 1;
+        longs &= longs - 1;
+        const uint32_t so = __shfl_sync(FULL, o, src), sA = __shfl_sync(FULL, A, src);
+        const uint32_t* lp;
+        uint32_t ll;
+        view(so, lp, ll);
+        const uint32_t lbase = view.bit_base(so, n_items);
+        for (uint32_t k = lane; k < ll; k += 32) serve(lp, k, lbase, sA);
+      }
+      head = min(head + 32u, np);
+    }
+    const uint32_t n_pairs = min(s.w.ctr[W_NPAIRS], ADV_PAIRS);
+    __syncwarp();
+    if (n_pairs * 8u > s.w.hset_mask) {
+      hset_clear_all(s.w.hset, s.w.hset_mask);  // the hash held (set, non-terminal) pairs
+    } else {
+      for (uint32_t i = lane; i < n_pairs; i += 32) {
+        const uint32_t key = s.pairs[i];
+        uint32_t hh = mix32(key) & s.w.hset_mask;
+        for (uint32_t probe = 0; probe <= s.w.hset_mask; ++probe) {
+          if (s.w.hset[hh] == key) {
+            s.w.hset[hh] = EMPTY_SLOT;
+            break;
+          }
+          hh = (hh + 1) & s.w.hset_mask;
+        }
+      }
+      __syncwarp();
+    }
+    if (s.w.ctr[W_OVERFLOW]) {
+      hset_clear_all(s.w.hset, s.w.hset_mask);
+      clear_nt(G, s.w);
+      return -1;
+    }
+    // ---- live items per earlier set, new set numbers, new offsets
+    for (uint32_t k = lane; k < M; k += 32) {
+      const uint32_t* sp;
+      uint32_t sl;
+      view(k, sp, sl);
+      const uint32_t base = view.bit_base(k, n_items);
+      uint32_t c = 0;
+      for (uint32_t i = 0; i < sl; ++i) c += (s.live[(base + i) >> 5] >> ((base + i) & 31u)) & 1u;
+      s.sets[k] = c;
+    }
+    __syncwarp();
   }
-  if (s.w.ctr[W_OVERFLOW]) {
-    hset_clear_all(s.w.hset, s.w.hset_mask);
-    clear_nt(G, s.w);
-    return -1;
-  }
-  // ---- live items per earlier set, new set numbers, new offsets
-  const uint32_t M = last;  // earlier sets: 0..last-1
-  for (uint32_t k = lane; k < M; k += 32) {
-    const uint32_t* sp;
-    uint32_t sl;
-    view(k, sp, sl);
-    const uint32_t base = view.bit_base(k, n_items);
-    uint32_t c = 0;
-    for (uint32_t i = 0; i < sl; ++i) c += (s.live[(base + i) >> 5] >> ((base + i) & 31u)) & 1u;
-    s.sets[k] = c;
-  }
-  __syncwarp();
   HashAcc h;
   uint32_t m_new = 0, kept = 0;
   for (uint32_t base = 0; base < M; base += 32) {

@@ -54,7 +54,8 @@ __device__ __forceinline__ int hset_insert(uint32_t* hset, uint32_t mask, uint32
 
 __device__ __forceinline__ void hset_clear_all(uint32_t* hset, uint32_t mask) {
   __syncwarp();
-  for (uint32_t i = lane_id(); i <= mask; i += 32) hset[i] = EMPTY_SLOT;
+  for (uint32_t i = 4u * lane_id(); i <= mask; i += 128)  // (tables begin on 16 bytes and have a power of two of slots, at least 128)
+    *reinterpret_cast<uint4*>(hset + i) = make_uint4(EMPTY_SLOT, EMPTY_SLOT, EMPTY_SLOT, EMPTY_SLOT);
   __syncwarp();
 }
 
@@ -201,17 +202,27 @@ __device__ __forceinline__ void predict_into_cur(const GrammarDev& G, const Warp
   uint32_t* ntmask = w.nt;
   uint32_t* clos = w.nt + Nw;
   __syncwarp();
-  for (uint32_t i = lane; i < Nw; i += 32) {  // each lane owns some words of the closure
-    uint32_t acc = 0u;
-    for (uint32_t wi = 0; wi < Nw; ++wi) {
-      uint32_t bits = ntmask[wi];
-      while (bits) {
-        const uint32_t y = wi * 32u + (uint32_t)(__ffs(bits) - 1);
-        bits &= bits - 1;
-        acc |= G.nt_closure[y * Nw + i];
-      }
+  if (Nw <= 4u) {  // a lane for every non-terminal that is asked for: its row of the closure, joined over the lanes
+    for (uint32_t i = 0; i < Nw; ++i) {
+      uint32_t acc = 0u;
+      for (uint32_t wi = 0; wi < Nw; ++wi)
+        if ((ntmask[wi] >> lane) & 1u) acc |= G.nt_closure[(wi * 32u + lane) * Nw + i];
+      acc = __reduce_or_sync(FULL, acc);
+      if (lane == i) clos[i] = acc;
     }
-    clos[i] = acc;
+  } else {
+    for (uint32_t i = lane; i < Nw; i += 32) {  // each lane owns some words of the closure
+      uint32_t acc = 0u;
+      for (uint32_t wi = 0; wi < Nw; ++wi) {
+        uint32_t bits = ntmask[wi];
+        while (bits) {
+          const uint32_t y = wi * 32u + (uint32_t)(__ffs(bits) - 1);
+          bits &= bits - 1;
+          acc |= G.nt_closure[y * Nw + i];
+        }
+      }
+      clos[i] = acc;
+    }
   }
   __syncwarp();
   uint32_t n = min(w.ctr[W_NCUR], w.cur_cap);
@@ -387,11 +398,14 @@ __device__ __forceinline__ uint32_t small_drop_completed(const GrammarDev& G, co
 // Copy the grammar's hot tables into shared memory (all threads of the block take part, the
 // caller synchronizes) and return a view of the grammar that reads them from there.
 __device__ __forceinline__ GrammarDev stage_hot_tables(const GrammarDev& Gg, uint32_t* dst) {
-  for (uint32_t i = threadIdx.x; i < Gg.hot_words; i += blockDim.x) dst[i] = Gg.hot_block[i];
+  for (uint32_t i = threadIdx.x; i < Gg.hot_words / 4u; i += blockDim.x)  // (the block is a multiple of 16 bytes)
+    reinterpret_cast<uint4*>(dst)[i] = __ldg(reinterpret_cast<const uint4*>(Gg.hot_block) + i);
   GrammarDev G = Gg;
   G.info = dst + (Gg.info - Gg.hot_block);
   G.class_bits = dst + (Gg.class_bits - Gg.hot_block);
   G.eq_of_byte = reinterpret_cast<const uint8_t*>(dst + (reinterpret_cast<const uint32_t*>(Gg.eq_of_byte) - Gg.hot_block));
+  G.lhs = reinterpret_cast<const uint16_t*>(dst + (reinterpret_cast<const uint32_t*>(Gg.lhs) - Gg.hot_block));
+  G.nt_up = dst + (Gg.nt_up - Gg.hot_block);
   G.nt_closure = dst + (Gg.nt_closure - Gg.hot_block);
   G.direct_off = dst + (Gg.direct_off - Gg.hot_block);
   G.direct_items = reinterpret_cast<const uint16_t*>(dst + (reinterpret_cast<const uint32_t*>(Gg.direct_items) - Gg.hot_block));

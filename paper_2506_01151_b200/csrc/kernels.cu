@@ -31,6 +31,7 @@ __device__ int32_t intern_chart(const StateDev& S, const uint32_t* ch, uint64_t&
   uint32_t slot = hlo & S.ht_mask;
   int32_t my_id = -1;
   uint64_t my_off = 0;
+  const uint32_t taken = lane == 0 ? ld_acquire(&S.counters[CNT_N_STATES]) : 0u;  // (asked for together with the first probe)
   for (uint32_t probe = 0; probe < 512; ++probe) {
     uint32_t v = 0;
     if (lane == 0) v = ld_acquire(&S.ht[slot]);
@@ -40,13 +41,11 @@ __device__ int32_t intern_chart(const StateDev& S, const uint32_t* ch, uint64_t&
         unsigned long long off = 0;
         int32_t id = -1;
         if (lane == 0) {
-          if (ld_acquire(&S.counters[CNT_N_STATES]) < S.max_states) {
-            uint32_t got = atomicAdd(&S.counters[CNT_N_STATES], 1u);
-            if (got < S.max_states) {
-              unsigned long long need = (words + 31u) & ~31u;
-              off = atomicAdd(reinterpret_cast<unsigned long long*>(S.counters + CNT_POOL_LO), need);
-              if (off + need <= S.pool_words) id = (int32_t)got;
-            }
+          if (taken < S.max_states) {
+            const unsigned long long need = (words + 31u) & ~31u;
+            const uint32_t got = atomicAdd(&S.counters[CNT_N_STATES], 1u);
+            off = atomicAdd(reinterpret_cast<unsigned long long*>(S.counters + CNT_POOL_LO), need);
+            if (got < S.max_states && off + need <= S.pool_words) id = (int32_t)got;
           }
         }
         id = __shfl_sync(FULL, id, 0);
@@ -97,7 +96,7 @@ __device__ int32_t intern_chart(const StateDev& S, const uint32_t* ch, uint64_t&
 // ===================================================================================== transition cache
 //
 // What advancing the chart with cache id `sid` by `tok` leads to, if that is known: the next chart's
-// cache id, TR_REJECT, or TR_UNSET (not known).  Called by one lane.
+// cache id, TR_REJECT, or TR_UNSET (not known).
 __device__ __forceinline__ uint32_t tr_slot(const StateDev& S, unsigned long long key) {
   return (mix32((uint32_t)key) ^ mix32((uint32_t)(key >> 32) * 0x9E3779B9u)) & S.tr_mask;
 }
@@ -105,12 +104,11 @@ __device__ int32_t tr_lookup(const StateDev& S, int32_t sid, uint32_t tok) {
   const unsigned long long key = ((unsigned long long)((uint32_t)sid + 1u) << 32) | tok;
   uint32_t slot = tr_slot(S, key);
   for (uint32_t probe = 0; probe < 32; ++probe) {
+    // (a value read before its key may be one not written yet: the pair then counts as unknown)
+    const int32_t v = __ldcg(S.tr_val + slot);
     const unsigned long long k = __ldcg(S.tr_key + slot);
     if (k == 0ull) return TR_UNSET;
-    if (k == key) {
-      const int32_t v = (int32_t)ld_acquire(reinterpret_cast<const uint32_t*>(S.tr_val + slot));
-      return (v >= 0 || v == TR_REJECT) ? v : TR_UNSET;
-    }
+    if (k == key) return (v >= 0 || v == TR_REJECT) ? v : TR_UNSET;
     slot = (slot + 1u) & S.tr_mask;
   }
   return TR_UNSET;
@@ -172,55 +170,53 @@ __global__ void __launch_bounds__(ADV_WARPS * 32, 1) advance_kernel(GrammarDev G
   extern __shared__ __align__(16) uint32_t smem[];
   const uint32_t warp = threadIdx.x >> 5, lane = lane_id();
   const uint32_t row = blockIdx.x * ADV_WARPS + warp;
-  GrammarDev G = Gg;
-  if (Gg.hot_words * 4u <= HOT_TABLE_BYTES) {
-    G = stage_hot_tables(Gg, smem + (size_t)ADV_WARPS * ADV_WARP_WORDS);
-    __syncthreads();
-  }
-  if (row >= S.B) return;
-  AdvScratch s = adv_scratch(smem + (size_t)warp * ADV_WARP_WORDS);
+  const int32_t tok = row < S.B ? tokens[row] : -1;
+  uint32_t flags = 0, b0 = 0, b1 = 0;
+  int32_t sid = -1;
+  const uint32_t* cur = nullptr;
   auto finish = [&](int32_t st) {
     if (status && lane == 0) status[row] = st;
   };
-  const int32_t tok = tokens[row];
-  if (tok == -1) return finish(FMT_OK);
-  const uint32_t flags = S.row_flags[row];
-  if (flags & ROW_FINISHED) return finish(FMT_ERR_FINISHED);
-  if (tok < 0 || (uint32_t)tok >= G.V) return finish(FMT_ERR_INVALID_ARG);
-  if (flags & ROW_BROKEN) return finish(FMT_ERR_CAPACITY);
-  const uint32_t* cur = S.arena + S.row_chart[row];
-  const uint32_t b0 = __ldg(&G.vocab_off[tok]), b1 = __ldg(&G.vocab_off[tok + 1]);
-  if (tok == G.eos) {
-    if (cur[CH_FLAGS] & CHART_ACCEPTING) {
+  // What can be said without an Earley step; true: it takes one.  (Everything is asked for before anything is looked at: a row
+  // that is answered by the transition cache is three reads one after the other.)
+  auto first_look = [&]() -> bool {
+    if (row >= S.B) return false;
+    flags = S.row_flags[row];
+    sid = S.cache_on ? S.row_state[row] : -1;
+    cur = S.arena + S.row_chart[row];
+    if (tok == -1) return finish(FMT_OK), false;
+    if (flags & ROW_FINISHED) return finish(FMT_ERR_FINISHED), false;
+    if (tok < 0 || (uint32_t)tok >= Gg.V) return finish(FMT_ERR_INVALID_ARG), false;
+    if (flags & ROW_BROKEN) return finish(FMT_ERR_CAPACITY), false;
+    b0 = __ldg(&Gg.vocab_off[tok]), b1 = __ldg(&Gg.vocab_off[tok + 1]);
+    // has this chart been advanced by this token before?  (Section 5.2: the state cache)
+    const int32_t known = (sid >= 0 && tok != Gg.eos) ? tr_lookup(S, sid, (uint32_t)tok) : TR_UNSET;
+    if (tok == Gg.eos) {
+      if (!(cur[CH_FLAGS] & CHART_ACCEPTING)) return finish(FMT_ERR_TOKEN_REJECTED), false;
       if (lane == 0) S.row_flags[row] = flags | ROW_FINISHED;
-      return finish(FMT_OK);
+      return finish(FMT_OK), false;
     }
-    return finish(FMT_ERR_TOKEN_REJECTED);
-  }
-  if (b1 == b0) return finish(FMT_ERR_TOKEN_REJECTED);
-  // ---- has this chart been advanced by this token before?  (Section 5.2: the state cache)
-  const int32_t sid = S.cache_on ? S.row_state[row] : -1;
-  if (sid >= 0) {
-    int32_t known = TR_UNSET;
-    if (lane == 0) known = tr_lookup(S, sid, (uint32_t)tok);
-    known = __shfl_sync(FULL, known, 0);
-    if (known == TR_REJECT) return finish(FMT_ERR_TOKEN_REJECTED);
-    if (known >= 0 && (uint32_t)known < S.max_states) {
-      if (lane == 0) {
-        S.row_state[row] = known;
-        S.st_ref[known] = 1;
-        S.row_chart[row] = ld_cg64(&S.st_off[known]);
-        S.row_buf[row] = 255;
-        stat_add(S, CNT_STAT_ADV, 1u);
-        stat_add(S, CNT_STAT_ADV_HIT, 1u);
-      }
-      return finish(FMT_OK);
+    if (b1 == b0 || known == TR_REJECT) return finish(FMT_ERR_TOKEN_REJECTED), false;
+    if (known < 0 || (uint32_t)known >= S.max_states) return true;
+    if (lane == 0) {
+      S.row_state[row] = known;
+      S.st_ref[known] = 1;
+      S.row_chart[row] = ld_cg64(&S.st_off[known]);
+      S.row_buf[row] = 255;
+      stat_add(S, CNT_STAT_ADV, 1u);
+      stat_add(S, CNT_STAT_ADV_HIT, 1u);
     }
-  }
-
+    return finish(FMT_OK), false;
+  };
+  const bool steps = first_look();
+  if (!__syncthreads_or(steps)) return;  // (nothing is staged for rows that are all answered)
+  GrammarDev G = Gg;
+  if (Gg.hot_words * 4u <= HOT_TABLE_BYTES) G = stage_hot_tables(Gg, smem + (size_t)ADV_WARPS * ADV_WARP_WORDS);
+  AdvScratch s = adv_scratch(smem + (size_t)warp * ADV_WARP_WORDS);
   hset_clear_all(s.w.hset, s.w.hset_mask);
   for (uint32_t i = lane; i < ADV_NT_WORDS; i += 32) s.w.nt[i] = 0u;
-  __syncwarp();
+  __syncthreads();
+  if (!steps) return;
   // a private buffer that does not hold the current chart
   const uint32_t held = S.row_buf[row];
   const uint32_t final_buf = (held == 0) ? 1u : 0u;

@@ -104,3 +104,49 @@ def test_no_automaton_for_states_that_ask_for_earley_steps():
     a = _run(w.ebnf, w.start, w.vocab, JSON_PREFIXES)
     b = _run(w.ebnf, w.start, w.vocab, JSON_PREFIXES, sweep_states=4096)
     assert a["walk_states"] < b["walk_states"]
+
+
+def _feed(text, start, data, options, dfa=True):
+    """The chart words after feeding the bytes one by one, and in one token where they are at most 32."""
+    import torch
+
+    import paper_2506_01151_b200 as fmt
+
+    pieces = [data[i:i + 32] for i in range(0, len(data), 32)]
+    vocab = [bytes([b]) for b in range(256)] + pieces + [b""]
+    g = fmt.Grammar(text, start, vocab, len(vocab) - 1, dfa=dfa)
+    st = fmt.State(g, 2, **options)
+    status = torch.zeros(2, dtype=torch.int32, device="cuda")
+    for i in range(len(data)):
+        whole = 256 + i // 32 if i % 32 == 0 else -1
+        st.advance(torch.tensor([data[i], whole], dtype=torch.int32, device="cuda"), status)
+        assert status.tolist() == [fmt.FMT_OK, fmt.FMT_OK], (i, data[:i + 1])
+    q = st.query()
+    return st.chart_words(0), st.chart_words(1), q
+
+
+@pytest.mark.parametrize("nests", [1, 31, 32, 33, 70])
+@pytest.mark.parametrize("dfa", [True, False])
+def test_compact_down_a_deep_nesting(nests, dfa):
+    """Compact stops at a set that holds everything before it: charts around multiples of 32 sets, the same words whether it ran
+    after every byte or once per 32 bytes, every set still referenced."""
+    w = workloads.build(2, V=300, batch=1, steps=1)
+    data = b"".join(b'[1, {"k":' if i % 3 == 0 else b"[" for i in range(nests)) + b'"x'
+    a, b, _ = _feed(w.ebnf, w.start, data, {}, dfa)
+    assert a.tolist() == b.tolist()
+    closing = data + b'"' + b"".join(b"}]" if i % 3 == 0 else b"]" for i in reversed(range(nests)))
+    a, b, q = _feed(w.ebnf, w.start, closing, {}, dfa)
+    assert a.tolist() == b.tolist() and q["accepting"].tolist() == [1, 1]
+
+
+@pytest.mark.parametrize("letters", [8, 30, 33, 64, 200])
+def test_sets_with_a_bit_for_every_item(letters):
+    """Earley sets that outgrow a warp's lanes: around 32 items, and beyond what the bits hold (the hash takes over)."""
+    text = 's ::= "<" e ">"\ne ::= e e | e n "+" n e | "(" e ")" | "a" | "b"\nn ::= "!" | ""'
+    data = b"<" + b"".join(b"a" if i % 5 else b"(b+a)" for i in range(letters))
+    a, b, _ = _feed(text, "s", data, dict(chart_words=1 << 18), True)
+    assert a.tolist() == b.tolist()
+    og = oracle.Grammar(text, "s")
+    s = oracle.Sequence_(og, pruned=True)
+    assert s.advance(data)
+    assert int(a[0]) == s.num_sets and int(a[1]) == s.total_items
