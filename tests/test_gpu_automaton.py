@@ -150,3 +150,31 @@ def test_sets_with_a_bit_for_every_item(letters):
     s = oracle.Sequence_(og, pruned=True)
     assert s.advance(data)
     assert int(a[0]) == s.num_sets and int(a[1]) == s.total_items
+
+
+@pytest.mark.parametrize("dtype", ["bf16", "fp32"])
+@pytest.mark.parametrize("V", [1, 7, 8, 15, 16, 17, 31, 33, 63, 64, 65, 4095, 4097, 16 * 512 + 3])
+def test_masking_rows_that_begin_anywhere(dtype, V):
+    """Rows are masked in units of 32 bytes from their first 32-byte boundary on: every place in a unit a row can begin, vocabularies
+    around whole units, units that are all valid, all invalid and mixed, and nothing written beside the row."""
+    import torch
+
+    import paper_2506_01151_b200 as fmt
+
+    rng = np.random.default_rng(V)
+    kind, bits = (np.uint16, 16) if dtype == "bf16" else (np.uint32, 32)
+    stride, batch = V + 5, 9
+    keep = rng.random((batch, V)) < np.array([0.0, 1.0, 0.5, 0.9, 0.05, 0.5, 0.5, 0.5, 0.5])[:, None]
+    words = (V + 31) // 32
+    mask = np.zeros((batch, words * 32), np.uint8)
+    mask[:, :V] = keep
+    mask = np.packbits(mask, axis=1, bitorder="little").view(np.uint32)
+    for shift in range(0, 32 * 8 // bits, 3 if V > 100 else 1):
+        logits = rng.integers(0, 1 << bits, size=shift + batch * stride, dtype=np.uint64).astype(kind)
+        want = logits.copy()
+        rows = want[shift:].reshape(batch, stride)
+        rows[:, :V][~keep] = 0xFF80 if dtype == "bf16" else 0xFF800000
+        on_gpu = torch.from_numpy(logits.view(np.int16 if bits == 16 else np.int32)).cuda()
+        m = torch.from_numpy(np.ascontiguousarray(mask).view(np.int32)).cuda()
+        fmt.apply_mask(m, on_gpu.data_ptr() + shift * bits // 8, fmt.BF16 if dtype == "bf16" else fmt.FP32, batch, V, row_stride=stride)
+        assert np.array_equal(on_gpu.cpu().numpy().view(kind), want), shift
