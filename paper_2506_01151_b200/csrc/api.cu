@@ -482,6 +482,7 @@ fmt_status fmt_state_create(const fmt_grammar* g, uint32_t batch, const fmt_stat
   AL(d.row_state, batch, 0xFF);
   AL(d.row_flags, batch, 0);
   AL(d.row_mask, batch, 0xFF);
+  AL(d.row_job, batch, 0);
   AL(d.ht, ht, 0);
   AL(s->st_off2[0], d.max_states, 0);
   AL(s->st_mask2[0], d.max_states, 0xFF);

@@ -356,6 +356,7 @@ __device__ __forceinline__ uint32_t ga_next(const GrammarDev& G, uint32_t code, 
 
 __global__ void __launch_bounds__(AF_THREADS, 4) automaton_fill_kernel(const __grid_constant__ GrammarDev G,
                                                                        const __grid_constant__ StateDev S) {
+  before_me();
   const uint32_t n_jobs = S.counters[CNT_N_JOBS];
   if (n_jobs == 0u) return;  // (every block sees the same count)
   extern __shared__ __align__(16) uint32_t smem[];
@@ -386,6 +387,7 @@ __global__ void __launch_bounds__(AF_THREADS, 4) automaton_fill_kernel(const __g
   for (uint32_t i = tid * 8u; i < min(G.D, 8u * AF_THREADS); i += 8u * AF_THREADS) {
     uint32_t v;
     asm volatile("ld.global.nc.u32 %0, [%1];" : "=r"(v) : "l"(G.ga_item + 4u * i));
+    (void)v;
   }
   bool rows_left = true;
   const uint32_t parts = A.parts;
@@ -853,7 +855,7 @@ cudaError_t configure_automaton_fill() {
 }
 
 void launch_automaton_fill(const GrammarDev& G, const StateDev& S, cudaStream_t st) {
-  automaton_fill_kernel<<<S.af.grid, AF_THREADS, AF_SMEM, st>>>(G, S);
+  launch_overlapped(automaton_fill_kernel, dim3(S.af.grid), dim3(AF_THREADS), AF_SMEM, st, G, S);
 }
 
 }  // namespace fmt

@@ -1009,7 +1009,6 @@ void launch_fill(const GrammarDev& G, const StateDev& S, int sweep_grid, cudaStr
     if (S.af.on) launch_automaton_fill(G, S, st);
     else launch_sweep(G, S, sweep_grid, st);
     if (after_sweep) cudaEventRecord(after_sweep, st);
-    launch_publish(S, st);
     return;
   }
   if (before_roots) cudaEventRecord(before_roots, st);
@@ -1040,7 +1039,6 @@ void launch_fill(const GrammarDev& G, const StateDev& S, int sweep_grid, cudaStr
     cudaLaunchCooperativeKernel((const void*)fill_kernel, dim3((unsigned)sweep_grid), dim3(SWEEP_WARPS * 32), args, S.au.smem_bytes, st);
   }
   if (after_sweep) cudaEventRecord(after_sweep, st);
-  launch_publish(S, st);
 }
 
 }  // namespace fmt

@@ -285,6 +285,7 @@ struct StateDev {
   uint8_t* row_buf;           // [B] private buffer holding it (0..2) or 255 (pool / start chart)
   int32_t* row_state;         // [B] cache id or -1
   uint32_t* row_flags;        // [B]
+  uint32_t* row_job;          // [B] 1: the row's mask is computed by the fill that is under way
   int32_t* row_mask;          // [B] mask row holding the row's mask after a fill (or a special value)
   uint32_t* ht;               // [ht_mask+1] id+1, 0 = empty
   uint64_t* st_off;           // [max_states] word offset of the cached chart

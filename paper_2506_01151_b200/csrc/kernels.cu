@@ -1,4 +1,4 @@
-// CUDA kernels of the mask path (sm_100a): advance, plan / sweep / publish of the mask fill, gather
+// CUDA kernels of the mask path (sm_100a): advance, plan and sweep of the mask fill, gather
 // and the logits masking.  Integer work only: no tensor cores are involved anywhere.
 #include <cuda_runtime.h>
 
@@ -148,7 +148,8 @@ __global__ void __launch_bounds__(32) intern_init_kernel(StateDev S, int32_t* in
 }
 
 // rows[i] (or rows 0..n-1) go back to the start chart
-__global__ void reset_kernel(StateDev S, const uint32_t* rows, uint32_t n, const int32_t* init_state) {
+__global__ void reset_kernel(const __grid_constant__ StateDev S, const uint32_t* rows, uint32_t n, const int32_t* init_state) {
+  before_me();
   uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   uint32_t row = rows ? rows[i] : i;
@@ -165,8 +166,10 @@ __global__ void reset_kernel(StateDev S, const uint32_t* rows, uint32_t n, const
 constexpr int ADV_WARPS = 4;
 
 
-__global__ void __launch_bounds__(ADV_WARPS * 32, 1) advance_kernel(GrammarDev Gg, StateDev S, const int32_t* tokens,
-                                                                  int32_t* status) {
+__global__ void __launch_bounds__(ADV_WARPS * 32, 1) advance_kernel(const __grid_constant__ GrammarDev Gg,
+                                                                    const __grid_constant__ StateDev S, const int32_t* tokens,
+                                                                    int32_t* status) {
+  before_me();
   extern __shared__ __align__(16) uint32_t smem[];
   const uint32_t warp = threadIdx.x >> 5, lane = lane_id();
   const uint32_t row = blockIdx.x * ADV_WARPS + warp;
@@ -272,8 +275,10 @@ __global__ void __launch_bounds__(ADV_WARPS * 32, 1) advance_kernel(GrammarDev G
 // punctuation a JSON schema fixes, Section 5.1's JSON-Schema task): as long as the text is not a
 // sentence and the last Earley set can scan exactly one byte, that byte is taken and the chart is
 // stepped over it.  Nothing of the row changes: the sets made on the way live in the warp's scratch.
-__global__ void __launch_bounds__(ADV_WARPS * 32, 1) forced_kernel(GrammarDev Gg, StateDev S, uint8_t* bytes_out,
+__global__ void __launch_bounds__(ADV_WARPS * 32, 1) forced_kernel(const __grid_constant__ GrammarDev Gg,
+                                                                   const __grid_constant__ StateDev S, uint8_t* bytes_out,
                                                                    size_t stride, uint32_t* len_out, uint32_t max_len) {
+  before_me();
   extern __shared__ __align__(16) uint32_t smem[];
   const uint32_t warp = threadIdx.x >> 5, lane = lane_id();
   const uint32_t row = blockIdx.x * ADV_WARPS + warp;
@@ -301,24 +306,28 @@ __global__ void __launch_bounds__(ADV_WARPS * 32, 1) forced_kernel(GrammarDev Gg
 
 // One block decides, row by row, where each mask comes from: the state cache, another row of
 // this call with the same chart, or a fresh computation (a "job").
-__global__ void __launch_bounds__(1024) plan_kernel(GrammarDev G, StateDev S) {
+__global__ void __launch_bounds__(1024) plan_kernel(const __grid_constant__ GrammarDev G, const __grid_constant__ StateDev S) {
+  before_me();
+  __shared__ uint32_t n_jobs, n_rows, n_cached, n_shared;
   if (threadIdx.x < CNT_HASH_GEN - CNT_BAR) S.counters[CNT_BAR + threadIdx.x] = 0u;  // barrier and level counters
   if (threadIdx.x < CNT_LAST_LEVEL + 1 - CNT_LEVEL_TAKEN) S.counters[CNT_LEVEL_TAKEN + threadIdx.x] = 0u;
   if (threadIdx.x == 0) {
-    S.counters[CNT_N_JOBS] = 0u;
     S.counters[CNT_N_FJOBS] = 0u;
     S.counters[CNT_AUTO_ITEMS] = 0u;
     S.counters[CNT_AF_TICKET] = S.counters[CNT_AF_TAKEN] = S.counters[CNT_AF_POSTED] = 0u;
+    n_jobs = n_cached = n_shared = 0u;
+    n_rows = S.counters[CNT_N_MASK_ROWS];
   }
-  if (S.rt.counters) {  // the root sweep of this fill starts from clean counters, too
+  if (S.rt.on) {  // the root sweep of this fill starts from clean counters, too
     if (threadIdx.x < CNT_HASH_GEN - CNT_BAR) S.rt.counters[CNT_BAR + threadIdx.x] = 0u;
     if (threadIdx.x < CNT_LAST_LEVEL + 1 - CNT_LEVEL_TAKEN) S.rt.counters[CNT_LEVEL_TAKEN + threadIdx.x] = 0u;
     if (threadIdx.x == 0) S.rt.counters[CNT_N_JOBS] = 0u, S.rt.counters[CNT_AUTO_ITEMS] = 0u;
   }
   __syncthreads();
   for (uint32_t row = threadIdx.x; row < S.B; row += blockDim.x) {
-    stat_add(S, CNT_STAT_FILLS, 1u);
     const uint32_t flags = S.row_flags[row];
+    const int32_t sid = S.row_state[row];
+    S.row_job[row] = 0u;
     if (flags & ROW_BROKEN) {
       S.row_mask[row] = MASK_ZERO;
       continue;
@@ -327,37 +336,39 @@ __global__ void __launch_bounds__(1024) plan_kernel(GrammarDev G, StateDev S) {
       S.row_mask[row] = MASK_EOS_ONLY;
       continue;
     }
-    const int32_t sid = S.row_state[row];
+    int32_t mrow = (int32_t)row;
     if (sid >= 0) {
-      int32_t old = atomicCAS(&S.st_mask[sid], -1, -2 - (int32_t)row);
+      const int32_t old = atomicCAS(&S.st_mask[sid], -1, -2 - (int32_t)row);
       if (old >= 0) {  // cached
         S.st_ref[sid] = 1;  // (used again: it outlives the next emptying of the cache)
         S.row_mask[row] = old;
-        stat_add(S, CNT_STAT_CACHED, 1u);
+        atomicAdd(&n_cached, 1u);
         continue;
       }
       if (old <= -2) {  // another row of this call computes it
         S.row_mask[row] = MASK_ALIAS0 - (-2 - old);
-        stat_add(S, CNT_STAT_SHARED, 1u);
+        atomicAdd(&n_shared, 1u);
         continue;
       }
       // this row computes it, into a cache row if one is left
-      int32_t mrow = (int32_t)row;
-      if (ld_acquire(&S.counters[CNT_N_MASK_ROWS]) < S.max_mask_rows) {
-        uint32_t got = atomicAdd(&S.counters[CNT_N_MASK_ROWS], 1u);
-        if (got < S.max_mask_rows) mrow = (int32_t)(S.mrow_base + got);
-      }
-      if (mrow == (int32_t)row && S.full_flag) *reinterpret_cast<volatile uint32_t*>(S.full_flag) = 1u;  // no mask row left to cache it in
-      S.row_mask[row] = mrow;
-    } else {
-      S.row_mask[row] = (int32_t)row;
+      const uint32_t got = atomicAdd(&n_rows, 1u);
+      if (got < S.max_mask_rows) mrow = (int32_t)(S.mrow_base + got);
+      else if (S.full_flag) *reinterpret_cast<volatile uint32_t*>(S.full_flag) = 1u;  // no mask row left to cache it in
     }
-    stat_add(S, CNT_STAT_COMPUTED, 1u);
-    uint32_t j = atomicAdd(&S.counters[CNT_N_JOBS], 1u);
-    S.jobs[j] = row;
+    S.row_mask[row] = mrow;
+    S.row_job[row] = 1u;
+    S.jobs[atomicAdd(&n_jobs, 1u)] = row;
   }
   __syncthreads();
-  if (threadIdx.x == 0) S.counters[CNT_AF_ACTIVE] = ld_acquire(&S.counters[CNT_N_JOBS]) * S.af.parts;
+  if (threadIdx.x == 0) {
+    S.counters[CNT_N_JOBS] = n_jobs;
+    S.counters[CNT_N_MASK_ROWS] = min(n_rows, max(S.max_mask_rows, S.counters[CNT_N_MASK_ROWS]));
+    S.counters[CNT_AF_ACTIVE] = n_jobs * S.af.parts;
+    stat_add(S, CNT_STAT_FILLS, S.B);
+    if (n_cached) stat_add(S, CNT_STAT_CACHED, n_cached);
+    if (n_shared) stat_add(S, CNT_STAT_SHARED, n_shared);
+    if (n_jobs) stat_add(S, CNT_STAT_COMPUTED, n_jobs);
+  }
 }
 
 // ===================================================================================== fill: sweep
@@ -738,43 +749,35 @@ __global__ void __launch_bounds__(SWEEP_WARPS * 32, 1) sweep_kernel(GrammarDev G
   }
 }
 
-// Publish the masks computed in this call to the cache (or release the claim when the row had
-// no cache row, or broke).
-__global__ void publish_kernel(StateDev S) {
-  const uint32_t j = blockIdx.x * blockDim.x + threadIdx.x;
-  const uint32_t n_jobs = S.counters[CNT_N_JOBS];
-  if (j < n_jobs) {
-    const uint32_t row = S.jobs[j];
-    const int32_t sid = S.row_state[row];
-    // a fill that was given up (a bounded wait ran out) hands out all-zero masks, never a guess; the
-    // rows themselves are fine and the next fill computes them afresh
-    const bool aborted = S.counters[CNT_BAR_ERR] != 0u;
-    const bool broken = (S.row_flags[row] & ROW_BROKEN) || aborted;
-    if (sid >= 0) {
-      const int32_t mrow = S.row_mask[row];
-      S.st_mask[sid] = (!broken && mrow >= (int32_t)S.B) ? mrow : -1;
-    }
-    if (aborted) {
-      S.row_mask[row] = MASK_ZERO;
-      if (j == 0) stat_add(S, CNT_STAT_ABORTS, 1u);
-    }
-  }
-}
-
+// The mask row of a row after a fill.  A fill that was given up (a bounded wait ran out) hands out all-zero masks, never a guess;
+// the rows themselves are fine and the next fill computes them afresh.
 __device__ __forceinline__ int32_t resolve_mask_row(const StateDev& S, uint32_t row) {
   int32_t r = S.row_mask[row];
-  if (S.row_flags[row] & ROW_BROKEN) return MASK_ZERO;
+  const bool aborted = S.counters[CNT_BAR_ERR] != 0u;
+  if ((S.row_flags[row] & ROW_BROKEN) || (aborted && S.row_job[row])) return MASK_ZERO;
   if (r <= MASK_ALIAS0) {  // the mask another row of this call computed: not to be used if that row broke
     const uint32_t other = (uint32_t)(MASK_ALIAS0 - r);
-    if (S.row_flags[other] & ROW_BROKEN) return MASK_ZERO;
+    if (aborted || (S.row_flags[other] & ROW_BROKEN)) return MASK_ZERO;
     r = S.row_mask[other];
   }
   return r;
 }
+// (one thread per row, in the kernel that reads the masks) A mask computed in this call becomes the cache's, or its claim is
+// released: when the row had no cache row, or broke, or the fill was given up.
+__device__ __forceinline__ void publish_row(const StateDev& S, uint32_t row) {
+  if (!S.row_job[row]) return;
+  const bool aborted = S.counters[CNT_BAR_ERR] != 0u;
+  const int32_t sid = S.row_state[row], mrow = S.row_mask[row];
+  if (sid >= 0) S.st_mask[sid] = (!(S.row_flags[row] & ROW_BROKEN) && !aborted && mrow >= (int32_t)S.B) ? mrow : -1;
+  if (aborted && row == S.jobs[0]) stat_add(S, CNT_STAT_ABORTS, 1u);
+}
 
 // mask_out[row][w] for every row
-__global__ void gather_kernel(GrammarDev G, StateDev S, uint32_t* out, size_t stride_words) {
+__global__ void gather_kernel(const __grid_constant__ GrammarDev G, const __grid_constant__ StateDev S, uint32_t* out,
+                              size_t stride_words) {
+  before_me();
   const uint32_t row = blockIdx.y;
+  if (blockIdx.x == 0 && threadIdx.x == 0) publish_row(S, row);
   const int32_t r = resolve_mask_row(S, row);
   const uint32_t* src = (r >= 0) ? S.mask_rows + (size_t)r * G.Wm : nullptr;
   uint32_t* dst = out + (size_t)row * stride_words;
@@ -866,14 +869,17 @@ __device__ __forceinline__ void apply_row(const uint32_t* mask_row, int32_t spec
 
 template <typename T>
 __global__ void apply_kernel(const uint32_t* mask, size_t stride_words, T* logits, uint32_t V, size_t row_stride) {
+  before_me();
   const uint32_t row = blockIdx.y;
   apply_row<T>(mask + (size_t)row * stride_words, 0, -1, logits + (size_t)row * row_stride, V, nullptr);
 }
 
 template <typename T>
-__global__ void gather_apply_kernel(GrammarDev G, StateDev S, T* logits, size_t row_stride, uint32_t* mask_out,
-                                    size_t stride_words) {
+__global__ void gather_apply_kernel(const __grid_constant__ GrammarDev G, const __grid_constant__ StateDev S, T* logits,
+                                    size_t row_stride, uint32_t* mask_out, size_t stride_words) {
+  before_me();
   const uint32_t row = blockIdx.y;
+  if (blockIdx.x == 0 && threadIdx.x == 0) publish_row(S, row);
   const int32_t r = resolve_mask_row(S, row);
   const uint32_t* src = (r >= 0) ? S.mask_rows + (size_t)r * G.Wm : nullptr;
   uint32_t* mo = mask_out ? mask_out + (size_t)row * stride_words : nullptr;
@@ -1015,14 +1021,15 @@ void launch_intern_init(const StateDev& S, int32_t* init_state_dev, cudaStream_t
 }
 void launch_reset(const StateDev& S, const uint32_t* rows_dev, uint32_t n, const int32_t* init_state_dev, cudaStream_t st) {
   if (n == 0) return;
-  reset_kernel<<<(n + 127) / 128, 128, 0, st>>>(S, rows_dev, n, init_state_dev);
+  launch_overlapped(reset_kernel, dim3((n + 127) / 128), dim3(128), 0, st, S, rows_dev, n, init_state_dev);
 }
 void launch_forced(const GrammarDev& G, const StateDev& S, uint8_t* bytes_out, size_t stride, uint32_t* len_out,
                    uint32_t max_len, cudaStream_t st) {
-  forced_kernel<<<(S.B + ADV_WARPS - 1) / ADV_WARPS, ADV_WARPS * 32, adv_smem_bytes(G), st>>>(G, S, bytes_out, stride, len_out, max_len);
+  launch_overlapped(forced_kernel, dim3((S.B + ADV_WARPS - 1) / ADV_WARPS), dim3(ADV_WARPS * 32), adv_smem_bytes(G), st, G, S, bytes_out,
+                    stride, len_out, max_len);
 }
 void launch_advance(const GrammarDev& G, const StateDev& S, const int32_t* tokens, int32_t* status, cudaStream_t st) {
-  advance_kernel<<<(S.B + ADV_WARPS - 1) / ADV_WARPS, ADV_WARPS * 32, adv_smem_bytes(G), st>>>(G, S, tokens, status);
+  launch_overlapped(advance_kernel, dim3((S.B + ADV_WARPS - 1) / ADV_WARPS), dim3(ADV_WARPS * 32), adv_smem_bytes(G), st, G, S, tokens, status);
 }
 static void launch_sweep_coop(const GrammarDev& G, const StateDev& S, int grid, cudaStream_t st) {
   GrammarDev g = G;
@@ -1031,13 +1038,14 @@ static void launch_sweep_coop(const GrammarDev& G, const StateDev& S, int grid, 
   cudaLaunchCooperativeKernel((const void*)sweep_kernel, dim3((unsigned)grid), dim3(SWEEP_WARPS * 32), args,
                               S.au.smem_bytes, st);
 }
-void launch_plan(const GrammarDev& G, const StateDev& S, cudaStream_t st) { plan_kernel<<<1, 1024, 0, st>>>(G, S); }
-void launch_publish(const StateDev& S, cudaStream_t st) { publish_kernel<<<(S.B + 255) / 256, 256, 0, st>>>(S); }
+void launch_plan(const GrammarDev& G, const StateDev& S, cudaStream_t st) {
+  launch_overlapped(plan_kernel, dim3(1), dim3(std::min<uint32_t>(1024u, std::max<uint32_t>(64u, (S.B + 31u) / 32u * 32u))), 0, st, G, S);
+}
 // the sweep alone, for jobs the caller has already listed (used by the allocation-free entry point)
 void launch_sweep(const GrammarDev& G, const StateDev& S, int grid, cudaStream_t st) { launch_sweep_coop(G, S, grid, st); }
 void launch_gather(const GrammarDev& G, const StateDev& S, uint32_t* out, size_t stride_words, cudaStream_t st) {
   dim3 grid((unsigned)std::min<size_t>((stride_words + 255) / 256, 64), S.B);
-  gather_kernel<<<grid, 256, 0, st>>>(G, S, out, stride_words);
+  launch_overlapped(gather_kernel, grid, dim3(256), 0, st, G, S, out, stride_words);
 }
 static dim3 apply_grid(uint32_t V, int dtype, uint32_t batch) {
   const uint32_t units = V / (dtype == FMT_BF16 ? 16u : 8u) + 1u;
@@ -1047,16 +1055,16 @@ void launch_apply(const uint32_t* mask, size_t stride_words, void* logits, int d
                   size_t row_stride, cudaStream_t st) {
   if (batch == 0 || V == 0) return;
   const dim3 grid = apply_grid(V, dtype, batch);
-  if (dtype == FMT_BF16) apply_kernel<uint16_t><<<grid, 256, 0, st>>>(mask, stride_words, (uint16_t*)logits, V, row_stride);
-  else apply_kernel<uint32_t><<<grid, 256, 0, st>>>(mask, stride_words, (uint32_t*)logits, V, row_stride);
+  if (dtype == FMT_BF16) launch_overlapped(apply_kernel<uint16_t>, grid, dim3(256), 0, st, mask, stride_words, (uint16_t*)logits, V, row_stride);
+  else launch_overlapped(apply_kernel<uint32_t>, grid, dim3(256), 0, st, mask, stride_words, (uint32_t*)logits, V, row_stride);
 }
 void launch_gather_apply(const GrammarDev& G, const StateDev& S, void* logits, int dtype, size_t row_stride,
                          uint32_t* mask_out, size_t stride_words, cudaStream_t st) {
   const dim3 grid = apply_grid(G.V, dtype, S.B);
   if (dtype == FMT_BF16)
-    gather_apply_kernel<uint16_t><<<grid, 256, 0, st>>>(G, S, (uint16_t*)logits, row_stride, mask_out, stride_words);
+    launch_overlapped(gather_apply_kernel<uint16_t>, grid, dim3(256), 0, st, G, S, (uint16_t*)logits, row_stride, mask_out, stride_words);
   else
-    gather_apply_kernel<uint32_t><<<grid, 256, 0, st>>>(G, S, (uint32_t*)logits, row_stride, mask_out, stride_words);
+    launch_overlapped(gather_apply_kernel<uint32_t>, grid, dim3(256), 0, st, G, S, (uint32_t*)logits, row_stride, mask_out, stride_words);
 }
 void launch_evacuate(const StateDev& S, cudaStream_t st) { evacuate_kernel<<<S.B, 128, 0, st>>>(S); }
 void launch_reintern(const StateDev& S, int32_t* init_state_dev, cudaStream_t st) {

@@ -6,6 +6,28 @@
 
 namespace fmt {
 
+// A launch that may begin while the kernel before it in the stream is still running: its blocks are set up meanwhile, and wait
+// at before_me() until that kernel is through and its writes are visible.  The kernels of a decoding step are launched this way:
+// several of them last a few microseconds, and the gap between two launches is as long (five launches for one row whose
+// answers are all cached: @A us one after the other, @B us overlapped).
+template <class... P, class... A>
+inline cudaError_t launch_overlapped(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A&&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid, cfg.blockDim = block, cfg.dynamicSmemBytes = smem, cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at, cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+#ifdef __CUDACC__
+// First thing in a kernel launched so (without effect in one launched otherwise): let the next one be set up, wait for the one before.
+__device__ __forceinline__ void before_me() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+#endif
+
 constexpr int SWEEP_WARPS = 24;  // warps of a CTA of the trie sweep: one CTA per SM, so that the grid barrier has few arrivals
 
 cudaError_t configure_kernels();
@@ -26,7 +48,6 @@ void launch_advance(const GrammarDev& G, const StateDev& S, const int32_t* token
 void launch_forced(const GrammarDev& G, const StateDev& S, uint8_t* bytes_out, size_t stride, uint32_t* len_out, uint32_t max_len,
                    cudaStream_t st);
 void launch_plan(const GrammarDev& G, const StateDev& S, cudaStream_t st);
-void launch_publish(const StateDev& S, cudaStream_t st);
 cudaError_t configure_walk_kernels();
 void launch_fill(const GrammarDev& G, const StateDev& S, int sweep_grid, cudaStream_t st, cudaEvent_t before_roots = nullptr,
                  cudaEvent_t after_roots = nullptr, cudaEvent_t before_sweep = nullptr, cudaEvent_t after_sweep = nullptr);
