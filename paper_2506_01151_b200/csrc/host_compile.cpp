@@ -414,7 +414,7 @@ class DfaBuilder {
       while (!call.empty()) {
         Frame& f = call.back();
         bool descended = false;
-        while (f.rule < by_lhs_[f.v].size() && !descended) {
+        while (!descended && f.rule < by_lhs_[f.v].size()) {  // (f is gone once a callee has been pushed)
           const Production& p = rules_[by_lhs_[f.v][f.rule]];
           while (f.sym < p.rhs.size()) {
             const int w = p.rhs[f.sym++];
