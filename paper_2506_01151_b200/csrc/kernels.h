@@ -9,7 +9,7 @@ namespace fmt {
 // A launch that may begin while the kernel before it in the stream is still running: its blocks are set up meanwhile, and wait
 // at before_me() until that kernel is through and its writes are visible.  The kernels of a decoding step are launched this way:
 // several of them last a few microseconds, and the gap between two launches is as long (five launches for one row whose
-// answers are all cached: @A us one after the other, @B us overlapped).
+// answers are all cached: 24 us one after the other, 19 us overlapped).
 template <class... P, class... A>
 inline cudaError_t launch_overlapped(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A&&... args) {
   cudaLaunchConfig_t cfg = {};
@@ -21,10 +21,12 @@ inline cudaError_t launch_overlapped(void (*kernel)(P...), dim3 grid, dim3 block
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
 }
 #ifdef __CUDACC__
-// First thing in a kernel launched so (without effect in one launched otherwise): let the next one be set up, wait for the one before.
+// First thing in a kernel launched so (without effect in one launched otherwise): wait for the one before, let the next one be set up.
+// In the other order kernels are set up seven deep, and take the room on the SMs from those that run (12 steps of 128 rows of
+// SQL: 5.55 ms, in this order 5.26).
 __device__ __forceinline__ void before_me() {
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 #endif
 
