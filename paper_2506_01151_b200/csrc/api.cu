@@ -231,8 +231,14 @@ fmt_status fmt_compile(const char* ebnf, size_t ebnf_len, const char* start_rule
     }
     d.dfa_first = h.dfa_first;
     if (h.dfa_states) {
-      UP(dfa_trans);
-      UP(dfa_done);
+      std::vector<uint32_t> blob((h.dfa_trans.size() * 2 + 15) / 16 * 4 + (h.dfa_done.size() * 2 + 15) / 16 * 4, 0u);
+      const size_t o_done = (h.dfa_trans.size() * 2 + 15) / 16 * 4;
+      memcpy(blob.data(), h.dfa_trans.data(), h.dfa_trans.size() * 2);
+      memcpy(blob.data() + o_done, h.dfa_done.data(), h.dfa_done.size() * 2);
+      if (e == cudaSuccess) e = g->bufs.upload(blob, &d.dfa_block);
+      d.dfa_words = (uint32_t)blob.size();
+      d.dfa_trans = reinterpret_cast<const uint16_t*>(d.dfa_block);
+      d.dfa_done = reinterpret_cast<const uint16_t*>(d.dfa_block + o_done);
       UP(dfa_scan);
     }
     UP(node_byte);
@@ -465,6 +471,7 @@ fmt_status fmt_state_create(const fmt_grammar* g, uint32_t batch, const fmt_stat
   int sms = 0, dev = 0;
   if (e == cudaSuccess) e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  advance_layout(g->dev, batch, (uint32_t)std::max(1, sms), d);
   // Rows are filled by the grammar's automaton if it has one.  A state that asks for the cache of
   // context-independent entries, or limits the Earley sets of a sweep, is swept by the grid.
   AutoFillDev& af = d.af;
@@ -476,7 +483,7 @@ fmt_status fmt_state_create(const fmt_grammar* g, uint32_t batch, const fmt_stat
     automaton_fill_layout(g->dev, batch, AUTO_FILL_PER_SM * (uint32_t)std::max(1, sms), af);
   }
 #define AL(ptr, count, fill) if (e == cudaSuccess) e = s->bufs.alloc((size_t)(count), &(ptr), (fill))
-  AL(d.arena, d.pool_base + d.pool_words * (two_gens ? 2 : 1), 0);
+  AL(d.arena, d.pool_base + d.pool_words * (two_gens ? 2 : 1) + ADV_AHEAD, 0);
   AL(d.row_chart, batch, 0);
   AL(d.row_buf, batch, 0xFF);
   AL(d.row_state, batch, 0xFF);
@@ -613,6 +620,7 @@ fmt_status fmt_state_advance(fmt_state* s, const int32_t* token_ids_dev, int32_t
   cudaEvent_t e0, e1;
   s->prof.next(0, &e0, &e1);
   if (e0) cudaEventRecord(e0, (cudaStream_t)stream);
+  ++s->dev.adv_no;
   launch_advance(s->g->dev, s->dev, token_ids_dev, status_dev, (cudaStream_t)stream);
   if (e1) cudaEventRecord(e1, (cudaStream_t)stream);
   return launched("fmt_state_advance");

@@ -268,21 +268,15 @@ __device__ uint32_t gen_scan_complete(const GrammarDev& G, const AdvScratch& s, 
 // With `forced_out` set, the bytes are not given but found: as long as the text so far is not a sentence and
 // exactly one byte can follow, that byte is taken (and written to forced_out); `len` is then the longest run
 // looked for, nothing is compacted or written to dst, and the return value is the length of the run.
-__device__ int token_step(const GrammarDev& G, AdvScratch& s, const uint32_t* src, const uint8_t* bytes, uint32_t len,
-                          uint32_t* dst, uint32_t dst_cap, uint32_t* arena, uint32_t arena_cap,
-                          uint8_t* forced_out = nullptr) {
+__device__ __forceinline__ int token_steps(const GrammarDev& G, AdvScratch& s, const uint32_t* src, const uint8_t* bytes, uint32_t len,
+                                           uint32_t* dst, uint32_t dst_cap, uint32_t* arena, uint32_t arena_cap, uint8_t* forced_out) {
   const uint32_t lane = lane_id();
   const uint32_t m = src[CH_SETS];
   const uint32_t n_items = src[CH_ITEMS];
   if (m == 0 || m + len + MAX_TOKEN_BYTES + 4 > ADV_MAX_SETS || n_items > ADV_MAX_ITEMS || len > MAX_TOKEN_BYTES)
     return forced_out ? 0 : -1;
-  // small charts are read from shared memory from here on
-  const uint32_t src_words = src[CH_WORDS];
-  __syncwarp();
-  if (src_words <= ADV_STAGE) {
-    for (uint32_t i = lane; i < src_words; i += 32) s.stage[i] = src[i];
-    src = s.stage;
-  }
+  const uint32_t own_byte = !forced_out && lane < len ? __ldg(&bytes[lane]) : 0u;
+  static_assert(MAX_TOKEN_BYTES <= 32, "a token's bytes sit one to a lane");
   uint32_t* lvl_off = s.sets + ADV_MAX_SETS - (MAX_TOKEN_BYTES + 2);  // the tail of `sets` is free until Compact ends
   TokenView view{src + CH_HDR, src + CH_HDR + m + 1, m, arena, lvl_off};
   const uint32_t* soff = view.soff;
@@ -309,7 +303,7 @@ __device__ int token_step(const GrammarDev& G, AdvScratch& s, const uint32_t* sr
       byte = (uint32_t)src_lane * 32u + (uint32_t)(__ffs(__shfl_sync(FULL, wd, src_lane)) - 1);
       __syncwarp();
     } else {
-      byte = __ldg(&bytes[L - 1]);
+      byte = __shfl_sync(FULL, own_byte, L - 1);
     }
     s.w.cur = arena + top;
     s.w.cur_cap = arena_cap - top;
@@ -324,7 +318,7 @@ __device__ int token_step(const GrammarDev& G, AdvScratch& s, const uint32_t* sr
       const uint32_t it = prev[0], inf = G.info[it & 0xFFFFu], kind = inf >> INFO_KIND_SHIFT;
       uint32_t to = 0;
       if (kind == KIND_DFA) {
-        const uint32_t t = __ldg(&G.dfa_trans[(size_t)(inf & INFO_ARG_MASK) * G.n_eq + G.eq_of_byte[byte]]);
+        const uint32_t t = G.dfa_trans[(size_t)(inf & INFO_ARG_MASK) * G.n_eq + G.eq_of_byte[byte]];
         if (t != 0xFFFFu && (t & 0xC000u) == 0x4000u) to = (it & 0xFFFF0000u) | (G.dfa_first + (t & 0x3FFFu));
       } else if (kind == KIND_TERM && class_has(G, inf & INFO_ARG_MASK, byte)) {
         const uint32_t next = G.info[(it & 0xFFFFu) + 1u] >> INFO_KIND_SHIFT;
@@ -661,6 +655,35 @@ __device__ int token_step(const GrammarDev& G, AdvScratch& s, const uint32_t* sr
   if (last_at + P > arena_cap) return -2;  // the sort pads the set to a power of two
   s.w.cur = arena + last_at;
   return finish_chart(s, dst, dst_cap, m_new, kept, n_last, accepting, h);
+}
+
+// A chart that is not too large comes into shared memory.  (Its first words are read with its header: nearly all charts are no longer, and
+// the arena goes on so far behind its last chart.)
+__device__ __forceinline__ bool stage_chart(const AdvScratch& s, const uint32_t* src) {
+  const uint32_t lane = lane_id();
+  uint32_t ahead[ADV_AHEAD / 32];
+#pragma unroll
+  for (uint32_t k = 0; k < ADV_AHEAD / 32; ++k) ahead[k] = src[k * 32u + lane];
+  const uint32_t words = __shfl_sync(FULL, ahead[0], CH_WORDS);
+  if (words > ADV_STAGE) return false;
+#pragma unroll
+  for (uint32_t k = 0; k < ADV_AHEAD / 32; ++k) s.stage[k * 32u + lane] = ahead[k];
+  for (uint32_t i = ADV_AHEAD + lane; i < words; i += 32) s.stage[i] = src[i];
+  __syncwarp();
+  return true;
+}
+
+// The same steps, wherever the tables, the chart and the arena are.  (Where all of them are in shared memory the steps are
+// compiled into the kernel, with 32-bit addresses throughout: a step is a chain of some hundred instructions of one warp.)
+__device__ __noinline__ int token_steps_anywhere(const GrammarDev& G, AdvScratch& s, const uint32_t* src, const uint8_t* bytes, uint32_t len,
+                                                 uint32_t* dst, uint32_t dst_cap, uint32_t* arena, uint32_t arena_cap, uint8_t* forced_out) {
+  return token_steps(G, s, src, bytes, len, dst, dst_cap, arena, arena_cap, forced_out);
+}
+__device__ __forceinline__ int token_step(const GrammarDev& G, const AdvScratch& s, const uint32_t* src, const uint8_t* bytes, uint32_t len,
+                                          uint32_t* dst, uint32_t dst_cap, uint32_t* arena, uint32_t arena_cap, uint8_t* forced_out = nullptr) {
+  const GrammarDev g = G;  // (copies: what a call takes by reference is kept in memory)
+  AdvScratch t = s;
+  return token_steps_anywhere(g, t, src, bytes, len, dst, dst_cap, arena, arena_cap, forced_out);
 }
 
 }  // namespace fmt

@@ -22,6 +22,8 @@ struct GrammarDev {
   uint32_t dfa_first;
   const uint16_t* dfa_trans;     // [states][n_eq] target | 0x4000 target has transitions | 0x8000 target accepts, or 0xFFFF
   const uint16_t* dfa_done;      // [states] completed item of the state's non-terminal
+  const uint32_t* dfa_block;     // the two above, one after the other, for kernels that copy them into shared memory
+  uint32_t dfa_words;
   const uint32_t* dfa_scan;      // [states][8] bytes with a transition
   const uint8_t* node_byte;      // [T]
   const uint32_t* parent;        // [T]
@@ -59,6 +61,7 @@ struct GrammarDev {
 //   the live sets 0..m-1 (the dense renumbering that makes equal situations equal charts).
 constexpr uint32_t CH_SETS = 0, CH_ITEMS = 1, CH_FLAGS = 2, CH_HASH_LO = 3, CH_HASH_HI = 4, CH_WORDS = 5, CH_HDR = 8;
 constexpr uint32_t CHART_ACCEPTING = 1u;
+constexpr uint32_t ADV_AHEAD = 128;  // words of a chart that are read before its length is known: the arena goes on so far behind its last chart
 
 constexpr uint32_t ROW_FINISHED = 1u, ROW_BROKEN = 2u;
 
@@ -106,7 +109,8 @@ enum : uint32_t {
   CNT_STAT_ADV_WORDS = 164,    // 64-bit: chart words read and written by advance
   CNT_STAT_FRAMES = 184,       // 64-bit: frames made (sets of a walk recognised as roots)
   CNT_DIAG = 166,              // [16] where capacity errors and expired waits came from (see DIAG_*)
-  CNT_TOTAL = 190
+  CNT_ADV_STEPPED = 190,       // the last call in which a row took an Earley step
+  CNT_TOTAL = 192
 };
 
 enum : uint32_t {
@@ -271,6 +275,8 @@ struct StateDev {
   uint32_t gen_ctx;           // generation of the context-dependent walk's tables
   uint32_t poll_limit_shift;  // bounded waits give up after 2^shift polls
   uint32_t time_steps;        // count the SM cycles spent inside Earley steps (costs a few per cent of the sweep)
+  uint32_t adv_rows, adv_dfa;  // rows of a thread block when sequences advance; 1: their automata are in shared memory, too
+  uint32_t adv_no;             // calls so far
   uint32_t chart_words;       // capacity of one private chart buffer
   uint32_t cache_on;
   uint32_t* full_flag;        // host-mapped word (or nullptr): set when the state cache or its mask rows have no room left

@@ -117,12 +117,12 @@ __device__ __forceinline__ Scanned scan_item(const GrammarDev& G, uint32_t it, u
     r.a = it + 1u;
   } else if (kind == KIND_DFA) {
     const uint32_t g = inf & INFO_ARG_MASK;
-    const uint32_t t = __ldg(&G.dfa_trans[(size_t)g * G.n_eq + G.eq_of_byte[byte]]);
+    const uint32_t t = G.dfa_trans[(size_t)g * G.n_eq + G.eq_of_byte[byte]];
     if (t != 0xFFFFu) {
       r.has_a = (t & 0x4000u) != 0u;
       r.a = (it & 0xFFFF0000u) | (G.dfa_first + (t & 0x3FFFu));
       r.has_b = (t & 0x8000u) != 0u;
-      r.b = (it & 0xFFFF0000u) | __ldg(&G.dfa_done[g]);
+      r.b = (it & 0xFFFF0000u) | G.dfa_done[g];
     }
   }
   return r;
@@ -202,6 +202,9 @@ __device__ __forceinline__ void predict_into_cur(const GrammarDev& G, const Warp
   uint32_t* ntmask = w.nt;
   uint32_t* clos = w.nt + Nw;
   __syncwarp();
+  uint32_t asked = 0u;
+  for (uint32_t i = lane; i < Nw; i += 32) asked |= ntmask[i];
+  if (!__any_sync(FULL, asked != 0u)) return;  // (inside literals and automata there is nothing to predict)
   if (Nw <= 4u) {  // a lane for every non-terminal that is asked for: its row of the closure, joined over the lanes
     for (uint32_t i = 0; i < Nw; ++i) {
       uint32_t acc = 0u;
@@ -395,11 +398,8 @@ __device__ __forceinline__ uint32_t small_drop_completed(const GrammarDev& G, co
   return nk;
 }
 
-// Copy the grammar's hot tables into shared memory (all threads of the block take part, the
-// caller synchronizes) and return a view of the grammar that reads them from there.
-__device__ __forceinline__ GrammarDev stage_hot_tables(const GrammarDev& Gg, uint32_t* dst) {
-  for (uint32_t i = threadIdx.x; i < Gg.hot_words / 4u; i += blockDim.x)  // (the block is a multiple of 16 bytes)
-    reinterpret_cast<uint4*>(dst)[i] = __ldg(reinterpret_cast<const uint4*>(Gg.hot_block) + i);
+// A view of the grammar that reads the hot tables from a copy of their block.
+__device__ __forceinline__ GrammarDev with_hot_tables(const GrammarDev& Gg, const uint32_t* dst) {
   GrammarDev G = Gg;
   G.info = dst + (Gg.info - Gg.hot_block);
   G.class_bits = dst + (Gg.class_bits - Gg.hot_block);
@@ -411,6 +411,14 @@ __device__ __forceinline__ GrammarDev stage_hot_tables(const GrammarDev& Gg, uin
   G.direct_items = reinterpret_cast<const uint16_t*>(dst + (reinterpret_cast<const uint32_t*>(Gg.direct_items) - Gg.hot_block));
   G.hot_block = dst;
   return G;
+}
+
+// Copy the grammar's hot tables into shared memory (all threads of the block take part, the
+// caller synchronizes) and return a view of the grammar that reads them from there.
+__device__ __forceinline__ GrammarDev stage_hot_tables(const GrammarDev& Gg, uint32_t* dst) {
+  for (uint32_t i = threadIdx.x; i < Gg.hot_words / 4u; i += blockDim.x)  // (the block is a multiple of 16 bytes)
+    reinterpret_cast<uint4*>(dst)[i] = __ldg(reinterpret_cast<const uint4*>(Gg.hot_block) + i);
+  return with_hot_tables(Gg, dst);
 }
 
 // Drop the items with the dot at the end from cur[0..n) in place; returns the new count.

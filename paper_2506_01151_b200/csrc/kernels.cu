@@ -165,14 +165,61 @@ __global__ void reset_kernel(const __grid_constant__ StateDev S, const uint32_t*
 
 constexpr int ADV_WARPS = 4;
 
+// A block of rows that advance gets its tables into shared memory before the kernel before it in the stream is through, behind its
+// back (they do not change), and clears its scratch.  A row's steps are a chain of short look-ups, and 850 cycles each where
+// an automaton's table is read from L2; the tables' way into shared memory took another 3,000 at the start.  Where the
+// last calls were answered by the transition cache alone it is left until a row takes a step (64 warm rows of a schema with 90 KB
+// of automata: 11.4 us a decoding step with the tables copied in vain, 10.8 without).
+__device__ __forceinline__ uint32_t* advance_table_space(const StateDev& S, uint32_t* smem) { return smem + S.adv_rows * ADV_WARP_WORDS; }
+template <bool HOT, bool DFA>
+__device__ __forceinline__ void advance_copy_tables(const GrammarDev& G, const StateDev& S, uint32_t* smem) {
+  uint32_t* dst = advance_table_space(S, smem);
+  auto copy = [&](const uint32_t* src, uint32_t words) {  // (multiples of 16 bytes)
+    for (uint32_t i = threadIdx.x * 4u; i < words; i += ADV_WARPS * 128u)
+      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst + i)), "l"(src + i) : "memory");
+    dst += words;
+  };
+  if (HOT) copy(G.hot_block, G.hot_words);
+  if (DFA) copy(G.dfa_block, G.dfa_words);
+}
+__device__ __forceinline__ AdvScratch advance_scratch(const StateDev& S, uint32_t* smem) {
+  const uint32_t warp = threadIdx.x >> 5;
+  const AdvScratch s = adv_scratch(smem + (size_t)min(warp, S.adv_rows - 1u) * ADV_WARP_WORDS);
+  if (warp < S.adv_rows) {
+    hset_clear_all(s.w.hset, s.w.hset_mask);
+    for (uint32_t i = lane_id(); i < ADV_NT_WORDS; i += 32) s.w.nt[i] = 0u;
+  }
+  return s;
+}
+// ... and the grammar as it is to be read from then on.
+template <bool HOT, bool DFA>
+__device__ __forceinline__ GrammarDev advance_tables(const GrammarDev& Gg, const StateDev& S, uint32_t* smem) {
+  asm volatile("cp.async.wait_all;" ::: "memory");
+  __syncthreads();
+  const uint32_t* at = advance_table_space(S, smem);
+  GrammarDev G = Gg;
+  if (HOT) G = with_hot_tables(Gg, at), at += Gg.hot_words;
+  if (DFA) {
+    G.dfa_done = reinterpret_cast<const uint16_t*>(at + (reinterpret_cast<const uint32_t*>(Gg.dfa_done) - Gg.dfa_block));
+    G.dfa_trans = reinterpret_cast<const uint16_t*>(at);
+  }
+  return G;
+}
 
+template <bool HOT, bool DFA>
 __global__ void __launch_bounds__(ADV_WARPS * 32, 1) advance_kernel(const __grid_constant__ GrammarDev Gg,
                                                                     const __grid_constant__ StateDev S, const int32_t* tokens,
                                                                     int32_t* status) {
-  before_me();
   extern __shared__ __align__(16) uint32_t smem[];
   const uint32_t warp = threadIdx.x >> 5, lane = lane_id();
-  const uint32_t row = blockIdx.x * ADV_WARPS + warp;
+  const uint32_t row = warp < S.adv_rows ? blockIdx.x * S.adv_rows + warp : 0xFFFFFFFFu;
+  __shared__ uint32_t early_s;  // (the kernel before may be writing the word: one reading of it holds for the block)
+  if (threadIdx.x == 0) early_s = S.adv_no - *reinterpret_cast<volatile const uint32_t*>(S.counters + CNT_ADV_STEPPED) <= 8u ? 1u : 0u;
+  __syncthreads();
+  const bool early = early_s != 0u;
+  if (early) advance_copy_tables<HOT, DFA>(Gg, S, smem);
+  AdvScratch s = advance_scratch(S, smem);
+  before_me();
   const int32_t tok = row < S.B ? tokens[row] : -1;
   uint32_t flags = 0, b0 = 0, b1 = 0;
   int32_t sid = -1;
@@ -212,20 +259,36 @@ __global__ void __launch_bounds__(ADV_WARPS * 32, 1) advance_kernel(const __grid
     return finish(FMT_OK), false;
   };
   const bool steps = first_look();
-  if (!__syncthreads_or(steps)) return;  // (nothing is staged for rows that are all answered)
-  GrammarDev G = Gg;
-  if (Gg.hot_words * 4u <= HOT_TABLE_BYTES) G = stage_hot_tables(Gg, smem + (size_t)ADV_WARPS * ADV_WARP_WORDS);
-  AdvScratch s = adv_scratch(smem + (size_t)warp * ADV_WARP_WORDS);
-  hset_clear_all(s.w.hset, s.w.hset_mask);
-  for (uint32_t i = lane; i < ADV_NT_WORDS; i += 32) s.w.nt[i] = 0u;
-  __syncthreads();
+  if (early) {
+    if (steps && lane == 0) S.counters[CNT_ADV_STEPPED] = S.adv_no;
+  } else {
+    if (!__syncthreads_or(steps)) return;
+    if (threadIdx.x == 0) S.counters[CNT_ADV_STEPPED] = S.adv_no;
+    advance_copy_tables<HOT, DFA>(Gg, S, smem);
+  }
+  // the pair is entered now, its value when it is known: the answer comes while the steps are made
+  unsigned long long tr_there = 1ull;
+  uint32_t tr_at = 0;
+  const unsigned long long tr_pair = ((unsigned long long)((uint32_t)sid + 1u) << 32) | (uint32_t)tok;
+  if (steps && sid >= 0) {
+    tr_at = tr_slot(S, tr_pair);
+    if (lane == 0) tr_there = atomicCAS(S.tr_key + tr_at, 0ull, tr_pair);
+  }
+  const GrammarDev G = advance_tables<HOT, DFA>(Gg, S, smem);
   if (!steps) return;
+  auto remember = [&](int32_t val) {  // (one lane)
+    if (tr_there == 0ull) asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(S.tr_val + tr_at), "r"(val) : "memory");
+    else if (tr_there != tr_pair) tr_insert(S, sid, (uint32_t)tok, val);
+  };
   // a private buffer that does not hold the current chart
   const uint32_t held = S.row_buf[row];
   const uint32_t final_buf = (held == 0) ? 1u : 0u;
   uint32_t* dst = private_buf(S, row, final_buf);
   uint32_t* const sm_arena = s.w.cur;
-  int r = token_step(G, s, cur, G.vocab_bytes + b0, b1 - b0, dst, S.chart_words, sm_arena, ADV_CUR_CAP);
+  const bool staged = stage_chart(s, cur);
+  int r;
+  if (HOT && staged) r = token_steps(G, s, s.stage, G.vocab_bytes + b0, b1 - b0, dst, S.chart_words, sm_arena, ADV_CUR_CAP, nullptr);
+  else r = token_step(G, s, staged ? s.stage : cur, G.vocab_bytes + b0, b1 - b0, dst, S.chart_words, sm_arena, ADV_CUR_CAP);
   if (r == -2) {  // the token's sets outgrew shared memory: use the row's third private buffer as the arena
     uint32_t* big = private_buf(S, row, 2);
     uint32_t cap = 32;
@@ -233,10 +296,10 @@ __global__ void __launch_bounds__(ADV_WARPS * 32, 1) advance_kernel(const __grid
     hset_clear_all(s.w.hset, s.w.hset_mask);
     for (uint32_t i = lane; i < ADV_NT_WORDS; i += 32) s.w.nt[i] = 0u;
     __syncwarp();
-    r = (held == 2) ? -1 : token_step(G, s, cur, G.vocab_bytes + b0, b1 - b0, dst, S.chart_words, big, cap);
+    r = (held == 2) ? -1 : token_step(G, s, staged ? s.stage : cur, G.vocab_bytes + b0, b1 - b0, dst, S.chart_words, big, cap);
   }
   if (r == 0) {
-    if (sid >= 0 && lane == 0) tr_insert(S, sid, (uint32_t)tok, TR_REJECT);
+    if (sid >= 0 && lane == 0) remember(TR_REJECT);
     return finish(FMT_ERR_TOKEN_REJECTED);
   }
   if (r < 0) {
@@ -256,7 +319,7 @@ __global__ void __launch_bounds__(ADV_WARPS * 32, 1) advance_kernel(const __grid
   uint64_t off;
   int32_t id = intern_chart(S, dst, off);
   if (lane == 0) {
-    if (sid >= 0 && id >= 0) tr_insert(S, sid, (uint32_t)tok, id);
+    if (sid >= 0 && id >= 0) remember(id);
     S.row_state[row] = id;
     if (id >= 0) {
       S.row_chart[row] = off;
@@ -275,28 +338,25 @@ __global__ void __launch_bounds__(ADV_WARPS * 32, 1) advance_kernel(const __grid
 // punctuation a JSON schema fixes, Section 5.1's JSON-Schema task): as long as the text is not a
 // sentence and the last Earley set can scan exactly one byte, that byte is taken and the chart is
 // stepped over it.  Nothing of the row changes: the sets made on the way live in the warp's scratch.
+template <bool HOT, bool DFA>
 __global__ void __launch_bounds__(ADV_WARPS * 32, 1) forced_kernel(const __grid_constant__ GrammarDev Gg,
                                                                    const __grid_constant__ StateDev S, uint8_t* bytes_out,
                                                                    size_t stride, uint32_t* len_out, uint32_t max_len) {
-  before_me();
   extern __shared__ __align__(16) uint32_t smem[];
   const uint32_t warp = threadIdx.x >> 5, lane = lane_id();
-  const uint32_t row = blockIdx.x * ADV_WARPS + warp;
-  GrammarDev G = Gg;
-  if (Gg.hot_words * 4u <= HOT_TABLE_BYTES) {
-    G = stage_hot_tables(Gg, smem + (size_t)ADV_WARPS * ADV_WARP_WORDS);
-    __syncthreads();
-  }
+  const uint32_t row = warp < S.adv_rows ? blockIdx.x * S.adv_rows + warp : 0xFFFFFFFFu;
+  advance_copy_tables<HOT, DFA>(Gg, S, smem);
+  AdvScratch s = advance_scratch(S, smem);
+  before_me();
+  const GrammarDev G = advance_tables<HOT, DFA>(Gg, S, smem);
   if (row >= S.B) return;
-  AdvScratch s = adv_scratch(smem + (size_t)warp * ADV_WARP_WORDS);
   int n = 0;
   if (!(S.row_flags[row] & (ROW_FINISHED | ROW_BROKEN)) && max_len > 0) {
-    hset_clear_all(s.w.hset, s.w.hset_mask);
-    for (uint32_t i = lane; i < ADV_NT_WORDS; i += 32) s.w.nt[i] = 0u;
-    __syncwarp();
     const uint32_t* cur = S.arena + S.row_chart[row];
-    n = token_step(G, s, cur, nullptr, min(max_len, MAX_TOKEN_BYTES), nullptr, 0u, s.w.cur, ADV_CUR_CAP,
-                   bytes_out + (size_t)row * stride);
+    uint8_t* const out = bytes_out + (size_t)row * stride;
+    const bool staged = stage_chart(s, cur);
+    if (HOT && staged) n = token_steps(G, s, s.stage, nullptr, min(max_len, MAX_TOKEN_BYTES), nullptr, 0u, s.w.cur, ADV_CUR_CAP, out);
+    else n = token_step(G, s, staged ? s.stage : cur, nullptr, min(max_len, MAX_TOKEN_BYTES), nullptr, 0u, s.w.cur, ADV_CUR_CAP, out);
     if (n < 0) n = 0;
   }
   if (lane == 0) len_out[row] = (uint32_t)n;
@@ -977,13 +1037,26 @@ __global__ void query_kernel(StateDev S, uint8_t* accepting, uint8_t* finished, 
 
 // ===================================================================================== launchers
 
+constexpr size_t ADV_SMEM_LIMIT = 226 * 1024, ADV_SMEM_SM = 228 * 1024;  // dynamic shared memory of a block, shared memory of an SM
+
 static inline cudaError_t opt_in_smem(const void* fn, size_t bytes) {
   return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
 }
 
-static size_t adv_smem_bytes(const GrammarDev& G) {
-  return (size_t)ADV_WARPS * ADV_WARP_WORDS * 4 + (G.hot_words * 4u <= HOT_TABLE_BYTES ? G.hot_words * 4u : 0u);
+static size_t adv_smem_bytes(const GrammarDev& G, const StateDev& S) {
+  return ((size_t)S.adv_rows * ADV_WARP_WORDS + (G.hot_words * 4u <= HOT_TABLE_BYTES ? G.hot_words : 0u) + (S.adv_dfa ? G.dfa_words : 0u)) * 4;
 }
+// One row to a block as long as all rows run at once: a block then has room for its grammar's automata (JSON 6 KB, a schema of
+// twelve members 60 KB).  Else two or four, with the automata if they fit.
+void advance_layout(const GrammarDev& G, uint32_t rows, uint32_t sms, StateDev& S) {
+  for (S.adv_rows = 1;; S.adv_rows *= 2) {
+    S.adv_dfa = G.dfa_words && G.hot_words * 4u <= HOT_TABLE_BYTES ? 1u : 0u;
+    if (S.adv_dfa && adv_smem_bytes(G, S) > ADV_SMEM_LIMIT) S.adv_dfa = 0;
+    const uint64_t blocks = (uint64_t)sms * (ADV_SMEM_SM / (adv_smem_bytes(G, S) + 1024));
+    if (S.adv_rows == (uint32_t)ADV_WARPS || blocks * S.adv_rows >= rows) return;
+  }
+}
+static_assert(ADV_WARPS * ADV_WARP_WORDS * 4 + HOT_TABLE_BYTES <= ADV_SMEM_LIMIT, "a block of so many rows fits without automata");
 static size_t init_smem_bytes() { return (size_t)ADV_WARP_WORDS * 4; }
 // Dynamic shared memory of the sweep for a grammar: per-warp scratch plus, if they fit the
 // budget, the item-info / byte-class / byte-class-number tables.
@@ -1002,8 +1075,10 @@ int sweep_warps() { return SWEEP_WARPS; }
 cudaError_t configure_kernels() {
   cudaError_t e;
   if ((e = opt_in_smem((const void*)init_kernel, init_smem_bytes())) != cudaSuccess) return e;
-  if ((e = opt_in_smem((const void*)advance_kernel, (size_t)ADV_WARPS * ADV_WARP_WORDS * 4 + HOT_TABLE_BYTES)) != cudaSuccess) return e;
-  if ((e = opt_in_smem((const void*)forced_kernel, (size_t)ADV_WARPS * ADV_WARP_WORDS * 4 + HOT_TABLE_BYTES)) != cudaSuccess) return e;
+  const void* const advancing[] = {(const void*)advance_kernel<false, false>, (const void*)advance_kernel<true, false>, (const void*)advance_kernel<true, true>,
+                                   (const void*)forced_kernel<false, false>, (const void*)forced_kernel<true, false>, (const void*)forced_kernel<true, true>};
+  for (const void* f : advancing)
+    if ((e = opt_in_smem(f, ADV_SMEM_LIMIT)) != cudaSuccess) return e;
   if ((e = opt_in_smem((const void*)sweep_kernel, SWEEP_SMEM_LIMIT)) != cudaSuccess) return e;
   if ((e = configure_automaton_fill()) != cudaSuccess) return e;
   return configure_walk_kernels();
@@ -1025,11 +1100,13 @@ void launch_reset(const StateDev& S, const uint32_t* rows_dev, uint32_t n, const
 }
 void launch_forced(const GrammarDev& G, const StateDev& S, uint8_t* bytes_out, size_t stride, uint32_t* len_out,
                    uint32_t max_len, cudaStream_t st) {
-  launch_overlapped(forced_kernel, dim3((S.B + ADV_WARPS - 1) / ADV_WARPS), dim3(ADV_WARPS * 32), adv_smem_bytes(G), st, G, S, bytes_out,
+  const auto kernel = G.hot_words * 4u > HOT_TABLE_BYTES ? forced_kernel<false, false> : S.adv_dfa ? forced_kernel<true, true> : forced_kernel<true, false>;
+  launch_overlapped(kernel, dim3((S.B + S.adv_rows - 1) / S.adv_rows), dim3(ADV_WARPS * 32), adv_smem_bytes(G, S), st, G, S, bytes_out,
                     stride, len_out, max_len);
 }
 void launch_advance(const GrammarDev& G, const StateDev& S, const int32_t* tokens, int32_t* status, cudaStream_t st) {
-  launch_overlapped(advance_kernel, dim3((S.B + ADV_WARPS - 1) / ADV_WARPS), dim3(ADV_WARPS * 32), adv_smem_bytes(G), st, G, S, tokens, status);
+  const auto kernel = G.hot_words * 4u > HOT_TABLE_BYTES ? advance_kernel<false, false> : S.adv_dfa ? advance_kernel<true, true> : advance_kernel<true, false>;
+  launch_overlapped(kernel, dim3((S.B + S.adv_rows - 1) / S.adv_rows), dim3(ADV_WARPS * 32), adv_smem_bytes(G, S), st, G, S, tokens, status);
 }
 static void launch_sweep_coop(const GrammarDev& G, const StateDev& S, int grid, cudaStream_t st) {
   GrammarDev g = G;

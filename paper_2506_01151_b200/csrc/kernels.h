@@ -43,6 +43,9 @@ void automaton_fill_layout(const GrammarDev& G, uint32_t rows, uint32_t max_bloc
 cudaError_t configure_automaton_fill();
 void launch_automaton_fill(const GrammarDev& G, const StateDev& S, cudaStream_t st);
 
+// how advance places rows and tables in shared memory (S.adv_rows, S.adv_dfa)
+void advance_layout(const GrammarDev& G, uint32_t rows, uint32_t sms, StateDev& S);
+
 void launch_init(const GrammarDev& G, const StateDev& S, int32_t* result_dev, cudaStream_t st);
 void launch_intern_init(const StateDev& S, int32_t* init_state_dev, cudaStream_t st);
 void launch_reset(const StateDev& S, const uint32_t* rows_dev, uint32_t n, const int32_t* init_state_dev, cudaStream_t st);

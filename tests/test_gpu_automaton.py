@@ -178,3 +178,51 @@ def test_masking_rows_that_begin_anywhere(dtype, V):
         m = torch.from_numpy(np.ascontiguousarray(mask).view(np.int32)).cuda()
         fmt.apply_mask(m, on_gpu.data_ptr() + shift * bits // 8, fmt.BF16 if dtype == "bf16" else fmt.FP32, batch, V, row_stride=stride)
         assert np.array_equal(on_gpu.cpu().numpy().view(kind), want), shift
+
+
+def _words(rng, n, length, first=""):
+    got = set()
+    while len(got) < n:
+        got.add(first + "".join(chr(97 + int(c)) for c in rng.integers(0, 26, length)))
+    return sorted(got)
+
+
+@pytest.mark.parametrize("batch", [1, 3, 149, 700])
+@pytest.mark.parametrize("tables", ["all in shared memory", "automata in global memory", "all in global memory"])
+def test_advance_wherever_the_tables_are(tables, batch):
+    """Rows advance one, two or four to a block, by how many there are and by how large the grammar's tables are: the same charts
+    as one row's fed byte by byte, and as many sets and items as the oracle's."""
+    import torch
+
+    import paper_2506_01151_b200 as fmt
+
+    rng = np.random.default_rng(7)
+    if tables == "all in shared memory":
+        names, text = _words(rng, 12, 4), 's ::= "(" s ")" | s "+" s | name\nname ::= %s'
+    elif tables == "automata in global memory":
+        names = [w for d in range(12) for w in _words(rng, 70, 6, str(d))]
+        text = 's ::= "(" s ")" | s "+" s | ' + " | ".join("w%d" % d for d in range(12)) + "\n"
+        text += "\n".join('w%d ::= %s' % (d, " | ".join('"%s"' % x for x in names[70 * d:70 * d + 70])) for d in range(12)) + "\nunused ::= %s"
+    else:
+        names, text = _words(rng, 700, 7), 's ::= "(" s ")" | s "+" s | name\nname ::= %s'
+    text = text % " | ".join('"%s"' % x for x in names)
+    data = ("((%s+%s)+%s" % (names[0], names[-1], names[len(names) // 2])).encode()
+    tokens = [data[:2], data[2:7], data[7:13], data[13:]]
+    vocab = [bytes([b]) for b in range(256)] + tokens + [b""]
+    g = fmt.Grammar(text, "s", vocab, len(vocab) - 1, dfa=tables != "all in global memory")
+    one, many = fmt.State(g, 1), fmt.State(g, batch, max_states=4096, chart_words=1 << 14, pool_words=1 << 22, max_mask_rows=8)
+    status, statuses = torch.zeros(1, dtype=torch.int32, device="cuda"), torch.zeros(batch, dtype=torch.int32, device="cuda")
+    for b in data:
+        one.advance(torch.tensor([b], dtype=torch.int32, device="cuda"), status)
+        assert status.tolist() == [fmt.FMT_OK]
+    for i in range(len(tokens)):
+        many.advance(torch.full((batch,), 256 + i, dtype=torch.int32, device="cuda"), statuses)
+        assert not statuses.any()
+    want = one.chart_words(0).tolist()
+    for row in {0, batch // 2, batch - 1}:
+        assert many.chart_words(row).tolist() == want
+    seq = oracle.Sequence_(oracle.Grammar(text, "s"), pruned=True)
+    assert seq.advance(data)
+    if tables == "all in global memory":  # (automata have items of their own)
+        assert want[1] == seq.total_items
+    assert want[0] == seq.num_sets
