@@ -202,8 +202,8 @@ class Driver:
         self.state.advance(self.tokens[i], self.status, stream=s)
         lg = self.ring[i % self.n_ring] if logits is None else logits
         self.state.fill_and_apply(lg, self.fmt.BF16, stream=s)
-        # advance; plan, [entry look-up (2), sweep of new entries, its collection, job set-up], trie sweep, publish, mask+apply
-        self.launches += 10 if self.roots else 5
+        # advance; plan, [entry look-up (2), sweep of new entries, its collection, job set-up], fill, mask+apply
+        self.launches += 9 if self.roots else 4
 
     def restart(self, warmup: int, clear_caches: bool):
         """Back to the start of the token stream: all rows reset, prefixes fed, `warmup` untimed steps."""
@@ -345,7 +345,7 @@ def run_ours(args):
     apply_rw = B * (4 * Wm + 2 * 2 * V)   # mask words read, logits read and written
     apply_wo = B * (4 * Wm + 2 * V)       # if the logits only had to be written
     kinds = {
-        ("fill_kernel" if drv.roots else "sweep_kernel"): (prof["sweep_ms"], prof["sweep_launches"], sweep_bytes),
+        ("fill_kernel" if drv.roots else "automaton_fill_kernel"): (prof["sweep_ms"], prof["sweep_launches"], sweep_bytes),
         "sweep_kernel (new entries)": (prof["roots_ms"], prof["roots_launches"], trie_bytes),
         "gather_apply_kernel": (prof["apply_ms"], prof["apply_launches"], apply_rw),
         "advance_kernel": (prof["advance_ms"], prof["advance_launches"], B * 2 * 4 * 256),
