@@ -369,8 +369,11 @@ __global__ void __launch_bounds__(ADV_WARPS * 32, 1) forced_kernel(const __grid_
 __global__ void __launch_bounds__(1024) plan_kernel(const __grid_constant__ GrammarDev G, const __grid_constant__ StateDev S) {
   before_me();
   __shared__ uint32_t n_jobs, n_rows, n_cached, n_shared;
-  if (threadIdx.x < CNT_HASH_GEN - CNT_BAR) S.counters[CNT_BAR + threadIdx.x] = 0u;  // barrier and level counters
-  if (threadIdx.x < CNT_LAST_LEVEL + 1 - CNT_LEVEL_TAKEN) S.counters[CNT_LEVEL_TAKEN + threadIdx.x] = 0u;
+  auto clear = [&](uint32_t* counters) {  // barrier and level counters: there may be fewer threads than counters
+    for (uint32_t i = CNT_BAR + threadIdx.x; i < CNT_HASH_GEN; i += blockDim.x) counters[i] = 0u;
+    for (uint32_t i = CNT_LEVEL_TAKEN + threadIdx.x; i <= CNT_LAST_LEVEL; i += blockDim.x) counters[i] = 0u;
+  };
+  clear(S.counters);
   if (threadIdx.x == 0) {
     S.counters[CNT_N_FJOBS] = 0u;
     S.counters[CNT_AUTO_ITEMS] = 0u;
@@ -379,8 +382,7 @@ __global__ void __launch_bounds__(1024) plan_kernel(const __grid_constant__ Gram
     n_rows = S.counters[CNT_N_MASK_ROWS];
   }
   if (S.rt.on) {  // the root sweep of this fill starts from clean counters, too
-    if (threadIdx.x < CNT_HASH_GEN - CNT_BAR) S.rt.counters[CNT_BAR + threadIdx.x] = 0u;
-    if (threadIdx.x < CNT_LAST_LEVEL + 1 - CNT_LEVEL_TAKEN) S.rt.counters[CNT_LEVEL_TAKEN + threadIdx.x] = 0u;
+    clear(S.rt.counters);
     if (threadIdx.x == 0) S.rt.counters[CNT_N_JOBS] = 0u, S.rt.counters[CNT_AUTO_ITEMS] = 0u;
   }
   __syncthreads();

@@ -106,6 +106,29 @@ def test_no_automaton_for_states_that_ask_for_earley_steps():
     assert a["walk_states"] < b["walk_states"]
 
 
+@pytest.mark.parametrize("batch", [1, 3, 65])
+@pytest.mark.parametrize("options", [dict(sweep_states=4096), dict(roots=True)])
+def test_sweeps_in_a_row_with_the_longest_tokens(batch, options):
+    """Every fill starts from clean counters at every depth of the trie, however few rows (and so threads that clear them) there
+    are: sweeps one after the other, each with steps to be made at depth 32."""
+    import torch
+
+    import paper_2506_01151_b200 as fmt
+
+    w = workloads.build(2, V=300, batch=1, steps=1)
+    vocab = [bytes([b]) for b in range(256)] + [b'"' + b"a" * 30 + b'"', b"[" * 32, b"[]," * 10 + b"[]", b"]" * 32, b""]
+    g, og, ov = fmt.Grammar(w.ebnf, w.start, vocab, len(vocab) - 1), oracle.Grammar(w.ebnf, w.start), oracle.Vocab(vocab, len(vocab) - 1)
+    st, seq = fmt.State(g, batch, cache=False, **options), oracle.Sequence_(og)
+    mask = torch.zeros((batch, g.mask_words), dtype=torch.int32, device="cuda")
+    for token in [ord("["), ord("["), 257, ord('"'), ord("x")]:
+        st.advance(torch.full((batch,), token, dtype=torch.int32, device="cuda"))
+        assert seq.advance(vocab[token])
+        st.fill_mask(mask)
+        got = mask.cpu().numpy().view(np.uint32)
+        assert all(np.array_equal(row, seq.mask(ov)) for row in got), token
+    assert st.stats()["fills_aborted"] == 0 and st.stats()["capacity_errors"] == 0
+
+
 def _feed(text, start, data, options, dfa=True):
     """The chart words after feeding the bytes one by one, and in one token where they are at most 32."""
     import torch
