@@ -96,7 +96,8 @@ __device__ int32_t intern_chart(const StateDev& S, const uint32_t* ch, uint64_t&
 // ===================================================================================== transition cache
 //
 // What advancing the chart with cache id `sid` by `tok` leads to, if that is known: the next chart's
-// cache id, TR_REJECT, or TR_UNSET (not known).
+// cache id, TR_REJECT, or TR_UNSET (not known).  For one lane: other blocks of the launch enter pairs meanwhile, and lanes that
+// looked for themselves could see different answers.
 __device__ __forceinline__ uint32_t tr_slot(const StateDev& S, unsigned long long key) {
   return (mix32((uint32_t)key) ^ mix32((uint32_t)(key >> 32) * 0x9E3779B9u)) & S.tr_mask;
 }
@@ -104,9 +105,10 @@ __device__ int32_t tr_lookup(const StateDev& S, int32_t sid, uint32_t tok) {
   const unsigned long long key = ((unsigned long long)((uint32_t)sid + 1u) << 32) | tok;
   uint32_t slot = tr_slot(S, key);
   for (uint32_t probe = 0; probe < 32; ++probe) {
-    // (a value read before its key may be one not written yet: the pair then counts as unknown)
-    const int32_t v = __ldcg(S.tr_val + slot);
+    // Both are under way at once.  The value is acquired: what it names (the chart's offset) was written by another block, of this
+    // launch perhaps, before the value was.  (One that is not there yet, behind a key that is: the pair counts as unknown.)
     const unsigned long long k = __ldcg(S.tr_key + slot);
+    const int32_t v = (int32_t)ld_acquire(reinterpret_cast<const uint32_t*>(S.tr_val + slot));
     if (k == 0ull) return TR_UNSET;
     if (k == key) return (v >= 0 || v == TR_REJECT) ? v : TR_UNSET;
     slot = (slot + 1u) & S.tr_mask;
@@ -240,7 +242,9 @@ __global__ void __launch_bounds__(ADV_WARPS * 32, 1) advance_kernel(const __grid
     if (flags & ROW_BROKEN) return finish(FMT_ERR_CAPACITY), false;
     b0 = __ldg(&Gg.vocab_off[tok]), b1 = __ldg(&Gg.vocab_off[tok + 1]);
     // has this chart been advanced by this token before?  (Section 5.2: the state cache)
-    const int32_t known = (sid >= 0 && tok != Gg.eos) ? tr_lookup(S, sid, (uint32_t)tok) : TR_UNSET;
+    int32_t known = TR_UNSET;
+    if (lane == 0 && sid >= 0 && tok != Gg.eos) known = tr_lookup(S, sid, (uint32_t)tok);
+    known = __shfl_sync(FULL, known, 0);
     if (tok == Gg.eos) {
       if (!(cur[CH_FLAGS] & CHART_ACCEPTING)) return finish(FMT_ERR_TOKEN_REJECTED), false;
       if (lane == 0) S.row_flags[row] = flags | ROW_FINISHED;

@@ -203,6 +203,33 @@ def test_masking_rows_that_begin_anywhere(dtype, V):
         assert np.array_equal(on_gpu.cpu().numpy().view(kind), want), shift
 
 
+def test_transitions_met_by_several_blocks_of_a_launch():
+    """Rows at one chart take one token, from caches that know nothing: some rows of a launch find what others of it have entered a
+    moment before.  All of them end up at the same chart, the one a single row reaches."""
+    import torch
+
+    import paper_2506_01151_b200 as fmt
+
+    w = workloads.build(2, V=300, batch=1, steps=1)
+    g = fmt.Grammar(w.ebnf, w.start, w.vocab, w.eos)
+    batch = 3000
+    many, one = fmt.State(g, batch, chart_words=1 << 12), fmt.State(g, 1, cache=False)
+    status = torch.zeros(batch, dtype=torch.int32, device="cuda")
+    for _ in range(20):
+        many.cache_clear()
+        many.reset()
+        one.reset()
+        for b in b'{"a": [1, {"k": tr':
+            many.advance(torch.full((batch,), b, dtype=torch.int32, device="cuda"), status)
+            one.advance(torch.full((1,), b, dtype=torch.int32, device="cuda"))
+            assert not status.any()
+        q, want = many.query(), one.query()
+        assert len(set(q["state_id"].tolist())) == 1 and (q["n_items"] == want["n_items"][0]).all() and (q["n_sets"] == want["n_sets"][0]).all()
+        assert many.chart_words(batch - 1).tolist() == one.chart_words(0).tolist()
+    s = many.stats()
+    assert s["capacity_errors"] == 0 and 0 < s["advances_cached"] < s["steps_advanced"]
+
+
 def _words(rng, n, length, first=""):
     got = set()
     while len(got) < n:
