@@ -536,18 +536,16 @@ __global__ void __launch_bounds__(AF_THREADS, 4) automaton_fill_kernel(const __g
         const uint2 x = i < list.y ? reinterpret_cast<const uint2*>(C.pool)[list.x / 2u + i] : make_uint2(0u, 0u);
         const uint32_t wide = i < list.y ? __ldg(&G.ga_item[4u * (x.y >> 16) + 2u]) : GA_DEAD;
         uint4 en = make_uint4(root.x, root.y >> 8, x.x, x.y & 0xFFFFu);
+        bool take = i < list.y && en.y != 0u;
         if (wide != GA_DEAD) {  // most of the vocabulary follows from this item alone
           const uint4 r = __ldg(reinterpret_cast<const uint4*>(G.ga_wide_rec) + wide);
           const uint32_t at = atomicAdd(&ctl[AC_NWIDE], 1u);
-          if (at < AF_EXITS) {
+          if (at < AF_EXITS) {  // (those that find no room start threads like any other)
             ctl[AC_WIDE + at] = r.x;
             if (r.z) exits[atomicAdd(&ctl[AC_NEXITS], 1u)] = make_uint4(r.y, r.z, 0u, en.w);
-          } else {
-            ok = false;
+            take = false;
           }
         }
-        ok = __all_sync(FULL, ok);
-        const bool take = i < list.y && en.y != 0u && wide == GA_DEAD;
         const uint32_t bal = __ballot_sync(FULL, take);
         if (take) entries[top + __popc(bal & ((1u << lane) - 1u))] = en;
         top += __popc(bal);

@@ -89,6 +89,22 @@ def test_left_recursion_nullables_and_shared_prefixes():
     _run(text, "s", vocab, [list(p) for p in (b"", b"a", b"a_", b"(a_", b"bab", b"((b_", b"baaaab(a)")])
 
 
+def _union(variants):
+    """A union told apart by what follows a member that all variants begin with: as many items in the set, each followed by a string."""
+    text = "s ::= " + " | ".join("t%d" % i for i in range(variants)) + "\n"
+    text += "".join('t%d ::= "{\\"id\\":" str ",\\"k%d\\":" val "}"\n' % (i, i) for i in range(variants))
+    return text + 'str ::= "\\"" [^"\\\\]* "\\""\nval ::= str | "[" val "]"\n'
+
+
+@pytest.mark.parametrize("variants", [59, 60, 61, 100, 200])
+@pytest.mark.parametrize("batch", [1, 4, 75, 300])
+def test_more_wide_items_than_there_is_room_for(variants, batch):
+    """Up to 60 items of a row's last set are answered by the masks made for them; the others are walked like any item."""
+    w = workloads.build(3, V=20000, batch=1, steps=1)
+    prefixes = [list(p) for p in (b'{"id":', b'{"id":"x', b'{"id":"x","k1', b'{"id":"y","k%d":[[' % (variants - 1))]
+    _run(_union(variants), "s", w.vocab, prefixes, batch=batch, check=range(min(batch, 4)))
+
+
 def test_grammar_without_an_automaton():
     """Alternations of more than a thousand literals have none: their rows are swept by Earley steps."""
     names = sorted({"k%06d" % (i * 7919 % 999983) for i in range(1200)})
