@@ -48,7 +48,8 @@ constexpr uint32_t CTX_NEW = 0xFFFFFFFFu;
 
 enum : uint32_t {
   AC_NEXT = 0, AC_SPEC = 1, AC_OVF = 2, AC_GTOP = 3, AC_FAIL = 4, AC_NCTX = 5, AC_POOL = 6, AC_NWORK = 7, AC_WSUM = 8, AC_NBUF = 16, AC_OVER = 17,
-  AC_SPILLED = 18, AC_WAITING = 19, AC_BASE = 20, AC_JOB = 21, AC_NWIDE = 22, AC_SOVF = 23, AC_GSPEC = 24, AC_NEXITS = 25, AC_WIDE = 26, AC_WORDS = AC_WIDE + AF_EXITS + 2
+  AC_SPILLED = 18, AC_WAITING = 19, AC_BASE = 20, AC_JOB = 21, AC_NWIDE = 22, AC_SOVF = 23, AC_GSPEC = 24, AC_NEXITS = 25, AC_LIST = 26,
+  AC_LIST_AT = 27, AC_LIST_END = 28, AC_WIDE = 30, AC_WORDS = AC_WIDE + AF_EXITS + 2
 };
 
 // A unit of work handed out: AU_HDR words, then the giver's contexts, lists and the threads.
@@ -528,7 +529,6 @@ __global__ void __launch_bounds__(AF_THREADS, 4) automaton_fill_kernel(const __g
         spill_contexts(C, ctl, A);
         ok = group_items(G, C, ctl, b, n, list);  // (sorted and without repeats already)
       }
-      if (list.y > AF_BATCH) ok = false, list.y = 0u;
       const uint4 root = __ldg(reinterpret_cast<const uint4*>(G.ga_node));
       uint32_t top = 0;
       for (uint32_t base = 0; base < list.y; base += 32) {
@@ -547,11 +547,14 @@ __global__ void __launch_bounds__(AF_THREADS, 4) automaton_fill_kernel(const __g
           }
         }
         const uint32_t bal = __ballot_sync(FULL, take);
-        if (take) entries[top + __popc(bal & ((1u << lane) - 1u))] = en;
+        const uint32_t at = top + __popc(bal & ((1u << lane) - 1u));
+        if (take && at < AF_BATCH) entries[at] = en;
+        else if (take) reinterpret_cast<uint2*>(C.pool)[list.x / 2u + at - AF_BATCH] = x;  // they wait in the list, closed up
         top += __popc(bal);
       }
       if (lane == 0) {
-        ctl[AC_NEXT] = top;
+        ctl[AC_NEXT] = min(top, AF_BATCH);
+        ctl[AC_LIST] = list.x, ctl[AC_LIST_END] = top > AF_BATCH ? top - AF_BATCH : 0u;
         if (!ok) ctl[AC_FAIL] = 1u + DIAG_SET_SCRATCH;
       }
     }
@@ -618,7 +621,8 @@ __global__ void __launch_bounds__(AF_THREADS, 4) automaton_fill_kernel(const __g
     };
     for (;;) {  // ---- rounds
       uint32_t n = min(ctl[AC_NEXT], AF_BATCH), ns = min(ctl[AC_SPEC], AF_SPEC), gtop = ctl[AC_GTOP], gspec = ctl[AC_GSPEC], nx = ctl[AC_NEXITS];
-      if (ctl[AC_FAIL] || n + ns + gtop + gspec + nx == 0u) break;
+      const uint32_t first_at = ctl[AC_LIST_AT], first_left = ctl[AC_LIST_END] - first_at;  // items of the last set that have not started
+      if (ctl[AC_FAIL] || n + ns + gtop + gspec + nx + first_left == 0u) break;
       spilled = ctl[AC_SPILLED] != 0u;
       const uint32_t waiting = ctl[AC_WAITING];
       __syncthreads();
@@ -638,6 +642,15 @@ __global__ void __launch_bounds__(AF_THREADS, 4) automaton_fill_kernel(const __g
         const uint32_t take = min(most - n, gtop);
         for (uint32_t i = tid; i < take; i += AF_THREADS) cur[n + i] = stack[gtop - take + i];
         n += take, gtop -= take;
+      } else if (n < most && first_left) {
+        const uint32_t take = min(most - n, first_left);
+        const uint4 root = __ldg(reinterpret_cast<const uint4*>(G.ga_node));
+        for (uint32_t i = tid; i < take; i += AF_THREADS) {
+          const uint2 x = element(ctl[AC_LIST], first_at + i);
+          cur[n + i] = make_uint4(root.x, root.y >> 8, x.x, x.y & 0xFFFFu);
+        }
+        if (tid == 0) ctl[AC_LIST_AT] = first_at + take;
+        n += take;
       } else if (n > most) {
         for (uint32_t i = most + tid; i < n; i += AF_THREADS) stack[gtop + i - most] = cur[i];
         gtop += n - most, n = most;

@@ -105,6 +105,19 @@ def test_more_wide_items_than_there_is_room_for(variants, batch):
     _run(_union(variants), "s", w.vocab, prefixes, batch=batch, check=range(min(batch, 4)))
 
 
+@pytest.mark.parametrize("n", [511, 512, 513, 600, 1000])
+@pytest.mark.parametrize("batch", [1, 5, 300])
+def test_more_items_than_a_round_takes(n, batch):
+    """After the byte that all literals of an alternation begin with, the last set has an item for each: a round takes 512 threads."""
+    rng = np.random.default_rng(n)
+    names = _words(rng, n, 15, "k")
+    text = 's ::= "[" v ("," v)* "]"\nv ::= "\\"" name "\\"" | "[" v "]"\nname ::= ' + " | ".join('"%s"' % x for x in names)
+    vocab = [bytes([b]) for b in range(256)] + [x[1:9].encode() for x in names[::3]] + [(x[1:] + '","').encode() for x in names[1::3]] + [b"k" + x[1:3].encode() for x in names[2::3]] + [b""]
+    prefixes = [list(p) for p in (b'["k', b'["' + names[5].encode() + b'","k', b'["' + names[1][:9].encode(), b'["')]
+    s = _run(text, "s", vocab, prefixes, batch=batch, check=range(min(batch, 4)))
+    assert s["walk_states"] < 200 * batch  # (the automaton's contexts, not Earley sets)
+
+
 def test_grammar_without_an_automaton():
     """Alternations of more than a thousand literals have none: their rows are swept by Earley steps."""
     names = sorted({"k%06d" % (i * 7919 % 999983) for i in range(1200)})
