@@ -256,7 +256,7 @@ fmt_status fmt_compile(const char* ebnf, size_t ebnf_len, const char* start_rule
       UP(ga_acc);
       UP(ga_node);
       UP(ga_tok);
-      d.ga_lvl2 = h.ga_lvl2, d.ga_lvl3 = h.ga_lvl3;
+      d.ga_lvl2 = h.ga_lvl2, d.ga_lvl3 = h.ga_lvl3, d.ga_path = h.ga_path;
       UP(ga_wide_rec);
       UP(ga_wide_mask);
       UP(ga_wide_exit);
@@ -477,7 +477,7 @@ fmt_status fmt_state_create(const fmt_grammar* g, uint32_t batch, const fmt_stat
   AutoFillDev& af = d.af;
   af.on = (g->dev.ga_on && !rt.on && !(opt && opt->sweep_states)) ? 1u : 0u;
   if (af.on) {
-    af.stack_cap = 32u << 10;
+    af.stack_cap = std::max(32u << 10, automaton_fill_least_stack(g->dev) + (16u << 10));
     af.ctx_cap = 4096, af.pool_cap = 64u << 10, af.big_cap = 64u << 10;
     af.unit_cap = 4096;
     automaton_fill_layout(g->dev, batch, AUTO_FILL_PER_SM * (uint32_t)std::max(1, sms), af);

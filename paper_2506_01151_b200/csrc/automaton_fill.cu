@@ -33,7 +33,8 @@ constexpr uint32_t AF_BATCH = 512;        // threads of a round
 constexpr uint32_t AF_PER = AF_BATCH / AF_THREADS;
 constexpr uint32_t AF_SPEC = AF_THREADS;  // expansions to be made at the start of a round
 constexpr uint32_t AF_EXITS = 60;         // lists of nodes at which expansions are to be made (from wide items)
-constexpr uint32_t AF_SPEC_STACK = 4096;  // part of a block's stack that is kept for those that found no room
+constexpr uint32_t AF_TIGHT = 6144;       // free places of a block's stack, its reserve not counted, below which entries are taken one at a time
+constexpr uint32_t AF_LIST_STARTS = 64;   // expansions of more elements are started from a list's nodes by specials
 constexpr uint32_t AF_SEEN = 512;         // recently started threads (a lossy table: repeats only cost time)
 constexpr uint32_t AF_STAGE = 1024;       // a chart up to this many words is read from shared memory
 constexpr uint32_t AF_CTX = 64, AF_CTX_HASH = 128, AF_POOL = 2048;  // contexts in shared memory, words of their lists
@@ -42,14 +43,16 @@ constexpr uint32_t AF_OWNER = AF_BATCH * 8;  // pieces of 32 children a round ca
 constexpr uint32_t AF_HEAVY = 16384;      // after so many look-ups for a row, or for a unit of work,
 constexpr uint32_t AF_SHARE = 384;        // a block with so many threads gives some to blocks that wait,
 constexpr uint32_t AF_MAX_UNITS = 7;      // to so many at once, 128 threads at the least to each
-constexpr uint32_t AF_SPAWN = 0xFFFFFFFDu;  // code of a special: to start the threads of a context's expansion at a node (first child, children)
+// code of a special: to start the threads of a context's expansion at a node (first child, children, AF_SPAWN, elements that have been
+// started << 16 | context)
+constexpr uint32_t AF_SPAWN = 0xFFFFFFFDu;
 constexpr uint32_t AF_GIVEN_UP = 0xFFFFFFFFu;  // (AC_FAIL) a wait ran out: the fill is given up, the row itself is fine
 constexpr uint32_t CTX_NEW = 0xFFFFFFFFu;
 
 enum : uint32_t {
   AC_NEXT = 0, AC_SPEC = 1, AC_OVF = 2, AC_GTOP = 3, AC_FAIL = 4, AC_NCTX = 5, AC_POOL = 6, AC_NWORK = 7, AC_WSUM = 8, AC_NBUF = 16, AC_OVER = 17,
-  AC_SPILLED = 18, AC_WAITING = 19, AC_BASE = 20, AC_JOB = 21, AC_NWIDE = 22, AC_SOVF = 23, AC_GSPEC = 24, AC_NEXITS = 25, AC_LIST = 26,
-  AC_LIST_AT = 27, AC_LIST_END = 28, AC_WIDE = 30, AC_WORDS = AC_WIDE + AF_EXITS + 2
+  AC_SPILLED = 18, AC_WAITING = 19, AC_BASE = 20, AC_JOB = 21, AC_NWIDE = 22, AC_POPPED = 24, AC_NEXITS = 25, AC_LIST = 26,
+  AC_LIST_AT = 27, AC_LIST_END = 28, AC_POPPED_SPEC = 29, AC_WIDE = 30, AC_WORDS = AC_WIDE + AF_EXITS + 2
 };
 
 // A unit of work handed out: AU_HDR words, then the giver's contexts, lists and the threads.
@@ -620,9 +623,9 @@ __global__ void __launch_bounds__(AF_THREADS, 4) automaton_fill_kernel(const __g
       return fresh;
     };
     for (;;) {  // ---- rounds
-      uint32_t n = min(ctl[AC_NEXT], AF_BATCH), ns = min(ctl[AC_SPEC], AF_SPEC), gtop = ctl[AC_GTOP], gspec = ctl[AC_GSPEC], nx = ctl[AC_NEXITS];
+      uint32_t n = min(ctl[AC_NEXT], AF_BATCH), ns = min(ctl[AC_SPEC], AF_SPEC), gtop = ctl[AC_GTOP], nx = ctl[AC_NEXITS];
       const uint32_t first_at = ctl[AC_LIST_AT], first_left = ctl[AC_LIST_END] - first_at;  // items of the last set that have not started
-      if (ctl[AC_FAIL] || n + ns + gtop + gspec + nx + first_left == 0u) break;
+      if (ctl[AC_FAIL] || n + ns + gtop + nx + first_left == 0u) break;
       spilled = ctl[AC_SPILLED] != 0u;
       const uint32_t waiting = ctl[AC_WAITING];
       __syncthreads();
@@ -630,20 +633,38 @@ __global__ void __launch_bounds__(AF_THREADS, 4) automaton_fill_kernel(const __g
       uint4* const nxt = entries + (side ^ 1u) * AF_BATCH;
       uint4* const spec = specials + side * AF_SPEC;
       uint4* const spec_nxt = specials + (side ^ 1u) * AF_SPEC;
-      if (tid == 0) ctl[AC_NEXT] = 0u, ctl[AC_SPEC] = 0u, ctl[AC_OVF] = 0u, ctl[AC_SOVF] = 0u;
+      if (tid == 0) ctl[AC_NEXT] = 0u, ctl[AC_SPEC] = 0u, ctl[AC_OVF] = 0u;
       if (tid == AF_THREADS - 1) {  // (looked at in the next round)
         const uint32_t t = vload(&S.counters[CNT_AF_TAKEN]), p = vload(&S.counters[CNT_AF_POSTED]);
         ctl[AC_WAITING] = t > p ? t - p : 0u;
       }
-      // a crowded stack: fewer threads at once, which keeps it from growing (depth first)
-      const uint32_t threads_cap = A.stack_cap - AF_SPEC_STACK;
-      const uint32_t most = max(1u, min(AF_BATCH, (threads_cap - gtop) / 16u));
-      if (n < most && gtop) {
-        const uint32_t take = min(most - n, gtop);
-        for (uint32_t i = tid; i < take; i += AF_THREADS) cur[n + i] = stack[gtop - take + i];
-        n += take, gtop -= take;
-      } else if (n < most && first_left) {
-        const uint32_t take = min(most - n, first_left);
+      // The stack cannot run over.  A round pushes at most the threads that its specials and its list start and two entries for each
+      // child it looks up, and takes no more than fits above the reserve.  On a crowded stack one entry is taken at a time, from the top:
+      // depth first the stack grows by two entries a child along one path of the trie (A.reserve, which has room for `cur` and `spec`, too).
+      const bool tight = A.stack_cap - gtop < A.reserve + AF_TIGHT, pops = !tight && gtop && n < AF_BATCH && ns < AF_SPEC;
+      if (tight) {
+        for (uint32_t i = tid; i < n; i += AF_THREADS) stack[gtop + i] = cur[i];
+        for (uint32_t i = tid; i < ns; i += AF_THREADS) stack[gtop + n + i] = spec[i];
+        gtop += n + ns;
+        __syncthreads();
+        const uint4 v = stack[--gtop];
+        ns = v.z == AF_SPAWN ? 1u : 0u, n = 1u - ns, nx = 0u;
+        if (tid == 0) (ns ? spec : cur)[0] = v;
+      } else if (pops) {
+        const uint32_t take = min(min(AF_BATCH - n, AF_SPEC - ns), gtop);
+        static_assert(AF_SPEC <= AF_THREADS, "one entry to a thread");
+        gtop -= take;
+        const uint4 v = tid < take ? stack[gtop + tid] : make_uint4(0u, 0u, 0u, 0u);
+        const bool is_spec = tid < take && v.z == AF_SPAWN, is_thread = tid < take && v.z != AF_SPAWN;
+        const uint32_t bt = __ballot_sync(FULL, is_thread), bs = __ballot_sync(FULL, is_spec);
+        uint32_t at = 0, at_spec = 0;
+        if (lane == 0 && bt) at = atomicAdd(&ctl[AC_POPPED], __popc(bt));
+        if (lane == 0 && bs) at_spec = atomicAdd(&ctl[AC_POPPED_SPEC], __popc(bs));
+        at = __shfl_sync(FULL, at, 0), at_spec = __shfl_sync(FULL, at_spec, 0);
+        if (is_thread) cur[n + at + __popc(bt & lt)] = v;
+        if (is_spec) spec[ns + at_spec + __popc(bs & lt)] = v;
+      } else if (n < AF_BATCH && first_left) {
+        const uint32_t take = min(AF_BATCH - n, first_left);
         const uint4 root = __ldg(reinterpret_cast<const uint4*>(G.ga_node));
         for (uint32_t i = tid; i < take; i += AF_THREADS) {
           const uint2 x = element(ctl[AC_LIST], first_at + i);
@@ -651,38 +672,27 @@ __global__ void __launch_bounds__(AF_THREADS, 4) automaton_fill_kernel(const __g
         }
         if (tid == 0) ctl[AC_LIST_AT] = first_at + take;
         n += take;
-      } else if (n > most) {
-        for (uint32_t i = most + tid; i < n; i += AF_THREADS) stack[gtop + i - most] = cur[i];
-        gtop += n - most, n = most;
-      }
-      if (gspec && ns < AF_SPEC) {
-        const uint32_t take = min(AF_SPEC - ns, gspec);
-        if (tid < take) spec[ns + tid] = stack[threads_cap + gspec - take + tid];
-        ns += take, gspec -= take;
       }
       __syncthreads();
-      const uint32_t room = threads_cap - gtop;
+      if (pops) n += ctl[AC_POPPED], ns += ctl[AC_POPPED_SPEC];
+      const uint32_t places = tight ? 0u : A.stack_cap - A.reserve - gtop;  // (at least AF_TIGHT)
       auto overflow = [&](const uint4& v) {
         const uint32_t p = atomicAdd(&ctl[AC_OVF], 1u);
-        if (p < room) stack[gtop + p] = v;
-        else ctl[AC_FAIL] = 1u + DIAG_QUEUE_FULL;
-      };
-      auto overflow_special = [&](const uint4& v) {
-        const uint32_t p = atomicAdd(&ctl[AC_SOVF], 1u);
-        if (gspec + p < AF_SPEC_STACK) stack[threads_cap + gspec + p] = v;
-        else ctl[AC_FAIL] = 1u + DIAG_QUEUE_FULL;
+        if (gtop + p < A.stack_cap) stack[gtop + p] = v;
+        else ctl[AC_FAIL] = 1u + DIAG_QUEUE_FULL;  // (cannot happen, see above)
       };
       if (ns + nx) {
         // ---- expansions: contexts that have none yet, then the threads they start, in this very round as far as there is room
         const bool list = nx != 0u && n < AF_BATCH / 2u;  // a list of nodes waits its turn
         const uint4 ex = list ? exits[nx - 1u] : make_uint4(0u, 0u, 0u, 0u);
         const uint4 en = tid < ns ? spec[tid] : make_uint4(0u, 0u, 0u, 0u);
-        if (__syncthreads_or((tid < ns && expansion(en.w).y == CTX_NEW) || (list && tid == 0 && expansion(ex.w).y == CTX_NEW))) {
+        const uint32_t en_ctx = en.w & 0xFFFFu;
+        if (__syncthreads_or((tid < ns && expansion(en_ctx).y == CTX_NEW) || (list && tid == 0 && expansion(ex.w).y == CTX_NEW))) {
           if (warp == 0) {
             Contexts C = spilled ? global_contexts(A) : C0;
             for (uint32_t base = 0; base <= ns; base += 32) {  // (the list's comes last)
               const uint32_t i = base + lane;
-              const uint32_t c = i < ns ? spec[i].w : i == ns && list ? ex.w : CTX_NEW;
+              const uint32_t c = i < ns ? spec[i].w & 0xFFFFu : i == ns && list ? ex.w : CTX_NEW;
               for (uint32_t todo = __ballot_sync(FULL, c != CTX_NEW && C.exp[c].y == CTX_NEW); todo;) {
                 const uint32_t x = __shfl_sync(FULL, c, __ffs(todo) - 1);
                 if (!expand_context(G, A, C, J, x, ctl, work, hset, buf) && lane == 0) ctl[AC_FAIL] = 1u + DIAG_SET_TABLE;
@@ -707,19 +717,31 @@ __global__ void __launch_bounds__(AF_THREADS, 4) automaton_fill_kernel(const __g
           else if (yes) overflow(v);
         };
         if (warp * 32u < ns) {
-          const uint2 x = tid < ns ? expansion(en.w) : make_uint2(0u, 0u);
-          const uint32_t most_of = __reduce_max_sync(FULL, x.y);
-          for (uint32_t q = 0; q < most_of; ++q) begin(q < x.y, en.x, en.y, q < x.y ? element(x.x, q) : make_uint2(0u, 0u));
+          // (all of its elements as a rule; what might not fit the stack is left for another round)
+          const uint2 spawns = tid < ns ? expansion(en_ctx) : make_uint2(0u, 0u);
+          const uint32_t from = en.w >> 16, count = min(spawns.y - min(from, spawns.y), tight ? 1u : max(1u, places / (2u * ns)));
+          const uint32_t most_of = __reduce_max_sync(FULL, count);
+          if (from + count < spawns.y) overflow(make_uint4(en.x, en.y, AF_SPAWN, (from + count) << 16 | en_ctx));
+          for (uint32_t q = 0; q < most_of; ++q) begin(q < count, en.x, en.y, q < count ? element(spawns.x, from + q) : make_uint2(0u, 0u));
         }
         if (list) {
           const uint2 x = expansion(ex.w);
-          const uint32_t nodes = x.y ? min(ex.y, max(parts * (AF_BATCH / 2u / x.y), 32u)) : ex.y;
+          const uint32_t nodes = x.y ? min(ex.y, max(parts * (AF_BATCH / 2u / x.y), 32u)) : ex.y;  // (at most 2048 threads)
+          const bool by_specials = x.y > AF_LIST_STARTS;
           if (x.y)
             for (uint32_t base = warp * 32u; base < nodes; base += AF_THREADS) {
               bool v = base + lane < nodes;
               const uint2 nd = v ? __ldg(reinterpret_cast<const uint2*>(G.ga_wide_exit) + ex.x + base + lane) : make_uint2(0u, 0u);
               // (blocks that share a row all start the threads of nodes of depth 1, and deal out the others)
               if (parts > 1u && (nd.x < G.ga_lvl2 || nd.x >= G.ga_lvl3)) v = v && ((base + lane) & (parts - 1u)) == part;
+              if (by_specials) {
+                v = v && start(nd.x, 0xFFFF0000u | ex.w);
+                const uint4 b = make_uint4(nd.x, nd.y, AF_SPAWN, ex.w);
+                const uint32_t p = v ? atomicAdd(&ctl[AC_SPEC], 1u) : 0u;
+                if (v && p < AF_SPEC) spec_nxt[p] = b;
+                else if (v) overflow(b);
+                continue;
+              }
               for (uint32_t q = 0; q < x.y; ++q) begin(v, nd.x, nd.y, element(x.x, q));
             }
           __syncthreads();
@@ -804,8 +826,20 @@ __global__ void __launch_bounds__(AF_THREADS, 4) automaton_fill_kernel(const __g
         before += w[u];
       }
       if (n == AF_BATCH && tid == 0) pre[n] = total;
-      looked_up += total;
+      const uint32_t pushed = ctl[AC_OVF];
       __syncthreads();
+      if (!tight && 2u * total > places - pushed) {  // more children than can be pushed: the last threads wait
+        uint32_t fit = 0;
+#pragma unroll
+        for (uint32_t u = 0; u < AF_PER; ++u) {
+          const uint32_t i = u * AF_THREADS + tid;
+          fit += __syncthreads_count(i < n && 2u * pre[i + 1u] <= places - pushed);
+        }
+        for (uint32_t i = fit + tid; i < n; i += AF_THREADS) overflow(cur[i]);
+        n = fit, total = pre[n];
+        __syncthreads();
+      }
+      looked_up += total;
       for (uint32_t base = warp * 32u; base < total; base += AF_THREADS) {
         const uint32_t lo = owner[base / 32u];
         const uint32_t nb = lo + 1u + lane <= n ? pre[lo + 1u + lane] - base : 32u;  // where the threads after it begin
@@ -869,12 +903,12 @@ __global__ void __launch_bounds__(AF_THREADS, 4) automaton_fill_kernel(const __g
         if (special) {
           const uint32_t p = atomicAdd(&ctl[AC_SPEC], 1u);
           if (p < AF_SPEC) spec_nxt[p] = b;
-          else overflow_special(b);
+          else overflow(b);
         }
       }
       side ^= 1u;
       __syncthreads();
-      if (tid == 0) ctl[AC_GTOP] = gtop + ctl[AC_OVF], ctl[AC_GSPEC] = gspec + ctl[AC_SOVF];
+      if (tid == 0) ctl[AC_GTOP] = gtop + ctl[AC_OVF], ctl[AC_POPPED] = ctl[AC_POPPED_SPEC] = 0u;
       __syncthreads();
     }
     contexts += ctl[AC_NCTX];
@@ -898,7 +932,15 @@ __global__ void __launch_bounds__(AF_THREADS, 4) automaton_fill_kernel(const __g
 
 constexpr uint32_t AF_SMEM = (2 * AF_BATCH + 2 * AF_SPEC + AF_EXITS) * 16 + AF_SEEN * 8 + AF_OWNER * 2 + (5 * AF_CTX + AF_POOL + AF_CTX_HASH + AF_BATCH + 4 + AC_WORDS + AF_STAGE + AF_BUF + AF_WORK + AF_HSET) * 4;
 
+// Places of a block's stack that only its depth-first rounds use: two for each child along the longest path of the trie and one for
+// what is left of a special at each of its nodes, and what a round may hold or has put back when the last places above are taken.
+uint32_t automaton_fill_reserve(const GrammarDev& G) {
+  return 2u * G.ga_path + MAX_TOKEN_BYTES + 1u + 2u * (AF_BATCH + AF_SPEC) + 32u;
+}
+uint32_t automaton_fill_least_stack(const GrammarDev& G) { return automaton_fill_reserve(G) + AF_TIGHT; }
+
 void automaton_fill_layout(const GrammarDev& G, uint32_t rows, uint32_t max_blocks, AutoFillDev& A) {
+  A.reserve = automaton_fill_reserve(G);
   A.scratch_words = 7u * A.ctx_cap + A.pool_cap + A.big_cap / 4u + A.big_cap / 2u + A.big_cap;
   A.unit_words = AU_WORDS;
   // few rows: several blocks take one, so that the chip is filled (a small trie gives the others nothing to do)

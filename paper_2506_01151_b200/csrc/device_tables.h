@@ -46,6 +46,7 @@ struct GrammarDev {
   const uint32_t* ga_node;       // [nodes][4]
   const uint32_t* ga_tok;
   uint32_t ga_lvl2, ga_lvl3;     // first nodes of depth 2 and 3
+  uint32_t ga_path;              // most children along a path
   const uint32_t* ga_wide_rec;   // [entries][4]
   const uint32_t* ga_wide_mask;  // [entries][Wm]
   const uint32_t* ga_wide_exit;  // [][2]
@@ -258,7 +259,7 @@ struct AutoFillDev {
   uint32_t on;               // rows are filled by the automaton
   uint32_t grid, parts;      // thread blocks, and how many of them share a row
   uint4* stack;              // [grid][stack_cap] first child, children, code, context
-  uint32_t stack_cap;
+  uint32_t stack_cap, reserve;  // and the places that are kept for rounds of one entry
   uint32_t* scratch;         // [grid][scratch_words]
   uint32_t scratch_words;
   uint32_t ctx_cap, pool_cap, big_cap;  // contexts per row, words for their lists, items of the largest expansion (powers of two)

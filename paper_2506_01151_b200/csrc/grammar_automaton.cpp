@@ -284,8 +284,9 @@ class Builder {
       node[v] = val[s];
     }
     const u32 n = (u32)eq.size();
-    std::vector<u32> order(1, 0), number(n, 0), depth(1, 0);
+    std::vector<u32> order(1, 0), number(n, 0), depth(1, 0), path(1, 0);
     order.reserve(n);
+    h_.ga_path = 0;
     h_.ga_node.assign((size_t)n * 4, 0u);
     h_.ga_lvl2 = h_.ga_lvl3 = n;
     for (u32 i = 0; i < (u32)order.size(); ++i) {
@@ -294,6 +295,9 @@ class Builder {
       u32 kids = 0;
       for (u32 c = child[order[i]]; c; c = sibling[c], ++kids) number[c] = (u32)order.size(), order.push_back(c), depth.push_back(depth[i] + 1);
       r[1] = kids << 8 | eq[order[i]];
+      path[i] += kids;
+      h_.ga_path = std::max(h_.ga_path, path[i]);
+      path.resize(order.size(), path[i]);
       if (depth[i] == 2) h_.ga_lvl2 = std::min(h_.ga_lvl2, i);
       if (depth[i] == 3) h_.ga_lvl3 = std::min(h_.ga_lvl3, i);
     }

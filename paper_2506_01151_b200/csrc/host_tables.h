@@ -95,6 +95,7 @@ struct HostTables {
   std::vector<uint32_t> ga_node;   // [nodes][4] first child, children << 8 | byte class, the token (or where in ga_tok they begin), tokens
   std::vector<uint32_t> ga_tok;    // token ids by node
   uint32_t ga_lvl2 = 0, ga_lvl3 = 0;  // first nodes of depth 2 and 3
+  uint32_t ga_path = 0;            // the children of a node and of all nodes above it, at most
   // wide items: what follows from them alone
   std::vector<uint32_t> ga_wide;       // [D] entry or GA_DEAD
   std::vector<uint32_t> ga_wide_rec;   // [entries][4] mask row, first exit, exits

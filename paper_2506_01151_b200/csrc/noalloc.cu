@@ -227,7 +227,7 @@ extern "C" fmt_status fmt_fill_mask_noalloc(const fmt_grammar* g, const uint32_t
   S.au.req_cap = NA_REQ_CAP;
   S.au.job_info = reinterpret_cast<uint4*>(scratch + NA_OFF_JOBINFO);
   sweep_layout(*G, &S.au.smem_bytes, &S.au.tables_in_smem);
-  if (G->ga_on) {
+  if (G->ga_on && automaton_fill_least_stack(*G) <= NA_STACK) {
     AutoFillDev& A = S.af;
     A.on = 1;
     A.stack = reinterpret_cast<uint4*>(scratch + NA_HEADER_WORDS);

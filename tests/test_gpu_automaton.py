@@ -100,7 +100,7 @@ def _union(variants):
 @pytest.mark.parametrize("batch", [1, 4, 75, 300])
 def test_more_wide_items_than_there_is_room_for(variants, batch):
     """Up to 60 items of a row's last set are answered by the masks made for them; the others are walked like any item."""
-    w = workloads.build(3, V=20000, batch=1, steps=1)
+    w = workloads.build(2, V=32000, batch=1, steps=1)
     prefixes = [list(p) for p in (b'{"id":', b'{"id":"x', b'{"id":"x","k1', b'{"id":"y","k%d":[[' % (variants - 1))]
     _run(_union(variants), "s", w.vocab, prefixes, batch=batch, check=range(min(batch, 4)))
 
@@ -116,6 +116,33 @@ def test_more_items_than_a_round_takes(n, batch):
     prefixes = [list(p) for p in (b'["k', b'["' + names[5].encode() + b'","k', b'["' + names[1][:9].encode(), b'["')]
     s = _run(text, "s", vocab, prefixes, batch=batch, check=range(min(batch, 4)))
     assert s["walk_states"] < 200 * batch  # (the automaton's contexts, not Earley sets)
+
+
+def _braces():
+    """Text whose every byte ends a rule, at any depth of braces; each byte a class of its own.  Three quarters of the vocabulary
+    are no text (a vocabulary in which rules end nearly everywhere is swept by Earley steps)."""
+    kw = " | ".join('"\\x%02x!"' % b for b in range(33, 256) if chr(b) not in "{}")
+    text = 'doc ::= piece*\npiece ::= char | "{" doc "}" | "}}" kw\nchar ::= [^{}\\x80-\\xff]\nkw ::= "!" | ' + kw + "\n"
+    rng = np.random.default_rng(11)
+    vocab, seen = [bytes([b]) for b in range(256)], set()
+    while len(vocab) < 60000:
+        n = 2 + int(rng.integers(0, 5))
+        t = bytes(rng.integers(32, 126, n).astype(np.uint8)) if len(vocab) % 4 == 0 else bytes(rng.integers(128, 256, n).astype(np.uint8))
+        if rng.random() < 0.2:
+            t += b"}" * int(rng.integers(1, 4))
+        if t not in seen:
+            seen.add(t)
+            vocab.append(t)
+    return text, vocab + [b""]
+
+
+@pytest.mark.parametrize("batch", [1, 64, 149, 300])
+def test_rounds_that_push_more_than_the_stack_holds(batch):
+    """Threads and expansions that find no room in a round go to the block's stack, which is never pushed more than it holds: a row
+    has its mask, however many rows share the grid and however many children its nodes have."""
+    text, vocab = _braces()
+    s = _run(text, "doc", vocab, [list(p) for p in (b"x {a{b{c", b"{" * 30, b"a{}b{{", b"")], batch=batch, check=range(min(batch, 4)))
+    assert s["walk_transitions"] > 20000 * batch  # (look-ups)
 
 
 def test_grammar_without_an_automaton():
