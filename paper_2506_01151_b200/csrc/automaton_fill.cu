@@ -153,12 +153,12 @@ __device__ void spill_contexts(Contexts& C, uint32_t* ctl, const AutoFillDev& A)
   __syncwarp();
 }
 
-// buf[0..n), values rule << 16 | origin in any order, room for the next power of two: sorted, grouped by rule, as the expansion
-// list (offset, count) in the pool.  False when there is no room.
-__device__ bool group_items(const GrammarDev& G, const Contexts& C, uint32_t* ctl, uint32_t* buf, uint32_t n, uint2& out) {
+// buf[0..n), room for the next power of two: sorted, without repeats.  How many are left, and how many rules they are of.
+__device__ uint32_t sort_unique(uint32_t* buf, uint32_t n, uint32_t& groups) {
   const uint32_t lane = lane_id();
   sort_items(buf, n, 1u << 30);
-  uint32_t k = 0, groups = 0;  // repeats go
+  uint32_t k = 0;
+  groups = 0;
   for (uint32_t base = 0, last = 0xFFFFFFFFu; base < n; base += 32) {
     const uint32_t i = base + lane;
     const uint32_t v = i < n ? buf[i] : 0xFFFFFFFFu;
@@ -172,6 +172,15 @@ __device__ bool group_items(const GrammarDev& G, const Contexts& C, uint32_t* ct
     k += __popc(b);
   }
   __syncwarp();
+  return k;
+}
+
+// buf[0..n), values rule << 16 | origin in any order, room for the next power of two: sorted, grouped by rule, as the expansion
+// list (offset, count) in the pool.  False when there is no room.
+__device__ bool group_items(const GrammarDev& G, const Contexts& C, uint32_t* ctl, uint32_t* buf, uint32_t n, uint2& out) {
+  const uint32_t lane = lane_id();
+  uint32_t groups;
+  const uint32_t k = sort_unique(buf, n, groups);
   const uint32_t at = (ctl[AC_POOL] + 1u) & ~1u;
   __syncwarp();
   if (at + 2u * groups > C.pool_cap) return false;
@@ -208,7 +217,8 @@ __device__ bool expand_into(const GrammarDev& G, const Contexts& C, const AfChar
                             uint32_t work_cap, uint32_t* hset, uint32_t hset_mask, uint32_t* buf, uint32_t buf_cap) {
   const uint32_t lane = lane_id();
   __syncwarp();
-  if (lane == 0) ctl[AC_NWORK] = 0u, ctl[AC_NBUF] = 0u, ctl[AC_OVER] = 0u;
+  uint32_t nbuf = 0;
+  if (lane == 0) ctl[AC_NWORK] = 0u, ctl[AC_OVER] = 0u;
   __syncwarp();
   auto need = [&](uint32_t a, uint32_t o) {  // "a, begun in set o, is complete"
     const uint32_t key = a << 16 | o;
@@ -229,18 +239,25 @@ __device__ bool expand_into(const GrammarDev& G, const Contexts& C, const AfChar
     if (head >= n) break;
     const uint32_t a = work[head] >> 16, o = work[head] & 0xFFFFu;
     const uint32_t lo = J.off[o], hi = J.off[o + 1u];
-    for (uint32_t k = lo + lane; k < hi; k += 32) {
-      const uint32_t it = J.items[k];
+    for (uint32_t base = lo; base < hi; base += 32) {
+      const uint32_t k = base + lane;
+      const uint32_t it = k < hi ? J.items[k] : 0u;
       const uint4 rec = __ldg(reinterpret_cast<const uint4*>(G.ga_item) + (it & 0xFFFFu));
-      if ((rec.y >> 16) != a) continue;
-      if (rec.w & GA_GOES_ON) {
-        const uint32_t at = atomicAdd(&ctl[AC_NBUF], 1u);
-        if (at < buf_cap) buf[at] = ((it & 0xFFFFu) + 1u) << 16 | (it >> 16);
-        else ctl[AC_OVER] = 1u;
+      const bool match = k < hi && (rec.y >> 16) == a, on = match && (rec.w & GA_GOES_ON);
+      const uint32_t b = __ballot_sync(FULL, on);
+      if (nbuf + __popc(b) > buf_cap) {  // an item comes once for every set that it waits in: the repeats go
+        uint32_t groups;
+        __syncwarp();
+        nbuf = sort_unique(buf, nbuf, groups);
+        if (nbuf > buf_cap / 2u) return false;
       }
-      if ((rec.w & 0xFFFFu) != 0xFFFFu) need(rec.w & 0xFFFFu, it >> 16);
+      if (on) buf[nbuf + __popc(b & ((1u << lane) - 1u))] = ((it & 0xFFFFu) + 1u) << 16 | (it >> 16);
+      nbuf += __popc(b);
+      if (match && (rec.w & 0xFFFFu) != 0xFFFFu) need(rec.w & 0xFFFFu, it >> 16);
     }
   }
+  if (lane == 0) ctl[AC_NBUF] = nbuf;
+  __syncwarp();
   return true;
 }
 

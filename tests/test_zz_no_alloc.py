@@ -130,3 +130,34 @@ def test_noalloc_checks_every_word_of_a_chart():
     got = mask.cpu().numpy().view(np.uint32)
     assert not got[0].any() and not got[2].any() and not got[3].any()
     assert got[1, 0] == 0b0111  # after "a": a, b, ab
+
+
+@pytest.mark.parametrize("letters", [20, 100, 200, 300])
+def test_noalloc_expansions_of_many_repeats(letters):
+    """In an ambiguous text an item waits in as many sets as there are ways to begin what follows it: what a completion yields is
+    counted without its repeats, of which there are forty thousand at 200 letters."""
+    import torch
+
+    import oracle
+    import paper_2506_01151_b200 as fmt
+
+    text = 's ::= "<" e ">"\ne ::= e e e | e "+" e | "a"'
+    vocab = [bytes([b]) for b in range(256)] + [b"aa", b"a+a", b"a>", b"+a>", b">a", b"aaa>", b""]
+    data = b"<" + b"a" * letters
+    g = fmt.Grammar(text, "s", vocab, len(vocab) - 1)
+    st = fmt.State(g, 1, chart_words=1 << 18)
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    for b in data:
+        st.advance(torch.tensor([b], dtype=torch.int32, device="cuda"), status)
+        assert status.item() == fmt.FMT_OK
+    chart = st.chart_words(0)
+    mask = torch.full((2, g.mask_words), -1, dtype=torch.int32, device="cuda")
+    offs = np.array([0, len(chart), 2 * len(chart)], dtype=np.uint64)
+    status = torch.full((2,), -1, dtype=torch.int32, device="cuda")
+    fmt.fill_mask_noalloc(g, torch.from_numpy(np.tile(chart, 2).view(np.int32)).cuda(), offs, mask, status)
+    seq = oracle.Sequence_(oracle.Grammar(text, "s"))
+    assert seq.advance(data)
+    want = seq.mask(oracle.Vocab(vocab, len(vocab) - 1))
+    assert status.tolist() == [fmt.FMT_OK, fmt.FMT_OK]
+    got = mask.cpu().numpy().view(np.uint32)
+    assert np.array_equal(got[0], want) and np.array_equal(got[1], want)
