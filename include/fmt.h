@@ -159,6 +159,8 @@ typedef struct {
                                    blocks, [7] a context-independent entry that could not be kept;
                                    [8..15] the same for the sweeps that fill such entries */
   uint64_t cache_flushes;       /* times the state cache was turned over because it had no room left */
+  uint64_t rows_swept_again;    /* computed rows that outgrew what the fill by the grammar's automaton has room for, or took
+                                   too long there, and were swept by Earley steps in the same call */
 } fmt_stats;
 
 /*
@@ -369,7 +371,7 @@ fmt_status fmt_state_read_profile_series(fmt_state* s, int kind, float* ms_out, 
  * but it needs an fmt_state, whose creation allocates gigabytes (fmt_stats.device_bytes).  This call needs no
  * fmt_state: it sweeps the vocabulary trie for charts the caller already holds in device memory
  * (in the layout fmt_state_copy_chart documents) and uses a fixed scratch array that is part of
- * the loaded library image (about 55 MB of device memory on every GPU that loads the library,
+ * the loaded library image (about 70 MB of device memory on every GPU that loads the library,
  * held until the process exits).
  *
  *   g              a grammar compiled for the current device

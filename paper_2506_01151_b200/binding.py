@@ -58,7 +58,7 @@ class Stats(C.Structure):
         "mask_rows_cached", "pool_words_used", "chart_items_max", "chart_sets_max", "capacity_errors",
         "big_mode_units", "sweep_transitions", "sweep_states", "advances_cached", "roots", "root_sweeps",
         "rows_mask_only", "rows_from_root", "rows_plain", "walk_transitions", "walk_states", "walk_frames",
-        "fills_aborted", "device_bytes", "earley_step_cycles", "advance_chart_words")] + [("diag", C.c_uint64 * 16), ("cache_flushes", C.c_uint64)]
+        "fills_aborted", "device_bytes", "earley_step_cycles", "advance_chart_words")] + [("diag", C.c_uint64 * 16), ("cache_flushes", C.c_uint64), ("rows_swept_again", C.c_uint64)]
 
     def as_dict(self):
         d = {n: int(getattr(self, n)) for n, _ in self._fields_ if n != "diag"}

@@ -27,6 +27,8 @@ fmt_status cuda_fail(cudaError_t e, const char* what) {
               std::string(what) + ": " + cudaGetErrorString(e));
 }
 
+constexpr int kAsIs = -1;  // memory that is written before it is read
+
 struct DeviceBuffers {
   std::vector<void*> ptrs;
   size_t bytes = 0;
@@ -55,7 +57,7 @@ struct DeviceBuffers {
     if (e != cudaSuccess) return e;
     ptrs.push_back(p);
     this->bytes += bytes;
-    e = cudaMemset(p, fill_byte, bytes);
+    if (fill_byte != kAsIs) e = cudaMemset(p, fill_byte, bytes);
     if (e != cudaSuccess) return e;
     *out = static_cast<T*>(p);
     return cudaSuccess;
@@ -141,7 +143,7 @@ static cudaError_t next_generations(fmt_state* s, cudaStream_t st) {
   StateDev& d = s->dev;
   cudaError_t e = cudaSuccess;
   if (s->next_gen + 1u > 65534u) {
-    if (d.af.on) e = cudaMemsetAsync(d.af.unit_flag, 0, ((size_t)d.af.unit_cap + d.B) * 4, st);
+    if (d.af.on) e = cudaMemsetAsync(d.af.unit_flag, 0, (size_t)d.af.flag_words * 4, st);
     if (e == cudaSuccess && !d.af.on) e = cudaMemsetAsync(d.au.hash, 0, (size_t)d.B * (d.au.hash_mask + 1u) * 4, st);
     if (e == cudaSuccess && !d.af.on) e = cudaMemsetAsync(d.au.req, 0, (size_t)d.au.req_cap * 8, st);
     if (e == cudaSuccess && d.rt.on) e = cudaMemsetAsync(d.cx.ctab, 0, (size_t)d.B * CT_SLOTS * 8, st);
@@ -405,6 +407,34 @@ static cudaError_t alloc_sweep(fmt_state* s) {
   return e;
 }
 
+// The tables of rows that the automaton's fill gives up (af.sweep_slots of them at a time), in one allocation: nothing there is read
+// before it is written.  The capacities are the grid-wide sweep's, but for the pool of items, which such rows share.
+static cudaError_t alloc_row_sweeps(fmt_state* s) {
+  StateDev& d = s->dev;
+  AutoDev& au = d.au;
+  const size_t n = d.af.sweep_slots;
+  au.st_stride = (s->g->dev.T + 63u) & ~63u;
+  au.req_cap = 128u << 10;
+  au.items_cap = 64u << 20;
+  size_t words = 0;
+  auto take = [&](size_t w) {
+    const size_t at = words;
+    words += (w + 63u) & ~(size_t)63u;
+    return at;
+  };
+  const size_t o_big = take(n * automaton_fill_warps() * ((size_t)d.big_arena_items + d.big_hset_slots));
+  const size_t o_recs = take(n * au.cap * au.rec_words), o_hash = take(n * (au.hash_mask + 1u)), o_n = take(n);
+  const size_t o_st = take((n * au.st_stride + 1u) / 2u), o_req = take(n * au.req_cap), o_items = take(au.items_cap);
+  uint32_t* base = nullptr;
+  const cudaError_t e = s->bufs.alloc(words, &base, kAsIs);
+  if (e != cudaSuccess) return e;
+  d.big_scratch = base + o_big;
+  au.recs = base + o_recs, au.hash = base + o_hash, au.n_states = base + o_n, au.items = base + o_items;
+  au.st = reinterpret_cast<uint16_t*>(base + o_st);
+  au.req = reinterpret_cast<unsigned long long*>(base + o_req);
+  return cudaSuccess;
+}
+
 fmt_status fmt_state_create(const fmt_grammar* g, uint32_t batch, const fmt_state_options* opt, void* stream,
                             fmt_state** out) {
   if (!out) return fail(FMT_ERR_INVALID_ARG, "out is NULL");
@@ -513,7 +543,13 @@ fmt_status fmt_state_create(const fmt_grammar* g, uint32_t batch, const fmt_stat
     AL(af.stack, (size_t)af.grid * af.stack_cap, 0);
     AL(af.scratch, (size_t)af.grid * af.scratch_words, 0);
     AL(af.units, (size_t)af.unit_cap * af.unit_words, 0);
-    AL(af.unit_flag, af.unit_cap + batch, 0);
+    // (behind the flags, which carry the fills' generations, the locks of the tables below)
+    af.sweep_slots = std::min(batch, 16u);
+    const uint32_t rows4 = (batch + 3u) & ~3u;
+    af.flag_words = af.unit_cap + 3u * rows4;
+    AL(af.unit_flag, af.flag_words + af.sweep_slots, 0);
+    af.row_gone = af.unit_flag + af.unit_cap + rows4, af.given = af.row_gone + rows4, af.sweep_lock = af.given + rows4;
+    if (e == cudaSuccess) e = alloc_row_sweeps(s);
   } else if (e == cudaSuccess) {
     e = alloc_sweep(s);
   }
@@ -867,6 +903,7 @@ fmt_status fmt_get_stats(fmt_state* s, fmt_stats* out, void* stream) {
   out->walk_frames = u64(CNT_STAT_FRAMES);
   out->root_sweeps = u64(CNT_STAT_ROOT_SWEEPS);
   out->fills_aborted = u64(CNT_STAT_ABORTS);
+  out->rows_swept_again = u64(CNT_STAT_SWEPT);
   out->device_bytes = s->device_bytes;
   out->cache_flushes = s->flushes;
   out->earley_step_cycles = u64(CNT_STAT_STEP_CYCLES);

@@ -18,12 +18,14 @@
 //   128 rows of SQL, 152,064 tokens             667 -> 231 us
 //   37 rows of JSON, 50,001 tokens              362 -> 129 us
 //   256 rows of ambiguous JSON, 128,256 tokens  3.51 -> 1.06 ms (2.65 ms when no work is handed on)
-// The sweep stays for grammars without an automaton and for the cache of context-independent entries.
+// The sweep stays for grammars without an automaton and for the cache of context-independent entries.  A row that outgrows the
+// contexts' storage, or takes far longer than rows do, is swept by Earley steps within the call (block_sweep.cuh).
 #include <cuda_runtime.h>
 
 #include <algorithm>
 
 #include "kernels.h"
+#include "block_sweep.cuh"
 #include "sweep_warp.cuh"
 
 namespace fmt {
@@ -46,14 +48,20 @@ constexpr uint32_t AF_MAX_UNITS = 7;      // to so many at once, 128 threads at 
 // code of a special: to start the threads of a context's expansion at a node (first child, children, AF_SPAWN, elements that have been
 // started << 16 | context)
 constexpr uint32_t AF_SPAWN = 0xFFFFFFFDu;
-constexpr uint32_t AF_GIVEN_UP = 0xFFFFFFFFu;  // (AC_FAIL) a wait ran out: the fill is given up, the row itself is fine
+constexpr uint32_t AF_KCYCLES = 1u << 14;      // a share of a row that takes longer (2^24 cycles, 8.5 ms) is given up for a sweep by Earley steps
+// AC_FAIL: 0, 1 + the capacity that was exceeded, or
+constexpr uint32_t AF_GIVEN_UP = 0xFFFFFFFFu;  // a wait ran out: the fill is given up, the row itself is fine
+constexpr uint32_t AF_GONE = 0xFFFFFFFEu;      // another block has given the row up
+constexpr uint32_t AF_LATE = 0xFFFFFFFDu;      // the share takes too long
 constexpr uint32_t CTX_NEW = 0xFFFFFFFFu;
 
 enum : uint32_t {
   AC_NEXT = 0, AC_SPEC = 1, AC_OVF = 2, AC_GTOP = 3, AC_FAIL = 4, AC_NCTX = 5, AC_POOL = 6, AC_NWORK = 7, AC_WSUM = 8, AC_NBUF = 16, AC_OVER = 17,
   AC_SPILLED = 18, AC_WAITING = 19, AC_BASE = 20, AC_JOB = 21, AC_NWIDE = 22, AC_POPPED = 24, AC_NEXITS = 25, AC_LIST = 26,
-  AC_LIST_AT = 27, AC_LIST_END = 28, AC_POPPED_SPEC = 29, AC_WIDE = 30, AC_WORDS = AC_WIDE + AF_EXITS + 2
+  AC_LIST_AT = 27, AC_LIST_END = 28, AC_POPPED_SPEC = 29, AC_BEGAN = 30,
+  AC_PEEK = 32, AC_WIDE = 40, AC_WORDS = (AC_WIDE + AF_EXITS + 3) & ~3u
 };
+static_assert(AC_WORDS % 4 == 0 && AC_WORDS <= AF_THREADS, "what follows in shared memory is cleared in 16-byte pieces; a thread clears a word");
 
 // A unit of work handed out: AU_HDR words, then the giver's contexts, lists and the threads.
 enum : uint32_t { AU_ROWJOB = 0, AU_N = 1, AU_NCTX = 2, AU_POOL = 3, AU_PART = 4, AU_HDR = 8 };
@@ -70,6 +78,10 @@ struct Contexts {
   uint32_t* pool;
   uint32_t cap, hash_mask, pool_cap;
 };
+// Four words of global memory (16-byte aligned, read past L1) on their way into shared memory.
+__device__ __forceinline__ void peek(uint32_t* to, const uint32_t* from) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(to)), "l"(from) : "memory");
+}
 __device__ __forceinline__ uint32_t vload(const uint32_t* p) { return *reinterpret_cast<const volatile uint32_t*>(p); }
 __device__ __forceinline__ Contexts global_contexts(const AutoFillDev& A) {
   uint32_t* p = A.scratch + (size_t)blockIdx.x * A.scratch_words;
@@ -473,6 +485,7 @@ __global__ void __launch_bounds__(AF_THREADS, 4) automaton_fill_kernel(const __g
           }
         }
         ctl[AC_JOB] = got ? ticket : 0xFFFFFFFFu;
+        ctl[AC_BASE] = vload(&S.counters[CNT_AF_GIVEN]);
       }
       __syncthreads();
       const uint32_t u = ctl[AC_JOB];
@@ -622,6 +635,7 @@ __global__ void __launch_bounds__(AF_THREADS, 4) automaton_fill_kernel(const __g
       }
     }
     const uint32_t looked_up_before = looked_up;
+    if (tid == AF_THREADS - 1) ctl[AC_BEGAN] = (uint32_t)(clock64() >> 10);
 
     bool spilled = false;
     // the expansion of a context (offset into pool, count), and its elements
@@ -651,9 +665,9 @@ __global__ void __launch_bounds__(AF_THREADS, 4) automaton_fill_kernel(const __g
       uint4* const spec = specials + side * AF_SPEC;
       uint4* const spec_nxt = specials + (side ^ 1u) * AF_SPEC;
       if (tid == 0) ctl[AC_NEXT] = 0u, ctl[AC_SPEC] = 0u, ctl[AC_OVF] = 0u;
-      if (tid == AF_THREADS - 1) {  // (looked at in the next round)
-        const uint32_t t = vload(&S.counters[CNT_AF_TAKEN]), p = vload(&S.counters[CNT_AF_POSTED]);
-        ctl[AC_WAITING] = t > p ? t - p : 0u;
+      if (tid == AF_THREADS - 1) {  // (looked at when the round ends; nobody waits for them until then)
+        peek(ctl + AC_PEEK, S.counters + CNT_AF_TICKET);
+        peek(ctl + AC_PEEK + 4u, A.row_gone + (j & ~3u));
       }
       // The stack cannot run over.  A round pushes at most the threads that its specials and its list start and two entries for each
       // child it looks up, and takes no more than fits above the reserve.  On a crowded stack one entry is taken at a time, from the top:
@@ -925,14 +939,24 @@ __global__ void __launch_bounds__(AF_THREADS, 4) automaton_fill_kernel(const __g
       }
       side ^= 1u;
       __syncthreads();
-      if (tid == 0) ctl[AC_GTOP] = gtop + ctl[AC_OVF], ctl[AC_POPPED] = ctl[AC_POPPED_SPEC] = 0u;
+      if (tid == 0) {
+        ctl[AC_GTOP] = gtop + ctl[AC_OVF];
+        if (pops) ctl[AC_POPPED] = ctl[AC_POPPED_SPEC] = 0u;
+      }
+      if (tid == AF_THREADS - 1) {
+        asm volatile("cp.async.wait_all;" ::: "memory");
+        const uint32_t t = ctl[AC_PEEK + CNT_AF_TAKEN - CNT_AF_TICKET], p = ctl[AC_PEEK + CNT_AF_POSTED - CNT_AF_TICKET];
+        const bool gone = ctl[AC_PEEK + 4u + (j & 3u)] == S.gen, late = (uint32_t)(clock64() >> 10) - ctl[AC_BEGAN] > AF_KCYCLES;
+        ctl[AC_WAITING] = t > p ? t - p : 0u;
+        if ((gone || late) && !ctl[AC_FAIL]) ctl[AC_FAIL] = gone ? AF_GONE : AF_LATE;
+      }
       __syncthreads();
     }
     contexts += ctl[AC_NCTX];
-    if (tid == 0 && ctl[AC_FAIL] && ctl[AC_FAIL] != AF_GIVEN_UP) {  // a capacity was exceeded: the row's mask cannot be trusted
-      diag(S, ctl[AC_FAIL] - 1u);
-      if (!(atomicOr(&S.row_flags[row], ROW_BROKEN) & ROW_BROKEN)) stat_add(S, CNT_STAT_CAPERR, 1u);
-      atomicExch(&S.counters[CNT_ERR], 1u);
+    if (tid == 0 && ctl[AC_FAIL] && ctl[AC_FAIL] < AF_GONE) {  // too many contexts, or too long a time: the row is left to a sweep by Earley steps
+      if (ctl[AC_FAIL] != AF_LATE) diag(S, ctl[AC_FAIL] - 1u);
+      if (atomicExch(A.row_gone + j, S.gen) != S.gen)  // (its other blocks stop when they see that)
+        *reinterpret_cast<volatile uint32_t*>(A.given + atomicAdd(&S.counters[CNT_AF_GIVEN], 1u)) = S.gen << 16 | j;
     }
     // ---- the next row
     __threadfence();
@@ -943,17 +967,73 @@ __global__ void __launch_bounds__(AF_THREADS, 4) automaton_fill_kernel(const __g
     stat_add(S, CNT_STAT_TRANS, looked_up);
     stat_add(S, CNT_STAT_LOCAL, contexts);
   }
+  // ---- rows that were given up, swept by blocks that have nothing else to do any more: who gives one up comes here later itself.  Only
+  // blocks that look for tables wait, and who has tables waits for nobody.
+  for (bool given = ctl[AC_BASE] != 0u; given;) {
+    __syncthreads();
+    if (tid == 0) {
+      uint32_t at = vload(&S.counters[CNT_AF_GIVEN_TAKEN]), got = 0xFFFFFFFFu, slot = 0xFFFFFFFFu;
+      while (at < ld_acquire(&S.counters[CNT_AF_GIVEN])) {
+        const uint32_t was = atomicCAS(&S.counters[CNT_AF_GIVEN_TAKEN], at, at + 1u);
+        if (was == at) {
+          got = at;
+          break;
+        }
+        at = was;
+      }
+      if (got != 0xFFFFFFFFu) {
+        uint32_t k = blockIdx.x % A.sweep_slots, v = 0u;
+        for (uint32_t polls = 0; slot == 0xFFFFFFFFu; ++polls, k = (k + 1u) % A.sweep_slots) {
+          if ((v >> 16) != S.gen) v = vload(A.given + got);  // (written right after its number was drawn)
+          if ((v >> 16) == S.gen && atomicCAS(A.sweep_lock + k, 0u, 1u) == 0u) slot = k;
+          else if (ld_acquire(&S.counters[CNT_BAR_ERR])) break;
+          else if (polls > poll_limit(S, 22)) {
+            diag(S, DIAG_WAIT_VALUE);
+            atomicExch(&S.counters[CNT_BAR_ERR], 1u);
+            break;
+          } else {
+            __nanosleep(400);
+          }
+        }
+        ctl[AC_BASE] = v & 0xFFFFu;
+        __threadfence();
+      }
+      ctl[AC_JOB] = slot;
+    }
+    __syncthreads();
+    const uint32_t slot = ctl[AC_JOB], row = slot == 0xFFFFFFFFu ? 0u : S.jobs[ctl[AC_BASE]];
+    __syncthreads();
+    if (slot == 0xFFFFFFFFu) break;
+    // (copies: if the parameters themselves were passed by reference, the rounds above would read them anew each time they are used; 12
+    // steps of 128 rows of SQL 5.42 ms, with copies 5.22)
+    const GrammarDev g = G;
+    const StateDev s = S;
+    const bool ok = sweep_row_by_block(g, s, row, slot, smem);
+    __threadfence();
+    __syncthreads();
+    if (tid == 0) {
+      atomicExch(A.sweep_lock + slot, 0u);
+      stat_add(S, CNT_STAT_SWEPT, 1u);
+      if (!ok) {  // a capacity was exceeded there, too: the row's mask cannot be trusted
+        diag(S, DIAG_SET_SCRATCH);
+        if (!(atomicOr(&S.row_flags[row], ROW_BROKEN) & ROW_BROKEN)) stat_add(S, CNT_STAT_CAPERR, 1u);
+        atomicExch(&S.counters[CNT_ERR], 1u);
+      }
+    }
+  }
 }
 
 // ===================================================================================== launchers
 
 constexpr uint32_t AF_SMEM = (2 * AF_BATCH + 2 * AF_SPEC + AF_EXITS) * 16 + AF_SEEN * 8 + AF_OWNER * 2 + (5 * AF_CTX + AF_POOL + AF_CTX_HASH + AF_BATCH + 4 + AC_WORDS + AF_STAGE + AF_BUF + AF_WORK + AF_HSET) * 4;
+static_assert(block_sweep_words(AF_WARPS, MAX_NONTERMINALS / 32u) * 4u <= AF_SMEM, "a row that is given up is swept in the same shared memory");
 
 // Places of a block's stack that only its depth-first rounds use: two for each child along the longest path of the trie and one for
 // what is left of a special at each of its nodes, and what a round may hold or has put back when the last places above are taken.
 uint32_t automaton_fill_reserve(const GrammarDev& G) {
   return 2u * G.ga_path + MAX_TOKEN_BYTES + 1u + 2u * (AF_BATCH + AF_SPEC) + 32u;
 }
+uint32_t automaton_fill_warps() { return AF_WARPS; }
 uint32_t automaton_fill_least_stack(const GrammarDev& G) { return automaton_fill_reserve(G) + AF_TIGHT; }
 
 void automaton_fill_layout(const GrammarDev& G, uint32_t rows, uint32_t max_blocks, AutoFillDev& A) {

@@ -101,17 +101,20 @@ enum : uint32_t {
   CNT_STAT_JOBS_ROOT = 152,    // 64-bit: computed rows that started from a swept root
   CNT_STAT_JOBS_PLAIN = 154,   // 64-bit: computed rows that walked the whole trie themselves
   CNT_STAT_JOBS_MASK = 156,    // 64-bit: computed rows answered by their root's mask row alone
-  CNT_AF_TICKET = 186,         // rows handed out to the blocks of the automaton's fill, beyond one for each
-  CNT_AF_TAKEN = 187,          // tickets drawn for units of work
-  CNT_AF_POSTED = 188,         // units given
-  CNT_AF_ACTIVE = 189,         // shares of rows, and units, that are not finished
   CNT_STAT_ABORTS = 160,       // 64-bit: fills abandoned because a bounded wait ran out
   CNT_STAT_STEP_CYCLES = 162,  // 64-bit: SM cycles spent inside Earley steps of the fill (summed over warps)
   CNT_STAT_ADV_WORDS = 164,    // 64-bit: chart words read and written by advance
   CNT_STAT_FRAMES = 184,       // 64-bit: frames made (sets of a walk recognised as roots)
   CNT_DIAG = 166,              // [16] where capacity errors and expired waits came from (see DIAG_*)
   CNT_ADV_STEPPED = 190,       // the last call in which a row took an Earley step
-  CNT_TOTAL = 192
+  CNT_STAT_SWEPT = 192,        // 64-bit: rows that the automaton's fill gave up, and a block swept
+  CNT_AF_GIVEN = 194,          // rows given up in this fill
+  CNT_AF_GIVEN_TAKEN = 195,    // how many of them a block has taken
+  CNT_AF_TICKET = 196,         // shares of rows handed out to the blocks of the automaton's fill (these four are read together)
+  CNT_AF_TAKEN = 197,          // tickets drawn for units of work
+  CNT_AF_POSTED = 198,         // units given
+  CNT_AF_ACTIVE = 199,         // shares of rows, and units, that are not finished
+  CNT_TOTAL = 200
 };
 
 enum : uint32_t {
@@ -266,7 +269,11 @@ struct AutoFillDev {
   uint32_t* units;           // [unit_cap][unit_words]
   uint32_t* unit_flag;       // [unit_cap] the generation (StateDev::gen) of the fill whose unit is there; then per row that of the fill
                              // in which its mask has been begun
-  uint32_t unit_cap, unit_words;
+  uint32_t* row_gone;        // [rows, a multiple of four; 16-byte aligned] the generation of the fill in which the row was given up
+  uint32_t* given;           // [rows] the rows given up, generation << 16 | job
+  uint32_t* sweep_lock;      // [sweep_slots] 1: a block sweeps a row in these tables (StateDev::au); 0 between launches
+  uint32_t sweep_slots;
+  uint32_t unit_cap, unit_words, flag_words;  // (flag_words: unit_flag, row_gone and given together)
 };
 
 struct StateDev {

@@ -382,6 +382,7 @@ __global__ void __launch_bounds__(1024) plan_kernel(const __grid_constant__ Gram
     S.counters[CNT_N_FJOBS] = 0u;
     S.counters[CNT_AUTO_ITEMS] = 0u;
     S.counters[CNT_AF_TICKET] = S.counters[CNT_AF_TAKEN] = S.counters[CNT_AF_POSTED] = 0u;
+    S.counters[CNT_AF_GIVEN] = S.counters[CNT_AF_GIVEN_TAKEN] = 0u;
     n_jobs = n_cached = n_shared = 0u;
     n_rows = S.counters[CNT_N_MASK_ROWS];
   }

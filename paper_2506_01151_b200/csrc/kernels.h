@@ -41,6 +41,7 @@ int sweep_warps();
 constexpr uint32_t AUTO_FILL_PER_SM = 4;  // thread blocks on an SM
 void automaton_fill_layout(const GrammarDev& G, uint32_t rows, uint32_t max_blocks, AutoFillDev& A);
 uint32_t automaton_fill_least_stack(const GrammarDev& G);  // entries
+uint32_t automaton_fill_warps();                            // of a block
 cudaError_t configure_automaton_fill();
 void launch_automaton_fill(const GrammarDev& G, const StateDev& S, cudaStream_t st);
 

@@ -145,6 +145,29 @@ def test_rounds_that_push_more_than_the_stack_holds(batch):
     assert s["walk_transitions"] > 20000 * batch  # (look-ups)
 
 
+def _endings(n):
+    """Brackets of n kinds, told apart after they close: every level of the text is completed to n kinds, n contexts a level.  Half of
+    the vocabulary are words that are no text."""
+    kinds = [chr(97 + i) if i < 20 else "z%c%c" % (97 + i // 26, 97 + i % 26) for i in range(n)]
+    text = "s ::= t\nt ::= \"x\" | " + " | ".join("t%d" % i for i in range(n)) + "\n"
+    text += "".join('t%d ::= "(" t ")" "%s"\n' % (i, k) for i, k in enumerate(kinds))
+    rng = np.random.default_rng(n)
+    chains = [b"".join(b")" + kinds[int(i)].encode() for i in rng.integers(0, n if k % 2 else 20, 16))[:32] for k in range(60)]
+    vocab = [bytes([b]) for b in range(256)] + [b"x" + c[:3 * k + 1] for k, c in enumerate(chains[:10])] + chains + [b")(", b"(("]
+    letters = np.frombuffer(b"abcdefghijklmnopqrstuvwxyz", np.uint8)
+    return text, vocab + sorted({bytes(letters[rng.integers(0, 26, 6)]) for _ in range(40000)}) + [b""]
+
+
+@pytest.mark.parametrize("n, batch", [(20, 3), (100, 3), (340, 1), (340, 9), (340, 80)])
+def test_rows_that_outgrow_the_storage_of_contexts(n, batch):
+    """Contexts begin in shared memory (64) and go on in storage of the block's own (4,096).  A row that needs more is swept by
+    Earley steps in the same call, by one of its blocks; the rows beside it are not touched by that."""
+    text, vocab = _endings(n)
+    prefixes = [list(p) for p in (b"(" * 20, b"(" * 20 + b"x", b"(" * 20 + b"x)a", b"((x)a")]
+    s = _run(text, "s", vocab, prefixes, batch=batch, check=range(min(batch, 4)))
+    assert s["rows_swept_again"] <= batch and (n == 20 or s["rows_swept_again"] > 0)
+
+
 def test_grammar_without_an_automaton():
     """Alternations of more than a thousand literals have none: their rows are swept by Earley steps."""
     names = sorted({"k%06d" % (i * 7919 % 999983) for i in range(1200)})

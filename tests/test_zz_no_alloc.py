@@ -161,3 +161,31 @@ def test_noalloc_expansions_of_many_repeats(letters):
     assert status.tolist() == [fmt.FMT_OK, fmt.FMT_OK]
     got = mask.cpu().numpy().view(np.uint32)
     assert np.array_equal(got[0], want) and np.array_equal(got[1], want)
+
+
+def test_noalloc_rows_that_outgrow_the_storage_of_contexts():
+    """More contexts than a block's part of the scratch holds (1,024): the chart is swept by Earley steps, one chart after the other."""
+    import torch
+
+    import oracle
+    import paper_2506_01151_b200 as fmt
+    from test_gpu_automaton import _endings
+
+    text, vocab = _endings(300)
+    g = fmt.Grammar(text, "s", vocab, len(vocab) - 1)
+    st = fmt.State(g, 3)
+    og, ov = oracle.Grammar(text, "s"), oracle.Vocab(vocab, len(vocab) - 1)
+    texts = [b"(" * 14, b"(" * 14 + b"x", b"(" * 13 + b"x)a"]
+    for i in range(max(map(len, texts))):
+        st.advance(torch.tensor([t[i] if i < len(t) else -1 for t in texts], dtype=torch.int32, device="cuda"))
+    charts = [st.chart_words(b) for b in range(3)] * 4
+    offs = np.concatenate([[0], np.cumsum([len(c) for c in charts])]).astype(np.uint64)
+    mask = torch.full((12, g.mask_words), -1, dtype=torch.int32, device="cuda")
+    status = torch.full((12,), -1, dtype=torch.int32, device="cuda")
+    fmt.fill_mask_noalloc(g, torch.from_numpy(np.concatenate(charts).view(np.int32)).cuda(), offs, mask, status)
+    assert not status.any()
+    got = mask.cpu().numpy().view(np.uint32)
+    for b in range(12):
+        seq = oracle.Sequence_(og)
+        assert seq.advance(texts[b % 3])
+        assert np.array_equal(got[b], seq.mask(ov)), b
