@@ -165,6 +165,40 @@ __device__ void spill_contexts(Contexts& C, uint32_t* ctl, const AutoFillDev& A)
   __syncwarp();
 }
 
+// The contexts (lhs, {origin}) of the lanes with `valid`, all looked up at once: each lane's number, or CTX_NEW for all of them when there
+// is no room.  (Nearly all contexts have one origin.  One after the other, each with its own chain of look-ups, those of a union of 60
+// variants took 2.4 ms a fill of 4 rows, see below.)
+__device__ uint32_t intern_singles(const Contexts& C, uint32_t* ctl, bool valid, uint32_t lhs, uint32_t origin) {
+  const uint32_t lane = lane_id();
+  const uint32_t peers = __match_any_sync(FULL, valid ? lhs << 16 | origin : 0xFFFFFFFFu);
+  const int leader = __ffs(peers) - 1;
+  const uint32_t home = mix32(mix32(origin + 1u) + lhs * 0x9E3779B9u + 1u) & C.hash_mask;  // (as context_hash has it)
+  uint32_t id = CTX_NEW;
+  if (valid && (int)lane == leader)
+    for (uint32_t slot = home; id == CTX_NEW; slot = (slot + 1u) & C.hash_mask) {
+      const uint32_t v = C.hash[slot];
+      if (v == 0u) break;
+      const uint2 o = C.org[v - 1u];
+      if (o.y == 1u && C.lhs[v - 1u] == lhs && C.pool[o.x] == origin) id = v - 1u;
+    }
+  const bool fresh = valid && (int)lane == leader && id == CTX_NEW;
+  const uint32_t b = __ballot_sync(FULL, fresh), n = __popc(b), first = ctl[AC_NCTX], at = ctl[AC_POOL];
+  __syncwarp();
+  if (first + n > C.cap || n > C.pool_cap - at) return CTX_NEW;
+  if (fresh) {
+    const uint32_t r = __popc(b & ((1u << lane) - 1u));
+    id = first + r;
+    C.pool[at + r] = origin;
+    C.org[id] = make_uint2(at + r, 1u);
+    C.exp[id] = make_uint2(0u, CTX_NEW);
+    C.lhs[id] = lhs;
+    for (uint32_t slot = home; atomicCAS(&C.hash[slot], 0u, id + 1u) != 0u;) slot = (slot + 1u) & C.hash_mask;
+  }
+  if (lane == 0) ctl[AC_NCTX] = first + n, ctl[AC_POOL] = at + n;
+  __syncwarp();
+  return __shfl_sync(FULL, id, leader);
+}
+
 // buf[0..n), room for the next power of two: sorted, without repeats.  How many are left, and how many rules they are of.
 __device__ uint32_t sort_unique(uint32_t* buf, uint32_t n, uint32_t& groups) {
   const uint32_t lane = lane_id();
@@ -200,6 +234,23 @@ __device__ bool group_items(const GrammarDev& G, const Contexts& C, uint32_t* ct
   __syncwarp();
   uint32_t g = 0;
   for (uint32_t i = 0; i < k;) {
+    {  // rules with one item each, up to 32 of them together
+      const uint32_t x = i + lane < k ? buf[i + lane] : 0xFFFFFFFFu, y = i + lane + 1u < k ? buf[i + lane + 1u] >> 16 : 0xFFFFu;
+      const uint32_t before = __shfl_up_sync(FULL, x >> 16, 1);
+      const uint32_t other = __ballot_sync(FULL, i + lane >= k || y == x >> 16 || (lane && before == x >> 16));
+      const uint32_t run = other ? (uint32_t)__ffs(other) - 1u : 32u;
+      if (run) {
+        const uint4 rec = lane < run ? __ldg(reinterpret_cast<const uint4*>(G.ga_item) + (x >> 16)) : make_uint4(GA_DEAD, 0u, 0u, 0u);
+        const bool v = lane < run && rec.x != GA_DEAD;
+        const uint32_t alive = __ballot_sync(FULL, v);
+        const uint32_t c = intern_singles(C, ctl, v, rec.y & 0xFFFFu, x & 0xFFFFu);
+        if (__any_sync(FULL, v && c == CTX_NEW)) return false;
+        if (v) reinterpret_cast<uint2*>(C.pool)[at / 2u + g + __popc(alive & ((1u << lane) - 1u))] = make_uint2(rec.x, (x & 0xFFFF0000u) | c);
+        g += __popc(alive);
+        i += run;
+        continue;
+      }
+    }
     const uint32_t d = buf[i] >> 16;
     const uint4 rec = __ldg(reinterpret_cast<const uint4*>(G.ga_item) + d);
     uint32_t e = i + 1u;
@@ -317,7 +368,23 @@ __device__ bool expand_small(const GrammarDev& G, const Contexts& C, const AfCha
   __syncwarp();
   if (lane == 0) ctl[AC_POOL] = at + 2u * ni;
   __syncwarp();
-  for (uint32_t left = ni == 32u ? FULL : (1u << ni) - 1u; left;) {
+  uint32_t left = ni == 32u ? FULL : (1u << ni) - 1u;
+  {  // rules with one item
+    const bool mine = (left >> lane) & 1u;
+    const uint32_t same = __match_any_sync(FULL, mine ? item >> 16 : 0x10000u + lane);
+    const bool single = mine && same == 1u << lane;
+    const uint4 rec = single ? __ldg(reinterpret_cast<const uint4*>(G.ga_item) + (item >> 16)) : make_uint4(GA_DEAD, 0u, 0u, 0u);
+    const bool v = single && rec.x != GA_DEAD;
+    const uint32_t alive = __ballot_sync(FULL, v);
+    left &= ~__ballot_sync(FULL, single);
+    if (alive) {
+      const uint32_t ctx = intern_singles(C, ctl, v, rec.y & 0xFFFFu, item & 0xFFFFu);
+      if (__any_sync(FULL, v && ctx == CTX_NEW)) return false;
+      if (v) reinterpret_cast<uint2*>(C.pool)[at / 2u + __popc(alive & ((1u << lane) - 1u))] = make_uint2(rec.x, (item & 0xFFFF0000u) | ctx);
+      g = __popc(alive);
+    }
+  }
+  while (left) {
     const uint32_t d = __shfl_sync(FULL, item >> 16, __ffs(left) - 1);
     const bool in = ((left >> lane) & 1u) && (item >> 16) == d;
     const uint32_t members = __ballot_sync(FULL, in), n = __popc(members);
