@@ -33,6 +33,17 @@ constexpr size_t GA_WIDE_NODES = 1024;    // an item is wide from so many trie n
 constexpr size_t GA_MAX_ITEMS = 1024;     // items of one set, predicted ones included: alternations of thousands of literals
                                           // would be scanned again for every set that predicts them
 
+// Where the chart has to be asked at many places a fill by the automaton is the slower one: its threads walk the trie one by one, and
+// each exit starts a thread for every item that completing the rule yields.  Two counts over the walk tell such grammars; they go without.
+// Fills of 64 rows of 128,256 tokens by the automaton and by the sweep, us (share of nodes with an exit; starts a node):
+//   JSON 94 and 239 (0.09; 0.6)   ambiguous JSON 400 and 1,000 (0.12; 1.4)   SQL 231 and 667 (0.03; 1.1)   JSON schema 77 and 263 (0.02; 0.04)
+//   HTML 923 and 457 (0.75; 69)   braces 1,758 and 753 (0.72; 1.4)   XML 14,000 and 1,280 (0.75; 4.6)   two like texts 1,750 and 603 (0.51; 3.3)
+//   a union of 60 variants 2,607 and 430 (0.05; 5.1)   a C-like language 1,883 and 669 (0.17; 36)   a union of 20 485 and 411 (0.05; 1.7)
+constexpr u32 GA_EXIT_SHARE = 4;          // no automaton if more than one in so many nodes has an exit
+constexpr u32 GA_EXITS = 1024;            // (and more than so many nodes: a small trie is walked in no time)
+constexpr u32 GA_STARTS = 2;              // nor if there are more starts than so many a node
+constexpr u64 GA_STARTS_FREE = 64u << 10; // and so many
+
 struct VecHash {
   size_t operator()(const std::vector<u64>& v) const {
     u64 h = 0x9E3779B97F4A7C15ull;
@@ -85,7 +96,7 @@ class Builder {
   std::vector<u64> cur_;
   std::vector<u32> arena_;
   std::vector<std::vector<u32>> follow_;      // per non-terminal: codes of the items that completing it can yield
-  u64 walked_ = 0;
+  u64 walked_ = 0, starts_ = 0, exit_nodes_ = 0;
   bool too_big_ = false;
 
   const u32* node(u32 n) const { return &h_.ga_node[(size_t)n * 4]; }
@@ -321,6 +332,7 @@ class Builder {
     for (u32 c = first; c < end && !too_big_; ++c) {
       const size_t base = arena_.size();
       const u32 e = node(c)[1] & 0xFFu, kids = node(c)[1] >> 8;
+      bool asks = false;
       for (size_t i = lo; i < hi; ++i) {
         const u32 code = arena_[i], r = next(code, e);
         if (r == GA_DEAD || kids == 0) continue;
@@ -328,8 +340,13 @@ class Builder {
         if (r & GA_EXIT) {
           const auto& f = follow_[lhs_of(code)];
           arena_.insert(arena_.end(), f.begin(), f.end());
+          asks = true, starts_ += f.size();
         }
       }
+      if (asks) ++exit_nodes_;
+      const u64 nodes = h_.ga_node.size() / 4;
+      if (exit_nodes_ > GA_EXITS && exit_nodes_ * GA_EXIT_SHARE > nodes) too_big_ = true;
+      if (starts_ > GA_STARTS * nodes + GA_STARTS_FREE) too_big_ = true;
       if (walked_ > GA_MAX_WALK) too_big_ = true;
       dedupe(arena_, base);
       if (arena_.size() > base) walk(c, base, arena_.size());

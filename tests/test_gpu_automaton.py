@@ -96,13 +96,16 @@ def _union(variants):
     return text + 'str ::= "\\"" [^"\\\\]* "\\""\nval ::= str | "[" val "]"\n'
 
 
-@pytest.mark.parametrize("variants", [59, 60, 61, 100, 200])
+@pytest.mark.parametrize("variants", [59, 60, 61, 100, 180])
 @pytest.mark.parametrize("batch", [1, 4, 75, 300])
 def test_more_wide_items_than_there_is_room_for(variants, batch):
     """Up to 60 items of a row's last set are answered by the masks made for them; the others are walked like any item."""
-    w = workloads.build(2, V=32000, batch=1, steps=1)
+    rng = np.random.default_rng(variants)
+    some = np.frombuffer(b"0123456789kid[]{}:,", np.uint8)
+    vocab = workloads.build(2, V=32000, batch=1, steps=1).vocab[:-1] + sorted({bytes(some[rng.integers(0, 19, 6)]) for _ in range(70000)}) + [b""]
     prefixes = [list(p) for p in (b'{"id":', b'{"id":"x', b'{"id":"x","k1', b'{"id":"y","k%d":[[' % (variants - 1))]
-    _run(_union(variants), "s", w.vocab, prefixes, batch=batch, check=range(min(batch, 4)))
+    s = _run(_union(variants), "s", vocab, prefixes, batch=batch, check=range(min(batch, 4)))
+    assert batch == 1 or s["walk_transitions"] > 1000 * batch  # (look-ups: the rows were not swept)
 
 
 @pytest.mark.parametrize("n", [511, 512, 513, 600, 1000])
@@ -146,8 +149,8 @@ def test_rounds_that_push_more_than_the_stack_holds(batch):
 
 
 def _endings(n):
-    """Brackets of n kinds, told apart after they close: every level of the text is completed to n kinds, n contexts a level.  Half of
-    the vocabulary are words that are no text."""
+    """Brackets of n kinds, told apart after they close: every level of the text is completed to n kinds, n contexts a level.  Nearly
+    all of the vocabulary are words that are no text (where the chart is asked at most of the trie, grammars have no automaton)."""
     kinds = [chr(97 + i) if i < 20 else "z%c%c" % (97 + i // 26, 97 + i % 26) for i in range(n)]
     text = "s ::= t\nt ::= \"x\" | " + " | ".join("t%d" % i for i in range(n)) + "\n"
     text += "".join('t%d ::= "(" t ")" "%s"\n' % (i, k) for i, k in enumerate(kinds))
@@ -155,7 +158,7 @@ def _endings(n):
     chains = [b"".join(b")" + kinds[int(i)].encode() for i in rng.integers(0, n if k % 2 else 20, 16))[:32] for k in range(60)]
     vocab = [bytes([b]) for b in range(256)] + [b"x" + c[:3 * k + 1] for k, c in enumerate(chains[:10])] + chains + [b")(", b"(("]
     letters = np.frombuffer(b"abcdefghijklmnopqrstuvwxyz", np.uint8)
-    return text, vocab + sorted({bytes(letters[rng.integers(0, 26, 6)]) for _ in range(40000)}) + [b""]
+    return text, vocab + sorted({bytes(letters[rng.integers(0, 26, 6)]) for _ in range(100000)}) + [b""]
 
 
 @pytest.mark.parametrize("n, batch", [(20, 3), (100, 3), (340, 1), (340, 9), (340, 80)])
@@ -166,6 +169,19 @@ def test_rows_that_outgrow_the_storage_of_contexts(n, batch):
     prefixes = [list(p) for p in (b"(" * 20, b"(" * 20 + b"x", b"(" * 20 + b"x)a", b"((x)a")]
     s = _run(text, "s", vocab, prefixes, batch=batch, check=range(min(batch, 4)))
     assert s["rows_swept_again"] <= batch and (n == 20 or s["rows_swept_again"] > 0)
+
+
+@pytest.mark.parametrize("text, start, prefixes", [
+    ('content ::= node*\nnode ::= char | entity | "<p>" content "</p>" | "<b>" content "</b>"\nchar ::= [^<&]\nentity ::= "&" [a-z]+ ";"\n', "content",
+     [b"<p>some <b>bold", b"text &am", b"", b"<p><b>x</"]),
+    ('doc ::= el\nel ::= "<" name ">" (el | text)* "</" name ">"\ntext ::= [^<&]+\nname ::= [a-zA-Z] [a-zA-Z0-9-]*\n', "doc",
+     [b"<a><b>some words of text", b"<a", b"<a><b>x</b>yz", b"<a>x</"])])
+@pytest.mark.parametrize("batch", [1, 64, 300])
+def test_text_whose_rules_end_everywhere(text, start, prefixes, batch):
+    """Grammars whose chart is asked at most nodes of the trie have no automaton: their rows are swept, a few steps each."""
+    w = workloads.build(2, V=20000, batch=1, steps=1)
+    s = _run(text, start, w.vocab, [list(p) for p in prefixes], batch=batch, check=range(min(batch, 4)))
+    assert s["walk_transitions"] < 2000 * batch and s["rows_swept_again"] == 0
 
 
 def test_grammar_without_an_automaton():
