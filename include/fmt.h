@@ -177,9 +177,10 @@ typedef struct {
  * no string), CAPACITY (more than 65535 dotted rules, more than 4096 non-terminals, or a token
  * longer than 32 bytes), OOM, CUDA.
  * Along with the tables goes the grammar's automaton over the vocabulary: what a token's bytes do to one unfinished
- * Earley item, whatever the chart holds, worked out on the host (0.03 to 0.15 s for a 128 K vocabulary in the
+ * Earley item, whatever the chart holds, worked out on the host (0.04 to 0.25 s for a 128 K vocabulary in the
  * measured workloads) and used by every fill.  A grammar for which it grows too large (sets of more than 1024 items,
- * 2^18 sets, about half a second of work) goes without; its rows are then swept by Earley steps.
+ * 2^18 sets, half a second of work), or whose rules end inside tokens so often that its fills would be slower
+ * with it (text character by character, unions of dozens of variants), goes without; its rows are then swept by Earley steps.
  * The grammar is immutable and may be shared by any number of states.
  */
 fmt_status fmt_compile(const char* ebnf, size_t ebnf_len, const char* start_rule, const uint8_t* vocab_bytes,

@@ -27,7 +27,10 @@ using u64 = uint64_t;
 // limits; a grammar beyond them has no automaton and its fills run the Earley steps themselves
 constexpr u32 GA_MAX_SETS = 1u << 18;
 constexpr u64 GA_MAX_TRANS = 32u << 20;   // table entries (4 bytes each)
-constexpr u64 GA_MAX_WALK = 60u << 20;    // look-ups of the walk over the trie (about half a second)
+// Look-ups of the walk over the trie, items scanned and every eighth comparison for a new transition; as many again for the wide items.
+// Together half a second at most (10 to 15 ns each: HTML with 90 tags, 44 million 0.69 s; JSON, SQL and JSON schemas over 128 K tokens have
+// 0.5 to 4 million, 0.04 to 0.2 s).
+constexpr u64 GA_MAX_WORK = 16u << 20;
 constexpr size_t GA_MAX_WIDE = 32u << 20;  // words of the masks and lists of wide items
 constexpr size_t GA_WIDE_NODES = 1024;    // an item is wide from so many trie nodes on
 constexpr size_t GA_MAX_ITEMS = 1024;     // items of one set, predicted ones included: alternations of thousands of literals
@@ -96,7 +99,7 @@ class Builder {
   std::vector<u64> cur_;
   std::vector<u32> arena_;
   std::vector<std::vector<u32>> follow_;      // per non-terminal: codes of the items that completing it can yield
-  u64 walked_ = 0, starts_ = 0, exit_nodes_ = 0;
+  u64 work_ = 0, starts_ = 0, exit_nodes_ = 0;
   bool too_big_ = false;
 
   const u32* node(u32 n) const { return &h_.ga_node[(size_t)n * 4]; }
@@ -151,10 +154,12 @@ class Builder {
         for (u32 k = h_.direct_off[z]; k < h_.direct_off[z + 1]; ++k) put((u64)(s + 1) << 32 | h_.direct_items[k]);
       }
     std::sort(set.wait.begin(), set.wait.end());
+    work_ += set.scan.size() + set.wait.size();
     if (set.scan.size() + set.wait.size() > GA_MAX_ITEMS) too_big_ = true;
   }
 
   void add(u64 it) {
+    work_ += cur_.size() / 8u;
     for (u32 j = 0; j <= h_.skip[(u32)it]; ++j)
       if (std::find(cur_.begin(), cur_.end(), it + j) == cur_.end()) cur_.push_back(it + j);
   }
@@ -185,7 +190,7 @@ class Builder {
   }
 
   u32 next(u32 code, u32 e) {
-    ++walked_;
+    ++work_;
     if (code & GA_ITEM) {
       const u32 org = (code >> 14) & 0xFFFFu, g = code & 0x3FFFu;
       const u32 t = h_.dfa_trans[(size_t)g * n_eq_ + e];
@@ -206,6 +211,7 @@ class Builder {
     if (trans_[slot] != GA_UNKNOWN) return trans_[slot];
     expand(code);
     cur_.clear();
+    work_ += sets_[code].scan.size();
     const u32 b = rep_[e];
     for (u64 it : sets_[code].scan) {
       const u32 d = (u32)it, a = arg(d);
@@ -333,7 +339,7 @@ class Builder {
       const size_t base = arena_.size();
       const u32 e = node(c)[1] & 0xFFu, kids = node(c)[1] >> 8;
       bool asks = false;
-      for (size_t i = lo; i < hi; ++i) {
+      for (size_t i = lo; i < hi && work_ <= GA_MAX_WORK; ++i) {
         const u32 code = arena_[i], r = next(code, e);
         if (r == GA_DEAD || kids == 0) continue;
         if ((r & ~GA_EXIT) != GA_NONE) arena_.push_back(r & ~GA_EXIT);
@@ -347,7 +353,7 @@ class Builder {
       const u64 nodes = h_.ga_node.size() / 4;
       if (exit_nodes_ > GA_EXITS && exit_nodes_ * GA_EXIT_SHARE > nodes) too_big_ = true;
       if (starts_ > GA_STARTS * nodes + GA_STARTS_FREE) too_big_ = true;
-      if (walked_ > GA_MAX_WALK) too_big_ = true;
+      if (work_ > GA_MAX_WORK) too_big_ = true;
       dedupe(arena_, base);
       if (arena_.size() > base) walk(c, base, arena_.size());
       arena_.resize(base);
@@ -359,7 +365,7 @@ class Builder {
   void wide_roots() {
     h_.ga_wide.assign(h_.D, GA_DEAD);
     h_.ga_wide_rec.clear(), h_.ga_wide_mask.clear(), h_.ga_wide_exit.clear();
-    walked_ = 0;
+    work_ = 0;
     std::unordered_map<u32, u32> known;  // items with one code share an entry
     std::vector<u32> alive, mask(h_.Wm);
     std::vector<std::pair<u32, u32>> work;  // (node, code)
@@ -371,7 +377,7 @@ class Builder {
         h_.ga_wide[d] = it->second;
         continue;
       }
-      if (walked_ > GA_MAX_WALK || h_.ga_wide_mask.size() + h_.ga_wide_exit.size() > GA_MAX_WIDE) break;
+      if (work_ > GA_MAX_WORK || h_.ga_wide_mask.size() + h_.ga_wide_exit.size() > GA_MAX_WIDE) break;
       alive.clear(), exits.clear();
       work.assign(1, {0u, h_.ga_root[d]});
       while (!work.empty()) {

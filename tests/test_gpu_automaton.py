@@ -184,6 +184,24 @@ def test_text_whose_rules_end_everywhere(text, start, prefixes, batch):
     assert s["walk_transitions"] < 2000 * batch and s["rows_swept_again"] == 0
 
 
+def test_compiling_takes_a_bounded_time():
+    """The automaton's tables take half a second at most, whether the grammar gets them or not (300 kinds of elements around text)."""
+    import time
+
+    import paper_2506_01151_b200 as fmt
+
+    w = workloads.build(2, V=128256, batch=1, steps=1)
+    tags = _words(np.random.default_rng(1), 300, 4)
+    text = "content ::= node*\nnode ::= char | entity | " + " | ".join('"<%s>" content "</%s>"' % (x, x) for x in tags)
+    text += '\nchar ::= [^<&]\nentity ::= "&" [a-z]+ ";"\n'
+    took = []
+    for host_only in (True, True, False):  # (the first call builds or loads the library)
+        t = time.process_time()
+        fmt.Grammar(text, "content", w.vocab, w.eos, host_only=host_only)
+        took.append(time.process_time() - t)
+    assert took[2] - took[1] < 0.7, took  # (half a second, and the upload)
+
+
 def test_grammar_without_an_automaton():
     """Alternations of more than a thousand literals have none: their rows are swept by Earley steps."""
     names = sorted({"k%06d" % (i * 7919 % 999983) for i in range(1200)})
