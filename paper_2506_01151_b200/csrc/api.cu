@@ -204,7 +204,7 @@ fmt_status fmt_compile(const char* ebnf, size_t ebnf_len, const char* start_rule
     cudaError_t e = cudaGetDevice(&g->device);
 #define UP(field) if (e == cudaSuccess) e = g->bufs.upload(h.field, &d.field)
     d.n_eq = h.n_eq;
-    {  // info | lhs | class_bits | eq_of_byte | nt_closure | nt_up | direct_off | direct_items, each 16-byte aligned
+    {  // info | lhs | class_bits | eq_of_byte | nt_closure | direct_off | direct_items, each 16-byte aligned
       std::vector<uint32_t> blob;
       auto put = [&](const void* src, size_t bytes) {
         size_t at = blob.size();
@@ -214,7 +214,6 @@ fmt_status fmt_compile(const char* ebnf, size_t ebnf_len, const char* start_rule
       };
       const size_t o_info = put(h.info.data(), h.info.size() * 4);
       const size_t o_lhs = put(h.lhs.data(), h.lhs.size() * 2);
-      const size_t o_up = put(h.nt_up.data(), h.nt_up.size() * 4);
       const size_t o_cls = put(h.class_bits.data(), h.class_bits.size() * 4);
       const size_t o_eq = put(h.eq_of_byte.data(), 256);
       const size_t o_clo = put(h.nt_closure.data(), h.nt_closure.size() * 4);
@@ -224,7 +223,6 @@ fmt_status fmt_compile(const char* ebnf, size_t ebnf_len, const char* start_rule
       d.hot_words = (uint32_t)blob.size();
       d.info = d.hot_block + o_info;
       d.lhs = reinterpret_cast<const uint16_t*>(d.hot_block + o_lhs);
-      d.nt_up = d.hot_block + o_up;
       d.class_bits = d.hot_block + o_cls;
       d.eq_of_byte = reinterpret_cast<const uint8_t*>(d.hot_block + o_eq);
       d.nt_closure = d.hot_block + o_clo;

@@ -397,8 +397,8 @@ __device__ __forceinline__ int token_steps(const GrammarDev& G, AdvScratch& s, c
   for (uint32_t i = lane; i < (n_bits + 31) / 32; i += 32) s.live[i] = 0u;
   __syncwarp();
   // ---- the needs, "somebody may complete a non-terminal begun in this set".  An item begun in a set lies in that set or
-  // in a later one, so one pass over the sets from the last to the first finds them all: per set a bit for every non-terminal;
-  // with a non-terminal come at once those whose prediction pulls it in (nt_up), which settles the items begun in the set itself.  One
+  // in a later one, so one pass over the sets from the last to the first finds them all: per set a bit for every non-terminal.
+  // An item whose non-terminal pulls an asked one in by prediction is waited for, too, which settles the items begun in the set itself.  One
   // pass over a set's items per set: with a list of (set, non-terminal) pairs served one after the other Compact
   // took 31,000 cycles for a JSON chart of 12 sets and 280,000 for an ambiguous one of 60, now 8,500 and 90,000.
   const uint32_t M = last;  // earlier sets: 0..last-1
@@ -435,10 +435,7 @@ __device__ __forceinline__ int token_steps(const GrammarDev& G, AdvScratch& s, c
     uint32_t first_asked = 0xFFFFFFFFu;  // (each lane: the earliest set it has asked)
     auto ask = [&](uint32_t o, uint32_t A) {
       first_asked = min(first_asked, o);
-      for (uint32_t w = 0; w < Nw; ++w) {
-        const uint32_t bits = G.nt_up[A * Nw + w];
-        if (bits) atomicOr(&need[o * Nw + w], bits);
-      }
+      atomicOr(&need[o * Nw + (A >> 5)], 1u << (A & 31u));
     };
     for (uint32_t i = lane; i < n_last; i += 32) {
       const uint32_t it = arena[last_at + i];
@@ -466,7 +463,9 @@ __device__ __forceinline__ int token_steps(const GrammarDev& G, AdvScratch& s, c
       for (uint32_t base = 0; base < sl; base += 32) {
         const uint32_t it = base + lane < sl ? sp[base + lane] : 0u;
         const uint32_t inf = G.info[it & 0xFFFFu], A = inf & INFO_ARG_MASK;
-        const bool keep = base + lane < sl && (inf >> INFO_KIND_SHIFT) == KIND_NT && ((need[o * Nw + (A >> 5)] >> (A & 31u)) & 1u);
+        bool keep = false;
+        if (base + lane < sl && (inf >> INFO_KIND_SHIFT) == KIND_NT)
+          for (uint32_t w = 0; w < Nw; ++w) keep = keep || (need[o * Nw + w] & G.nt_closure[A * Nw + w]);
         const uint32_t kb = __ballot_sync(FULL, keep);
         if (kb == 0u) continue;
         live += __popc(kb);

@@ -15,7 +15,6 @@ struct GrammarDev {
   const uint8_t* eq_of_byte;     // [256] equivalence class of each byte (same membership in all byte classes)
   uint32_t n_eq;
   const uint32_t* nt_closure;    // [N][Nw]
-  const uint32_t* nt_up;         // [N][Nw] its transpose
   const uint32_t* direct_off;    // [N+1]
   const uint16_t* direct_items;
   // regular non-terminals run as automata: item id dfa_first + g is automaton state g
@@ -28,7 +27,7 @@ struct GrammarDev {
   const uint8_t* node_byte;      // [T]
   const uint32_t* parent;        // [T]
   const uint8_t* node_depth;     // [T]
-  // The tables above that every Earley step reads (info, lhs, class_bits, eq_of_byte, nt_closure, nt_up,
+  // The tables above that every Earley step reads (info, lhs, class_bits, eq_of_byte, nt_closure,
   // direct_off, direct_items) sit in one contiguous block so that a kernel can copy them into
   // shared memory at once and shift the pointers.
   const uint32_t* hot_block;

@@ -405,7 +405,6 @@ __device__ __forceinline__ GrammarDev with_hot_tables(const GrammarDev& Gg, cons
   G.class_bits = dst + (Gg.class_bits - Gg.hot_block);
   G.eq_of_byte = reinterpret_cast<const uint8_t*>(dst + (reinterpret_cast<const uint32_t*>(Gg.eq_of_byte) - Gg.hot_block));
   G.lhs = reinterpret_cast<const uint16_t*>(dst + (reinterpret_cast<const uint32_t*>(Gg.lhs) - Gg.hot_block));
-  G.nt_up = dst + (Gg.nt_up - Gg.hot_block);
   G.nt_closure = dst + (Gg.nt_closure - Gg.hot_block);
   G.direct_off = dst + (Gg.direct_off - Gg.hot_block);
   G.direct_items = reinterpret_cast<const uint16_t*>(dst + (reinterpret_cast<const uint32_t*>(Gg.direct_items) - Gg.hot_block));

@@ -900,10 +900,6 @@ void compile_grammar(const char* text, size_t len, const std::string& start, Hos
       }
     }
   }
-  out.nt_up.assign((size_t)N * out.Nw, 0);
-  for (int y = 0; y < N; ++y)
-    for (int z = 0; z < N; ++z)
-      if ((out.nt_closure[(size_t)y * out.Nw + (z >> 5)] >> (z & 31)) & 1u) out.nt_up[(size_t)z * out.Nw + (y >> 5)] |= 1u << (y & 31);
 }
 
 // ------------------------------------------------------------------------------------ trie

@@ -53,7 +53,6 @@ struct HostTables {
   std::vector<uint8_t> skip;           // [D] how many nullable non-terminals follow the dot in a row
   std::vector<uint32_t> class_bits;    // [C][8] 256-bit byte classes
   std::vector<uint32_t> nt_closure;    // [N][Nw] non-terminals predicted (transitively) with Y
-  std::vector<uint32_t> nt_up;         // [N][Nw] the same seen from below: non-terminals whose prediction pulls Y in
   std::vector<uint32_t> direct_off;    // [N+1]
   std::vector<uint16_t> direct_items;  // start items of each non-terminal's rules, dots moved over
                                        // leading nullable symbols, completed items left out

@@ -27,7 +27,7 @@ __device__ __forceinline__ void stat_add64(const StateDev& S, uint32_t slot, uns
 __device__ __forceinline__ void diag(const StateDev& S, uint32_t what) { atomicAdd(S.counters + CNT_DIAG + what, 1u); }
 __device__ __forceinline__ void stat_max(const StateDev& S, uint32_t slot, uint32_t v) { atomicMax(S.counters + slot, v); }
 
-constexpr uint32_t HOT_TABLE_BYTES = 32 * 1024;  // grammar tables up to this size are staged in shared memory
+constexpr uint32_t HOT_TABLE_BYTES = 36 * 1024;  // grammar tables up to this size are staged in shared memory (four rows of an advance leave as much)
 
 constexpr uint32_t SWEEP_CUR = 512;     // items of a set under construction per warp (fast mode, power of two)
 constexpr uint32_t SWEEP_HSET = 1024;   // uniqueness hash slots per warp (fast mode)

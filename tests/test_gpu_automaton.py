@@ -288,6 +288,21 @@ def test_sets_with_a_bit_for_every_item(letters):
     assert int(a[0]) == s.num_sets and int(a[1]) == s.total_items
 
 
+@pytest.mark.parametrize("n", [31, 32, 33, 64, 130, 300])
+def test_compact_with_many_non_terminals(n):
+    """What Compact keeps, with the non-terminals in one and in several words: chains of prediction and left recursion among them."""
+    text = "s ::= n0 | s \",\" n1\n"
+    text += "".join('n%d ::= n%d | "(" n%d ")" "%c" | n%d "+" "x"\n' % (i, i + 1, i * 7 % (n - 2), 97 + i % 26, i) for i in range(n - 2))
+    text += 'n%d ::= "x" | "[" s "]"' % (n - 2)
+    data = b"x,((x+x"
+    for dfa in (True, False):
+        a, b, _ = _feed(text, "s", data, {}, dfa)
+        assert a.tolist() == b.tolist()
+        seq = oracle.Sequence_(oracle.Grammar(text, "s"), pruned=True)
+        assert seq.advance(data)
+        assert int(a[0]) == seq.num_sets and int(a[1]) == seq.total_items
+
+
 @pytest.mark.parametrize("dtype", ["bf16", "fp32"])
 @pytest.mark.parametrize("V", [1, 7, 8, 15, 16, 17, 31, 33, 63, 64, 65, 4095, 4097, 16 * 512 + 3])
 def test_masking_rows_that_begin_anywhere(dtype, V):
