@@ -243,7 +243,7 @@ def stat_delta(a, b, keys):
 
 STAT_KEYS = ["fills", "fills_computed", "fills_from_cache", "fills_shared", "rows_mask_only", "rows_from_root", "rows_plain",
              "root_sweeps", "sweep_transitions", "sweep_states", "walk_transitions", "walk_states", "walk_frames",
-             "big_mode_units", "steps_advanced", "advances_cached", "earley_step_cycles", "capacity_errors", "fills_aborted"]
+             "big_mode_units", "rows_swept_again", "steps_advanced", "advances_cached", "earley_step_cycles", "capacity_errors", "fills_aborted"]
 
 
 def read_traffic(config: int, kernel: str):
@@ -344,8 +344,10 @@ def run_ours(args):
     sweep_bytes = trie_bytes + (sweep_jobs / max(1, K)) * (4 * Wm + 2048)  # + per job: its mask row and its chart
     apply_rw = B * (4 * Wm + 2 * 2 * V)   # mask words read, logits read and written
     apply_wo = B * (4 * Wm + 2 * V)       # if the logits only had to be written
+    # (the automaton's fill looks tables up and takes no Earley steps but for rows it gives up)
+    by_tables = not drv.roots and st_cyc["walk_transitions"] > 0 and st_cyc["earley_step_cycles"] < st_cyc["walk_transitions"]
     kinds = {
-        ("fill_kernel" if drv.roots else "automaton_fill_kernel"): (prof["sweep_ms"], prof["sweep_launches"], sweep_bytes),
+        ("fill_kernel" if drv.roots else "automaton_fill_kernel" if by_tables else "sweep_kernel"): (prof["sweep_ms"], prof["sweep_launches"], sweep_bytes),
         "sweep_kernel (new entries)": (prof["roots_ms"], prof["roots_launches"], trie_bytes),
         "gather_apply_kernel": (prof["apply_ms"], prof["apply_launches"], apply_rw),
         "advance_kernel": (prof["advance_ms"], prof["advance_launches"], B * 2 * 4 * 256),
@@ -371,6 +373,11 @@ def run_ours(args):
                 "spent inside Earley steps / (resident warps x SM clock) = the sweeps' time if no warp ever waited for a "
                 "trie level, a queue or a barrier; frac = that time / the sweeps' time in the same run",
     }
+    if by_tables:
+        second = {"bound": "latency (rounds of look-ups)", "lookups_per_step": steps_earley / K,
+                  "lookups_per_computed_row": steps_earley / max(1, st_cyc["fills_computed"]), "sweeps_ms_per_step": sweeps_ms / K,
+                  "rows_swept_again": st["rows_swept_again"],
+                  "what": "the fill by the grammar's automaton: table look-ups, and the rows that were given up and swept by Earley steps"}
     floor_rw = (apply_rw + trie_bytes) / (peak * 1e9) * 1e3
     floor_wo = (apply_wo + trie_bytes) / (peak * 1e9) * 1e3
     ms_step = t_ms / K
@@ -411,7 +418,8 @@ def run_ours(args):
                   "computed_by": {"context_independent_row_only": st["rows_mask_only"], "sweep_in_frames": st["rows_from_root"],
                                   "sweep_from_chart": st["rows_plain"]},
                   "new_entries_swept": st["root_sweeps"], "entries": stats_end["roots"],
-                  "earley_steps": {"rows": st["walk_transitions"], "new_entries": st["sweep_transitions"]},
+                  ("lookups" if by_tables else "earley_steps"): {"rows": st["walk_transitions"], "new_entries": st["sweep_transitions"]},
+                  "rows_swept_again": st["rows_swept_again"],
                   "states_cached": stats_end["states_cached"], "chart_items_max": stats_end["chart_items_max"],
                   "chart_sets_max": stats_end["chart_sets_max"], "capacity_errors": stats_end["capacity_errors"],
                   "fills_aborted": stats_end["fills_aborted"], "big_mode": st["big_mode_units"],
@@ -438,7 +446,7 @@ def measure_passes(drv: "Driver", W: int, K: int, n_passes: int, first):
     finds what passes 1..p-1 left."""
     out = [{"pass": 1, "ms_per_step": first["t_ms"] / K, "hit_rate": 1.0 - first["stats"]["fills_computed"] / max(1, first["stats"]["fills"]),
             "computed": first["stats"]["fills_computed"], "new_entries_swept": first["stats"]["root_sweeps"],
-            "earley_steps": first["stats"]["walk_transitions"] + first["stats"]["sweep_transitions"],
+            "transitions": first["stats"]["walk_transitions"] + first["stats"]["sweep_transitions"],
             "p50_ms": percentile(first["per_step"], 0.5), "p99_ms": percentile(first["per_step"], 0.99)}]
     # the last repeat has left the caches as one pass leaves them
     for p in range(2, n_passes + 1):
@@ -448,7 +456,7 @@ def measure_passes(drv: "Driver", W: int, K: int, n_passes: int, first):
         d = stat_delta(s0, drv.state.stats(), STAT_KEYS)
         out.append({"pass": p, "ms_per_step": total_ms / K, "hit_rate": 1.0 - d["fills_computed"] / max(1, d["fills"]),
                     "computed": d["fills_computed"], "new_entries_swept": d["root_sweeps"],
-                    "earley_steps": d["walk_transitions"] + d["sweep_transitions"],
+                    "transitions": d["walk_transitions"] + d["sweep_transitions"],
                     "p50_ms": percentile(per_step, 0.5), "p99_ms": percentile(per_step, 0.99)})
     return out
 
@@ -492,7 +500,7 @@ def measure_cold(drv: "Driver", w, start: int, n: int, clear_ci: bool):
     d = stat_delta(s0, drv.state.stats(), STAT_KEYS)
     return {"fills": n, "ms_per_fill": statistics.median(times), "min": min(times), "max": max(times),
             "rows_computed_per_fill": d["fills_computed"] / n,
-            "earley_steps_per_computed_row": (d["walk_transitions"] + d["sweep_transitions"]) / max(1, d["fills_computed"]),
+            "transitions_per_computed_row": (d["walk_transitions"] + d["sweep_transitions"]) / max(1, d["fills_computed"]),
             "token_checks_per_s": w.batch * w.V / (statistics.median(times) * 1e-3),
             "what": "fmt_fill_mask with the state cache emptied before each call%s: every distinct row state is computed"
                     % (" and the context-independent entries too" if clear_ci else ", context-independent entries kept")}

@@ -9,15 +9,19 @@
 //
 // What bounds it: at the sizes measured, latency - rounds of "take threads, look their children up, push what is alive", each
 // two or three dependent reads in L2 and four block barriers, about as many rounds as the longest token has bytes.  Hence
-// the threads, the contexts and the chart sit in shared memory (with a way out to global memory), and four blocks
-// share an SM.  Rows differ by a factor of a hundred in work (measured: 800 to 290,000 look-ups), so blocks that have no row left wait
+// the threads, the contexts and the chart sit in shared memory (with a way out to global memory), and three blocks
+// share an SM (58 KB each).  The grid has four for each all the same: a row's blocks are a power of two, and with three 128 rows of SQL
+// got two blocks each in the place of four.  Rows differ by a factor of a hundred in work (measured: 800 to 290,000 look-ups), so blocks that have no row left wait
 // for work, and a block with many threads hands parts of them out, with its contexts.
 // Measured on a B200, the fill alone, against the sweep of the whole grid by Earley steps (kernels.cu) before:
 //   8 rows of JSON, 32,000 tokens               239 -> 94 us    (where about half of the rows are computed)
 //   64 rows of a JSON schema, 128,256 tokens    263 -> 77 us
 //   128 rows of SQL, 152,064 tokens             667 -> 231 us
-//   37 rows of JSON, 50,001 tokens              362 -> 129 us
-//   256 rows of ambiguous JSON, 128,256 tokens  3.51 -> 1.06 ms (2.65 ms when no work is handed on)
+//   37 rows of JSON, 50,001 tokens              362 -> 138 us
+//   256 rows of ambiguous JSON, 128,256 tokens  3.51 -> 1.04 ms (2.65 ms when no work is handed on)
+// Blocks of an SM, us for those 37 rows of JSON, those 256 ambiguous rows and 12 decoding steps of the SQL rows: three resident of four
+// asked for 150, 1,076 and 5,437; four resident, with half the specials 176, 1,372 and 6,055; three of three asked for 153, 1,223 and 7,454;
+// three of four with 80 registers a thread 153, 1,107 and 5,340.
 // The sweep stays for grammars without an automaton and for the cache of context-independent entries.  A row that outgrows the
 // contexts' storage, or takes far longer than rows do, is swept by Earley steps within the call (block_sweep.cuh).
 #include <cuda_runtime.h>

@@ -722,7 +722,8 @@ void compile_grammar(const char* text, size_t len, const std::string& start, Hos
           // too large: it stays a set of rules, and the regular non-terminals in those are tried one by one.  (A JSON schema is
           // often regular as a whole, but with too many states; its strings, numbers and members are small.  The schema of the
           // timed cases went from no automaton to seven with 764 states: an advance of 64 rows 57 -> 40 us, a sweep of their masks
-          // by Earley steps 374 -> 263 us.)
+          // by Earley steps 374 -> 263 us.  With parts of at most 128 states instead of 512 that schema's 64 rows decode 16 steps in 2.99 ms
+          // instead of 2.43, with 2,048 in 2.42.)
           for (auto& p : rules)
             if (p.lhs == (int)x)
               for (int s : p.rhs)

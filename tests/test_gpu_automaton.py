@@ -51,9 +51,9 @@ def test_rows_of_every_share_of_the_grid(batch):
 
 
 @pytest.mark.parametrize("size", [258, 6144 * 32, 6144 * 32 + 1])
-def test_masks_in_and_out_of_shared_memory(size):
-    """Rows of more than 6144 mask words are collected in global memory.  Thousands of tokens end at one node of the trie over
-    byte classes (words no terminal tells apart), duplicates among them."""
+def test_many_tokens_at_a_node(size):
+    """Thousands of tokens end at one node of the trie over byte classes (words no terminal tells apart), duplicates among them, in
+    vocabularies up to 196,609 tokens."""
     rng = np.random.default_rng(3)
     letters = b"ghijkmopqvwxyzGHIJ"
     vocab = [bytes([b]) for b in range(256)]
