@@ -17,9 +17,9 @@
 //   8 rows of JSON, 32,000 tokens               239 -> 94 us    (where about half of the rows are computed)
 //   64 rows of a JSON schema, 128,256 tokens    263 -> 77 us
 //   128 rows of SQL, 152,064 tokens             667 -> 231 us
-//   37 rows of JSON, 50,001 tokens              362 -> 138 us
-//   256 rows of ambiguous JSON, 128,256 tokens  3.51 -> 1.04 ms (2.65 ms when no work is handed on)
-// Blocks of an SM, us for those 37 rows of JSON, those 256 ambiguous rows and 12 decoding steps of the SQL rows: three resident of four
+//   37 rows of JSON, 50,001 tokens              362 -> 126 us
+//   256 rows of ambiguous JSON, 128,256 tokens  3.51 -> 0.93 ms (2.65 ms when no work is handed on)
+// Blocks of an SM, us (timed call by call) for those 37 rows of JSON, those 256 ambiguous rows and 12 decoding steps of the SQL rows: three resident of four
 // asked for 150, 1,076 and 5,437; four resident, with half the specials 176, 1,372 and 6,055; three of three asked for 153, 1,223 and 7,454;
 // three of four with 80 registers a thread 153, 1,107 and 5,340.
 // The sweep stays for grammars without an automaton and for the cache of context-independent entries.  A row that outgrows the
