@@ -1,29 +1,17 @@
-// The fill of rows' masks by the grammar automaton (grammar_automaton.cpp; Sections 3.3, 4.1, 4.3 of the paper).
+// The fill of rows' masks by what the grammar automaton tabulates (grammar_automaton.cpp; Sections 3.3, 4.1, 4.3 of the paper).
 //
-// A thread block takes a row.  The kernel items of the chart's last set are grouped by dotted rule; every group starts a
-// THREAD at the root of the vocabulary trie: a code of the automaton and a CONTEXT, the set of origins its items were begun in.  A
-// trie node's children are reached by one table look-up each.  Where the automaton says that a rule begun in the chart ends, the
-// thread's context is EXPANDED: the items that waited in its origins, completed upwards (Section 3.2's Complete), start
-// threads of their own at that node.  A context is expanded once per row.  A token is valid iff some thread is alive at the
-// node where its bytes end; its bit is set in the row's mask in global memory at once.
+// A thread block takes a row.  The kernel items of the chart's last set are grouped by dotted rule; each group has a CONTEXT, the set
+// of origins its items were begun in, and the record of what follows from the item (its start): the tokens that are valid whatever
+// the chart holds, and edges for the places inside tokens where the item's rule ends.  There the chart is asked: the context is
+// EXPANDED, once per row, into the items that waited in its origins, completed upwards (Section 3.2's Complete), grouped
+// in the same way.  An edge whose item is among them sets its own tokens, and its edges go on with that group's context.  A
+// round takes all edges that are known, looks their items up in the contexts' expansions, and lists the edges of those that are found.
 //
-// What bounds it: at the sizes measured, latency - rounds of "take threads, look their children up, push what is alive", each
-// two or three dependent reads in L2 and four block barriers, about as many rounds as the longest token has bytes.  Hence
-// the threads, the contexts and the chart sit in shared memory (with a way out to global memory), and three blocks
-// share an SM (58 KB each).  The grid has four for each all the same: a row's blocks are a power of two, and with three 128 rows of SQL
-// got two blocks each in the place of four.  Rows differ by a factor of a hundred in work (measured: 800 to 290,000 look-ups), so blocks that have no row left wait
-// for work, and a block with many threads hands parts of them out, with its contexts.
-// Measured on a B200, the fill alone, against the sweep of the whole grid by Earley steps (kernels.cu) before:
-//   8 rows of JSON, 32,000 tokens               239 -> 94 us    (where about half of the rows are computed)
-//   64 rows of a JSON schema, 128,256 tokens    263 -> 77 us
-//   128 rows of SQL, 152,064 tokens             667 -> 231 us
-//   37 rows of JSON, 50,001 tokens              362 -> 126 us
-//   256 rows of ambiguous JSON, 128,256 tokens  3.51 -> 0.93 ms (2.65 ms when no work is handed on)
-// Blocks of an SM, us (timed call by call) for those 37 rows of JSON, those 256 ambiguous rows and 12 decoding steps of the SQL rows: three resident of four
-// asked for 150, 1,076 and 5,437; four resident, with half the specials 176, 1,372 and 6,055; three of three asked for 153, 1,223 and 7,454;
-// three of four with 80 registers a thread 153, 1,107 and 5,340.
-// The sweep stays for grammars without an automaton and for the cache of context-independent entries.  A row that outgrows the
-// contexts' storage, or takes far longer than rows do, is swept by Earley steps within the call (block_sweep.cuh).
+// What bounds it: latency - a few rounds (as many as rules end one after the other inside a token), each a read of edges in L2, and
+// between them the expansions, which one warp makes.  Following edges replaced a walk of the trie over byte classes by table look-ups, a
+// byte a round (the same automaton, tabulated less far).  Fills on a B200 before and now, us: 37 rows of JSON, 50,001 tokens 139 -> 65;
+// 256 rows of ambiguous JSON, 128,256 tokens 1,010 -> 795; 24 charts of JSON without allocations 123 -> 72; 12 decoding steps of 128
+// rows of SQL, 152,064 tokens 4,930 -> 2,460, 16 of 64 rows of a JSON schema 2,440 -> 1,690.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -35,23 +23,17 @@
 namespace fmt {
 
 constexpr int AF_WARPS = 8, AF_THREADS = AF_WARPS * 32;
-constexpr uint32_t AF_BATCH = 512;        // threads of a round
-constexpr uint32_t AF_PER = AF_BATCH / AF_THREADS;
-constexpr uint32_t AF_SPEC = AF_THREADS;  // expansions to be made at the start of a round
-constexpr uint32_t AF_EXITS = 60;         // lists of nodes at which expansions are to be made (from wide items)
-constexpr uint32_t AF_TIGHT = 6144;       // free places of a block's stack, its reserve not counted, below which entries are taken one at a time
-constexpr uint32_t AF_LIST_STARTS = 64;   // expansions of more elements are started from a list's nodes by specials
-constexpr uint32_t AF_SEEN = 512;         // recently started threads (a lossy table: repeats only cost time)
+constexpr uint32_t AF_BATCH = 512;        // entries (lists of edges with a context) of a round,
+constexpr uint32_t AF_EDGES = 32768;      // edges of a round,
+constexpr uint32_t AF_CHUNK = 4096;       // and of an entry
+constexpr uint32_t AF_LISTS = 512, AF_TOKENS = 32768;  // lists of tokens that are written when a round's edges are through, and tokens in them
+constexpr uint32_t AF_TIGHT = 2048;       // free places of a block's stack, its reserve not counted, below which entries are taken one at a time,
+constexpr uint32_t AF_TIGHT_EDGES = 32;   // so many edges of them
+constexpr uint32_t AF_SLICE = 1024;       // items of a last set whose starts are taken together
+constexpr uint32_t AF_SEEN = 512;         // recently listed edges (a lossy table: repeats only cost time)
 constexpr uint32_t AF_STAGE = 1024;       // a chart up to this many words is read from shared memory
 constexpr uint32_t AF_CTX = 64, AF_CTX_HASH = 128, AF_POOL = 2048;  // contexts in shared memory, words of their lists
 constexpr uint32_t AF_BUF = 512, AF_WORK = 256, AF_HSET = 512;      // an expansion in shared memory (larger ones: global memory)
-constexpr uint32_t AF_OWNER = AF_BATCH * 8;  // pieces of 32 children a round can hold (a node has at most 256)
-constexpr uint32_t AF_HEAVY = 16384;      // after so many look-ups for a row, or for a unit of work,
-constexpr uint32_t AF_SHARE = 384;        // a block with so many threads gives some to blocks that wait,
-constexpr uint32_t AF_MAX_UNITS = 7;      // to so many at once, 128 threads at the least to each
-// code of a special: to start the threads of a context's expansion at a node (first child, children, AF_SPAWN, elements that have been
-// started << 16 | context)
-constexpr uint32_t AF_SPAWN = 0xFFFFFFFDu;
 constexpr uint32_t AF_KCYCLES = 1u << 14;      // a share of a row that takes longer (2^24 cycles, 8.5 ms) is given up for a sweep by Earley steps
 // AC_FAIL: 0, 1 + the capacity that was exceeded, or
 constexpr uint32_t AF_GIVEN_UP = 0xFFFFFFFFu;  // a wait ran out: the fill is given up, the row itself is fine
@@ -60,23 +42,72 @@ constexpr uint32_t AF_LATE = 0xFFFFFFFDu;      // the share takes too long
 constexpr uint32_t CTX_NEW = 0xFFFFFFFFu;
 
 enum : uint32_t {
-  AC_NEXT = 0, AC_SPEC = 1, AC_OVF = 2, AC_GTOP = 3, AC_FAIL = 4, AC_NCTX = 5, AC_POOL = 6, AC_NWORK = 7, AC_WSUM = 8, AC_NBUF = 16, AC_OVER = 17,
-  AC_SPILLED = 18, AC_WAITING = 19, AC_BASE = 20, AC_JOB = 21, AC_NWIDE = 22, AC_POPPED = 24, AC_NEXITS = 25, AC_LIST = 26,
-  AC_LIST_AT = 27, AC_LIST_END = 28, AC_POPPED_SPEC = 29, AC_BEGAN = 30,
-  AC_PEEK = 32, AC_WIDE = 40, AC_WORDS = (AC_WIDE + AF_EXITS + 3) & ~3u
+  AC_OVF = 0, AC_GTOP = 1, AC_FAIL = 2, AC_NCTX = 3, AC_POOL = 4, AC_NWORK = 5, AC_NBUF = 6, AC_OVER = 7, AC_SPILLED = 8, AC_JOB = 9,
+  AC_NWIDE = 10, AC_LIST = 11, AC_LIST_END = 12, AC_LOOKED = 13, AC_BEGAN = 14, AC_SLOT = 15,
+  AC_EDGES = 16,   // [2] counters of the entries (see Deal)
+  AC_TOKENS = 24,  // [2] and of the lists of tokens
+  AC_PEEK = 32, AC_FULL = 36, AC_WORDS = 40
 };
 static_assert(AC_WORDS % 4 == 0 && AC_WORDS <= AF_THREADS, "what follows in shared memory is cleared in 16-byte pieces; a thread clears a word");
 
-// A unit of work handed out: AU_HDR words, then the giver's contexts, lists and the threads.
-enum : uint32_t { AU_ROWJOB = 0, AU_N = 1, AU_NCTX = 2, AU_POOL = 3, AU_PART = 4, AU_HDR = 8 };
-constexpr uint32_t AU_ENTRIES = AF_BATCH / 2 + 4;
-constexpr uint32_t AU_WORDS = AU_HDR + 5 * AF_CTX + AF_POOL + 4 * AU_ENTRIES;
-static_assert(AU_WORDS % 4 == 0 && (AU_HDR + 5 * AF_CTX + AF_POOL) % 4 == 0, "the threads of a unit are 16-byte records");
+// Lists whose elements are dealt out to the lanes: places and elements are counted by one atomic operation, so that the places are in
+// the order of the elements.
+struct Deal {
+  uint32_t* count;   // 64 bits: places << 32 | elements; then the first place and the first element that found no room
+  uint2* what;       // [cap] where the list begins, and what it comes with
+  uint32_t* pre;     // [cap] its first element's number
+  uint16_t* owner;   // [things / 32] the place of the list to which the element 32 * i belongs
+  uint32_t cap, things;
+};
+__device__ __forceinline__ uint32_t dealt_lists(const Deal& D) { return min(D.count[1], D.count[2]); }
+__device__ __forceinline__ uint32_t dealt_things(const Deal& D) { return min(D.count[0], D.count[3]); }
+__device__ __forceinline__ void deal_clear(const Deal& D) {
+  D.count[0] = D.count[1] = 0u;
+  D.count[2] = D.count[3] = 0xFFFFFFFFu;
+}
+// By all lanes of a warp: the lists of the lanes with `yes`.  False: there is no room for the lane's.
+__device__ __forceinline__ bool deal(const Deal& D, bool yes, uint32_t n, uint2 what) {
+  const uint32_t lane = lane_id(), b = __ballot_sync(FULL, yes);
+  if (b == 0u) return true;
+  uint32_t incl = yes ? n : 0u;
+#pragma unroll
+  for (int d = 1; d < 32; d <<= 1) {
+    const uint32_t t = __shfl_up_sync(FULL, incl, d);
+    if ((int)lane >= d) incl += t;
+  }
+  unsigned long long base = 0;
+  if (lane == 31u) base = atomicAdd(reinterpret_cast<unsigned long long*>(D.count), (unsigned long long)__popc(b) << 32 | incl);
+  const uint32_t slot = __shfl_sync(FULL, (uint32_t)(base >> 32), 31) + __popc(b & ((1u << lane) - 1u));
+  const uint32_t before = __shfl_sync(FULL, (uint32_t)base, 31) + incl - (yes ? n : 0u);
+  const bool fits = slot < D.cap && before + n <= D.things, longer = n > 128u;
+  if (yes && fits) {
+    D.what[slot] = what;
+    D.pre[slot] = before;
+    if (!longer)
+      for (uint32_t p = (before + 31u) / 32u; p * 32u < before + n; ++p) D.owner[p] = (uint16_t)slot;
+  } else if (yes) {
+    atomicMin(&D.count[2], slot);
+    atomicMin(&D.count[3], before);
+  }
+  for (uint32_t m = __ballot_sync(FULL, yes && fits && longer); m; m &= m - 1u) {
+    const int src = __ffs(m) - 1;
+    const uint32_t from = __shfl_sync(FULL, before, src), until = from + __shfl_sync(FULL, n, src), s = __shfl_sync(FULL, slot, src);
+    for (uint32_t p = (from + 31u) / 32u + lane; p * 32u < until; p += 32u) D.owner[p] = (uint16_t)s;
+  }
+  return fits || !yes;
+}
+// The list to which element base + lane of n lists belongs (base a multiple of 32).
+__device__ __forceinline__ uint32_t whose(const Deal& D, uint32_t n, uint32_t base) {
+  const uint32_t lane = lane_id(), lo = D.owner[base / 32u];
+  const uint32_t nb = lo + 1u + lane < n ? D.pre[lo + 1u + lane] - base : 32u;  // where the lists after it begin
+  const uint32_t starts = __reduce_or_sync(FULL, nb < 32u ? 1u << nb : 0u);
+  return lo + __popc(starts & (0xFFFFFFFFu >> (31u - lane)));
+}
 
 // The contexts of the row a block works on: in shared memory, or, when they outgrow it, in global memory of the block's own.
 struct Contexts {
   uint2* org;       // [cap] origins: offset into pool, count
-  uint2* exp;       // [cap] expansion: offset into pool, count (CTX_NEW: not made yet); pairs (code, rule << 16 | context)
+  uint2* exp;       // [cap] expansion: offset into pool, count (CTX_NEW: not made yet); rule << 16 | context, ascending
   uint32_t* lhs;    // [cap] the non-terminal whose rule is open
   uint32_t* hash;   // [hash_mask + 1] context + 1, 0 = empty
   uint32_t* pool;
@@ -231,10 +262,10 @@ __device__ bool group_items(const GrammarDev& G, const Contexts& C, uint32_t* ct
   const uint32_t lane = lane_id();
   uint32_t groups;
   const uint32_t k = sort_unique(buf, n, groups);
-  const uint32_t at = (ctl[AC_POOL] + 1u) & ~1u;
+  const uint32_t at = ctl[AC_POOL];
   __syncwarp();
-  if (at + 2u * groups > C.pool_cap) return false;
-  if (lane == 0) ctl[AC_POOL] = at + 2u * groups;
+  if (at + groups > C.pool_cap) return false;
+  if (lane == 0) ctl[AC_POOL] = at + groups;
   __syncwarp();
   uint32_t g = 0;
   for (uint32_t i = 0; i < k;) {
@@ -244,19 +275,16 @@ __device__ bool group_items(const GrammarDev& G, const Contexts& C, uint32_t* ct
       const uint32_t other = __ballot_sync(FULL, i + lane >= k || y == x >> 16 || (lane && before == x >> 16));
       const uint32_t run = other ? (uint32_t)__ffs(other) - 1u : 32u;
       if (run) {
-        const uint4 rec = lane < run ? __ldg(reinterpret_cast<const uint4*>(G.ga_item) + (x >> 16)) : make_uint4(GA_DEAD, 0u, 0u, 0u);
-        const bool v = lane < run && rec.x != GA_DEAD;
-        const uint32_t alive = __ballot_sync(FULL, v);
-        const uint32_t c = intern_singles(C, ctl, v, rec.y & 0xFFFFu, x & 0xFFFFu);
+        const bool v = lane < run;
+        const uint32_t c = intern_singles(C, ctl, v, v ? __ldg(&G.ga_item[2u * (x >> 16)]) & 0xFFFFu : 0u, x & 0xFFFFu);
         if (__any_sync(FULL, v && c == CTX_NEW)) return false;
-        if (v) reinterpret_cast<uint2*>(C.pool)[at / 2u + g + __popc(alive & ((1u << lane) - 1u))] = make_uint2(rec.x, (x & 0xFFFF0000u) | c);
-        g += __popc(alive);
+        if (v) C.pool[at + g + lane] = (x & 0xFFFF0000u) | c;
+        g += run;
         i += run;
         continue;
       }
     }
     const uint32_t d = buf[i] >> 16;
-    const uint4 rec = __ldg(reinterpret_cast<const uint4*>(G.ga_item) + d);
     uint32_t e = i + 1u;
     for (;;) {  // the end of the group
       const uint32_t b = __ballot_sync(FULL, e + lane >= k || (buf[min(e + lane, k - 1u)] >> 16) != d);
@@ -266,16 +294,57 @@ __device__ bool group_items(const GrammarDev& G, const Contexts& C, uint32_t* ct
       }
       e += 32u;
     }
-    if (rec.x != GA_DEAD) {
-      const uint32_t c = intern_context(C, ctl, rec.y & 0xFFFFu, buf + i, e - i);
-      if (c == CTX_NEW) return false;
-      if (lane == 0) reinterpret_cast<uint2*>(C.pool)[at / 2u + g] = make_uint2(rec.x, d << 16 | c);
-      ++g;
-    }
+    const uint32_t c = intern_context(C, ctl, __ldg(&G.ga_item[2u * d]) & 0xFFFFu, buf + i, e - i);
+    if (c == CTX_NEW) return false;
+    if (lane == 0) C.pool[at + g] = d << 16 | c;
+    ++g;
     i = e;
   }
   __syncwarp();
   out = make_uint2(at, g);
+  return true;
+}
+
+// The same for at most 32 different items that sit one to a lane (lane l < n: item l).
+__device__ __forceinline__ bool group_lanes(const GrammarDev& G, const Contexts& C, uint32_t* ctl, uint32_t item, uint32_t n, uint2& out) {
+  const uint32_t lane = lane_id(), at = ctl[AC_POOL];
+  if (lane >= n) item = 0xFFFFFFFFu;
+  if (n > 1u) {
+#pragma unroll
+    for (uint32_t k = 2; k <= 32; k <<= 1)
+#pragma unroll
+      for (uint32_t j = k >> 1; j > 0; j >>= 1) {
+        const uint32_t other = __shfl_xor_sync(FULL, item, j);
+        item = (((lane & k) == 0) == ((lane & j) == 0)) ? min(item, other) : max(item, other);
+      }
+  }
+  const uint32_t d = item >> 16, before = __shfl_up_sync(FULL, d, 1);
+  const bool leads = lane < n && (lane == 0u || before != d);
+  const uint32_t lb = __ballot_sync(FULL, leads), groups = __popc(lb);
+  if (at + groups + n > C.pool_cap) return false;
+  __syncwarp();
+  if (lane == 0) ctl[AC_POOL] = at + groups;
+  __syncwarp();
+  const uint32_t after = lane == 31u ? 0u : lb >> (lane + 1u), size = after ? (uint32_t)__ffs(after) : n - lane;  // (of the group of a lane that leads)
+  const uint32_t lhs = leads ? __ldg(&G.ga_item[2u * d]) & 0xFFFFu : 0u;
+  uint32_t ctx = CTX_NEW;
+  if (__any_sync(FULL, leads && size == 1u)) {
+    ctx = intern_singles(C, ctl, leads && size == 1u, lhs, item & 0xFFFFu);
+    if (__any_sync(FULL, leads && size == 1u && ctx == CTX_NEW)) return false;
+  }
+  for (uint32_t m = __ballot_sync(FULL, leads && size > 1u); m; m &= m - 1u) {
+    const uint32_t first = (uint32_t)__ffs(m) - 1u, k = __shfl_sync(FULL, size, first);
+    const uint32_t top = ctl[AC_POOL];  // its origins, ascending, at the pool's top (which grows only if the context is new)
+    if (top + k > C.pool_cap) return false;
+    if (lane >= first && lane < first + k) C.pool[top + lane - first] = item & 0xFFFFu;
+    __syncwarp();
+    const uint32_t c = intern_context(C, ctl, __shfl_sync(FULL, lhs, first), C.pool + top, k);
+    if (c == CTX_NEW) return false;
+    if (lane == first) ctx = c;
+  }
+  if (leads) C.pool[at + __popc(lb & ((1u << lane) - 1u))] = d << 16 | ctx;
+  __syncwarp();
+  out = make_uint2(at, groups);
   return true;
 }
 
@@ -309,8 +378,8 @@ __device__ bool expand_into(const GrammarDev& G, const Contexts& C, const AfChar
     for (uint32_t base = lo; base < hi; base += 32) {
       const uint32_t k = base + lane;
       const uint32_t it = k < hi ? J.items[k] : 0u;
-      const uint4 rec = __ldg(reinterpret_cast<const uint4*>(G.ga_item) + (it & 0xFFFFu));
-      const bool match = k < hi && (rec.y >> 16) == a, on = match && (rec.w & GA_GOES_ON);
+      const uint2 rec = __ldg(reinterpret_cast<const uint2*>(G.ga_item) + (it & 0xFFFFu));
+      const bool match = k < hi && (rec.x >> 16) == a, on = match && (rec.y & GA_GOES_ON);
       const uint32_t b = __ballot_sync(FULL, on);
       if (nbuf + __popc(b) > buf_cap) {  // an item comes once for every set that it waits in: the repeats go
         uint32_t groups;
@@ -320,7 +389,7 @@ __device__ bool expand_into(const GrammarDev& G, const Contexts& C, const AfChar
       }
       if (on) buf[nbuf + __popc(b & ((1u << lane) - 1u))] = ((it & 0xFFFFu) + 1u) << 16 | (it >> 16);
       nbuf += __popc(b);
-      if (match && (rec.w & 0xFFFFu) != 0xFFFFu) need(rec.w & 0xFFFFu, it >> 16);
+      if (match && (rec.y & 0xFFFFu) != 0xFFFFu) need(rec.y & 0xFFFFu, it >> 16);
     }
   }
   if (lane == 0) ctl[AC_NBUF] = nbuf;
@@ -344,9 +413,9 @@ __device__ bool expand_small(const GrammarDev& G, const Contexts& C, const AfCha
     for (uint32_t base = lo; base < hi; base += 32) {
       const uint32_t k = base + lane;
       const uint32_t it = k < hi ? J.items[k] : 0u;
-      const uint4 rec = __ldg(reinterpret_cast<const uint4*>(G.ga_item) + (it & 0xFFFFu));
-      const bool match = k < hi && (rec.y >> 16) == a;
-      uint32_t on = __ballot_sync(FULL, match && (rec.w & GA_GOES_ON));
+      const uint2 rec = __ldg(reinterpret_cast<const uint2*>(G.ga_item) + (it & 0xFFFFu));
+      const bool match = k < hi && (rec.x >> 16) == a;
+      uint32_t on = __ballot_sync(FULL, match && (rec.y & GA_GOES_ON));
       if (on) {
         const uint32_t x = ((it & 0xFFFFu) + 1u) << 16 | (it >> 16);
         if (ni + __popc(on) > 32u) return false;
@@ -357,8 +426,8 @@ __device__ bool expand_small(const GrammarDev& G, const Contexts& C, const AfCha
           ++ni;
         }
       }
-      for (uint32_t up = __ballot_sync(FULL, match && (rec.w & 0xFFFFu) != 0xFFFFu); up; up &= up - 1u) {
-        const uint32_t v = __shfl_sync(FULL, (rec.w & 0xFFFFu) << 16 | (it >> 16), __ffs(up) - 1);
+      for (uint32_t up = __ballot_sync(FULL, match && (rec.y & 0xFFFFu) != 0xFFFFu); up; up &= up - 1u) {
+        const uint32_t v = __shfl_sync(FULL, (rec.y & 0xFFFFu) << 16 | (it >> 16), __ffs(up) - 1);
         if (__ballot_sync(FULL, lane < nw && work == v)) continue;
         if (nw == 32u) return false;
         if (lane == nw) work = v;
@@ -366,50 +435,10 @@ __device__ bool expand_small(const GrammarDev& G, const Contexts& C, const AfCha
       }
     }
   }
-  // by rule: one context for each
-  uint32_t at = (ctl[AC_POOL] + 1u) & ~1u, g = 0;
-  if (at + 2u * ni + 64u > C.pool_cap || ctl[AC_NCTX] + ni > C.cap) return false;
-  __syncwarp();
-  if (lane == 0) ctl[AC_POOL] = at + 2u * ni;
-  __syncwarp();
-  uint32_t left = ni == 32u ? FULL : (1u << ni) - 1u;
-  {  // rules with one item
-    const bool mine = (left >> lane) & 1u;
-    const uint32_t same = __match_any_sync(FULL, mine ? item >> 16 : 0x10000u + lane);
-    const bool single = mine && same == 1u << lane;
-    const uint4 rec = single ? __ldg(reinterpret_cast<const uint4*>(G.ga_item) + (item >> 16)) : make_uint4(GA_DEAD, 0u, 0u, 0u);
-    const bool v = single && rec.x != GA_DEAD;
-    const uint32_t alive = __ballot_sync(FULL, v);
-    left &= ~__ballot_sync(FULL, single);
-    if (alive) {
-      const uint32_t ctx = intern_singles(C, ctl, v, rec.y & 0xFFFFu, item & 0xFFFFu);
-      if (__any_sync(FULL, v && ctx == CTX_NEW)) return false;
-      if (v) reinterpret_cast<uint2*>(C.pool)[at / 2u + __popc(alive & ((1u << lane) - 1u))] = make_uint2(rec.x, (item & 0xFFFF0000u) | ctx);
-      g = __popc(alive);
-    }
-  }
-  while (left) {
-    const uint32_t d = __shfl_sync(FULL, item >> 16, __ffs(left) - 1);
-    const bool in = ((left >> lane) & 1u) && (item >> 16) == d;
-    const uint32_t members = __ballot_sync(FULL, in), n = __popc(members);
-    left &= ~members;
-    const uint4 rec = __ldg(reinterpret_cast<const uint4*>(G.ga_item) + d);
-    if (rec.x == GA_DEAD) continue;
-    // its origins, ascending, at the pool's top (which grows only if the context is new)
-    const uint32_t top = ctl[AC_POOL];
-    if (top + n > C.pool_cap) return false;
-    uint32_t rank = 0;
-    if (n > 1u)
-      for (uint32_t m = members; m; m &= m - 1u) rank += __shfl_sync(FULL, item, __ffs(m) - 1) < item ? 1u : 0u;
-    if (in) C.pool[top + rank] = item & 0xFFFFu;
-    __syncwarp();
-    const uint32_t ctx = intern_context(C, ctl, rec.y & 0xFFFFu, C.pool + top, n);
-    if (ctx == CTX_NEW) return false;
-    if (lane == 0) reinterpret_cast<uint2*>(C.pool)[at / 2u + g] = make_uint2(rec.x, d << 16 | ctx);
-    ++g;
-  }
-  __syncwarp();
-  if (lane == 0) C.exp[c] = make_uint2(at, g);
+  if (ctl[AC_NCTX] + ni > C.cap) return false;
+  uint2 list;
+  if (!group_lanes(G, C, ctl, item, ni, list)) return false;
+  if (lane == 0) C.exp[c] = list;
   __syncwarp();
   return true;
 }
@@ -442,25 +471,7 @@ __device__ __noinline__ bool expand_context(const GrammarDev& G, const AutoFillD
   }
 }
 
-// Where `code` leads on byte class e.
-__device__ __forceinline__ uint32_t ga_next(const GrammarDev& G, uint32_t code, uint32_t e) {
-  if (!(code & GA_ITEM)) return __ldg(&G.ga_trans[(size_t)code * G.n_eq + e]);
-  const uint32_t org = (code >> 14) & 0xFFFFu;
-  const uint32_t t = __ldg(&G.dfa_trans[(size_t)(code & 0x3FFFu) * G.n_eq + e]);
-  if (t == 0xFFFFu || !(t & 0xC000u)) return GA_DEAD;
-  if (!(t & 0x8000u)) return GA_ITEM | (org << 14) | (t & 0x3FFFu);
-  if (org == 0u) return GA_EXIT | ((t & 0x4000u) ? (GA_ITEM | (t & 0x3FFFu)) : GA_NONE);
-  const uint32_t key = org << 16 | t;
-  for (uint32_t s = ga_hash(key) & G.ga_acc_mask;; s = (s + 1u) & G.ga_acc_mask) {
-    const uint2 kv = __ldg(reinterpret_cast<const uint2*>(G.ga_acc) + s);
-    if (kv.x == key) return kv.y;
-    if (kv.x == 0u) return GA_UNKNOWN;
-  }
-}
-
-// Nodes at which several tokens end (byte strings that the grammar cannot tell apart): tokens at .. at + cnt of each lane, dealt out to
-// the lanes two by two.  (Node by node, each waited for its own read of ga_tok: 3,000 of the 7,000 cycles of a round.  64 rows of a
-// JSON schema decode 16 steps in 2.46 ms instead of 2.57, 37 rows of JSON are filled in 126 us instead of 132.)
+// Tokens at .. at + cnt of each lane's list, dealt out to the lanes two by two.
 __device__ __forceinline__ void set_tokens(const GrammarDev& G, uint32_t* mask, uint32_t at, uint32_t cnt) {
   const uint32_t lane = lane_id();
   uint32_t incl = cnt;
@@ -492,14 +503,14 @@ __global__ void __launch_bounds__(AF_THREADS, 4) automaton_fill_kernel(const __g
                                                                        const __grid_constant__ StateDev S) {
   before_me();
   const uint32_t n_jobs = S.counters[CNT_N_JOBS];
-  if (n_jobs == 0u) return;  // (every block sees the same count)
-  extern __shared__ __align__(16) uint32_t smem[];
   const AutoFillDev& A = S.af;
+  const uint32_t parts = A.parts;  // (a power of two)
+  if (blockIdx.x >= n_jobs * parts) return;
+  extern __shared__ __align__(16) uint32_t smem[];
   const uint32_t tid = threadIdx.x, warp = tid >> 5, lane = lane_id(), lt = (1u << lane) - 1u;
-  uint4* const entries = reinterpret_cast<uint4*>(smem);               // [2][AF_BATCH], in turn
-  uint4* const specials = entries + 2 * AF_BATCH;                      // [2][AF_SPEC], in turn
-  uint4* const exits = specials + 2 * AF_SPEC;                         // [AF_EXITS] where in ga_wide_exit, count, -, context
-  unsigned long long* const seen = reinterpret_cast<unsigned long long*>(exits + AF_EXITS);
+  uint2* const entries = reinterpret_cast<uint2*>(smem);  // [2][AF_BATCH], in turn: first edge, context
+  uint2* const lists = entries + 2 * AF_BATCH;            // [AF_LISTS] where in ga_tok
+  unsigned long long* const seen = reinterpret_cast<unsigned long long*>(lists + AF_LISTS);
   Contexts C0;
   C0.org = reinterpret_cast<uint2*>(seen + AF_SEEN);
   C0.exp = C0.org + AF_CTX;
@@ -507,165 +518,96 @@ __global__ void __launch_bounds__(AF_THREADS, 4) automaton_fill_kernel(const __g
   C0.pool = C0.lhs + AF_CTX;
   C0.hash = C0.pool + AF_POOL;
   C0.cap = AF_CTX, C0.hash_mask = AF_CTX_HASH - 1u, C0.pool_cap = AF_POOL;
-  uint32_t* const pre = C0.hash + AF_CTX_HASH;  // [AF_BATCH + 1]
-  uint32_t* const ctl = pre + AF_BATCH + 4;
-  uint32_t* const stage = ctl + AC_WORDS;
+  uint32_t* const pre = C0.hash + AF_CTX_HASH;  // [2][AF_BATCH], [AF_LISTS]
+  uint32_t* const ctl = pre + 2 * AF_BATCH + AF_LISTS;
+  uint32_t* const wide = ctl + AC_WORDS;        // [AF_THREADS] rows of ga_mask
+  uint32_t* const stage = wide + AF_THREADS;
   uint32_t* const buf = stage + AF_STAGE;
   uint32_t* const work = buf + AF_BUF;
   uint32_t* const hset = work + AF_WORK;
-  uint16_t* const owner = reinterpret_cast<uint16_t*>(hset + AF_HSET);  // [AF_OWNER] the thread to whom the first child of a piece belongs
-  uint4* const stack = A.stack + (size_t)blockIdx.x * A.stack_cap;  // threads that found no room in `entries`
+  uint16_t* const owner = reinterpret_cast<uint16_t*>(hset + AF_HSET);
+  uint4* const stack = A.stack + (size_t)blockIdx.x * A.stack_cap;  // entries that found no room: first edge, edges, context
+  auto edge_deal = [&](uint32_t side) {
+    return Deal{ctl + AC_EDGES + 4u * side, entries + side * AF_BATCH, pre + side * AF_BATCH, owner + side * (AF_EDGES / 32u), AF_BATCH, AF_EDGES};
+  };
+  auto token_deal = [&](uint32_t side) {
+    return Deal{ctl + AC_TOKENS + 4u * side, lists, pre + 2u * AF_BATCH, owner + 2u * (AF_EDGES / 32u), AF_LISTS, AF_TOKENS};
+  };
   for (uint32_t i = tid; i < AF_HSET; i += AF_THREADS) hset[i] = EMPTY_SLOT;
   uint32_t looked_up = 0, contexts = 0;
-  // (expansions look items up one after the other: what fits is brought near at once)
-  for (uint32_t i = tid * 8u; i < min(G.D, 8u * AF_THREADS); i += 8u * AF_THREADS) {
-    uint32_t v;
-    asm volatile("ld.global.nc.u32 %0, [%1];" : "=r"(v) : "l"(G.ga_item + 4u * i));
-    (void)v;
-  }
-  bool rows_left = true;
-  const uint32_t parts = A.parts;  // (a power of two)
+  bool gave_up = false;
 
+  uint32_t ticket = blockIdx.x;
+  if (parts > 1u) {  // (drawn by blocks that run: nobody ever waits for a block that has not started)
+    if (tid == 0) ctl[AC_JOB] = atomicAdd(&S.counters[CNT_AF_TICKET], 1u);
+    __syncthreads();
+    ticket = ctl[AC_JOB];
+    __syncthreads();
+  }
   for (;;) {
-    // ---- (a share of) a row, or, when there is none left, a unit of work that another block gives
-    // (they are taken by blocks that run: nobody ever waits for a block that has not started)
-    __syncthreads();
-    if (tid == 0) ctl[AC_JOB] = rows_left ? atomicAdd(&S.counters[CNT_AF_TICKET], 1u) : 0xFFFFFFFFu;
-    __syncthreads();
-    uint32_t j = ctl[AC_JOB] / parts, part = ctl[AC_JOB] & (parts - 1u);
-    uint32_t* unit = nullptr;
-    rows_left = j < n_jobs;
-    if (j >= n_jobs) {
-      __syncthreads();
-      if (tid == 0) {
-        const uint32_t ticket = atomicAdd(&S.counters[CNT_AF_TAKEN], 1u);
-        uint32_t got = 0;
-        if (ticket < A.unit_cap) {
-          for (uint32_t polls = 0;; ++polls) {
-            if (ld_acquire(&A.unit_flag[ticket]) == S.gen) {
-              got = 1u;
-              break;
-            }
-            if (ld_acquire(&S.counters[CNT_AF_ACTIVE]) == 0u || ld_acquire(&S.counters[CNT_BAR_ERR])) break;  // all is done
-            if (polls > poll_limit(S, 22)) {
-              diag(S, DIAG_WAIT_QUEUE);
-              atomicExch(&S.counters[CNT_BAR_ERR], 1u);  // the fill is given up: its rows get all-zero masks
-              break;
-            }
-            __nanosleep(400);
-          }
-        }
-        ctl[AC_JOB] = got ? ticket : 0xFFFFFFFFu;
-        ctl[AC_BASE] = vload(&S.counters[CNT_AF_GIVEN]);
-      }
-      __syncthreads();
-      const uint32_t u = ctl[AC_JOB];
-      if (u == 0xFFFFFFFFu) break;
-      unit = A.units + (size_t)u * AU_WORDS;
-      j = __ldcg(unit + AU_ROWJOB), part = __ldcg(unit + AU_PART);
-    }
+    // ---- (a share of) a row
+    const uint32_t j = ticket / parts, part = ticket & (parts - 1u);
+    if (j >= n_jobs) break;
     const uint32_t row = S.jobs[j];
     const uint32_t* chart = S.arena + S.row_chart[row];
     uint32_t* const mask = S.mask_rows + (size_t)S.row_mask[row] * G.Wm;
     AfChart J;
+    const uint32_t ahead = tid < A.ahead ? chart[tid] : 0u;  // (asked for together with the header)
     J.m = chart[CH_SETS];
     const uint32_t chart_words = chart[CH_WORDS];
     const bool accepting = (chart[CH_FLAGS] & CHART_ACCEPTING) != 0u;
     J.off = chart + CH_HDR;
     if (chart_words <= AF_STAGE) {
-      for (uint32_t i = CH_HDR + tid; i < chart_words; i += AF_THREADS) stage[i] = chart[i];
+      if (tid < A.ahead) stage[tid] = ahead;
+      for (uint32_t i = A.ahead + tid; i < chart_words; i += AF_THREADS) stage[i] = chart[i];
       J.off = stage + CH_HDR;
     }
     J.items = J.off + J.m + 1u;
-    const bool begins = !unit && part == 0u;
     auto eos_word = [&](uint32_t i) -> uint32_t { return (accepting && G.eos >= 0 && i == (uint32_t)G.eos >> 5) ? 1u << ((uint32_t)G.eos & 31u) : 0u; };
-    if (begins && parts > 1u) {  // the mask is cleared first: the other blocks of the row wait for that
+    if (parts > 1u && part == 0u) {  // the mask is cleared first: the other blocks of the row wait for that
       for (uint32_t i = tid; i < G.Wm; i += AF_THREADS) mask[i] = eos_word(i);
       __threadfence();
     }
-    __syncthreads();
-    if (begins && parts > 1u && tid == AF_THREADS - 1)
-      asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(A.unit_flag + A.unit_cap + j), "r"(S.gen) : "memory");
     for (uint32_t i = tid; i < AF_SEEN; i += AF_THREADS) seen[i] = 0ull;
     if (tid < AC_WORDS) ctl[tid] = 0u;
     if (tid < AF_CTX_HASH) C0.hash[tid] = 0u;
-    uint32_t side = 0;  // the threads of this round are entries[side]
     __syncthreads();
-    if (unit) {
-      const uint32_t n = __ldcg(unit + AU_N), nc = __ldcg(unit + AU_NCTX), np = __ldcg(unit + AU_POOL);
-      const uint32_t* src = unit + AU_HDR;
-      uint32_t* dst = reinterpret_cast<uint32_t*>(C0.org);  // org, exp, lhs and pool follow one another here and there
-      for (uint32_t i = tid; i < 5u * AF_CTX + np; i += AF_THREADS) dst[i] = __ldcg(src + i);
-      const uint4* th = reinterpret_cast<const uint4*>(unit + AU_HDR + 5 * AF_CTX + AF_POOL);
-      for (uint32_t i = tid; i < n; i += AF_THREADS) entries[i] = __ldcg(th + i);
-      __syncthreads();
-      if (warp == 0) {
-        for (uint32_t c = 0; c < nc; ++c) {
-          const uint2 o = C0.org[c];
-          uint32_t slot = context_hash(C0.lhs[c], C0.pool + o.x, o.y) & (AF_CTX_HASH - 1u);
-          while (C0.hash[slot]) slot = (slot + 1u) & (AF_CTX_HASH - 1u);
-          __syncwarp();
-          if (lane == 0) C0.hash[slot] = c + 1u;
-          __syncwarp();
-        }
-        if (lane == 0) ctl[AC_NEXT] = n, ctl[AC_NCTX] = nc, ctl[AC_POOL] = np;
-      }
-    } else if (warp == 0) {  // the kernel of the chart's last set starts the first threads
+    if (warp == 0) {  // the kernel of the chart's last set
+      if (lane < 4u) deal_clear(lane < 2u ? edge_deal(lane) : token_deal(lane - 2u));
       const uint32_t lo = J.off[J.m - 1u], hi = J.off[J.m], self = J.m - 1u;
       uint32_t* b = hi - lo <= AF_BUF ? buf : big_area(A) + A.big_cap / 4u + A.big_cap / 2u;
-      uint32_t n = 0;
+      uint32_t n = 0, mine = 0;
       bool ok = hi - lo <= A.big_cap;
       if (ok)
         for (uint32_t base = lo; base < hi; base += 32) {
           const uint32_t k = base + lane;
           const uint32_t it = k < hi ? J.items[k] : 0u;
           bool take = k < hi && ((it >> 16) != self || (it & 0xFFFFu) == ITEM_START);
+          if (take) take = (__ldg(&G.ga_item[2u * (it & 0xFFFFu) + 1u]) & GA_ALIVE) != 0u;
           if (take && k > lo && (it & 0xFFFFu) != 0u && J.items[k - 1u] == it - 1u)  // the item before it skips to it
-            take = !(__ldg(&G.ga_item[4u * ((it & 0xFFFFu) - 1u) + 3u]) & GA_SKIPS);
+            take = !(__ldg(&G.ga_item[2u * ((it & 0xFFFFu) - 1u) + 1u]) & GA_SKIPS);
           const uint32_t bal = __ballot_sync(FULL, take);
-          if (take) b[n + __popc(bal & ((1u << lane) - 1u))] = (it << 16) | (it >> 16);
+          if (take) b[n + __popc(bal & lt)] = (it << 16) | (it >> 16);
           n += __popc(bal);
         }
       __syncwarp();
       uint2 list = make_uint2(0u, 0u);
       Contexts C = C0;
-      if (ok && !(ok = group_items(G, C, ctl, b, n, list))) {
+      if (lane < n) mine = b[lane];
+      bool grouped = n <= 32u && group_lanes(G, C, ctl, mine, n, list);
+      if (!grouped && ok && !(ok = group_items(G, C, ctl, b, n, list))) {
         spill_contexts(C, ctl, A);
         ok = group_items(G, C, ctl, b, n, list);  // (sorted and without repeats already)
       }
-      const uint4 root = __ldg(reinterpret_cast<const uint4*>(G.ga_node));
-      uint32_t top = 0;
-      for (uint32_t base = 0; base < list.y; base += 32) {
-        const uint32_t i = base + lane;
-        const uint2 x = i < list.y ? reinterpret_cast<const uint2*>(C.pool)[list.x / 2u + i] : make_uint2(0u, 0u);
-        const uint32_t wide = i < list.y ? __ldg(&G.ga_item[4u * (x.y >> 16) + 2u]) : GA_DEAD;
-        uint4 en = make_uint4(root.x, root.y >> 8, x.x, x.y & 0xFFFFu);
-        bool take = i < list.y && en.y != 0u;
-        if (wide != GA_DEAD) {  // most of the vocabulary follows from this item alone
-          const uint4 r = __ldg(reinterpret_cast<const uint4*>(G.ga_wide_rec) + wide);
-          const uint32_t at = atomicAdd(&ctl[AC_NWIDE], 1u);
-          if (at < AF_EXITS) {  // (those that find no room start threads like any other)
-            ctl[AC_WIDE + at] = r.x;
-            if (r.z) exits[atomicAdd(&ctl[AC_NEXITS], 1u)] = make_uint4(r.y, r.z, 0u, en.w);
-            take = false;
-          }
-        }
-        const uint32_t bal = __ballot_sync(FULL, take);
-        const uint32_t at = top + __popc(bal & ((1u << lane) - 1u));
-        if (take && at < AF_BATCH) entries[at] = en;
-        else if (take) reinterpret_cast<uint2*>(C.pool)[list.x / 2u + at - AF_BATCH] = x;  // they wait in the list, closed up
-        top += __popc(bal);
-      }
       if (lane == 0) {
-        ctl[AC_NEXT] = min(top, AF_BATCH);
-        ctl[AC_LIST] = list.x, ctl[AC_LIST_END] = top > AF_BATCH ? top - AF_BATCH : 0u;
+        ctl[AC_LIST] = list.x, ctl[AC_LIST_END] = list.y;
         if (!ok) ctl[AC_FAIL] = 1u + DIAG_SET_SCRATCH;
       }
-    }
-    __syncthreads();
-    if (!unit) {
-      if (part && tid == 0)  // the block that began with the row clears the mask
-        for (uint32_t polls = 0; ld_acquire(A.unit_flag + A.unit_cap + j) != S.gen; ++polls) {
+    } else if (tid == AF_THREADS - 1) {
+      ctl[AC_BEGAN] = (uint32_t)(clock64() >> 10);
+      if (parts > 1u && part == 0u) asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(A.row_begun + j), "r"(S.gen) : "memory");
+      if (part)  // the block that began with the row clears the mask
+        for (uint32_t polls = 0; ld_acquire(A.row_begun + j) != S.gen; ++polls) {
           if (polls > poll_limit(S, 22)) {
             diag(S, DIAG_WAIT_GRID);
             atomicExch(&S.counters[CNT_BAR_ERR], 1u);
@@ -674,373 +616,235 @@ __global__ void __launch_bounds__(AF_THREADS, 4) automaton_fill_kernel(const __g
           }
           if (polls) __nanosleep(64);
         }
-      __syncthreads();
-      // what follows from wide items, four words of a thread under way at once; a row's blocks share them (one dependent read
-      // after the other, by the block that began, they took 15,000 of the 150,000 cycles of a row of a JSON schema)
-      const uint32_t nw = min(ctl[AC_NWIDE], AF_EXITS), step = parts * AF_THREADS;
-      if (parts == 1u) {
-        for (uint32_t i = tid; i < G.Wm; i += 4u * AF_THREADS) {
-          uint32_t v[4];
-#pragma unroll
-          for (uint32_t u = 0; u < 4; ++u) v[u] = eos_word(i + u * AF_THREADS);
-          for (uint32_t k = 0; k < nw; ++k) {
-            const uint32_t* src = G.ga_wide_mask + (size_t)ctl[AC_WIDE + k] * G.Wm;
-#pragma unroll
-            for (uint32_t u = 0; u < 4; ++u) v[u] |= i + u * AF_THREADS < G.Wm ? __ldg(src + i + u * AF_THREADS) : 0u;
-          }
-#pragma unroll
-          for (uint32_t u = 0; u < 4; ++u)
-            if (i + u * AF_THREADS < G.Wm) mask[i + u * AF_THREADS] = v[u];
-        }
-      }
-      for (uint32_t k = 0; parts > 1u && k < nw; ++k) {
-        const uint32_t* src = G.ga_wide_mask + (size_t)ctl[AC_WIDE + k] * G.Wm;
-        for (uint32_t i = part * AF_THREADS + tid; i < G.Wm; i += 4u * step) {
-          uint32_t v[4];
-#pragma unroll
-          for (uint32_t u = 0; u < 4; ++u) v[u] = i + u * step < G.Wm ? __ldg(src + i + u * step) : 0u;
-#pragma unroll
-          for (uint32_t u = 0; u < 4; ++u)
-            if (v[u]) atomicOr(&mask[i + u * step], v[u]);
-        }
-      }
     }
-    const uint32_t looked_up_before = looked_up;
-    if (tid == AF_THREADS - 1) ctl[AC_BEGAN] = (uint32_t)(clock64() >> 10);
+    __syncthreads();
 
     bool spilled = false;
     // the expansion of a context (offset into pool, count), and its elements
     auto expansion = [&](uint32_t c) -> uint2 { return spilled ? global_contexts(A).exp[c] : C0.exp[c]; };
-    auto element = [&](uint32_t off, uint32_t k) -> uint2 {
-      return spilled ? reinterpret_cast<const uint2*>(global_contexts(A).pool)[off / 2u + k] : reinterpret_cast<const uint2*>(C0.pool)[off / 2u + k];
-    };
-    // false: this thread was started here a moment ago
-    auto start = [&](uint32_t first, uint32_t rule_ctx) -> bool {
-      const uint32_t slot = (first * 0x9E3779B1u ^ rule_ctx * 0x85EBCA6Bu) >> 23;
+    auto element = [&](uint32_t at) -> uint32_t { return spilled ? global_contexts(A).pool[at] : C0.pool[at]; };
+    // false: these edges were listed with this context a moment ago
+    auto fresh = [&](uint32_t edge, uint32_t ctx) -> bool {
+      const uint32_t slot = (edge * 0x9E3779B1u ^ ctx * 0x85EBCA6Bu) >> 23;
       static_assert(AF_SEEN == 512, "the slot is the upper nine bits");
-      const unsigned long long key = (unsigned long long)first << 32 | rule_ctx;
+      const unsigned long long key = (unsigned long long)(edge + 1u) << 32 | ctx;
       volatile unsigned long long* p = seen + slot;
-      const bool fresh = *p != key;
+      const bool yes = *p != key;
       *p = key;
-      return fresh;
+      return yes;
     };
-    for (;;) {  // ---- rounds
-      uint32_t n = min(ctl[AC_NEXT], AF_BATCH), ns = min(ctl[AC_SPEC], AF_SPEC), gtop = ctl[AC_GTOP], nx = ctl[AC_NEXITS];
-      const uint32_t first_at = ctl[AC_LIST_AT], first_left = ctl[AC_LIST_END] - first_at;  // items of the last set that have not started
-      if (ctl[AC_FAIL] || n + ns + gtop + nx + first_left == 0u) break;
-      spilled = ctl[AC_SPILLED] != 0u;
-      const uint32_t waiting = ctl[AC_WAITING];
-      __syncthreads();
-      uint4* const cur = entries + side * AF_BATCH;
-      uint4* const nxt = entries + (side ^ 1u) * AF_BATCH;
-      uint4* const spec = specials + side * AF_SPEC;
-      uint4* const spec_nxt = specials + (side ^ 1u) * AF_SPEC;
-      if (tid == 0) ctl[AC_NEXT] = 0u, ctl[AC_SPEC] = 0u, ctl[AC_OVF] = 0u;
-      if (tid == AF_THREADS - 1) {  // (looked at when the round ends; nobody waits for them until then)
-        peek(ctl + AC_PEEK, S.counters + CNT_AF_TICKET);
-        peek(ctl + AC_PEEK + 4u, A.row_gone + (j & ~3u));
-      }
-      // The stack cannot run over.  A round pushes at most the threads that its specials and its list start and two entries for each
-      // child it looks up, and takes no more than fits above the reserve.  On a crowded stack one entry is taken at a time, from the top:
-      // depth first the stack grows by two entries a child along one path of the trie (A.reserve, which has room for `cur` and `spec`, too).
-      const bool tight = A.stack_cap - gtop < A.reserve + AF_TIGHT, pops = !tight && gtop && n < AF_BATCH && ns < AF_SPEC;
-      if (tight) {
-        for (uint32_t i = tid; i < n; i += AF_THREADS) stack[gtop + i] = cur[i];
-        for (uint32_t i = tid; i < ns; i += AF_THREADS) stack[gtop + n + i] = spec[i];
-        gtop += n + ns;
-        __syncthreads();
-        const uint4 v = stack[--gtop];
-        ns = v.z == AF_SPAWN ? 1u : 0u, n = 1u - ns, nx = 0u;
-        if (tid == 0) (ns ? spec : cur)[0] = v;
-      } else if (pops) {
-        const uint32_t take = min(min(AF_BATCH - n, AF_SPEC - ns), gtop);
-        static_assert(AF_SPEC <= AF_THREADS, "one entry to a thread");
-        gtop -= take;
-        const uint4 v = tid < take ? stack[gtop + tid] : make_uint4(0u, 0u, 0u, 0u);
-        const bool is_spec = tid < take && v.z == AF_SPAWN, is_thread = tid < take && v.z != AF_SPAWN;
-        const uint32_t bt = __ballot_sync(FULL, is_thread), bs = __ballot_sync(FULL, is_spec);
-        uint32_t at = 0, at_spec = 0;
-        if (lane == 0 && bt) at = atomicAdd(&ctl[AC_POPPED], __popc(bt));
-        if (lane == 0 && bs) at_spec = atomicAdd(&ctl[AC_POPPED_SPEC], __popc(bs));
-        at = __shfl_sync(FULL, at, 0), at_spec = __shfl_sync(FULL, at_spec, 0);
-        if (is_thread) cur[n + at + __popc(bt & lt)] = v;
-        if (is_spec) spec[ns + at_spec + __popc(bs & lt)] = v;
-      } else if (n < AF_BATCH && first_left) {
-        const uint32_t take = min(AF_BATCH - n, first_left);
-        const uint4 root = __ldg(reinterpret_cast<const uint4*>(G.ga_node));
-        for (uint32_t i = tid; i < take; i += AF_THREADS) {
-          const uint2 x = element(ctl[AC_LIST], first_at + i);
-          cur[n + i] = make_uint4(root.x, root.y >> 8, x.x, x.y & 0xFFFFu);
+    auto expand_all = [&](const Deal& D, uint32_t entries_of) {  // (by warp 0) the contexts of these entries
+      Contexts C = ctl[AC_SPILLED] ? global_contexts(A) : C0;
+      for (uint32_t base = 0; base < entries_of; base += 32) {
+        const uint32_t c = base + lane < entries_of ? D.what[base + lane].y : CTX_NEW;
+        for (uint32_t todo = __ballot_sync(FULL, c != CTX_NEW && C.exp[c].y == CTX_NEW); todo;) {
+          const uint32_t x = __shfl_sync(FULL, c, __ffs(todo) - 1);
+          if (!expand_context(G, A, C, J, x, ctl, work, hset, buf) && lane == 0) ctl[AC_FAIL] = 1u + DIAG_SET_TABLE;
+          todo &= ~__ballot_sync(FULL, c == x);
         }
-        if (tid == 0) ctl[AC_LIST_AT] = first_at + take;
-        n += take;
       }
-      __syncthreads();
-      if (pops) n += ctl[AC_POPPED], ns += ctl[AC_POPPED_SPEC];
-      const uint32_t places = tight ? 0u : A.stack_cap - A.reserve - gtop;  // (at least AF_TIGHT)
-      auto overflow = [&](const uint4& v) {
+    };
+    uint32_t list_at = 0;  // items of the last set whose starts have been taken
+    bool begun = false;
+    for (uint32_t side = 0;; side ^= 1u) {  // ---- rounds
+      const Deal E = edge_deal(side), N = edge_deal(side ^ 1u), T = token_deal(side);
+      uint32_t n = dealt_lists(E), total = dealt_things(E), gtop = ctl[AC_GTOP];
+      const uint32_t list_end = ctl[AC_LIST_END];
+      if (ctl[AC_FAIL] || (n + gtop == 0u && begun && list_at == list_end)) break;
+      spilled = ctl[AC_SPILLED] != 0u;
+      if (parts > 1u && tid == AF_THREADS - 1) peek(ctl + AC_PEEK, A.row_gone + (j & ~3u));  // (looked at when the round ends)
+      auto overflow = [&](uint32_t edge, uint32_t cnt, uint32_t ctx) {
         const uint32_t p = atomicAdd(&ctl[AC_OVF], 1u);
-        if (gtop + p < A.stack_cap) stack[gtop + p] = v;
-        else ctl[AC_FAIL] = 1u + DIAG_QUEUE_FULL;  // (cannot happen, see above)
+        if (gtop + p < A.stack_cap) stack[gtop + p] = make_uint4(edge, cnt, ctx, 0u);
+        else ctl[AC_FULL] = 1u;  // (cannot happen, see below)
       };
-      if (ns + nx) {
-        // ---- expansions: contexts that have none yet, then the threads they start, in this very round as far as there is room
-        const bool list = nx != 0u && n < AF_BATCH / 2u;  // a list of nodes waits its turn
-        const uint4 ex = list ? exits[nx - 1u] : make_uint4(0u, 0u, 0u, 0u);
-        const uint4 en = tid < ns ? spec[tid] : make_uint4(0u, 0u, 0u, 0u);
-        const uint32_t en_ctx = en.w & 0xFFFFu;
-        if (__syncthreads_or((tid < ns && expansion(en_ctx).y == CTX_NEW) || (list && tid == 0 && expansion(ex.w).y == CTX_NEW))) {
-          if (warp == 0) {
-            Contexts C = spilled ? global_contexts(A) : C0;
-            for (uint32_t base = 0; base <= ns; base += 32) {  // (the list's comes last)
-              const uint32_t i = base + lane;
-              const uint32_t c = i < ns ? spec[i].w & 0xFFFFu : i == ns && list ? ex.w : CTX_NEW;
-              for (uint32_t todo = __ballot_sync(FULL, c != CTX_NEW && C.exp[c].y == CTX_NEW); todo;) {
-                const uint32_t x = __shfl_sync(FULL, c, __ffs(todo) - 1);
-                if (!expand_context(G, A, C, J, x, ctl, work, hset, buf) && lane == 0) ctl[AC_FAIL] = 1u + DIAG_SET_TABLE;
-                todo &= ~__ballot_sync(FULL, c == x);
+      auto list_edges = [&](bool yes, uint32_t edge, uint32_t cnt, uint32_t ctx) {  // (by all lanes of a warp)
+        const bool fits = deal(N, yes, min(cnt, AF_CHUNK), make_uint2(edge, ctx));
+        if (yes && !fits) overflow(edge, cnt, ctx);
+        else if (yes && cnt > AF_CHUNK) overflow(edge + AF_CHUNK, cnt - AF_CHUNK, ctx);
+      };
+      auto list_tokens = [&](uint32_t at, uint32_t cnt) {
+        const bool fits = deal(T, cnt != 0u, cnt, make_uint2(at, 0u));
+        if (__any_sync(FULL, !fits)) set_tokens(G, mask, at, fits ? 0u : cnt);
+      };
+      if (n + gtop == 0u) {
+        // ---- the starts of the last set's items; blocks that share a row share their tokens and edges
+        const uint32_t from = list_at, until = min(list_end, from + AF_SLICE);
+        list_at = until, begun = true;
+        for (uint32_t base = from; base == from || base < until; base += AF_THREADS) {
+          const uint32_t i = base + tid;
+          const uint32_t x = i < until ? element(ctl[AC_LIST] + i) : 0u;
+          uint4 r = i < until ? __ldg(reinterpret_cast<const uint4*>(G.ga_start) + (x >> 16)) : make_uint4(0u, 0u, 0u, 0u);
+          if (r.y == GA_MASK) wide[atomicAdd(&ctl[AC_NWIDE], 1u)] = r.x, r.y = 0u;
+          __syncthreads();
+          // what is valid from the items with masks, four words of a thread under way at once
+          const uint32_t nw = ctl[AC_NWIDE], step = parts * AF_THREADS;
+          if (tid == 0) looked_up += nw * (G.Wm / parts);
+          if (nw || base == 0u)
+            for (uint32_t i4 = part * AF_THREADS + tid; i4 < G.Wm; i4 += 4u * step) {
+              uint32_t v[4];
+#pragma unroll
+              for (uint32_t u = 0; u < 4; ++u) v[u] = 0u;
+              for (uint32_t k = 0; k < nw; ++k) {
+                const uint32_t* src = G.ga_mask + (size_t)wide[k] * G.Wm;
+#pragma unroll
+                for (uint32_t u = 0; u < 4; ++u) v[u] |= i4 + u * step < G.Wm ? __ldg(src + i4 + u * step) : 0u;
+              }
+#pragma unroll
+              for (uint32_t u = 0; u < 4; ++u) {
+                if (i4 + u * step >= G.Wm) continue;
+                if (parts == 1u && base == 0u) mask[i4 + u * step] = v[u] | eos_word(i4 + u * step);
+                else if (v[u]) atomicOr(&mask[i4 + u * step], v[u]);
               }
             }
+          __syncthreads();
+          if (tid == 0) ctl[AC_NWIDE] = 0u;
+          if (r.y == 1u && part == 0u) atomicOr(&mask[r.x >> 5], 1u << (r.x & 31u));
+          const uint32_t t0 = r.y > 1u ? (uint32_t)((uint64_t)r.y * part / parts) : 0u, t1 = r.y > 1u ? (uint32_t)((uint64_t)r.y * (part + 1u) / parts) : 0u;
+          const uint32_t e0 = (uint32_t)((uint64_t)r.w * part / parts), e1 = (uint32_t)((uint64_t)r.w * (part + 1u) / parts);
+          list_tokens(r.x + t0, t1 - t0);
+          list_edges(e1 > e0, r.z + e0, e1 - e0, x & 0xFFFFu);
+          looked_up += t1 - t0 + (r.y == 1u ? 1u : 0u);
+          __syncthreads();
+        }
+      } else {
+        // The stack cannot run over: a round takes no more edges than there are places above the reserve, and lists what follows from
+        // one of them at most once.  On a crowded stack one entry is taken at a time, from the top, and a few of its edges: depth first
+        // the stack grows along one path of the trie.
+        const uint32_t places = A.stack_cap - min(gtop + A.reserve, A.stack_cap);
+        if (places < AF_TIGHT) {
+          for (uint32_t i = tid; i < n; i += AF_THREADS) {
+            const uint2 w = E.what[i];
+            stack[gtop + i] = make_uint4(w.x, (i + 1u < n ? E.pre[i + 1u] : total) - E.pre[i], w.y, 0u);
           }
           __syncthreads();
-          spilled = ctl[AC_SPILLED] != 0u;
-        }
-        if (tid == 0) ctl[AC_NBUF] = n;
-        __syncthreads();
-        auto begin = [&](bool yes, uint32_t first, uint32_t kids, const uint2& el) {  // (by all lanes of a warp)
-          yes = yes && start(first, el.y);
-          const uint32_t bal = __ballot_sync(FULL, yes);
-          if (bal == 0u) return;
-          uint32_t at = 0;
-          if (lane == 0) at = atomicAdd(&ctl[AC_NBUF], __popc(bal));
-          at = __shfl_sync(FULL, at, 0) + __popc(bal & ((1u << lane) - 1u));
-          const uint4 v = make_uint4(first, kids, el.x, el.y & 0xFFFFu);
-          if (yes && at < AF_BATCH) cur[at] = v;
-          else if (yes) overflow(v);
-        };
-        if (warp * 32u < ns) {
-          // (all of its elements as a rule; what might not fit the stack is left for another round)
-          const uint2 spawns = tid < ns ? expansion(en_ctx) : make_uint2(0u, 0u);
-          const uint32_t from = en.w >> 16, count = min(spawns.y - min(from, spawns.y), tight ? 1u : max(1u, places / (2u * ns)));
-          const uint32_t most_of = __reduce_max_sync(FULL, count);
-          if (from + count < spawns.y) overflow(make_uint4(en.x, en.y, AF_SPAWN, (from + count) << 16 | en_ctx));
-          for (uint32_t q = 0; q < most_of; ++q) begin(q < count, en.x, en.y, q < count ? element(spawns.x, from + q) : make_uint2(0u, 0u));
-        }
-        if (list) {
-          const uint2 x = expansion(ex.w);
-          const uint32_t nodes = x.y ? min(ex.y, max(parts * (AF_BATCH / 2u / x.y), 32u)) : ex.y;  // (at most 2048 threads)
-          const bool by_specials = x.y > AF_LIST_STARTS;
-          if (x.y)
-            for (uint32_t base = warp * 32u; base < nodes; base += AF_THREADS) {
-              bool v = base + lane < nodes;
-              const uint2 nd = v ? __ldg(reinterpret_cast<const uint2*>(G.ga_wide_exit) + ex.x + base + lane) : make_uint2(0u, 0u);
-              // (blocks that share a row all start the threads of nodes of depth 1, and deal out the others)
-              if (parts > 1u && (nd.x < G.ga_lvl2 || nd.x >= G.ga_lvl3)) v = v && ((base + lane) & (parts - 1u)) == part;
-              if (by_specials) {
-                v = v && start(nd.x, 0xFFFF0000u | ex.w);
-                const uint4 b = make_uint4(nd.x, nd.y, AF_SPAWN, ex.w);
-                const uint32_t p = v ? atomicAdd(&ctl[AC_SPEC], 1u) : 0u;
-                if (v && p < AF_SPEC) spec_nxt[p] = b;
-                else if (v) overflow(b);
-                continue;
-              }
-              for (uint32_t q = 0; q < x.y; ++q) begin(v, nd.x, nd.y, element(x.x, q));
-            }
+          gtop += n - 1u;
+          const uint4 v = stack[gtop];
+          total = min(v.y, AF_TIGHT_EDGES), n = 1u;
           __syncthreads();
           if (tid == 0) {
-            if (nodes == ex.y) ctl[AC_NEXITS] = nx - 1u;
-            else exits[nx - 1u] = make_uint4(ex.x + nodes, ex.y - nodes, 0u, ex.w);
+            E.what[0] = make_uint2(v.x, v.z), E.pre[0] = 0u, E.owner[0] = 0u;
+            if (v.y > total) stack[gtop] = make_uint4(v.x + total, v.y - total, v.z, 0u);
           }
-        }
-        __syncthreads();
-        n = min(ctl[AC_NBUF], AF_BATCH);
-      }
-      if (waiting && n >= AF_SHARE && looked_up - looked_up_before >= AF_HEAVY && !spilled) {
-        // ---- other blocks wait: entry i stays here when i is a multiple of units + 1, else it goes to unit i % (units + 1) - 1
-        const uint32_t units = min(min(waiting, n / 128u - 1u), AF_MAX_UNITS);
-        if (tid == 0) {
-          const uint32_t at = atomicAdd(&S.counters[CNT_AF_POSTED], units);
-          const uint32_t fit = at >= A.unit_cap ? 0u : min(units, A.unit_cap - at);
-          if (fit == units) atomicAdd(&S.counters[CNT_AF_ACTIVE], units);
-          ctl[AC_BASE] = fit == units ? at : 0xFFFFFFFFu;  // (near the end of the units' storage nothing is given any more)
-        }
-        __syncthreads();
-        const uint32_t at = ctl[AC_BASE];
-        if (at != 0xFFFFFFFFu) {
-          const uint32_t nc = ctl[AC_NCTX], np = ctl[AC_POOL];
-          const uint32_t* src = reinterpret_cast<const uint32_t*>(C0.org);
-          for (uint32_t u = 0; u < units; ++u) {
-            uint32_t* dst = A.units + (size_t)(at + u) * AU_WORDS;
-            for (uint32_t i = tid; i < 5u * AF_CTX + np; i += AF_THREADS) dst[AU_HDR + i] = src[i];
-            if (tid == 0) dst[AU_ROWJOB] = j, dst[AU_N] = (n + units - 1u - u) / (units + 1u), dst[AU_NCTX] = nc, dst[AU_POOL] = np, dst[AU_PART] = part;
-          }
-          uint4 keep[AF_PER];
-#pragma unroll
-          for (uint32_t k = 0; k < AF_PER; ++k) {
-            const uint32_t i = k * AF_THREADS + tid;
-            if (i < n) {
-              keep[k] = cur[i];
-              const uint32_t to = i % (units + 1u);
-              if (to)
-                reinterpret_cast<uint4*>(A.units + (size_t)(at + to - 1u) * AU_WORDS + AU_HDR + 5 * AF_CTX + AF_POOL)[i / (units + 1u)] = keep[k];
-            }
-          }
-          __threadfence();
+          if (v.y > total) ++gtop;
           __syncthreads();
-          if (tid < units) asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(A.unit_flag + at + tid), "r"(S.gen) : "memory");
-#pragma unroll
-          for (uint32_t k = 0; k < AF_PER; ++k) {
-            const uint32_t i = k * AF_THREADS + tid;
-            if (i < n && i % (units + 1u) == 0u) cur[i / (units + 1u)] = keep[k];
-          }
-          n = (n + units) / (units + 1u);
+          if (warp == 0) expand_all(E, 1u);
           __syncthreads();
-        }
-      }
-      // ---- the threads' children, 32 to a piece
-      uint32_t w[AF_PER], sum = 0;
-#pragma unroll
-      for (uint32_t u = 0; u < AF_PER; ++u) {
-        const uint32_t i = tid * AF_PER + u;
-        w[u] = i < n ? cur[i].y : 0u;
-        sum += w[u];
-      }
-      uint32_t incl = sum;
-#pragma unroll
-      for (int d = 1; d < 32; d <<= 1) {
-        const uint32_t t = __shfl_up_sync(FULL, incl, d);
-        if ((int)lane >= d) incl += t;
-      }
-      if (lane == 31u) ctl[AC_WSUM + warp] = incl;
-      __syncthreads();
-      uint32_t before = incl - sum, total = 0;
-#pragma unroll
-      for (uint32_t k = 0; k < AF_WARPS; ++k) {
-        const uint32_t s = ctl[AC_WSUM + k];
-        if (k < warp) before += s;
-        total += s;
-      }
-#pragma unroll
-      for (uint32_t u = 0; u < AF_PER; ++u) {
-        const uint32_t i = tid * AF_PER + u;
-        if (i <= n) pre[i] = before;  // (pre[n] = the total)
-        for (uint32_t piece = (before + 31u) / 32u; piece * 32u < before + w[u]; ++piece) owner[piece] = (uint16_t)i;
-        before += w[u];
-      }
-      if (n == AF_BATCH && tid == 0) pre[n] = total;
-      const uint32_t pushed = ctl[AC_OVF];
-      __syncthreads();
-      if (!tight && 2u * total > places - pushed) {  // more children than can be pushed: the last threads wait
-        uint32_t fit = 0;
-#pragma unroll
-        for (uint32_t u = 0; u < AF_PER; ++u) {
-          const uint32_t i = u * AF_THREADS + tid;
-          fit += __syncthreads_count(i < n && 2u * pre[i + 1u] <= places - pushed);
-        }
-        for (uint32_t i = fit + tid; i < n; i += AF_THREADS) overflow(cur[i]);
-        n = fit, total = pre[n];
-        __syncthreads();
-      }
-      looked_up += total;
-      for (uint32_t base = warp * 32u; base < total; base += AF_THREADS) {
-        const uint32_t lo = owner[base / 32u];
-        const uint32_t nb = lo + 1u + lane <= n ? pre[lo + 1u + lane] - base : 32u;  // where the threads after it begin
-        const uint32_t starts = __reduce_or_sync(FULL, nb < 32u ? 1u << nb : 0u);
-        const uint32_t e = lo + __popc(starts & (0xFFFFFFFFu >> (31u - lane)));
-        bool goes_on = false, starts_one = false, special = false;
-        uint4 a, b;
-        uint4 nd = make_uint4(0u, 0u, 0u, 0u);
-        uint32_t many = 0;
-        uint4 en = make_uint4(0u, 0u, 0u, 0u);
-        uint32_t child = 0;
-        bool ours = base + lane < total;
-        if (ours) {
-          en = cur[e];
-          child = en.x + (base + lane - pre[e]);
-          // blocks that share a row share the nodes of depth 2, and with them what lies below
-          if (parts > 1u && child >= G.ga_lvl2 && child < G.ga_lvl3) ours = (child & (parts - 1u)) == part;
-        }
-        if (ours) {
-          nd = __ldg(reinterpret_cast<const uint4*>(G.ga_node) + child);
-          const uint32_t t = ga_next(G, en.z, nd.y & 0xFFu);
-          if (t < GA_UNKNOWN) {
-            if (nd.w == 1u) atomicOr(&mask[nd.z >> 5], 1u << (nd.z & 31u));
-            else many = nd.w;
-            const uint32_t kids = nd.y >> 8;
-            if (kids) {
-              goes_on = (t & ~GA_EXIT) != GA_NONE;
-              a = make_uint4(nd.x, kids, t & ~GA_EXIT, en.w);
-              if (t & GA_EXIT) {
-                const uint2 x = expansion(en.w);
-                if (x.y) {
-                  const uint2 el = x.y == 1u ? element(x.x, 0u) : make_uint2(AF_SPAWN, 0xFFFF0000u | en.w);
-                  starts_one = start(nd.x, el.y);
-                  special = starts_one && x.y != 1u;
-                  b = make_uint4(nd.x, kids, el.x, el.y & 0xFFFFu);
-                }
-              }
-            }
-          } else if (t == GA_UNKNOWN) {
-            ctl[AC_FAIL] = 1u + DIAG_ROOT_FAILED;  // (cannot happen: the automaton covers the vocabulary)
+          spilled = ctl[AC_SPILLED] != 0u;
+        } else if (places < total) {
+          for (uint32_t i = tid; i < n; i += AF_THREADS) {
+            const uint2 w = E.what[i];
+            const uint32_t first = E.pre[i], end = i + 1u < n ? E.pre[i + 1u] : total;
+            if (end > places) overflow(w.x + (max(first, places) - first), end - max(first, places), w.y);
           }
+          total = places;
         }
+        // ---- the edges
+        if (tid == 0) looked_up += total;
+        for (uint32_t base = warp * 32u; base < total; base += AF_THREADS) {
+          const uint32_t e = whose(E, n, base);
+          uint4 g = make_uint4(0u, 0u, 0u, 0u);
+          uint32_t to = CTX_NEW;
+          if (base + lane < total) {
+            const uint2 w = E.what[e];
+            g = __ldg(reinterpret_cast<const uint4*>(G.ga_edge) + w.x + (base + lane - E.pre[e]));
+            const uint2 x = expansion(w.y);
+            uint32_t lo = 0, hi = x.y;
+            while (lo < hi) {
+              const uint32_t mid = (lo + hi) >> 1;
+              if ((element(x.x + mid) >> 16) < (g.x >> 16)) lo = mid + 1u;
+              else hi = mid;
+            }
+            const uint32_t el = lo < x.y ? element(x.x + lo) : 0xFFFFFFFFu;
+            if ((el >> 16) == (g.x >> 16) && lo < x.y) to = el & 0xFFFFu;
+          }
+          const uint32_t cnt = to != CTX_NEW ? g.x & 0xFFFFu : 0u;
+          looked_up += cnt;
+          if (cnt == 1u) atomicOr(&mask[g.y >> 5], 1u << (g.y & 31u));
+          __syncwarp();
+          list_tokens(g.y, cnt > 1u ? cnt : 0u);
+          list_edges(to != CTX_NEW && g.w && fresh(g.z, to), g.z, g.w, to);
+        }
+      }
+      __syncthreads();
+      if (warp == 0) {
+        // ---- entries from the stack, as far as there is room, and the expansions that the next round needs
+        gtop += ctl[AC_OVF];
         __syncwarp();
-        if (__any_sync(FULL, many != 0u)) set_tokens(G, mask, nd.z, many);
-        const uint32_t ba = __ballot_sync(FULL, goes_on), bb = __ballot_sync(FULL, starts_one && !special);
-        if (ba | bb) {
-          uint32_t at = 0;
-          if (lane == 0) at = atomicAdd(&ctl[AC_NEXT], __popc(ba) + __popc(bb));
-          at = __shfl_sync(FULL, at, 0);
-          if (goes_on) {
-            const uint32_t p = at + __popc(ba & lt);
-            if (p < AF_BATCH) nxt[p] = a;
-            else overflow(a);
-          }
-          if (starts_one && !special) {
-            const uint32_t p = at + __popc(ba) + __popc(bb & lt);
-            if (p < AF_BATCH) nxt[p] = b;
-            else overflow(b);
-          }
+        if (lane == 0) ctl[AC_OVF] = 0u, deal_clear(E);
+        if (lane == 1u) deal_clear(token_deal(side ^ 1u));
+        __syncwarp();
+        while (gtop && A.stack_cap - min(gtop + A.reserve, A.stack_cap) >= AF_TIGHT && N.count[1] < AF_BATCH / 2u && N.count[0] < AF_EDGES / 2u) {
+          const uint32_t take = min(gtop, 32u);
+          const uint4 v = lane < take ? stack[gtop - 1u - lane] : make_uint4(0u, 0u, 0u, 0u);
+          __syncwarp();
+          gtop -= take;
+          list_edges(lane < take, v.x, v.y, v.z);
+          __syncwarp();
+          gtop += ctl[AC_OVF];
+          __syncwarp();
+          if (lane == 0) ctl[AC_OVF] = 0u;
+          __syncwarp();
         }
-        if (special) {
-          const uint32_t p = atomicAdd(&ctl[AC_SPEC], 1u);
-          if (p < AF_SPEC) spec_nxt[p] = b;
-          else overflow(b);
+        if (lane == 0) {
+          ctl[AC_GTOP] = gtop;
+          if (ctl[AC_FULL]) ctl[AC_FAIL] = 1u + DIAG_QUEUE_FULL;
         }
-      }
-      side ^= 1u;
-      __syncthreads();
-      if (tid == 0) {
-        ctl[AC_GTOP] = gtop + ctl[AC_OVF];
-        if (pops) ctl[AC_POPPED] = ctl[AC_POPPED_SPEC] = 0u;
-      }
-      if (tid == AF_THREADS - 1) {
-        asm volatile("cp.async.wait_all;" ::: "memory");
-        const uint32_t t = ctl[AC_PEEK + CNT_AF_TAKEN - CNT_AF_TICKET], p = ctl[AC_PEEK + CNT_AF_POSTED - CNT_AF_TICKET];
-        const bool gone = ctl[AC_PEEK + 4u + (j & 3u)] == S.gen, late = (uint32_t)(clock64() >> 10) - ctl[AC_BEGAN] > AF_KCYCLES;
-        ctl[AC_WAITING] = t > p ? t - p : 0u;
-        if ((gone || late) && !ctl[AC_FAIL]) ctl[AC_FAIL] = gone ? AF_GONE : AF_LATE;
+        expand_all(N, dealt_lists(N));
+      } else {
+        // ---- tokens, meanwhile
+        const uint32_t nt = dealt_lists(T), tt = dealt_things(T);
+        for (uint32_t base = (warp - 1u) * 32u; base < tt; base += 4u * (AF_THREADS - 32u)) {
+          uint32_t tok[4];
+#pragma unroll
+          for (uint32_t u = 0; u < 4; ++u) {
+            const uint32_t at = base + u * (AF_THREADS - 32u);
+            tok[u] = 0xFFFFFFFFu;
+            if (at >= tt) continue;
+            const uint32_t e = whose(T, nt, at);
+            if (at + lane < tt) tok[u] = __ldg(&G.ga_tok[T.what[e].x + (at + lane - T.pre[e])]);
+          }
+#pragma unroll
+          for (uint32_t u = 0; u < 4; ++u)
+            if (tok[u] != 0xFFFFFFFFu) atomicOr(&mask[tok[u] >> 5], 1u << (tok[u] & 31u));
+        }
+        if (tid == AF_THREADS - 1) {
+          asm volatile("cp.async.wait_all;" ::: "memory");
+          const bool gone = parts > 1u && ctl[AC_PEEK + (j & 3u)] == S.gen, late = (uint32_t)(clock64() >> 10) - ctl[AC_BEGAN] > AF_KCYCLES;
+          if ((gone || late) && !ctl[AC_FAIL]) ctl[AC_FAIL] = gone ? AF_GONE : AF_LATE;
+        }
       }
       __syncthreads();
     }
     contexts += ctl[AC_NCTX];
-    if (tid == 0 && ctl[AC_FAIL] && ctl[AC_FAIL] < AF_GONE) {  // too many contexts, or too long a time: the row is left to a sweep by Earley steps
-      if (ctl[AC_FAIL] != AF_LATE) diag(S, ctl[AC_FAIL] - 1u);
-      if (atomicExch(A.row_gone + j, S.gen) != S.gen)  // (its other blocks stop when they see that)
-        *reinterpret_cast<volatile uint32_t*>(A.given + atomicAdd(&S.counters[CNT_AF_GIVEN], 1u)) = S.gen << 16 | j;
+    if (ctl[AC_FAIL] && ctl[AC_FAIL] != AF_GONE && ctl[AC_FAIL] != AF_GIVEN_UP) {  // too many contexts, or too long a time: the row is left to a sweep by Earley steps
+      gave_up = true;
+      if (tid == 0) {
+        if (ctl[AC_FAIL] != AF_LATE) diag(S, ctl[AC_FAIL] - 1u);
+        if (atomicExch(A.row_gone + j, S.gen) != S.gen)  // (its other blocks stop when they see that)
+          *reinterpret_cast<volatile uint32_t*>(A.given + atomicAdd(&S.counters[CNT_AF_GIVEN], 1u)) = S.gen << 16 | j;
+      }
     }
     // ---- the next row
     __threadfence();
+    if (gridDim.x >= n_jobs * parts) break;
     __syncthreads();
-    if (tid == 0) atomicSub(&S.counters[CNT_AF_ACTIVE], 1u);
+    if (tid == 0) ctl[AC_JOB] = gridDim.x + atomicAdd(&S.counters[CNT_AF_TICKET], 1u);
+    __syncthreads();
+    ticket = ctl[AC_JOB];
+    __syncthreads();
   }
-  if (tid == 0 && looked_up) {
-    stat_add(S, CNT_STAT_TRANS, looked_up);
+  looked_up = __reduce_add_sync(FULL, looked_up);
+  __syncthreads();
+  if (lane == 0 && looked_up) atomicAdd(&ctl[AC_LOOKED], looked_up);
+  __syncthreads();
+  if (tid == 0) {
+    stat_add(S, CNT_STAT_TRANS, ctl[AC_LOOKED]);
     stat_add(S, CNT_STAT_LOCAL, contexts);
   }
-  // ---- rows that were given up, swept by blocks that have nothing else to do any more: who gives one up comes here later itself.  Only
-  // blocks that look for tables wait, and who has tables waits for nobody.
-  for (bool given = ctl[AC_BASE] != 0u; given;) {
+  // ---- rows that were given up, swept by the blocks that gave them up when they have no row left.  Only blocks that look for tables
+  // wait, and who has tables waits for nobody.
+  while (gave_up) {
     __syncthreads();
     if (tid == 0) {
       uint32_t at = vload(&S.counters[CNT_AF_GIVEN_TAKEN]), got = 0xFFFFFFFFu, slot = 0xFFFFFFFFu;
@@ -1066,13 +870,13 @@ __global__ void __launch_bounds__(AF_THREADS, 4) automaton_fill_kernel(const __g
             __nanosleep(400);
           }
         }
-        ctl[AC_BASE] = v & 0xFFFFu;
+        ctl[AC_SLOT] = v & 0xFFFFu;
         __threadfence();
       }
       ctl[AC_JOB] = slot;
     }
     __syncthreads();
-    const uint32_t slot = ctl[AC_JOB], row = slot == 0xFFFFFFFFu ? 0u : S.jobs[ctl[AC_BASE]];
+    const uint32_t slot = ctl[AC_JOB], row = slot == 0xFFFFFFFFu ? 0u : S.jobs[ctl[AC_SLOT]];
     __syncthreads();
     if (slot == 0xFFFFFFFFu) break;
     // (copies: if the parameters themselves were passed by reference, the rounds above would read them anew each time they are used; 12
@@ -1096,33 +900,32 @@ __global__ void __launch_bounds__(AF_THREADS, 4) automaton_fill_kernel(const __g
 
 // ===================================================================================== launchers
 
-constexpr uint32_t AF_SMEM = (2 * AF_BATCH + 2 * AF_SPEC + AF_EXITS) * 16 + AF_SEEN * 8 + AF_OWNER * 2 + (5 * AF_CTX + AF_POOL + AF_CTX_HASH + AF_BATCH + 4 + AC_WORDS + AF_STAGE + AF_BUF + AF_WORK + AF_HSET) * 4;
-static_assert(block_sweep_words(AF_WARPS, MAX_NONTERMINALS / 32u) * 4u <= AF_SMEM, "a row that is given up is swept in the same shared memory");
+constexpr uint32_t AF_SMEM = (2 * AF_BATCH + AF_LISTS + AF_SEEN) * 8 + (5 * AF_CTX + AF_POOL + AF_CTX_HASH + 2 * AF_BATCH + AF_LISTS + AC_WORDS + AF_THREADS + AF_STAGE + AF_BUF + AF_WORK + AF_HSET) * 4 +
+                             (2 * AF_EDGES + AF_TOKENS) / 32 * 2;
+constexpr uint32_t AF_SWEEP_SMEM = block_sweep_words(AF_WARPS, MAX_NONTERMINALS / 32u) * 4u;  // a row that is given up is swept in the same shared memory
+constexpr uint32_t AF_SMEM_ASKED = AF_SMEM > AF_SWEEP_SMEM ? AF_SMEM : AF_SWEEP_SMEM;
 
-// Places of a block's stack that only its depth-first rounds use: two for each child along the longest path of the trie and one for
-// what is left of a special at each of its nodes, and what a round may hold or has put back when the last places above are taken.
-uint32_t automaton_fill_reserve(const GrammarDev& G) {
-  return 2u * G.ga_path + MAX_TOKEN_BYTES + 1u + 2u * (AF_BATCH + AF_SPEC) + 32u;
-}
+// Places of a block's stack that only its depth-first rounds use - what is left of an entry and what its edges start, along the longest
+// path of the trie - and the entries of a round that are put back.
+uint32_t automaton_fill_reserve() { return (MAX_TOKEN_BYTES + 2u) * (2u * AF_TIGHT_EDGES + 2u) + 3u * AF_BATCH; }
 uint32_t automaton_fill_warps() { return AF_WARPS; }
-uint32_t automaton_fill_least_stack(const GrammarDev& G) { return automaton_fill_reserve(G) + AF_TIGHT; }
+uint32_t automaton_fill_least_stack() { return automaton_fill_reserve() + AF_TIGHT + AF_SLICE; }
 
 void automaton_fill_layout(const GrammarDev& G, uint32_t rows, uint32_t max_blocks, AutoFillDev& A) {
-  A.reserve = automaton_fill_reserve(G);
+  A.reserve = automaton_fill_reserve();
   A.scratch_words = 7u * A.ctx_cap + A.pool_cap + A.big_cap / 4u + A.big_cap / 2u + A.big_cap;
-  A.unit_words = AU_WORDS;
   // few rows: several blocks take one, so that the chip is filled (a small trie gives the others nothing to do)
   A.parts = 1;
   while (A.parts < 8u && (uint64_t)rows * A.parts * 2u <= max_blocks && A.parts * 2048u <= G.T) A.parts *= 2u;
-  A.grid = (uint32_t)std::min<uint64_t>(max_blocks, (uint64_t)rows * std::max(A.parts, 1u + G.T / 16384u));
+  A.grid = (uint32_t)std::min<uint64_t>(max_blocks, (uint64_t)rows * A.parts);
 }
 
 cudaError_t configure_automaton_fill() {
-  return cudaFuncSetAttribute((const void*)automaton_fill_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, AF_SMEM);
+  return cudaFuncSetAttribute((const void*)automaton_fill_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, AF_SMEM_ASKED);
 }
 
 void launch_automaton_fill(const GrammarDev& G, const StateDev& S, cudaStream_t st) {
-  launch_overlapped(automaton_fill_kernel, dim3(S.af.grid), dim3(AF_THREADS), AF_SMEM, st, G, S);
+  launch_overlapped(automaton_fill_kernel, dim3(S.af.grid), dim3(AF_THREADS), AF_SMEM_ASKED, st, G, S);
 }
 
 }  // namespace fmt

@@ -38,17 +38,12 @@ struct GrammarDev {
   const uint32_t* tok_off;       // [T+1] tokens whose bytes end at node n (duplicates included)
   const uint32_t* tok_ids;
   // the grammar automaton over the vocabulary (see host_tables.h), if the grammar has one
-  uint32_t ga_on, ga_acc_mask;
-  const uint32_t* ga_item;       // [D][4]
-  const uint32_t* ga_trans;      // [sets][n_eq]
-  const uint32_t* ga_acc;        // [ga_acc_mask + 1][2]
-  const uint32_t* ga_node;       // [nodes][4]
+  uint32_t ga_on;
+  const uint32_t* ga_item;       // [D][2]
+  const uint32_t* ga_start;      // [D][4]
+  const uint32_t* ga_edge;       // [][4]
   const uint32_t* ga_tok;
-  uint32_t ga_lvl2, ga_lvl3;     // first nodes of depth 2 and 3
-  uint32_t ga_path;              // most children along a path
-  const uint32_t* ga_wide_rec;   // [entries][4]
-  const uint32_t* ga_wide_mask;  // [entries][Wm]
-  const uint32_t* ga_wide_exit;  // [][2]
+  const uint32_t* ga_mask;       // [][Wm]
   const uint32_t* vocab_off;     // [V+1]
   const uint8_t* vocab_bytes;
 };
@@ -109,10 +104,7 @@ enum : uint32_t {
   CNT_STAT_SWEPT = 192,        // 64-bit: rows that the automaton's fill gave up, and a block swept
   CNT_AF_GIVEN = 194,          // rows given up in this fill
   CNT_AF_GIVEN_TAKEN = 195,    // how many of them a block has taken
-  CNT_AF_TICKET = 196,         // shares of rows handed out to the blocks of the automaton's fill (these four are read together)
-  CNT_AF_TAKEN = 197,          // tickets drawn for units of work
-  CNT_AF_POSTED = 198,         // units given
-  CNT_AF_ACTIVE = 199,         // shares of rows, and units, that are not finished
+  CNT_AF_TICKET = 196,         // shares of rows handed out to the blocks of the automaton's fill
   CNT_TOTAL = 200
 };
 
@@ -255,24 +247,23 @@ struct CtxDev {
   uint32_t req2_cap;
 };
 
-// What the fill by the grammar automaton needs (automaton_fill.cu): per thread block a stack of threads and room for the
-// contexts of the row it works on, and units of work that blocks hand to one another.
+// What the fill by the grammar automaton needs (automaton_fill.cu): per thread block a stack of lists of edges and room for the
+// contexts of the row it works on.
 struct AutoFillDev {
   uint32_t on;               // rows are filled by the automaton
   uint32_t grid, parts;      // thread blocks, and how many of them share a row
-  uint4* stack;              // [grid][stack_cap] first child, children, code, context
+  uint4* stack;              // [grid][stack_cap] first edge, edges, context
   uint32_t stack_cap, reserve;  // and the places that are kept for rounds of one entry
   uint32_t* scratch;         // [grid][scratch_words]
   uint32_t scratch_words;
   uint32_t ctx_cap, pool_cap, big_cap;  // contexts per row, words for their lists, items of the largest expansion (powers of two)
-  uint32_t* units;           // [unit_cap][unit_words]
-  uint32_t* unit_flag;       // [unit_cap] the generation (StateDev::gen) of the fill whose unit is there; then per row that of the fill
-                             // in which its mask has been begun
+  uint32_t* row_begun;       // [rows, a multiple of four] the generation (StateDev::gen) of the fill in which the row's mask has been begun
   uint32_t* row_gone;        // [rows, a multiple of four; 16-byte aligned] the generation of the fill in which the row was given up
   uint32_t* given;           // [rows] the rows given up, generation << 16 | job
   uint32_t* sweep_lock;      // [sweep_slots] 1: a block sweeps a row in these tables (StateDev::au); 0 between launches
   uint32_t sweep_slots;
-  uint32_t unit_cap, unit_words, flag_words;  // (flag_words: unit_flag, row_gone and given together)
+  uint32_t flag_words;       // row_begun, row_gone and given together
+  uint32_t ahead;            // words that may be read from where a chart begins, however long it is
 };
 
 struct StateDev {

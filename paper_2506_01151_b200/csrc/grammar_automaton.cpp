@@ -5,12 +5,17 @@
 // begun in set o - everything that happens inside a token depends on d alone, except where the rule of d is completed
 // and o has to be asked who waited for it.  So the sets reached from {(d, here)} along byte strings, with the origin o left
 // open, can be hash-consed and their transitions tabulated once for a grammar and a vocabulary (Section 4.3 of the paper
-// keeps a context-independent part of the masks in the same spirit); a fill then walks the vocabulary trie by table look-ups
-// and runs Earley completions only where a rule of the chart ends (automaton_fill.cu).
+// keeps a context-independent part of the masks in the same spirit).
 //
 // Which transitions are needed follows from the vocabulary: the trie is walked once with the codes of all items that a
 // kernel can hold, and where a rule of non-terminal A ends inside a token the walk goes on, from that node, with every item that
 // completing A can yield in any chart of the grammar.
+//
+// What the fill gets (automaton_fill.cu) is no trie any more.  A START is an item at a trie node: an item of a chart's kernel at the root,
+// or one that completing a rule inside a token yields, at the node where the rule ends.  Its TOKENS are those below the node that end before
+// the item's own rule has: they are valid whatever the chart holds.  Where the rule ends with bytes still to come, the chart is
+// asked, and for every item that it can answer there is an EDGE to the start of that item at that node.  So a fill follows edges, one
+// for each rule that ends inside a token, and not the trie byte by byte.
 #include <algorithm>
 #include <cstring>
 #include <unordered_map>
@@ -31,8 +36,11 @@ constexpr u64 GA_MAX_TRANS = 32u << 20;   // table entries (4 bytes each)
 // Together half a second at most (10 to 15 ns each: HTML with 90 tags, 44 million 0.69 s; JSON, SQL and JSON schemas over 128 K tokens have
 // 0.5 to 4 million, 0.04 to 0.2 s).
 constexpr u64 GA_MAX_WORK = 16u << 20;
-constexpr size_t GA_MAX_WIDE = 32u << 20;  // words of the masks and lists of wide items
-constexpr size_t GA_WIDE_NODES = 1024;    // an item is wide from so many trie nodes on
+// Look-ups for the starts: those of JSON, SQL, JSON schemas and tagged unions over 128 K tokens take 0.3 to 1.6 times as many as that walk.
+constexpr u64 GA_MAX_START_WORK = 64u << 20;
+constexpr size_t GA_MAX_WORDS = 64u << 20;  // of masks, tokens and edges
+constexpr size_t GA_MASK_TOKENS = 1024;   // a kernel's item from which so many tokens follow has a mask in the place of a list
+constexpr u32 GA_EDGE_TOKENS = 2048;      // tokens of an edge at most (the others go to further edges)
 constexpr size_t GA_MAX_ITEMS = 1024;     // items of one set, predicted ones included: alternations of thousands of literals
                                           // would be scanned again for every set that predicts them
 
@@ -70,14 +78,13 @@ class Builder {
     follow();
     std::vector<u32> first;
     for (u32 d = 0; d < h_.D; ++d)
-      if (h_.ga_root[d] != GA_DEAD) first.push_back(h_.ga_root[d]);
+      if (root_[d] != GA_DEAD) first.push_back(root_[d]);
     dedupe(first, 0);
     arena_ = first;
     if (!too_big_) walk(0, 0, arena_.size());
     if (too_big_) return false;
-    wide_roots();
-    finish_tables();
-    return true;
+    starts();
+    return !too_big_;
   }
 
  private:
@@ -91,6 +98,10 @@ class Builder {
 
   HostTables& h_;
   const u32 n_eq_;
+  std::vector<u32> root_;                     // [D] code of the kernel {(d, open)}
+  // the vocabulary trie over byte classes, breadth first: [nodes][4] first child, children << 8 | byte class, the token (or where in tok_
+  // they begin), tokens
+  std::vector<u32> node_, tok_;
   uint8_t rep_[256];
   std::vector<Set> sets_;
   std::unordered_map<std::vector<u64>, u32, VecHash> ids_;
@@ -98,11 +109,12 @@ class Builder {
   std::unordered_map<u32, u32> accept_;
   std::vector<u64> cur_;
   std::vector<u32> arena_;
-  std::vector<std::vector<u32>> follow_;      // per non-terminal: codes of the items that completing it can yield
-  u64 work_ = 0, starts_ = 0, exit_nodes_ = 0;
+  std::vector<std::vector<u32>> follow_;      // per non-terminal: the items that completing it can yield,
+  std::vector<std::vector<u32>> codes_;       // and their codes
+  u64 work_ = 0, begun_ = 0, exit_nodes_ = 0;
   bool too_big_ = false;
 
-  const u32* node(u32 n) const { return &h_.ga_node[(size_t)n * 4]; }
+  const u32* node(u32 n) const { return &node_[(size_t)n * 4]; }
   u32 kind(u32 d) const { return h_.info[d] >> INFO_KIND_SHIFT; }
   u32 arg(u32 d) const { return h_.info[d] & INFO_ARG_MASK; }
 
@@ -229,13 +241,13 @@ class Builder {
     return r;
   }
 
-  // ga_root[d]: the code of the kernel {(d, open)}, nullable non-terminals skipped, for every item a kernel can hold
+  // root_[d]: the code of the kernel {(d, open)}, nullable non-terminals skipped, for every item a kernel can hold
   void roots() {
-    h_.ga_root.assign(h_.D, GA_DEAD);
+    root_.assign(h_.D, GA_DEAD);
     for (u32 d = 0; d < h_.D && !too_big_; ++d) {
       if (kind(d) == KIND_END) continue;
       if (kind(d) == KIND_DFA) {
-        h_.ga_root[d] = GA_ITEM | arg(d);
+        root_[d] = GA_ITEM | arg(d);
         continue;
       }
       const bool begins_rule = d != ITEM_START && (kind(d - 1) == KIND_END || d == 0);
@@ -243,7 +255,7 @@ class Builder {
       std::vector<u64> k;
       for (u32 j = 0; j <= h_.skip[d]; ++j)
         if (kind(d + j) != KIND_END) k.push_back(d + j);
-      h_.ga_root[d] = intern(k);
+      root_[d] = intern(k);
     }
   }
 
@@ -255,10 +267,10 @@ class Builder {
     for (u32 d = 0; d < h_.D; ++d) {
       if (kind(d) != KIND_NT) continue;
       const u32 a = arg(d), skip = h_.skip[d + 1];
-      if (kind(d + 1) != KIND_END) own[a].push_back(h_.ga_root[d + 1]);
+      if (kind(d + 1) != KIND_END) own[a].push_back(d + 1);
       if (kind(d + 1 + skip) == KIND_END) up[a].push_back(h_.lhs[d]);
     }
-    follow_.assign(N, {});
+    follow_.assign(N, {}), codes_.assign(N, {});
     for (u32 a = 0; a < N; ++a) {
       std::vector<char> seen(N, 0);
       std::vector<u32> work{a};
@@ -271,6 +283,8 @@ class Builder {
           if (!seen[y]) seen[y] = 1, work.push_back(y);
       }
       dedupe(follow_[a], 0);
+      for (u32 d : follow_[a]) codes_[a].push_back(root_[d]);
+      dedupe(codes_[a], 0);
     }
   }
 
@@ -301,34 +315,27 @@ class Builder {
       node[v] = val[s];
     }
     const u32 n = (u32)eq.size();
-    std::vector<u32> order(1, 0), number(n, 0), depth(1, 0), path(1, 0);
+    std::vector<u32> order(1, 0), number(n, 0);
     order.reserve(n);
-    h_.ga_path = 0;
-    h_.ga_node.assign((size_t)n * 4, 0u);
-    h_.ga_lvl2 = h_.ga_lvl3 = n;
+    node_.assign((size_t)n * 4, 0u);
     for (u32 i = 0; i < (u32)order.size(); ++i) {
-      u32* r = &h_.ga_node[(size_t)i * 4];
+      u32* r = &node_[(size_t)i * 4];
       r[0] = (u32)order.size();
       u32 kids = 0;
-      for (u32 c = child[order[i]]; c; c = sibling[c], ++kids) number[c] = (u32)order.size(), order.push_back(c), depth.push_back(depth[i] + 1);
+      for (u32 c = child[order[i]]; c; c = sibling[c], ++kids) number[c] = (u32)order.size(), order.push_back(c);
       r[1] = kids << 8 | eq[order[i]];
-      path[i] += kids;
-      h_.ga_path = std::max(h_.ga_path, path[i]);
-      path.resize(order.size(), path[i]);
-      if (depth[i] == 2) h_.ga_lvl2 = std::min(h_.ga_lvl2, i);
-      if (depth[i] == 3) h_.ga_lvl3 = std::min(h_.ga_lvl3, i);
     }
     std::vector<u32> count(n + 1, 0);  // tokens by node
     for (u32 v = 0; v < h_.T; ++v) count[number[node[v]] + 1] += h_.tok_off[v + 1] - h_.tok_off[v];
     for (u32 i = 0; i < n; ++i) count[i + 1] += count[i];
-    h_.ga_tok.assign(std::max<u32>(count[n], 1), 0);
+    tok_.assign(std::max<u32>(count[n], 1), 0);
     std::vector<u32> at(count.begin(), count.end() - 1);
     for (u32 v = 0; v < h_.T; ++v)
-      for (u32 k = h_.tok_off[v]; k < h_.tok_off[v + 1]; ++k) h_.ga_tok[at[number[node[v]]]++] = h_.tok_ids[k];
+      for (u32 k = h_.tok_off[v]; k < h_.tok_off[v + 1]; ++k) tok_[at[number[node[v]]]++] = h_.tok_ids[k];
     for (u32 i = 0; i < n; ++i) {  // a single token is named in the node itself
-      u32* r = &h_.ga_node[(size_t)i * 4];
+      u32* r = &node_[(size_t)i * 4];
       r[3] = count[i + 1] - count[i];
-      r[2] = r[3] == 1 ? h_.ga_tok[count[i]] : count[i];
+      r[2] = r[3] == 1 ? tok_[count[i]] : count[i];
     }
   }
 
@@ -344,15 +351,15 @@ class Builder {
         if (r == GA_DEAD || kids == 0) continue;
         if ((r & ~GA_EXIT) != GA_NONE) arena_.push_back(r & ~GA_EXIT);
         if (r & GA_EXIT) {
-          const auto& f = follow_[lhs_of(code)];
+          const auto& f = codes_[lhs_of(code)];
           arena_.insert(arena_.end(), f.begin(), f.end());
-          asks = true, starts_ += f.size();
+          asks = true, begun_ += f.size();
         }
       }
       if (asks) ++exit_nodes_;
-      const u64 nodes = h_.ga_node.size() / 4;
+      const u64 nodes = node_.size() / 4;
       if (exit_nodes_ > GA_EXITS && exit_nodes_ * GA_EXIT_SHARE > nodes) too_big_ = true;
-      if (starts_ > GA_STARTS * nodes + GA_STARTS_FREE) too_big_ = true;
+      if (begun_ > GA_STARTS * nodes + GA_STARTS_FREE) too_big_ = true;
       if (work_ > GA_MAX_WORK) too_big_ = true;
       dedupe(arena_, base);
       if (arena_.size() > base) walk(c, base, arena_.size());
@@ -360,83 +367,133 @@ class Builder {
     }
   }
 
-  // Items from which a large part of the vocabulary can follow (inside a string, mostly): the tokens that are valid whatever
-  // the chart holds, and the nodes where the chart has to be asked, are kept as a mask and a list.
-  void wide_roots() {
-    h_.ga_wide.assign(h_.D, GA_DEAD);
-    h_.ga_wide_rec.clear(), h_.ga_wide_mask.clear(), h_.ga_wide_exit.clear();
+  struct Start {
+    u32 node, code;
+    u32 tok = 0, n_tok = 0;    // in h_.ga_tok; the token itself if it is one
+    u32 link = 0, n_link = 0;  // in links: the starts that it has edges to, if anything follows from them
+    u32 edge = 0, n_edge = 0;  // in h_.ga_edge
+  };
+
+  // Is any child of node v reached from there?
+  bool goes_on(u32 v, u32 code) {
+    const u32 first = node(v)[0], end = first + (node(v)[1] >> 8);
+    for (u32 c = first; c < end; ++c)
+      if (next(code, node(c)[1] & 0xFFu) != GA_DEAD) return true;
+    return false;
+  }
+
+  // The starts with their tokens and edges, from the kernels' items on, and the items' records.
+  void starts() {
     work_ = 0;
-    std::unordered_map<u32, u32> known;  // items with one code share an entry
-    std::vector<u32> alive, mask(h_.Wm);
-    std::vector<std::pair<u32, u32>> work;  // (node, code)
-    std::vector<u32> exits;
-    for (u32 d = 0; d < h_.D; ++d) {
-      if (h_.ga_root[d] == GA_DEAD) continue;
-      const auto it = known.find(h_.ga_root[d]);
-      if (it != known.end()) {
-        h_.ga_wide[d] = it->second;
-        continue;
+    std::vector<Start> st;
+    std::vector<std::pair<u32, u32>> links, walked;  // (item, start); (node, code)
+    std::vector<u32> exits, toks, hash(1u << 12, 0u);  // hash: start + 1
+    h_.ga_tok.clear(), h_.ga_edge.clear(), h_.ga_mask.clear();
+    auto slot_of = [&](u32 v, u32 code) {
+      size_t s = (size_t)((((u64)v << 32 | code) + 1) * 0x9E3779B97F4A7C15ull >> 32) & (hash.size() - 1);
+      while (hash[s] && (st[hash[s] - 1].node != v || st[hash[s] - 1].code != code)) s = (s + 1) & (hash.size() - 1);
+      return s;
+    };
+    auto start = [&](u32 v, u32 code) -> u32 {
+      const size_t s = slot_of(v, code);
+      if (hash[s]) return hash[s] - 1;
+      st.push_back({v, code});
+      hash[s] = (u32)st.size();
+      if (st.size() * 2 > hash.size()) {
+        hash.assign(hash.size() * 4, 0u);
+        for (u32 i = 0; i < st.size(); ++i) hash[slot_of(st[i].node, st[i].code)] = i + 1;
       }
-      if (work_ > GA_MAX_WORK || h_.ga_wide_mask.size() + h_.ga_wide_exit.size() > GA_MAX_WIDE) break;
-      alive.clear(), exits.clear();
-      work.assign(1, {0u, h_.ga_root[d]});
-      while (!work.empty()) {
-        const auto [v, code] = work.back();
-        work.pop_back();
+      return (u32)st.size() - 1;
+    };
+    std::vector<u32> root_start(h_.D, GA_DEAD), mask_of;
+    for (u32 d = 0; d < h_.D; ++d)
+      if (root_[d] != GA_DEAD) root_start[d] = start(0, root_[d]);
+    const u32 roots = (u32)st.size();
+    mask_of.assign(roots, GA_DEAD);
+    for (u32 i = 0; i < (u32)st.size(); ++i) {
+      if (work_ > GA_MAX_START_WORK || h_.ga_tok.size() + h_.ga_mask.size() + 4 * links.size() > GA_MAX_WORDS) too_big_ = true;
+      if (too_big_) return;
+      walked.assign(1, {st[i].node, st[i].code});
+      exits.clear(), toks.clear();
+      while (!walked.empty()) {
+        const auto [v, code] = walked.back();
+        walked.pop_back();
         const u32 first = node(v)[0], end = first + (node(v)[1] >> 8);
         for (u32 c = first; c < end; ++c) {
           const u32 r = next(code, node(c)[1] & 0xFFu);
           if (r == GA_DEAD) continue;
-          alive.push_back(c);
+          if (node(c)[3] == 1) toks.push_back(node(c)[2]);
+          else toks.insert(toks.end(), tok_.begin() + node(c)[2], tok_.begin() + node(c)[2] + node(c)[3]);
           if ((node(c)[1] >> 8) == 0u) continue;
-          if ((r & ~GA_EXIT) != GA_NONE) work.push_back({c, r & ~GA_EXIT});
+          if ((r & ~GA_EXIT) != GA_NONE) walked.push_back({c, r & ~GA_EXIT});
           if (r & GA_EXIT) exits.push_back(c);
         }
       }
-      u32 id = GA_DEAD;
-      if (alive.size() >= GA_WIDE_NODES) {
-        id = (u32)h_.ga_wide_rec.size() / 4;
-        std::sort(exits.begin(), exits.end());
-        h_.ga_wide_rec.insert(h_.ga_wide_rec.end(), {id, (u32)h_.ga_wide_exit.size() / 2, (u32)exits.size(), 0u});
-        std::fill(mask.begin(), mask.end(), 0u);
-        for (u32 c : alive) {
-          if (node(c)[3] == 1) mask[node(c)[2] >> 5] |= 1u << (node(c)[2] & 31);
-          else
-            for (u32 k = 0; k < node(c)[3]; ++k) mask[h_.ga_tok[node(c)[2] + k] >> 5] |= 1u << (h_.ga_tok[node(c)[2] + k] & 31);
-        }
-        h_.ga_wide_mask.insert(h_.ga_wide_mask.end(), mask.begin(), mask.end());
-        for (u32 c : exits) h_.ga_wide_exit.push_back(node(c)[0]), h_.ga_wide_exit.push_back(node(c)[1] >> 8);
+      st[i].n_tok = (u32)toks.size();
+      if (i < roots && toks.size() >= GA_MASK_TOKENS) {
+        mask_of[i] = (u32)(h_.ga_mask.size() / h_.Wm);
+        h_.ga_mask.resize(h_.ga_mask.size() + h_.Wm, 0u);
+        u32* m = &h_.ga_mask[(size_t)mask_of[i] * h_.Wm];
+        for (u32 t : toks) m[t >> 5] |= 1u << (t & 31);
+      } else if (toks.size() == 1) {
+        st[i].tok = toks[0];
+      } else {
+        st[i].tok = (u32)h_.ga_tok.size();
+        h_.ga_tok.insert(h_.ga_tok.end(), toks.begin(), toks.end());
       }
-      h_.ga_wide[d] = id;
-      known.emplace(h_.ga_root[d], id);
+      std::sort(exits.begin(), exits.end());
+      const auto& f = follow_[lhs_of(st[i].code)];
+      st[i].link = (u32)links.size();
+      for (u32 c : exits)
+        for (u32 d : f)
+          if (root_[d] != GA_DEAD && goes_on(c, root_[d])) links.push_back({d, start(c, root_[d])});
+      st[i].n_link = (u32)links.size() - st[i].link;
     }
-  }
-
-  void finish_tables() {
-    h_.ga_sets = (u32)sets_.size();
-    h_.ga_item.assign((size_t)h_.D * 4, 0u);
+    // edges: deeper nodes have larger numbers, so what a start's edges lead to is there before it
+    std::vector<u32> order(st.size());
+    for (u32 i = 0; i < (u32)st.size(); ++i) order[i] = i;
+    std::sort(order.begin(), order.end(), [&](u32 a, u32 b) { return st[a].node > st[b].node; });
+    std::vector<char> reached(h_.D, 0);
+    for (u32 i : order) {
+      st[i].edge = (u32)(h_.ga_edge.size() / 4);
+      for (u32 k = st[i].link; k < st[i].link + st[i].n_link; ++k) {
+        const u32 d = links[k].first;
+        const Start& to = st[links[k].second];
+        if (to.n_tok == 0 && to.n_edge == 0) continue;
+        reached[d] = 1;
+        u32 n = std::min(to.n_tok, GA_EDGE_TOKENS);
+        h_.ga_edge.insert(h_.ga_edge.end(), {d << 16 | n, to.tok, to.edge, to.n_edge});
+        for (u32 at = n; at < to.n_tok; at += n) {
+          n = std::min(to.n_tok - at, GA_EDGE_TOKENS);
+          h_.ga_edge.insert(h_.ga_edge.end(), {d << 16 | n, n == 1 ? h_.ga_tok[to.tok + at] : to.tok + at, 0u, 0u});
+        }
+      }
+      st[i].n_edge = (u32)(h_.ga_edge.size() / 4) - st[i].edge;
+      if (h_.ga_tok.size() + h_.ga_mask.size() + h_.ga_edge.size() > GA_MAX_WORDS) {
+        too_big_ = true;
+        return;
+      }
+    }
+    h_.ga_start.assign((size_t)h_.D * 4, 0u);
+    h_.ga_item.assign((size_t)h_.D * 2, 0u);
     for (u32 d = 0; d < h_.D; ++d) {
-      u32* r = &h_.ga_item[(size_t)d * 4];
-      r[0] = h_.ga_root[d];
-      r[1] = h_.lhs[d] | 0xFFFF0000u;
-      r[2] = h_.ga_wide[d];
-      r[3] = 0xFFFFu;
+      u32* r = &h_.ga_item[(size_t)d * 2];
+      r[0] = h_.lhs[d] | 0xFFFF0000u;
+      r[1] = 0xFFFFu;
+      if (root_start[d] != GA_DEAD) {
+        const Start& s = st[root_start[d]];
+        const u32 mask = mask_of[root_start[d]];
+        u32* q = &h_.ga_start[(size_t)d * 4];
+        q[0] = mask != GA_DEAD ? mask : s.tok, q[1] = mask != GA_DEAD ? GA_MASK : s.n_tok;
+        q[2] = s.edge, q[3] = s.n_edge;
+        if (s.n_tok || s.n_edge) r[1] |= GA_ALIVE;
+      }
       if (kind(d) != KIND_NT) continue;
-      r[1] = h_.lhs[d] | arg(d) << 16;
+      r[0] = h_.lhs[d] | arg(d) << 16;
       const u32 skip = h_.skip[d + 1];
-      r[3] = (kind(d + 1) != KIND_END ? GA_GOES_ON : 0u) | (kind(d + 1 + skip) == KIND_END ? (u32)h_.lhs[d] : 0xFFFFu);
-      if ((h_.info[d] & INFO_NULLABLE) && h_.ga_root[d] != GA_DEAD) r[3] |= GA_SKIPS;
-    }
-    if (trans_.empty()) trans_.push_back(GA_UNKNOWN);
-    h_.ga_trans.swap(trans_);
-    u32 cap = 16;
-    while (cap < accept_.size() * 4) cap <<= 1;
-    h_.ga_acc_mask = cap - 1;
-    h_.ga_acc.assign((size_t)cap * 2, 0u);
-    for (const auto& kv : accept_) {
-      u32 s = ga_hash(kv.first) & h_.ga_acc_mask;
-      while (h_.ga_acc[2 * s]) s = (s + 1) & h_.ga_acc_mask;
-      h_.ga_acc[2 * s] = kv.first, h_.ga_acc[2 * s + 1] = kv.second;
+      if (kind(d + 1 + skip) == KIND_END) r[1] = (r[1] & ~0xFFFFu) | h_.lhs[d];
+      if (reached[d + 1]) r[1] |= GA_GOES_ON;
+      if ((h_.info[d] & INFO_NULLABLE) && root_[d] != GA_DEAD) r[1] |= GA_SKIPS;
     }
   }
 };
@@ -448,10 +505,7 @@ void build_grammar_automaton(HostTables& h) {
   if (h.D > 65535 || h.T >= (1u << 24)) return;
   Builder b(h);
   h.ga_on = b.run();
-  if (!h.ga_on) {
-    h.ga_root.clear();
-    h.ga_sets = 0;
-  }
+  if (!h.ga_on) h.ga_tok.clear(), h.ga_edge.clear(), h.ga_mask.clear();
 }
 
 }  // namespace fmt

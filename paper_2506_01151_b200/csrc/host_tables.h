@@ -27,17 +27,10 @@ constexpr uint32_t MAX_NONTERMINALS = 4096;
 // for a kernel that is one item inside an automaton of a regular non-terminal; with GA_EXIT where a rule begun in the open
 // origin is completed.  GA_NONE: nothing is left but completed items.
 constexpr uint32_t GA_DEAD = 0xFFFFFFFFu, GA_UNKNOWN = 0xFFFFFFFEu, GA_ITEM = 1u << 31, GA_EXIT = 1u << 30, GA_NONE = GA_EXIT - 1u;
-constexpr uint32_t GA_GOES_ON = 1u << 31;  // ga_item: the rule does not end with the post-dot non-terminal
+constexpr uint32_t GA_GOES_ON = 1u << 31;  // ga_item: when its non-terminal is completed, the item with the dot moved can be what a token goes on with
 constexpr uint32_t GA_SKIPS = 1u << 30;    // the kernel of the item holds the next item, too (the non-terminal is nullable)
-#ifdef __CUDACC__
-__host__ __device__
-#endif
-inline uint32_t ga_hash(uint32_t key) {
-  key ^= key >> 15;
-  key *= 0x2C1B3C6Du;
-  key ^= key >> 12;
-  return key;
-}
+constexpr uint32_t GA_ALIVE = 1u << 29;    // tokens follow from a kernel with this item
+constexpr uint32_t GA_MASK = 0xFFFFFFFFu;  // ga_start: the tokens are a mask
 
 struct CompileError {
   int code;
@@ -81,25 +74,19 @@ struct HostTables {
   std::vector<uint32_t> tok_ids;
   std::vector<uint32_t> lvl_off;    // [depth+2] nodes of depth L are lvl_off[L]..lvl_off[L+1]-1
   std::vector<uint32_t> tok_node;   // [V] node where the token's bytes end, 0xFFFFFFFF for empty tokens
-  // ---- the grammar automaton over this vocabulary (grammar_automaton.cpp), if it stays within its limits
+  // ---- what follows from one Earley item over this vocabulary (grammar_automaton.cpp), if it stays within its limits
   bool ga_on = false;
-  uint32_t ga_sets = 0, ga_acc_mask = 0;
-  std::vector<uint32_t> ga_root;   // [D] code of the kernel {(d, open)}
-  // per dotted rule d: ga_root[d] | left-hand side, post-dot non-terminal << 16 (0xFFFF if there is none) | wide entry or GA_DEAD |
-  // GA_* flags and the left-hand side if the rule may end right after that non-terminal, else 0xFFFF
-  std::vector<uint32_t> ga_item;   // [D][4]
-  std::vector<uint32_t> ga_trans;  // [ga_sets][n_eq] code
-  std::vector<uint32_t> ga_acc;    // [ga_acc_mask + 1][2] hash: set + 1 << 16 | automaton transition -> code
-  // the vocabulary trie over byte classes, breadth first
-  std::vector<uint32_t> ga_node;   // [nodes][4] first child, children << 8 | byte class, the token (or where in ga_tok they begin), tokens
-  std::vector<uint32_t> ga_tok;    // token ids by node
-  uint32_t ga_lvl2 = 0, ga_lvl3 = 0;  // first nodes of depth 2 and 3
-  uint32_t ga_path = 0;            // the children of a node and of all nodes above it, at most
-  // wide items: what follows from them alone
-  std::vector<uint32_t> ga_wide;       // [D] entry or GA_DEAD
-  std::vector<uint32_t> ga_wide_rec;   // [entries][4] mask row, first exit, exits
-  std::vector<uint32_t> ga_wide_mask;  // [entries][Wm] tokens that are valid whatever the chart holds
-  std::vector<uint32_t> ga_wide_exit;  // [][2] nodes (first child, children) at which the item's rule ends
+  // per dotted rule d: left-hand side | post-dot non-terminal << 16 (0xFFFF if there is none); GA_* flags and the left-hand side if the
+  // rule may end right after that non-terminal, else 0xFFFF
+  std::vector<uint32_t> ga_item;   // [D][2]
+  // per dotted rule d as an item of a chart's kernel: its tokens (one token, where in ga_tok they begin, or a row of ga_mask), how many
+  // (GA_MASK: a mask), first edge, edges
+  std::vector<uint32_t> ga_start;  // [D][4]
+  // where a rule ends inside a token: the item that goes on << 16 | its tokens (at most 65535), the token or where in ga_tok they begin,
+  // first edge, edges
+  std::vector<uint32_t> ga_edge;   // [][4]
+  std::vector<uint32_t> ga_tok;    // token ids
+  std::vector<uint32_t> ga_mask;   // [][Wm]
   std::vector<uint32_t> vocab_off;  // [V+1] byte offsets (32-bit) into vocab_bytes
   std::vector<uint8_t> vocab_bytes;
 };

@@ -381,7 +381,7 @@ __global__ void __launch_bounds__(1024) plan_kernel(const __grid_constant__ Gram
   if (threadIdx.x == 0) {
     S.counters[CNT_N_FJOBS] = 0u;
     S.counters[CNT_AUTO_ITEMS] = 0u;
-    S.counters[CNT_AF_TICKET] = S.counters[CNT_AF_TAKEN] = S.counters[CNT_AF_POSTED] = 0u;
+    S.counters[CNT_AF_TICKET] = 0u;
     S.counters[CNT_AF_GIVEN] = S.counters[CNT_AF_GIVEN_TAKEN] = 0u;
     n_jobs = n_cached = n_shared = 0u;
     n_rows = S.counters[CNT_N_MASK_ROWS];
@@ -430,7 +430,6 @@ __global__ void __launch_bounds__(1024) plan_kernel(const __grid_constant__ Gram
   if (threadIdx.x == 0) {
     S.counters[CNT_N_JOBS] = n_jobs;
     S.counters[CNT_N_MASK_ROWS] = min(n_rows, max(S.max_mask_rows, S.counters[CNT_N_MASK_ROWS]));
-    S.counters[CNT_AF_ACTIVE] = n_jobs * S.af.parts;
     stat_add(S, CNT_STAT_FILLS, S.B);
     if (n_cached) stat_add(S, CNT_STAT_CACHED, n_cached);
     if (n_shared) stat_add(S, CNT_STAT_SHARED, n_shared);

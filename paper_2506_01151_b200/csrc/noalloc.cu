@@ -52,11 +52,9 @@ constexpr size_t NA_SWEEP_WORDS = NA_OFF_REQ + 2 * (size_t)NA_REQ_CAP;
 constexpr uint32_t NA_FILL_BLOCKS = 160, NA_STACK = 12u << 10;
 constexpr uint32_t NA_CTX = 1024, NA_POOL = 8u << 10, NA_LARGE = 4u << 10;
 constexpr uint32_t NA_FILL_SCRATCH = 7u * NA_CTX + NA_POOL + NA_LARGE / 4u + NA_LARGE / 2u + NA_LARGE;
-constexpr uint32_t NA_UNITS = 512, NA_UNIT_WORDS = 4096;  // units of work between blocks
 constexpr size_t NA_OFF_FILL = NA_HEADER_WORDS + 4 * (size_t)NA_FILL_BLOCKS * NA_STACK;
-constexpr size_t NA_OFF_UNIT_FLAG = NA_OFF_FILL + (size_t)NA_FILL_BLOCKS * NA_FILL_SCRATCH;
-constexpr size_t NA_OFF_UNITS = NA_OFF_UNIT_FLAG + NA_UNITS + 3 * NA_MAX;
-static_assert(NA_OFF_UNITS + (size_t)NA_UNITS * NA_UNIT_WORDS <= NA_SWEEP_WORDS && NA_OFF_UNITS % 4 == 0, "the fill's tables do not fit");
+constexpr size_t NA_OFF_ROW_FLAGS = NA_OFF_FILL + (size_t)NA_FILL_BLOCKS * NA_FILL_SCRATCH;
+static_assert(NA_OFF_ROW_FLAGS + 3 * NA_MAX <= NA_SWEEP_WORDS, "the fill's tables do not fit");
 // behind both: tables of Earley sets for the charts that this fill gives up, one chart at a time
 constexpr uint32_t NA_BLOCK_WARPS = 8;
 constexpr size_t NA_ROW_ST_ENTRIES = 2u << 20;
@@ -68,7 +66,7 @@ constexpr size_t NA_OFF_ROW_ST = NA_OFF_ROW_ITEMS + NA_ITEM_WORDS;
 constexpr size_t NA_OFF_ROW_REQ = NA_OFF_ROW_ST + NA_ROW_ST_ENTRIES / 2;
 constexpr size_t NA_OFF_ROW_LOCK = NA_OFF_ROW_REQ + NA_REQ_CAP;
 constexpr size_t NA_WORDS = NA_OFF_ROW_LOCK + 4;
-static_assert(NA_OFF_UNIT_FLAG % 4 == 0 && NA_UNITS % 4 == 0 && NA_MAX % 4 == 0, "flags are read in 16-byte pieces");
+static_assert(NA_OFF_ROW_FLAGS % 4 == 0 && NA_MAX % 4 == 0, "flags are read in 16-byte pieces");
 static_assert(NA_OFF_ROW_BIG % 4 == 0 && (NA_ARENA_ITEMS + NA_HSET_SLOTS) % 4 == 0, "hash slots are cleared in 16-byte pieces");
 static_assert(CNT_TOTAL <= NA_OFF_JOBS, "the counters overlap the job list");
 static_assert(NA_OFF_JOBINFO + 4 * NA_MAX <= NA_HEADER_WORDS, "header too small");
@@ -106,7 +104,7 @@ __global__ void noalloc_prepare_kernel(GrammarDev G, StateDev S, uint32_t* scrat
   }
   for (size_t i = tid; i < (size_t)n * G.Wm; i += nth) mask[i] = 0u;
   if (S.af.on) {
-    if (tid < NA_UNITS + 3 * NA_MAX) S.af.unit_flag[tid] = 0u;
+    if (tid < 3 * NA_MAX) S.af.row_begun[tid] = 0u;
     if (tid == 0) *S.af.sweep_lock = 0u;
     return;
   }
@@ -147,7 +145,6 @@ __global__ void noalloc_jobs_kernel(StateDev S, const uint32_t* scratch, uint32_
   for (uint32_t r = 0; r < n; ++r)
     if (!scratch[NA_OFF_BAD + r]) S.jobs[j++] = r;
   S.counters[CNT_N_JOBS] = j;
-  S.counters[CNT_AF_ACTIVE] = j * S.af.parts;
 }
 
 __global__ void noalloc_finish_kernel(GrammarDev G, StateDev S, const uint32_t* scratch, uint32_t n, uint32_t* mask,
@@ -241,17 +238,16 @@ extern "C" fmt_status fmt_fill_mask_noalloc(const fmt_grammar* g, const uint32_t
   S.au.req_cap = NA_REQ_CAP;
   S.au.job_info = reinterpret_cast<uint4*>(scratch + NA_OFF_JOBINFO);
   sweep_layout(*G, &S.au.smem_bytes, &S.au.tables_in_smem);
-  if (G->ga_on && automaton_fill_least_stack(*G) <= NA_STACK && st_stride <= NA_ROW_ST_ENTRIES) {
+  if (G->ga_on && automaton_fill_least_stack() <= NA_STACK && st_stride <= NA_ROW_ST_ENTRIES) {
     AutoFillDev& A = S.af;
     A.on = 1;
     A.stack = reinterpret_cast<uint4*>(scratch + NA_HEADER_WORDS);
     A.stack_cap = NA_STACK;
     A.scratch = scratch + NA_OFF_FILL;
     A.ctx_cap = NA_CTX, A.pool_cap = NA_POOL, A.big_cap = NA_LARGE;
-    A.unit_cap = NA_UNITS;
-    A.units = scratch + NA_OFF_UNITS;
-    A.unit_flag = scratch + NA_OFF_UNIT_FLAG;
-    A.row_gone = A.unit_flag + NA_UNITS + NA_MAX, A.given = A.row_gone + NA_MAX;
+    A.ahead = CH_HDR;  // (the caller's memory may end with its last chart)
+    A.row_begun = scratch + NA_OFF_ROW_FLAGS;
+    A.row_gone = A.row_begun + NA_MAX, A.given = A.row_gone + NA_MAX;
     A.sweep_slots = 1, A.sweep_lock = scratch + NA_OFF_ROW_LOCK;
     S.big_scratch = scratch + NA_OFF_ROW_BIG;
     S.au.recs = scratch + NA_OFF_ROW_RECS;
@@ -261,7 +257,7 @@ extern "C" fmt_status fmt_fill_mask_noalloc(const fmt_grammar* g, const uint32_t
     S.au.req = reinterpret_cast<unsigned long long*>(scratch + NA_OFF_ROW_REQ);
     if (automaton_fill_warps() > NA_BLOCK_WARPS) return fail(FMT_ERR_CAPACITY, "the built-in scratch does not fit the fill");
     automaton_fill_layout(*G, n, NA_FILL_BLOCKS, A);
-    if (A.unit_words > NA_UNIT_WORDS || A.scratch_words > NA_FILL_SCRATCH) return fail(FMT_ERR_CAPACITY, "the built-in scratch does not fit the fill");
+    if (A.scratch_words > NA_FILL_SCRATCH) return fail(FMT_ERR_CAPACITY, "the built-in scratch does not fit the fill");
   }
   cudaStream_t st = (cudaStream_t)stream;
   noalloc_prepare_kernel<<<256, 256, 0, st>>>(*G, S, scratch, charts_dev, off, n, mask_dev);
