@@ -219,8 +219,18 @@ fmt_status fmt_compile(const char* ebnf, size_t ebnf_len, const char* start_rule
       const size_t o_clo = put(h.nt_closure.data(), h.nt_closure.size() * 4);
       const size_t o_doff = put(h.direct_off.data(), h.direct_off.size() * 4);
       const size_t o_dit = put(h.direct_items.data(), h.direct_items.size() * 2);
-      if (e == cudaSuccess) e = g->bufs.upload(blob, &d.hot_block);
       d.hot_words = (uint32_t)blob.size();
+      std::vector<uint16_t> pred(h.N + 1, 0);
+      for (uint32_t y = 0; y < h.N && pred.size() <= MAX_PREDICTED; ++y) {
+        for (uint32_t z = 0; z < h.N && pred.size() <= MAX_PREDICTED; ++z)
+          if ((h.nt_closure[(size_t)y * h.Nw + (z >> 5)] >> (z & 31)) & 1u)
+            pred.insert(pred.end(), h.direct_items.begin() + h.direct_off[z], h.direct_items.begin() + h.direct_off[z + 1]);
+        pred[y + 1] = (uint16_t)(pred.size() - (h.N + 1));
+      }
+      const size_t o_pred = pred.size() <= MAX_PREDICTED ? put(pred.data(), pred.size() * 2) : 0;
+      if (e == cudaSuccess) e = g->bufs.upload(blob, &d.hot_block);
+      d.pred_words = (uint32_t)blob.size() - d.hot_words;
+      d.pred = d.pred_words ? reinterpret_cast<const uint16_t*>(d.hot_block + o_pred) : nullptr;
       d.info = d.hot_block + o_info;
       d.lhs = reinterpret_cast<const uint16_t*>(d.hot_block + o_lhs);
       d.class_bits = d.hot_block + o_cls;

@@ -32,6 +32,9 @@ struct GrammarDev {
   // shared memory at once and shift the pointers.
   const uint32_t* hot_block;
   uint32_t hot_words;
+  // Behind them, if they are small: what is predicted with each non-terminal, [N+1] offsets and the items of its closure one after the other.
+  const uint16_t* pred;
+  uint32_t pred_words;
   const uint32_t* lvl_off;       // [depth+2]
   const uint32_t* tok_node;      // [V]
   const uint32_t* child_off;     // [T+1] children of node n are nodes child_off[n] .. child_off[n+1]-1
@@ -274,6 +277,7 @@ struct StateDev {
   uint32_t poll_limit_shift;  // bounded waits give up after 2^shift polls
   uint32_t time_steps;        // count the SM cycles spent inside Earley steps (costs a few per cent of the sweep)
   uint32_t adv_rows, adv_dfa;  // rows of a thread block when sequences advance; 1: their automata are in shared memory, too
+  uint32_t adv_pred;           // and the lists of predicted items
   uint32_t adv_no;             // calls so far
   uint32_t chart_words;       // capacity of one private chart buffer
   uint32_t cache_on;

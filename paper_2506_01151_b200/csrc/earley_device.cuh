@@ -43,6 +43,7 @@ struct WarpCtx {
 // 1 inserted, 0 already there, -1 table full
 __device__ __forceinline__ int hset_insert(uint32_t* hset, uint32_t mask, uint32_t key) {
   uint32_t h = mix32(key) & mask;
+  #pragma unroll 1
   for (uint32_t probe = 0; probe <= mask; ++probe) {
     uint32_t old = atomicCAS(&hset[h], EMPTY_SLOT, key);
     if (old == EMPTY_SLOT) return 1;
@@ -54,6 +55,7 @@ __device__ __forceinline__ int hset_insert(uint32_t* hset, uint32_t mask, uint32
 
 __device__ __forceinline__ void hset_clear_all(uint32_t* hset, uint32_t mask) {
   __syncwarp();
+  #pragma unroll 1
   for (uint32_t i = 4u * lane_id(); i <= mask; i += 128)  // (tables begin on 16 bytes and have a power of two of slots, at least 128)
     *reinterpret_cast<uint4*>(hset + i) = make_uint4(EMPTY_SLOT, EMPTY_SLOT, EMPTY_SLOT, EMPTY_SLOT);
   __syncwarp();
@@ -66,9 +68,11 @@ __device__ __forceinline__ void hset_clear_items(const WarpCtx& w, uint32_t n) {
     hset_clear_all(w.hset, w.hset_mask);
     return;
   }
+  #pragma unroll 1
   for (uint32_t i = lane_id(); i < n; i += 32) {
     uint32_t key = w.cur[i];
     uint32_t h = mix32(key) & w.hset_mask;
+    #pragma unroll 1
     for (uint32_t probe = 0; probe <= w.hset_mask; ++probe) {
       if (w.hset[h] == key) {
         w.hset[h] = EMPTY_SLOT;
@@ -84,6 +88,7 @@ __device__ __forceinline__ void hset_clear_items(const WarpCtx& w, uint32_t n) {
 // May be called by any subset of lanes.
 __device__ __forceinline__ void add_item(const GrammarDev& G, const WarpCtx& w, uint32_t key) {
   uint32_t n = (G.info[key & 0xFFFFu] >> INFO_SKIP_SHIFT) & INFO_SKIP_MASK;
+  #pragma unroll 1
   for (uint32_t j = 0; j <= n; ++j) {
     int r = hset_insert(w.hset, w.hset_mask, key + j);
     if (r == 1) {
@@ -132,6 +137,7 @@ __device__ __forceinline__ Scanned scan_item(const GrammarDev& G, uint32_t it, u
 // into cur.  Returns the number of items in cur afterwards (uniform over the warp).
 __device__ __forceinline__ uint32_t scan_into_cur(const GrammarDev& G, const WarpCtx& w, const uint32_t* set,
                                                   uint32_t len, uint32_t byte) {
+  #pragma unroll 1
   for (uint32_t k = lane_id(); k < len; k += 32) {
     uint32_t it = set[k];
     uint32_t inf = G.info[it & 0xFFFFu];
@@ -153,6 +159,7 @@ template <class View>
 __device__ __forceinline__ void complete_fixpoint(const GrammarDev& G, const WarpCtx& w, const View& view,
                                                   uint32_t cur_index, uint32_t head) {
   const uint32_t lane = lane_id();
+  #pragma unroll 1
   for (;;) {
     __syncwarp();
     uint32_t n = min(w.ctr[W_NCUR], w.cur_cap);
@@ -171,6 +178,7 @@ __device__ __forceinline__ void complete_fixpoint(const GrammarDev& G, const War
     if (have && kind == KIND_END && (it & 0xFFFFu) == ITEM_ACCEPT) w.ctr[W_ACCEPT] = 1u;
     bool done_item = have && kind == KIND_END && (it >> 16) != cur_index && (it & 0xFFFFu) != ITEM_ACCEPT;  // (nothing waits for the augmented start symbol)
     uint32_t bal = __ballot_sync(FULL, done_item);
+    #pragma unroll 1
     while (bal) {
       int src = __ffs(bal) - 1;
       bal &= bal - 1;
@@ -179,6 +187,7 @@ __device__ __forceinline__ void complete_fixpoint(const GrammarDev& G, const War
       const uint32_t* sp;
       uint32_t sl;
       view(o, sp, sl);
+      #pragma unroll 1
       for (uint32_t k = lane; k < sl; k += 32) {
         uint32_t wi = sp[k];
         uint32_t winf = G.info[wi & 0xFFFFu];
@@ -192,88 +201,132 @@ __device__ __forceinline__ void complete_fixpoint(const GrammarDev& G, const War
 }
 
 // Predict (Section 3.2) for all non-terminals collected in w.nt[0..Nw): append the start items of
-// every rule of every non-terminal in their closure, origin = cur_index.  These items are all new
-// (nothing else in the set has this origin), so no uniqueness check is needed.  One closure word
-// (32 non-terminals) per pass: a warp scan gives every lane the place of its non-terminal's items;
+// every rule of every non-terminal in their closure, origin = cur_index, to the n items of cur.  Returns their number, or
+// PREDICT_FULL.  These items are all new (nothing else in the set has this origin), so no uniqueness check is needed.  LISTS: where one
+// of the non-terminals pulls in all the others, and the items of its closure are listed (G.pred), they are copied.  Otherwise one
+// closure word (32 non-terminals) per pass: a warp scan gives every lane the place of its non-terminal's items;
 // short lists are copied by their lane, long ones (alternations of many literals) by the whole warp.
-__device__ __forceinline__ void predict_into_cur(const GrammarDev& G, const WarpCtx& w, uint32_t cur_index) {
+constexpr uint32_t PREDICT_FULL = 0xffffffffu;
+template <bool LISTS>
+__device__ __forceinline__ uint32_t predict_set(const GrammarDev& G, const WarpCtx& w, uint32_t n, uint32_t cur_index) {
   const uint32_t lane = lane_id();
   const uint32_t Nw = G.Nw;
   uint32_t* ntmask = w.nt;
   uint32_t* clos = w.nt + Nw;
   __syncwarp();
   uint32_t asked = 0u;
+#pragma unroll 1
   for (uint32_t i = lane; i < Nw; i += 32) asked |= ntmask[i];
-  if (!__any_sync(FULL, asked != 0u)) return;  // (inside literals and automata there is nothing to predict)
-  if (Nw <= 4u) {  // a lane for every non-terminal that is asked for: its row of the closure, joined over the lanes
-    for (uint32_t i = 0; i < Nw; ++i) {
-      uint32_t acc = 0u;
-      for (uint32_t wi = 0; wi < Nw; ++wi)
-        if ((ntmask[wi] >> lane) & 1u) acc |= G.nt_closure[(wi * 32u + lane) * Nw + i];
-      acc = __reduce_or_sync(FULL, acc);
-      if (lane == i) clos[i] = acc;
+  if (!__any_sync(FULL, asked != 0u)) return n;  // (inside literals and automata there is nothing to predict)
+  uint32_t one = 0xffffffffu;  // the non-terminal that pulls in all the others
+  if (LISTS && G.pred && Nw <= 4u) {
+#pragma unroll 1
+    for (uint32_t wi = 0; wi < Nw && one == 0xffffffffu; ++wi) {
+      bool mine = (ntmask[wi] >> lane) & 1u;
+      if (mine)
+#pragma unroll 1
+        for (uint32_t i = 0; i < Nw; ++i) mine = mine && (ntmask[i] & ~G.nt_closure[(wi * 32u + lane) * Nw + i]) == 0u;
+      const uint32_t b = __ballot_sync(FULL, mine);
+      if (b) one = wi * 32u + (uint32_t)__ffs(b) - 1u;
+    }
+  }
+  if (one != 0xffffffffu) {
+    const uint32_t lo = G.pred[one], len = G.pred[one + 1u] - lo;
+    const uint16_t* from = G.pred + G.N + 1u + lo;
+    if (n + len > w.cur_cap) n = PREDICT_FULL;
+    else {
+#pragma unroll 1
+      for (uint32_t i = lane; i < len; i += 32) w.cur[n + i] = (cur_index << 16) | (uint32_t)from[i];
+      n += len;
     }
   } else {
-    for (uint32_t i = lane; i < Nw; i += 32) {  // each lane owns some words of the closure
-      uint32_t acc = 0u;
-      for (uint32_t wi = 0; wi < Nw; ++wi) {
-        uint32_t bits = ntmask[wi];
-        while (bits) {
-          const uint32_t y = wi * 32u + (uint32_t)(__ffs(bits) - 1);
-          bits &= bits - 1;
-          acc |= G.nt_closure[y * Nw + i];
-        }
+    if (Nw <= 4u) {  // a lane for every non-terminal that is asked for: its row of the closure, joined over the lanes
+#pragma unroll 1
+      for (uint32_t i = 0; i < Nw; ++i) {
+        uint32_t acc = 0u;
+#pragma unroll 1
+        for (uint32_t wi = 0; wi < Nw; ++wi)
+          if ((ntmask[wi] >> lane) & 1u) acc |= G.nt_closure[(wi * 32u + lane) * Nw + i];
+        acc = __reduce_or_sync(FULL, acc);
+        if (lane == i) clos[i] = acc;
       }
-      clos[i] = acc;
+    } else {
+#pragma unroll 1
+      for (uint32_t i = lane; i < Nw; i += 32) {  // each lane owns some words of the closure
+        uint32_t acc = 0u;
+#pragma unroll 1
+        for (uint32_t wi = 0; wi < Nw; ++wi) {
+          uint32_t bits = ntmask[wi];
+#pragma unroll 1
+          while (bits) {
+            const uint32_t y = wi * 32u + (uint32_t)(__ffs(bits) - 1);
+            bits &= bits - 1;
+            acc |= G.nt_closure[y * Nw + i];
+          }
+        }
+        clos[i] = acc;
+      }
+    }
+    __syncwarp();
+#pragma unroll 1
+    for (uint32_t wi = 0; wi < Nw; ++wi) {
+      const uint32_t bits = clos[wi];
+      if (bits == 0u) continue;  // (uniform) most words of the closure are empty
+      uint32_t lo = 0, len = 0;
+      if ((bits >> lane) & 1u) {
+        const uint32_t z = wi * 32u + lane;
+        lo = G.direct_off[z];
+        len = G.direct_off[z + 1] - lo;
+      }
+      uint32_t incl = len;
+#pragma unroll
+      for (int d = 1; d < 32; d <<= 1) {
+        uint32_t t = __shfl_up_sync(FULL, incl, d);
+        if ((int)lane >= d) incl += t;
+      }
+      const uint32_t total = __shfl_sync(FULL, incl, 31);
+      if (n + total > w.cur_cap) {
+        n = PREDICT_FULL;
+        break;
+      }
+      const uint32_t at = n + incl - len;
+      const bool is_long = len > 8u;
+      if (!is_long)
+#pragma unroll 1
+        for (uint32_t i = 0; i < len; ++i) w.cur[at + i] = (cur_index << 16) | (uint32_t)G.direct_items[lo + i];
+      uint32_t longs = __ballot_sync(FULL, is_long);
+#pragma unroll 1
+      while (longs) {
+        const int src = __ffs(longs) - 1;
+        longs &= longs - 1;
+        const uint32_t slo = __shfl_sync(FULL, lo, src), slen = __shfl_sync(FULL, len, src), sat = __shfl_sync(FULL, at, src);
+#pragma unroll 1
+        for (uint32_t i = lane; i < slen; i += 32) w.cur[sat + i] = (cur_index << 16) | (uint32_t)G.direct_items[slo + i];
+      }
+      n += total;
     }
   }
   __syncwarp();
-  uint32_t n = min(w.ctr[W_NCUR], w.cur_cap);
-  bool over = false;
-  for (uint32_t wi = 0; wi < Nw; ++wi) {
-    const uint32_t bits = clos[wi];
-    if (bits == 0u) continue;  // (uniform) most words of the closure are empty
-    uint32_t lo = 0, len = 0;
-    if ((bits >> lane) & 1u) {
-      const uint32_t z = wi * 32u + lane;
-      lo = G.direct_off[z];
-      len = G.direct_off[z + 1] - lo;
-    }
-    uint32_t incl = len;
-    for (int d = 1; d < 32; d <<= 1) {
-      uint32_t t = __shfl_up_sync(FULL, incl, d);
-      if ((int)lane >= d) incl += t;
-    }
-    const uint32_t total = __shfl_sync(FULL, incl, 31);
-    if (n + total > w.cur_cap) {
-      over = true;
-      break;
-    }
-    const uint32_t at = n + incl - len;
-    const bool is_long = len > 8u;
-    if (!is_long)
-      for (uint32_t i = 0; i < len; ++i) w.cur[at + i] = (cur_index << 16) | (uint32_t)G.direct_items[lo + i];
-    uint32_t longs = __ballot_sync(FULL, is_long);
-    while (longs) {
-      const int src = __ffs(longs) - 1;
-      longs &= longs - 1;
-      const uint32_t slo = __shfl_sync(FULL, lo, src), slen = __shfl_sync(FULL, len, src), sat = __shfl_sync(FULL, at, src);
-      for (uint32_t i = lane; i < slen; i += 32) w.cur[sat + i] = (cur_index << 16) | (uint32_t)G.direct_items[slo + i];
-    }
-    n += total;
-  }
-  __syncwarp();
-  if (lane == 0) {
-    w.ctr[W_NCUR] = n;
-    if (over) w.ctr[W_OVERFLOW] = 1u;
-  }
+#pragma unroll 1
   for (uint32_t i = lane; i < Nw; i += 32) ntmask[i] = 0u;
+  __syncwarp();
+  return n;
+}
+// The same on the counters in shared memory.
+__device__ __forceinline__ void predict_into_cur(const GrammarDev& G, const WarpCtx& w, uint32_t cur_index) {
+  __syncwarp();
+  const uint32_t n = predict_set<false>(G, w, min(w.ctr[W_NCUR], w.cur_cap), cur_index);
+  if (lane_id() == 0) {
+    if (n == PREDICT_FULL) w.ctr[W_OVERFLOW] = 1u;
+    else w.ctr[W_NCUR] = n;
+  }
   __syncwarp();
 }
 
 // Is `key` in the uniqueness hash?
 __device__ __forceinline__ bool hset_contains(const uint32_t* hset, uint32_t mask, uint32_t key) {
   uint32_t h = mix32(key) & mask;
+  #pragma unroll 1
   for (uint32_t probe = 0; probe <= mask; ++probe) {
     const uint32_t v = hset[h];
     if (v == key) return true;
@@ -285,6 +338,7 @@ __device__ __forceinline__ bool hset_contains(const uint32_t* hset, uint32_t mas
 
 __device__ __forceinline__ void clear_nt(const GrammarDev& G, const WarpCtx& w) {
   __syncwarp();
+  #pragma unroll 1
   for (uint32_t i = lane_id(); i < 2 * G.Nw; i += 32) w.nt[i] = 0u;
   __syncwarp();
 }
@@ -301,10 +355,12 @@ constexpr uint32_t SMALL_OVERFLOW = 0xffffffffu;
 __device__ __forceinline__ uint32_t append_small(uint32_t c, bool v, uint32_t skip, uint32_t n, uint32_t& mine) {
   const uint32_t lane = lane_id();
   uint32_t vm = __ballot_sync(FULL, v);
+  #pragma unroll 1
   while (vm) {
     const int src = __ffs(vm) - 1;
     vm &= vm - 1;
     const uint32_t c0 = __shfl_sync(FULL, c, src), sk = __shfl_sync(FULL, skip, src);
+    #pragma unroll 1
     for (uint32_t j = 0; j <= sk; ++j) {
       const uint32_t cj = c0 + j;
       if (__ballot_sync(FULL, lane < n && mine == cj)) continue;  // already there
@@ -332,6 +388,7 @@ __device__ __forceinline__ uint32_t small_scan_complete(const GrammarDev& G, con
   mine = 0;
   accept = false;
   __syncwarp();
+  #pragma unroll 1
   for (uint32_t base = 0; base < len; base += 32) {
     const uint32_t k = base + lane;
     uint32_t it = k < len ? set[k] : 0u;
@@ -346,6 +403,7 @@ __device__ __forceinline__ uint32_t small_scan_complete(const GrammarDev& G, con
   }
   if (n == 0) return 0;
   uint32_t head = 0;  // lanes [head, n) hold the items not looked at yet
+  #pragma unroll 1
   while (head < n) {
     const bool have = lane >= head && lane < n;
     const uint32_t inf = have ? G.info[mine & 0xFFFFu] : 0u;
@@ -358,6 +416,7 @@ __device__ __forceinline__ uint32_t small_scan_complete(const GrammarDev& G, con
     uint32_t bal = __ballot_sync(FULL, have && kind == KIND_END && (mine >> 16) != cur_index && (mine & 0xFFFFu) != ITEM_ACCEPT);
     const uint32_t it = mine;
     head = n;
+    #pragma unroll 1
     while (bal) {
       const int src = __ffs(bal) - 1;
       bal &= bal - 1;
@@ -366,6 +425,7 @@ __device__ __forceinline__ uint32_t small_scan_complete(const GrammarDev& G, con
       const uint32_t* sp;
       uint32_t sl;
       view(o, sp, sl);
+      #pragma unroll 1
       for (uint32_t base = 0; base < sl; base += 32) {
         const uint32_t k = base + lane;
         const uint32_t wi = k < sl ? sp[k] : 0u;
@@ -408,6 +468,7 @@ __device__ __forceinline__ GrammarDev with_hot_tables(const GrammarDev& Gg, cons
   G.nt_closure = dst + (Gg.nt_closure - Gg.hot_block);
   G.direct_off = dst + (Gg.direct_off - Gg.hot_block);
   G.direct_items = reinterpret_cast<const uint16_t*>(dst + (reinterpret_cast<const uint32_t*>(Gg.direct_items) - Gg.hot_block));
+  if (Gg.pred) G.pred = reinterpret_cast<const uint16_t*>(dst + (reinterpret_cast<const uint32_t*>(Gg.pred) - Gg.hot_block));
   G.hot_block = dst;
   return G;
 }
@@ -415,6 +476,7 @@ __device__ __forceinline__ GrammarDev with_hot_tables(const GrammarDev& Gg, cons
 // Copy the grammar's hot tables into shared memory (all threads of the block take part, the
 // caller synchronizes) and return a view of the grammar that reads them from there.
 __device__ __forceinline__ GrammarDev stage_hot_tables(const GrammarDev& Gg, uint32_t* dst) {
+  #pragma unroll 1
   for (uint32_t i = threadIdx.x; i < Gg.hot_words / 4u; i += blockDim.x)  // (the block is a multiple of 16 bytes)
     reinterpret_cast<uint4*>(dst)[i] = __ldg(reinterpret_cast<const uint4*>(Gg.hot_block) + i);
   return with_hot_tables(Gg, dst);
@@ -425,6 +487,7 @@ __device__ __forceinline__ uint32_t drop_completed(const GrammarDev& G, const Wa
   const uint32_t lane = lane_id();
   uint32_t out = 0;
   __syncwarp();
+  #pragma unroll 1
   for (uint32_t base = 0; base < n; base += 32) {
     uint32_t idx = base + lane;
     bool have = idx < n;
@@ -446,6 +509,7 @@ __device__ __forceinline__ void scannable_bytes(const GrammarDev& G, const uint3
   uint32_t acc[8];
 #pragma unroll
   for (int i = 0; i < 8; ++i) acc[i] = 0u;
+  #pragma unroll 1
   for (uint32_t k = lane_id(); k < len; k += 32) {
     uint32_t inf = G.info[set[k] & 0xFFFFu];
     const uint32_t kind = inf >> INFO_KIND_SHIFT;
@@ -467,34 +531,22 @@ __device__ __forceinline__ void scannable_bytes(const GrammarDev& G, const uint3
   __syncwarp();
 }
 
-// Ascending bitonic sort of a[0..n); the array must have room for the next power of two >= max(n, 32),
-// which must not exceed cap_pow2.
-__device__ __forceinline__ void sort_items(uint32_t* a, uint32_t n, uint32_t cap_pow2) {
+// Ascending bitonic sort of a[0..n), n > 32; the array must have room for the next power of two >= n, which must not exceed cap_pow2.
+static __device__ __noinline__ void sort_large(uint32_t* a, uint32_t n, uint32_t cap_pow2) {
   const uint32_t lane = lane_id();
-  if (n <= 32) {  // one item per lane, compare-exchange through shuffles
-    __syncwarp();
-    uint32_t v = (lane < n) ? a[lane] : 0xffffffffu;
-#pragma unroll
-    for (uint32_t k = 2; k <= 32; k <<= 1) {
-#pragma unroll
-      for (uint32_t j = k >> 1; j > 0; j >>= 1) {
-        const uint32_t other = __shfl_xor_sync(FULL, v, j);
-        const bool up = (lane & k) == 0, lower = (lane & j) == 0;
-        v = (lower == up) ? min(v, other) : max(v, other);
-      }
-    }
-    if (lane < n) a[lane] = v;
-    __syncwarp();
-    return;
-  }
   uint32_t P = 32;
+#pragma unroll 1
   while (P < n) P <<= 1;
   if (P > cap_pow2) P = cap_pow2;
   __syncwarp();
+#pragma unroll 1
   for (uint32_t i = n + lane; i < P; i += 32) a[i] = 0xffffffffu;
   __syncwarp();
+#pragma unroll 1
   for (uint32_t k = 2; k <= P; k <<= 1) {
+#pragma unroll 1
     for (uint32_t j = k >> 1; j > 0; j >>= 1) {
+#pragma unroll 1
       for (uint32_t i = lane; i < P; i += 32) {
         uint32_t l = i ^ j;
         if (l > i) {
@@ -509,6 +561,25 @@ __device__ __forceinline__ void sort_items(uint32_t* a, uint32_t n, uint32_t cap
       __syncwarp();
     }
   }
+}
+
+// The same for any n (room for at least 32).
+__device__ __forceinline__ void sort_items(uint32_t* a, uint32_t n, uint32_t cap_pow2) {
+  if (n > 32) return sort_large(a, n, cap_pow2);
+  const uint32_t lane = lane_id();  // one item per lane, compare-exchange through shuffles
+  __syncwarp();
+  uint32_t v = (lane < n) ? a[lane] : 0xffffffffu;
+#pragma unroll
+  for (uint32_t k = 2; k <= 32; k <<= 1) {
+#pragma unroll
+    for (uint32_t j = k >> 1; j > 0; j >>= 1) {
+      const uint32_t other = __shfl_xor_sync(FULL, v, j);
+      const bool up = (lane & k) == 0, lower = (lane & j) == 0;
+      v = (lower == up) ? min(v, other) : max(v, other);
+    }
+  }
+  if (lane < n) a[lane] = v;
+  __syncwarp();
 }
 
 }  // namespace fmt

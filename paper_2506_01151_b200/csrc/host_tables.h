@@ -22,6 +22,7 @@ constexpr uint32_t ITEM_START = 0;   // $ -> . start
 constexpr uint32_t ITEM_ACCEPT = 1;  // $ -> start .
 constexpr uint32_t MAX_TOKEN_BYTES = 32;
 constexpr uint32_t MAX_NONTERMINALS = 4096;
+constexpr size_t MAX_PREDICTED = 4096;  // 16-bit words of the lists of what is predicted with each non-terminal (grammars with more have none)
 
 // Codes of the grammar automaton: the number of a set, or GA_ITEM | (set + 1, or 0 for the open origin) << 14 | state
 // for a kernel that is one item inside an automaton of a regular non-terminal; with GA_EXIT where a rule begun in the open

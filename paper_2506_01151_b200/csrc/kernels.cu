@@ -181,7 +181,7 @@ __device__ __forceinline__ void advance_copy_tables(const GrammarDev& G, const S
       asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst + i)), "l"(src + i) : "memory");
     dst += words;
   };
-  if (HOT) copy(G.hot_block, G.hot_words);
+  if (HOT) copy(G.hot_block, G.hot_words + (S.adv_pred ? G.pred_words : 0u));
   if (DFA) copy(G.dfa_block, G.dfa_words);
 }
 __device__ __forceinline__ AdvScratch advance_scratch(const StateDev& S, uint32_t* smem) {
@@ -200,7 +200,8 @@ __device__ __forceinline__ GrammarDev advance_tables(const GrammarDev& Gg, const
   __syncthreads();
   const uint32_t* at = advance_table_space(S, smem);
   GrammarDev G = Gg;
-  if (HOT) G = with_hot_tables(Gg, at), at += Gg.hot_words;
+  if (HOT) G = with_hot_tables(Gg, at), at += Gg.hot_words + (S.adv_pred ? Gg.pred_words : 0u);
+  if (!HOT || !S.adv_pred) G.pred = nullptr;
   if (DFA) {
     G.dfa_done = reinterpret_cast<const uint16_t*>(at + (reinterpret_cast<const uint32_t*>(Gg.dfa_done) - Gg.dfa_block));
     G.dfa_trans = reinterpret_cast<const uint16_t*>(at);
@@ -223,7 +224,8 @@ __global__ void __launch_bounds__(ADV_WARPS * 32, 1) advance_kernel(const __grid
   AdvScratch s = advance_scratch(S, smem);
   before_me();
   const int32_t tok = row < S.B ? tokens[row] : -1;
-  uint32_t flags = 0, b0 = 0, b1 = 0;
+  uint32_t flags = 0, b0 = 0, b1 = 0, own_byte = 0, held = 0;
+  ChartAhead ahead;
   int32_t sid = -1;
   const uint32_t* cur = nullptr;
   auto finish = [&](int32_t st) {
@@ -236,11 +238,13 @@ __global__ void __launch_bounds__(ADV_WARPS * 32, 1) advance_kernel(const __grid
     flags = S.row_flags[row];
     sid = S.cache_on ? S.row_state[row] : -1;
     cur = S.arena + S.row_chart[row];
+    held = S.row_buf[row];
     if (tok == -1) return finish(FMT_OK), false;
     if (flags & ROW_FINISHED) return finish(FMT_ERR_FINISHED), false;
     if (tok < 0 || (uint32_t)tok >= Gg.V) return finish(FMT_ERR_INVALID_ARG), false;
     if (flags & ROW_BROKEN) return finish(FMT_ERR_CAPACITY), false;
     b0 = __ldg(&Gg.vocab_off[tok]), b1 = __ldg(&Gg.vocab_off[tok + 1]);
+    ahead = read_ahead(cur);  // (under way while it is looked up whether they are needed)
     // has this chart been advanced by this token before?  (Section 5.2: the state cache)
     int32_t known = TR_UNSET;
     if (lane == 0 && sid >= 0 && tok != Gg.eos) known = tr_lookup(S, sid, (uint32_t)tok);
@@ -251,7 +255,10 @@ __global__ void __launch_bounds__(ADV_WARPS * 32, 1) advance_kernel(const __grid
       return finish(FMT_OK), false;
     }
     if (b1 == b0 || known == TR_REJECT) return finish(FMT_ERR_TOKEN_REJECTED), false;
-    if (known < 0 || (uint32_t)known >= S.max_states) return true;
+    if (known < 0 || (uint32_t)known >= S.max_states) {
+      if (lane < b1 - b0) own_byte = __ldg(&Gg.vocab_bytes[b0 + lane]);
+      return true;
+    }
     if (lane == 0) {
       S.row_state[row] = known;
       S.st_ref[known] = 1;
@@ -285,14 +292,15 @@ __global__ void __launch_bounds__(ADV_WARPS * 32, 1) advance_kernel(const __grid
     else if (tr_there != tr_pair) tr_insert(S, sid, (uint32_t)tok, val);
   };
   // a private buffer that does not hold the current chart
-  const uint32_t held = S.row_buf[row];
   const uint32_t final_buf = (held == 0) ? 1u : 0u;
   uint32_t* dst = private_buf(S, row, final_buf);
   uint32_t* const sm_arena = s.w.cur;
-  const bool staged = stage_chart(s, cur);
+  const bool staged = stage_chart(s, cur, ahead);
+  const uint32_t* const src = staged ? s.stage : cur;
+  const uint32_t src_words = src[CH_WORDS];
   int r;
-  if (HOT && staged) r = token_steps(G, s, s.stage, G.vocab_bytes + b0, b1 - b0, dst, S.chart_words, sm_arena, ADV_CUR_CAP, nullptr);
-  else r = token_step(G, s, staged ? s.stage : cur, G.vocab_bytes + b0, b1 - b0, dst, S.chart_words, sm_arena, ADV_CUR_CAP);
+  if (HOT && staged) r = token_steps(G, s, s.stage, own_byte, b1 - b0, dst, S.chart_words, sm_arena, ADV_CUR_CAP, nullptr);
+  else r = token_step(G, s, src, own_byte, b1 - b0, dst, S.chart_words, sm_arena, ADV_CUR_CAP);
   if (r == -2) {  // the token's sets outgrew shared memory: use the row's third private buffer as the arena
     uint32_t* big = private_buf(S, row, 2);
     uint32_t cap = 32;
@@ -300,7 +308,7 @@ __global__ void __launch_bounds__(ADV_WARPS * 32, 1) advance_kernel(const __grid
     hset_clear_all(s.w.hset, s.w.hset_mask);
     for (uint32_t i = lane; i < ADV_NT_WORDS; i += 32) s.w.nt[i] = 0u;
     __syncwarp();
-    r = (held == 2) ? -1 : token_step(G, s, staged ? s.stage : cur, G.vocab_bytes + b0, b1 - b0, dst, S.chart_words, big, cap);
+    r = (held == 2) ? -1 : token_step(G, s, src, own_byte, b1 - b0, dst, S.chart_words, big, cap);
   }
   if (r == 0) {
     if (sid >= 0 && lane == 0) remember(TR_REJECT);
@@ -314,14 +322,18 @@ __global__ void __launch_bounds__(ADV_WARPS * 32, 1) advance_kernel(const __grid
     }
     return finish(FMT_ERR_CAPACITY);
   }
+  const uint32_t* const made = s.out;
+  const uint32_t made_words = made[CH_WORDS];
   if (lane == 0) {
     stat_add(S, CNT_STAT_ADV, 1u);
-    stat_max(S, CNT_STAT_ITEMS_MAX, dst[CH_ITEMS]);
-    stat_max(S, CNT_STAT_SETS_MAX, dst[CH_SETS]);
-    stat_add(S, CNT_STAT_ADV_WORDS, cur[CH_WORDS] + dst[CH_WORDS]);
+    stat_max(S, CNT_STAT_ITEMS_MAX, made[CH_ITEMS]);
+    stat_max(S, CNT_STAT_SETS_MAX, made[CH_SETS]);
+    stat_add(S, CNT_STAT_ADV_WORDS, src_words + made_words);
   }
   uint64_t off;
-  int32_t id = intern_chart(S, dst, off);
+  int32_t id = intern_chart(S, made, off);
+  if (id < 0 && made != dst)  // it stays the row's own
+    for (uint32_t i = lane; i < made_words; i += 32) dst[i] = made[i];
   if (lane == 0) {
     if (sid >= 0 && id >= 0) remember(id);
     S.row_state[row] = id;
@@ -358,9 +370,9 @@ __global__ void __launch_bounds__(ADV_WARPS * 32, 1) forced_kernel(const __grid_
   if (!(S.row_flags[row] & (ROW_FINISHED | ROW_BROKEN)) && max_len > 0) {
     const uint32_t* cur = S.arena + S.row_chart[row];
     uint8_t* const out = bytes_out + (size_t)row * stride;
-    const bool staged = stage_chart(s, cur);
-    if (HOT && staged) n = token_steps(G, s, s.stage, nullptr, min(max_len, MAX_TOKEN_BYTES), nullptr, 0u, s.w.cur, ADV_CUR_CAP, out);
-    else n = token_step(G, s, staged ? s.stage : cur, nullptr, min(max_len, MAX_TOKEN_BYTES), nullptr, 0u, s.w.cur, ADV_CUR_CAP, out);
+    const bool staged = stage_chart(s, cur, read_ahead(cur));
+    if (HOT && staged) n = token_steps(G, s, s.stage, 0u, min(max_len, MAX_TOKEN_BYTES), nullptr, 0u, s.w.cur, ADV_CUR_CAP, out);
+    else n = token_step(G, s, staged ? s.stage : cur, 0u, min(max_len, MAX_TOKEN_BYTES), nullptr, 0u, s.w.cur, ADV_CUR_CAP, out);
     if (n < 0) n = 0;
   }
   if (lane == 0) len_out[row] = (uint32_t)n;
@@ -1050,14 +1062,18 @@ static inline cudaError_t opt_in_smem(const void* fn, size_t bytes) {
 }
 
 static size_t adv_smem_bytes(const GrammarDev& G, const StateDev& S) {
-  return ((size_t)S.adv_rows * ADV_WARP_WORDS + (G.hot_words * 4u <= HOT_TABLE_BYTES ? G.hot_words : 0u) + (S.adv_dfa ? G.dfa_words : 0u)) * 4;
+  const uint32_t tables = G.hot_words * 4u <= HOT_TABLE_BYTES ? G.hot_words + (S.adv_pred ? G.pred_words : 0u) : 0u;
+  return ((size_t)S.adv_rows * ADV_WARP_WORDS + tables + (S.adv_dfa ? G.dfa_words : 0u)) * 4;
 }
 // One row to a block as long as all rows run at once: a block then has room for its grammar's automata (JSON 6 KB, a schema of
 // twelve members 60 KB).  Else two or four, with the automata if they fit.
 void advance_layout(const GrammarDev& G, uint32_t rows, uint32_t sms, StateDev& S) {
   for (S.adv_rows = 1;; S.adv_rows *= 2) {
+    S.adv_pred = 0;
     S.adv_dfa = G.dfa_words && G.hot_words * 4u <= HOT_TABLE_BYTES ? 1u : 0u;
     if (S.adv_dfa && adv_smem_bytes(G, S) > ADV_SMEM_LIMIT) S.adv_dfa = 0;
+    S.adv_pred = 1u;
+    if (adv_smem_bytes(G, S) > ADV_SMEM_LIMIT) S.adv_pred = 0;
     const uint64_t blocks = (uint64_t)sms * (ADV_SMEM_SM / (adv_smem_bytes(G, S) + 1024));
     if (S.adv_rows == (uint32_t)ADV_WARPS || blocks * S.adv_rows >= rows) return;
   }
