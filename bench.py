@@ -202,8 +202,8 @@ class Driver:
         self.state.advance(self.tokens[i], self.status, stream=s)
         lg = self.ring[i % self.n_ring] if logits is None else logits
         self.state.fill_and_apply(lg, self.fmt.BF16, stream=s)
-        # advance; plan, [entry look-up (2), sweep of new entries, its collection, job set-up], fill, mask+apply
-        self.launches += 9 if self.roots else 4
+        # advance; [plan, entry look-up (2), sweep of new entries, its collection, job set-up,] fill, mask+apply
+        self.launches += 9 if self.roots else 3
 
     def restart(self, warmup: int, clear_caches: bool):
         """Back to the start of the token stream: all rows reset, prefixes fed, `warmup` untimed steps."""

@@ -143,7 +143,8 @@ static cudaError_t next_generations(fmt_state* s, cudaStream_t st) {
   StateDev& d = s->dev;
   cudaError_t e = cudaSuccess;
   if (s->next_gen + 1u > 65534u) {
-    if (d.af.on) e = cudaMemsetAsync(d.af.row_begun, 0, (size_t)d.af.flag_words * 4, st);
+    if (d.af.on) e = cudaMemsetAsync(d.af.given, 0, (size_t)d.B * 4, st);
+    if (e == cudaSuccess && d.af.on) e = cudaMemsetAsync(d.counters + CNT_BAR_ERR, 0, 4, st);
     if (e == cudaSuccess && !d.af.on) e = cudaMemsetAsync(d.au.hash, 0, (size_t)d.B * (d.au.hash_mask + 1u) * 4, st);
     if (e == cudaSuccess && !d.af.on) e = cudaMemsetAsync(d.au.req, 0, (size_t)d.au.req_cap * 8, st);
     if (e == cudaSuccess && d.rt.on) e = cudaMemsetAsync(d.cx.ctab, 0, (size_t)d.B * CT_SLOTS * 8, st);
@@ -266,6 +267,7 @@ fmt_status fmt_compile(const char* ebnf, size_t ebnf_len, const char* start_rule
       UP(ga_edge);
       UP(ga_tok);
       UP(ga_mask);
+      d.ga_mask_words = (h.Wm + 3u) & ~3u;
     }
     UP(vocab_off);
     UP(vocab_bytes);
@@ -514,7 +516,7 @@ fmt_status fmt_state_create(const fmt_grammar* g, uint32_t batch, const fmt_stat
     af.stack_cap = std::max(32u << 10, automaton_fill_least_stack());
     af.ctx_cap = 1024, af.pool_cap = 16u << 10, af.big_cap = 64u << 10;
     af.ahead = ADV_AHEAD;
-    automaton_fill_layout(g->dev, batch, AUTO_FILL_PER_SM * (uint32_t)std::max(1, sms), af);
+    automaton_fill_layout(batch, AUTO_FILL_PER_SM * (uint32_t)std::max(1, sms), af);
   }
 #define AL(ptr, count, fill) if (e == cudaSuccess) e = s->bufs.alloc((size_t)(count), &(ptr), (fill))
   AL(d.arena, d.pool_base + d.pool_words * (two_gens ? 2 : 1) + ADV_AHEAD, 0);
@@ -546,12 +548,9 @@ fmt_status fmt_state_create(const fmt_grammar* g, uint32_t batch, const fmt_stat
   if (af.on) {
     AL(af.stack, (size_t)af.grid * af.stack_cap, 0);
     AL(af.scratch, (size_t)af.grid * af.scratch_words, 0);
-    // (behind the flags, which carry the fills' generations, the locks of the tables below)
     af.sweep_slots = std::min(batch, 16u);
-    const uint32_t rows4 = (batch + 3u) & ~3u;
-    af.flag_words = 3u * rows4;
-    AL(af.row_begun, af.flag_words + af.sweep_slots, 0);
-    af.row_gone = af.row_begun + rows4, af.given = af.row_gone + rows4, af.sweep_lock = af.given + rows4;
+    AL(af.given, batch + af.sweep_slots, 0);
+    af.sweep_lock = af.given + batch;
     if (e == cudaSuccess) e = alloc_row_sweeps(s);
   } else if (e == cudaSuccess) {
     e = alloc_sweep(s);

@@ -1002,7 +1002,7 @@ cudaError_t configure_walk_kernels() {
 
 void launch_fill(const GrammarDev& G, const StateDev& S, int sweep_grid, cudaStream_t st, cudaEvent_t before_roots,
                  cudaEvent_t after_roots, cudaEvent_t before_sweep, cudaEvent_t after_sweep) {
-  launch_plan(G, S, st);
+  if (!S.af.on) launch_plan(G, S, st);
   if (!S.rt.on) {
     // without the cache of context-independent entries every row is swept from its chart's last set
     if (before_sweep) cudaEventRecord(before_sweep, st);

@@ -46,7 +46,8 @@ struct GrammarDev {
   const uint32_t* ga_start;      // [D][4]
   const uint32_t* ga_edge;       // [][4]
   const uint32_t* ga_tok;
-  const uint32_t* ga_mask;       // [][Wm]
+  const uint32_t* ga_mask;       // [][ga_mask_words]
+  uint32_t ga_mask_words;        // Wm, a multiple of four (rows are read in 16-byte pieces)
   const uint32_t* vocab_off;     // [V+1]
   const uint8_t* vocab_bytes;
 };
@@ -84,7 +85,7 @@ enum : uint32_t {
   CNT_STAT_TRANS = 26,  // transitions computed by the trie sweep (Earley steps)
   CNT_STAT_LOCAL = 28,  // local states created by the trie sweep
   CNT_BAR = 30,         // grid barrier of the trie sweep: arrivals
-  CNT_BAR_ERR = 31,     // a block gave up waiting at the barrier
+  CNT_BAR_ERR = 31,     // a block gave up waiting: 1, or, where rows are filled by the automaton, the generation of the fill in which one did
   CNT_LEVEL_ALIVE = 32, // [MAX_TOKEN_BYTES + 2] per trie depth: some node of some job was alive
   CNT_LEVEL_REQ = 68,   // [MAX_TOKEN_BYTES + 2] per trie depth: transitions queued for computation
   CNT_HASH_GEN = 104,   // (the depth counters that every fill clears end here; the fills' generations are handed out by the host)
@@ -107,7 +108,7 @@ enum : uint32_t {
   CNT_STAT_SWEPT = 192,        // 64-bit: rows that the automaton's fill gave up, and a block swept
   CNT_AF_GIVEN = 194,          // rows given up in this fill
   CNT_AF_GIVEN_TAKEN = 195,    // how many of them a block has taken
-  CNT_AF_TICKET = 196,         // shares of rows handed out to the blocks of the automaton's fill
+  CNT_AF_TICKET = 196,         // rows handed out to blocks of the automaton's fill that have filled their first
   CNT_TOTAL = 200
 };
 
@@ -254,18 +255,15 @@ struct CtxDev {
 // contexts of the row it works on.
 struct AutoFillDev {
   uint32_t on;               // rows are filled by the automaton
-  uint32_t grid, parts;      // thread blocks, and how many of them share a row
+  uint32_t grid;             // thread blocks
   uint4* stack;              // [grid][stack_cap] first edge, edges, context
   uint32_t stack_cap, reserve;  // and the places that are kept for rounds of one entry
   uint32_t* scratch;         // [grid][scratch_words]
   uint32_t scratch_words;
   uint32_t ctx_cap, pool_cap, big_cap;  // contexts per row, words for their lists, items of the largest expansion (powers of two)
-  uint32_t* row_begun;       // [rows, a multiple of four] the generation (StateDev::gen) of the fill in which the row's mask has been begun
-  uint32_t* row_gone;        // [rows, a multiple of four; 16-byte aligned] the generation of the fill in which the row was given up
-  uint32_t* given;           // [rows] the rows given up, generation << 16 | job
+  uint32_t* given;           // [rows] the rows given up, generation of the fill (StateDev::gen) << 16 | row
   uint32_t* sweep_lock;      // [sweep_slots] 1: a block sweeps a row in these tables (StateDev::au); 0 between launches
   uint32_t sweep_slots;
-  uint32_t flag_words;       // row_begun, row_gone and given together
   uint32_t ahead;            // words that may be read from where a chart begins, however long it is
 };
 

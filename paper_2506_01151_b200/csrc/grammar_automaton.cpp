@@ -17,6 +17,7 @@
 // asked, and for every item that it can answer there is an EDGE to the start of that item at that node.  So a fill follows edges, one
 // for each rule that ends inside a token, and not the trie byte by byte.
 #include <algorithm>
+#include <array>
 #include <cstring>
 #include <unordered_map>
 #include <utility>
@@ -40,7 +41,7 @@ constexpr u64 GA_MAX_WORK = 16u << 20;
 constexpr u64 GA_MAX_START_WORK = 64u << 20;
 constexpr size_t GA_MAX_WORDS = 64u << 20;  // of masks, tokens and edges
 constexpr size_t GA_MASK_TOKENS = 1024;   // a kernel's item from which so many tokens follow has a mask in the place of a list
-constexpr u32 GA_EDGE_TOKENS = 2048;      // tokens of an edge at most (the others go to further edges)
+constexpr size_t GA_LONG_LIST = 64;       // edges of a start from which on it has one for each item and the others behind it
 constexpr size_t GA_MAX_ITEMS = 1024;     // items of one set, predicted ones included: alternations of thousands of literals
                                           // would be scanned again for every set that predicts them
 
@@ -431,9 +432,10 @@ class Builder {
       }
       st[i].n_tok = (u32)toks.size();
       if (i < roots && toks.size() >= GA_MASK_TOKENS) {
-        mask_of[i] = (u32)(h_.ga_mask.size() / h_.Wm);
-        h_.ga_mask.resize(h_.ga_mask.size() + h_.Wm, 0u);
-        u32* m = &h_.ga_mask[(size_t)mask_of[i] * h_.Wm];
+        const u32 words = (h_.Wm + 3u) & ~3u;
+        mask_of[i] = (u32)(h_.ga_mask.size() / words);
+        h_.ga_mask.resize(h_.ga_mask.size() + words, 0u);
+        u32* m = &h_.ga_mask[(size_t)mask_of[i] * words];
         for (u32 t : toks) m[t >> 5] |= 1u << (t & 31);
       } else if (toks.size() == 1) {
         st[i].tok = toks[0];
@@ -454,20 +456,36 @@ class Builder {
     for (u32 i = 0; i < (u32)st.size(); ++i) order[i] = i;
     std::sort(order.begin(), order.end(), [&](u32 a, u32 b) { return st[a].node > st[b].node; });
     std::vector<char> reached(h_.D, 0);
+    using Edge = std::array<u32, 4>;
+    std::vector<Edge> out;
     for (u32 i : order) {
-      st[i].edge = (u32)(h_.ga_edge.size() / 4);
+      out.clear();
       for (u32 k = st[i].link; k < st[i].link + st[i].n_link; ++k) {
         const u32 d = links[k].first;
         const Start& to = st[links[k].second];
         if (to.n_tok == 0 && to.n_edge == 0) continue;
         reached[d] = 1;
         u32 n = std::min(to.n_tok, GA_EDGE_TOKENS);
-        h_.ga_edge.insert(h_.ga_edge.end(), {d << 16 | n, to.tok, to.edge, to.n_edge});
+        out.push_back({d << 16 | n, to.tok, to.edge, to.n_edge});
         for (u32 at = n; at < to.n_tok; at += n) {
           n = std::min(to.n_tok - at, GA_EDGE_TOKENS);
-          h_.ga_edge.insert(h_.ga_edge.end(), {d << 16 | n, n == 1 ? h_.ga_tok[to.tok + at] : to.tok + at, 0u, 0u});
+          out.push_back({d << 16 | n, n == 1 ? h_.ga_tok[to.tok + at] : to.tok + at, 0u, 0u});
         }
       }
+      if (out.size() > GA_LONG_LIST) {  // those of one item together, behind an edge to all of them
+        std::stable_sort(out.begin(), out.end(), [](const Edge& a, const Edge& b) { return a[0] >> 16 < b[0] >> 16; });
+        std::vector<Edge> heads;
+        for (size_t k = 0, e; k < out.size(); k = e) {
+          for (e = k; e < out.size() && e - k < GA_EDGE_GROUP && out[e][0] >> 16 == out[k][0] >> 16;) ++e;
+          if (e == k + 1) heads.push_back(out[k]);
+          else heads.push_back({(out[k][0] & 0xFFFF0000u) | GA_GROUP, 0u, (u32)(h_.ga_edge.size() / 4), (u32)(e - k)});
+          if (e > k + 1)
+            for (size_t x = k; x < e; ++x) h_.ga_edge.insert(h_.ga_edge.end(), out[x].begin(), out[x].end());
+        }
+        out.swap(heads);
+      }
+      st[i].edge = (u32)(h_.ga_edge.size() / 4);
+      for (const Edge& x : out) h_.ga_edge.insert(h_.ga_edge.end(), x.begin(), x.end());
       st[i].n_edge = (u32)(h_.ga_edge.size() / 4) - st[i].edge;
       if (h_.ga_tok.size() + h_.ga_mask.size() + h_.ga_edge.size() > GA_MAX_WORDS) {
         too_big_ = true;

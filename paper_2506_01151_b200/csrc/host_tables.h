@@ -32,6 +32,9 @@ constexpr uint32_t GA_GOES_ON = 1u << 31;  // ga_item: when its non-terminal is 
 constexpr uint32_t GA_SKIPS = 1u << 30;    // the kernel of the item holds the next item, too (the non-terminal is nullable)
 constexpr uint32_t GA_ALIVE = 1u << 29;    // tokens follow from a kernel with this item
 constexpr uint32_t GA_MASK = 0xFFFFFFFFu;  // ga_start: the tokens are a mask
+constexpr uint32_t GA_EDGE_TOKENS = 2047;   // tokens of an edge at most (the others go to further edges)
+constexpr uint32_t GA_EDGE_GROUP = 1024;    // edges behind one edge at most
+constexpr uint32_t GA_GROUP = 0xFFFFu;     // ga_edge, in the place of the tokens' number: the edges of this item in a long list
 
 struct CompileError {
   int code;
@@ -83,11 +86,11 @@ struct HostTables {
   // per dotted rule d as an item of a chart's kernel: its tokens (one token, where in ga_tok they begin, or a row of ga_mask), how many
   // (GA_MASK: a mask), first edge, edges
   std::vector<uint32_t> ga_start;  // [D][4]
-  // where a rule ends inside a token: the item that goes on << 16 | its tokens (at most 65535), the token or where in ga_tok they begin,
+  // where a rule ends inside a token: the item that goes on << 16 | its tokens (or GA_GROUP), the token or where in ga_tok they begin,
   // first edge, edges
   std::vector<uint32_t> ga_edge;   // [][4]
   std::vector<uint32_t> ga_tok;    // token ids
-  std::vector<uint32_t> ga_mask;   // [][Wm]
+  std::vector<uint32_t> ga_mask;   // [][Wm, a multiple of four]
   std::vector<uint32_t> vocab_off;  // [V+1] byte offsets (32-bit) into vocab_bytes
   std::vector<uint8_t> vocab_bytes;
 };

@@ -381,7 +381,7 @@ __global__ void __launch_bounds__(ADV_WARPS * 32, 1) forced_kernel(const __grid_
 // ===================================================================================== fill: plan
 
 // One block decides, row by row, where each mask comes from: the state cache, another row of
-// this call with the same chart, or a fresh computation (a "job").
+// this call with the same chart, or a fresh computation (a "job").  (For the sweeps; the automaton's fill decides by itself.)
 __global__ void __launch_bounds__(1024) plan_kernel(const __grid_constant__ GrammarDev G, const __grid_constant__ StateDev S) {
   before_me();
   __shared__ uint32_t n_jobs, n_rows, n_cached, n_shared;
@@ -393,8 +393,6 @@ __global__ void __launch_bounds__(1024) plan_kernel(const __grid_constant__ Gram
   if (threadIdx.x == 0) {
     S.counters[CNT_N_FJOBS] = 0u;
     S.counters[CNT_AUTO_ITEMS] = 0u;
-    S.counters[CNT_AF_TICKET] = 0u;
-    S.counters[CNT_AF_GIVEN] = S.counters[CNT_AF_GIVEN_TAKEN] = 0u;
     n_jobs = n_cached = n_shared = 0u;
     n_rows = S.counters[CNT_N_MASK_ROWS];
   }
@@ -831,7 +829,7 @@ __global__ void __launch_bounds__(SWEEP_WARPS * 32, 1) sweep_kernel(GrammarDev G
 // the rows themselves are fine and the next fill computes them afresh.
 __device__ __forceinline__ int32_t resolve_mask_row(const StateDev& S, uint32_t row) {
   int32_t r = S.row_mask[row];
-  const bool aborted = S.counters[CNT_BAR_ERR] != 0u;
+  const bool aborted = fill_aborted(S, S.counters[CNT_BAR_ERR]);
   if ((S.row_flags[row] & ROW_BROKEN) || (aborted && S.row_job[row])) return MASK_ZERO;
   if (r <= MASK_ALIAS0) {  // the mask another row of this call computed: not to be used if that row broke
     const uint32_t other = (uint32_t)(MASK_ALIAS0 - r);
@@ -844,10 +842,14 @@ __device__ __forceinline__ int32_t resolve_mask_row(const StateDev& S, uint32_t 
 // released: when the row had no cache row, or broke, or the fill was given up.
 __device__ __forceinline__ void publish_row(const StateDev& S, uint32_t row) {
   if (!S.row_job[row]) return;
-  const bool aborted = S.counters[CNT_BAR_ERR] != 0u;
+  const bool aborted = fill_aborted(S, S.counters[CNT_BAR_ERR]);
   const int32_t sid = S.row_state[row], mrow = S.row_mask[row];
   if (sid >= 0) S.st_mask[sid] = (!(S.row_flags[row] & ROW_BROKEN) && !aborted && mrow >= (int32_t)S.B) ? mrow : -1;
-  if (aborted && row == S.jobs[0]) stat_add(S, CNT_STAT_ABORTS, 1u);
+  if (aborted && !S.af.on && row == S.jobs[0]) stat_add(S, CNT_STAT_ABORTS, 1u);
+}
+// (one thread of that kernel) The automaton's fill counts from zero again.
+__device__ __forceinline__ void fill_is_through(const StateDev& S) {
+  if (S.af.on) S.counters[CNT_AF_TICKET] = S.counters[CNT_AF_GIVEN] = S.counters[CNT_AF_GIVEN_TAKEN] = 0u;
 }
 
 // mask_out[row][w] for every row
@@ -856,6 +858,7 @@ __global__ void gather_kernel(const __grid_constant__ GrammarDev G, const __grid
   before_me();
   const uint32_t row = blockIdx.y;
   if (blockIdx.x == 0 && threadIdx.x == 0) publish_row(S, row);
+  if (blockIdx.x == 0 && row == 0u && threadIdx.x == 32) fill_is_through(S);
   const int32_t r = resolve_mask_row(S, row);
   const uint32_t* src = (r >= 0) ? S.mask_rows + (size_t)r * G.Wm : nullptr;
   uint32_t* dst = out + (size_t)row * stride_words;
@@ -958,6 +961,7 @@ __global__ void gather_apply_kernel(const __grid_constant__ GrammarDev G, const 
   before_me();
   const uint32_t row = blockIdx.y;
   if (blockIdx.x == 0 && threadIdx.x == 0) publish_row(S, row);
+  if (blockIdx.x == 0 && row == 0u && threadIdx.x == 32) fill_is_through(S);
   const int32_t r = resolve_mask_row(S, row);
   const uint32_t* src = (r >= 0) ? S.mask_rows + (size_t)r * G.Wm : nullptr;
   uint32_t* mo = mask_out ? mask_out + (size_t)row * stride_words : nullptr;

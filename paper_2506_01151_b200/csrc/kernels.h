@@ -38,8 +38,8 @@ void sweep_layout(const GrammarDev& G, uint32_t* smem_bytes, uint32_t* tables_in
 int sweep_warps();
 
 // the fill by the grammar automaton (automaton_fill.cu); the layout sets what follows from the grammar, the rows and the capacities in A
-constexpr uint32_t AUTO_FILL_PER_SM = 4;  // thread blocks asked for on an SM (three of them run at a time, see automaton_fill.cu)
-void automaton_fill_layout(const GrammarDev& G, uint32_t rows, uint32_t max_blocks, AutoFillDev& A);
+constexpr uint32_t AUTO_FILL_PER_SM = 2;  // thread blocks that run on an SM at a time
+void automaton_fill_layout(uint32_t rows, uint32_t max_blocks, AutoFillDev& A);
 uint32_t automaton_fill_least_stack();  // entries
 uint32_t automaton_fill_warps();                            // of a block
 cudaError_t configure_automaton_fill();

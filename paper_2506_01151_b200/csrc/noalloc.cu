@@ -54,7 +54,7 @@ constexpr uint32_t NA_CTX = 1024, NA_POOL = 8u << 10, NA_LARGE = 4u << 10;
 constexpr uint32_t NA_FILL_SCRATCH = 7u * NA_CTX + NA_POOL + NA_LARGE / 4u + NA_LARGE / 2u + NA_LARGE;
 constexpr size_t NA_OFF_FILL = NA_HEADER_WORDS + 4 * (size_t)NA_FILL_BLOCKS * NA_STACK;
 constexpr size_t NA_OFF_ROW_FLAGS = NA_OFF_FILL + (size_t)NA_FILL_BLOCKS * NA_FILL_SCRATCH;
-static_assert(NA_OFF_ROW_FLAGS + 3 * NA_MAX <= NA_SWEEP_WORDS, "the fill's tables do not fit");
+static_assert(NA_OFF_ROW_FLAGS + NA_MAX <= NA_SWEEP_WORDS, "the fill's tables do not fit");
 // behind both: tables of Earley sets for the charts that this fill gives up, one chart at a time
 constexpr uint32_t NA_BLOCK_WARPS = 8;
 constexpr size_t NA_ROW_ST_ENTRIES = 2u << 20;
@@ -66,7 +66,6 @@ constexpr size_t NA_OFF_ROW_ST = NA_OFF_ROW_ITEMS + NA_ITEM_WORDS;
 constexpr size_t NA_OFF_ROW_REQ = NA_OFF_ROW_ST + NA_ROW_ST_ENTRIES / 2;
 constexpr size_t NA_OFF_ROW_LOCK = NA_OFF_ROW_REQ + NA_REQ_CAP;
 constexpr size_t NA_WORDS = NA_OFF_ROW_LOCK + 4;
-static_assert(NA_OFF_ROW_FLAGS % 4 == 0 && NA_MAX % 4 == 0, "flags are read in 16-byte pieces");
 static_assert(NA_OFF_ROW_BIG % 4 == 0 && (NA_ARENA_ITEMS + NA_HSET_SLOTS) % 4 == 0, "hash slots are cleared in 16-byte pieces");
 static_assert(CNT_TOTAL <= NA_OFF_JOBS, "the counters overlap the job list");
 static_assert(NA_OFF_JOBINFO + 4 * NA_MAX <= NA_HEADER_WORDS, "header too small");
@@ -100,11 +99,11 @@ __global__ void noalloc_prepare_kernel(GrammarDev G, StateDev S, uint32_t* scrat
     scratch[NA_OFF_BAD + r] = ok ? 0u : 1u;
     S.row_chart[r] = off.v[r];
     S.row_mask[r] = (int32_t)r;
-    S.row_flags[r] = 0u;
+    S.row_flags[r] = ok ? 0u : ROW_BROKEN;  // (the automaton's fill leaves such rows out)
   }
   for (size_t i = tid; i < (size_t)n * G.Wm; i += nth) mask[i] = 0u;
   if (S.af.on) {
-    if (tid < 3 * NA_MAX) S.af.row_begun[tid] = 0u;
+    if (tid < NA_MAX) S.af.given[tid] = 0u;
     if (tid == 0) *S.af.sweep_lock = 0u;
     return;
   }
@@ -119,7 +118,7 @@ __global__ void noalloc_prepare_kernel(GrammarDev G, StateDev S, uint32_t* scrat
 // One CTA per chart whose header was accepted: the rest of the chart.  The sweep indexes its tables
 // with what the chart says, so every word is checked here: the sets' offsets must not decrease, every
 // item must name a dotted rule of this grammar and start in a set of this chart.
-__global__ void noalloc_validate_kernel(GrammarDev G, uint32_t* scratch, const uint32_t* charts, Offsets off, uint32_t n) {
+__global__ void noalloc_validate_kernel(GrammarDev G, StateDev S, uint32_t* scratch, const uint32_t* charts, Offsets off, uint32_t n) {
   const uint32_t r = blockIdx.x;
   if (r >= n || scratch[NA_OFF_BAD + r]) return;
   const uint32_t* ch = charts + off.v[r];
@@ -135,7 +134,7 @@ __global__ void noalloc_validate_kernel(GrammarDev G, uint32_t* scratch, const u
     const uint32_t x = it[k];
     if ((x & 0xFFFFu) >= G.D || (x >> 16) >= m) bad = true;
   }
-  if (bad) scratch[NA_OFF_BAD + r] = 1u;  // (every writer writes the same value)
+  if (bad) scratch[NA_OFF_BAD + r] = 1u, S.row_flags[r] = ROW_BROKEN;  // (every writer writes the same values)
 }
 
 // One thread: the job list holds the charts that passed both checks.
@@ -246,8 +245,7 @@ extern "C" fmt_status fmt_fill_mask_noalloc(const fmt_grammar* g, const uint32_t
     A.scratch = scratch + NA_OFF_FILL;
     A.ctx_cap = NA_CTX, A.pool_cap = NA_POOL, A.big_cap = NA_LARGE;
     A.ahead = CH_HDR;  // (the caller's memory may end with its last chart)
-    A.row_begun = scratch + NA_OFF_ROW_FLAGS;
-    A.row_gone = A.row_begun + NA_MAX, A.given = A.row_gone + NA_MAX;
+    A.given = scratch + NA_OFF_ROW_FLAGS;
     A.sweep_slots = 1, A.sweep_lock = scratch + NA_OFF_ROW_LOCK;
     S.big_scratch = scratch + NA_OFF_ROW_BIG;
     S.au.recs = scratch + NA_OFF_ROW_RECS;
@@ -256,13 +254,13 @@ extern "C" fmt_status fmt_fill_mask_noalloc(const fmt_grammar* g, const uint32_t
     S.au.st = reinterpret_cast<uint16_t*>(scratch + NA_OFF_ROW_ST);
     S.au.req = reinterpret_cast<unsigned long long*>(scratch + NA_OFF_ROW_REQ);
     if (automaton_fill_warps() > NA_BLOCK_WARPS) return fail(FMT_ERR_CAPACITY, "the built-in scratch does not fit the fill");
-    automaton_fill_layout(*G, n, NA_FILL_BLOCKS, A);
+    automaton_fill_layout(n, NA_FILL_BLOCKS, A);
     if (A.scratch_words > NA_FILL_SCRATCH) return fail(FMT_ERR_CAPACITY, "the built-in scratch does not fit the fill");
   }
   cudaStream_t st = (cudaStream_t)stream;
   noalloc_prepare_kernel<<<256, 256, 0, st>>>(*G, S, scratch, charts_dev, off, n, mask_dev);
-  noalloc_validate_kernel<<<n, 256, 0, st>>>(*G, scratch, charts_dev, off, n);
-  noalloc_jobs_kernel<<<1, 32, 0, st>>>(S, scratch, n);
+  noalloc_validate_kernel<<<n, 256, 0, st>>>(*G, S, scratch, charts_dev, off, n);
+  if (!S.af.on) noalloc_jobs_kernel<<<1, 32, 0, st>>>(S, scratch, n);
   if (S.af.on) launch_automaton_fill(*G, S, st);
   else launch_sweep(*G, S, (int)NA_GRID, st);
   noalloc_finish_kernel<<<n, 128, 0, st>>>(*G, S, scratch, n, mask_dev, status_dev);
