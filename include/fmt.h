@@ -313,8 +313,8 @@ fmt_status fmt_state_cache_clear(fmt_state* s, void* stream);
 fmt_status fmt_state_ci_cache_clear(fmt_state* s, void* stream);
 
 /* Every wait inside a kernel of this library (for another thread block, for a queued work item, for
- * a transition another warp is computing) is a poll with an iteration limit; a wait that runs out
- * makes the fill give up: its computed rows get all-zero masks, fmt_stats.fills_aborted counts it,
+ * a transition another warp is computing) is a poll with an iteration limit, and a row's fill by the
+ * automaton has no more rounds than that; a wait that runs out makes the fill give up: its computed rows get all-zero masks, fmt_stats.fills_aborted counts it,
  * nothing hangs and the next fill starts afresh.  log2_polls = 0 restores the defaults.  (A test
  * aid: with a tiny limit the give-up path can be taken without anything being wrong.) */
 fmt_status fmt_state_set_wait_limit(fmt_state* s, uint32_t log2_polls);

@@ -48,6 +48,7 @@ constexpr uint32_t AF_CTX = AF_ITEMS + 96, AF_CTX_HASH = 1024, AF_POOL = 3072;  
 constexpr uint32_t AF_BUF = 512, AF_WORK = 256, AF_HSET = 512;      // an expansion in shared memory (larger ones: global memory)
 constexpr uint32_t AF_KCYCLES = 1u << 14;      // a row that takes longer (2^24 cycles, 8.5 ms) is given up for a sweep by Earley steps
 // AC_FAIL: 0, 1 + the capacity that was exceeded, or
+constexpr uint32_t AF_GIVEN_UP = 0xFFFFFFFFu;  // more rounds than a bounded wait has polls: the fill is given up, the row itself is fine
 constexpr uint32_t AF_LATE = 0xFFFFFFFDu;      // the row takes too long
 constexpr uint32_t CTX_NEW = 0xFFFFFFFFu;
 constexpr uint32_t AF_FOUND = 1u << 31;        // an entry whose edges are all of one item, with that item's context
@@ -863,7 +864,7 @@ __global__ void __launch_bounds__(AF_THREADS, 2) automaton_fill_kernel(const __g
         *p = rest;
         return yes;
       };
-      uint32_t list_at = 0, gtop = 0;  // items of the last set whose starts have been taken, entries on the stack
+      uint32_t list_at = 0, gtop = 0, rounds = 0;  // items of the last set whose starts have been taken, entries on the stack
       bool begun = false;
 #pragma unroll 1
       for (uint32_t side = 0;; side ^= 1u) {  // ---- rounds
@@ -1044,6 +1045,11 @@ __global__ void __launch_bounds__(AF_THREADS, 2) automaton_fill_kernel(const __g
           ctl[AC_OVF] = 0u;
           deal_clear(E), deal_clear(token_deal(side ^ 1u));
           if (ctl[AC_FULL]) ctl[AC_FAIL] = 1u + DIAG_QUEUE_FULL;
+          if (++rounds > poll_limit(S, 22)) {
+            diag(S, DIAG_WAIT_QUEUE);
+            if (atomicExch(&S.counters[CNT_BAR_ERR], S.gen) != S.gen) stat_add(S, CNT_STAT_ABORTS, 1u);
+            ctl[AC_FAIL] = AF_GIVEN_UP;
+          }
         }
         if (warp == 0 && ctl[AC_WANT]) {
           // ---- expansions that the next round needs
@@ -1086,7 +1092,7 @@ __global__ void __launch_bounds__(AF_THREADS, 2) automaton_fill_kernel(const __g
         __syncthreads();
       }
       contexts += ctl[AC_NCTX];
-      if (ctl[AC_FAIL]) {  // too many contexts, or too long a time: the row is left to a sweep by Earley steps
+      if (ctl[AC_FAIL] && ctl[AC_FAIL] != AF_GIVEN_UP) {  // too many contexts, or too long a time: the row is left to a sweep by Earley steps
         gave_up = true;
         __threadfence();
         if (tid == 0) {
