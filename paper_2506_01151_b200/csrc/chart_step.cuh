@@ -371,8 +371,8 @@ __device__ __forceinline__ int token_steps(const GrammarDev& G, AdvScratch& s, c
     // seldom is one (trying it all the same cost an advance of 32 ambiguous rows 90 us, not trying 80) ...
     uint32_t mine;
     const uint32_t ns = (prev_len <= (gen_fits(G, index) ? 32u : 96u)) ? small_scan_complete(G, s.w, view, prev, prev_len, byte, index,
-                                                                 [](uint32_t it) { return it; }, mine, accepting)
-                                           : SMALL_OVERFLOW;
+                                                                                                   [](uint32_t it) { return it; }, mine, accepting)
+                                                                       : SMALL_OVERFLOW;
     if (ns == 0) return forced_out ? (int)(L - 1) : 0;
     if (ns != SMALL_OVERFLOW) {
       n = small_drop_completed(G, s.w, ns, mine);
@@ -439,9 +439,12 @@ __device__ __forceinline__ int token_steps(const GrammarDev& G, AdvScratch& s, c
     // Where no item of the source chart's sets after set o begins before o, everything before o is held by o's items alone, and as the
     // source chart is pruned, all of it is needed if they all are: the way down a deep nesting ends at the first such set.
     uint32_t earliest = 0xFFFFFFFFu, looked_at = n_items;  // (each lane: over some of the items from looked_at on)
-    uint32_t first_asked = 0xFFFFFFFFu;  // (each lane: the earliest set it has asked)
+    const bool narrow = M <= 32u;        // (then the sets that have been asked are a word)
+    uint32_t first_asked = 0xFFFFFFFFu;  // (each lane: the earliest set it has asked, or all of them)
+    uint32_t asked_sets = 0u;
+    if (narrow) first_asked = 0u;
     auto ask = [&](uint32_t o, uint32_t A) {
-      first_asked = min(first_asked, o);
+      first_asked = narrow ? first_asked | 1u << o : min(first_asked, o);
       atomicOr(&need[o * Nw + (A >> 5)], 1u << (A & 31u));
     };
     #pragma unroll 1
@@ -452,19 +455,29 @@ __device__ __forceinline__ int token_steps(const GrammarDev& G, AdvScratch& s, c
     #pragma unroll 1
     for (uint32_t end = M; end;) {  // sets 0 .. end-1 are left: the last of them that is asked for
       __syncwarp();
-      const uint32_t k = end - 1u - lane;  // (wraps around for lanes beyond set 0)
-      bool asked = false;
-      if (k < end)
-        #pragma unroll 1
-        for (uint32_t w = 0; w < Nw; ++w) asked = asked || need[k * Nw + w] != 0u;
-      const uint32_t bal = __ballot_sync(FULL, asked);
-      if (bal == 0u) {
-        end -= min(end, 32u);
-        continue;
+      uint32_t o;
+      bool sole;  // nothing before it has been asked yet
+      if (narrow) {
+        asked_sets |= __reduce_or_sync(FULL, first_asked);
+        const uint32_t left = asked_sets & (0xFFFFFFFFu >> (32u - end));
+        if (left == 0u) break;
+        o = 31u - __clz(left);
+        sole = left == 1u << o;
+      } else {
+        const uint32_t k = end - 1u - lane;  // (wraps around for lanes beyond set 0)
+        bool asked = false;
+        if (k < end)
+#pragma unroll 1
+          for (uint32_t w = 0; w < Nw; ++w) asked = asked || need[k * Nw + w] != 0u;
+        const uint32_t bal = __ballot_sync(FULL, asked);
+        if (bal == 0u) {
+          end -= min(end, 32u);
+          continue;
+        }
+        o = end - (uint32_t)__ffs(bal);
+        sole = __reduce_min_sync(FULL, first_asked) == o;
       }
-      const uint32_t o = end - (uint32_t)__ffs(bal);
       end = o;
-      const bool sole = __reduce_min_sync(FULL, first_asked) == o;  // nothing before it has been asked yet
       const uint32_t* sp;
       uint32_t sl;
       view(o, sp, sl);
@@ -661,7 +674,8 @@ __device__ __forceinline__ int token_steps(const GrammarDev& G, AdvScratch& s, c
     const uint32_t a = dst[CH_HDR + nw], b = (nw + 1 < m_new) ? dst[CH_HDR + nw + 1] : kept;
     uint32_t* set = dst + items_at + a;
     const uint32_t ns = b - a;
-    if (ns <= 32) {
+    if (ns <= 1) {
+    } else if (ns <= 32) {
       sort_items(set, ns, 32);
     } else {  // rare: by rank, through the part of the arena whose sets have been copied out by now
       #pragma unroll 1

@@ -219,7 +219,9 @@ __device__ __forceinline__ uint32_t predict_set(const GrammarDev& G, const WarpC
   for (uint32_t i = lane; i < Nw; i += 32) asked |= ntmask[i];
   if (!__any_sync(FULL, asked != 0u)) return n;  // (inside literals and automata there is nothing to predict)
   uint32_t one = 0xffffffffu;  // the non-terminal that pulls in all the others
-  if (LISTS && G.pred && Nw <= 4u) {
+  if (LISTS && G.pred && Nw == 1u && __popc(ntmask[0]) == 1) {
+    one = (uint32_t)__ffs(ntmask[0]) - 1u;
+  } else if (LISTS && G.pred && Nw <= 4u) {
 #pragma unroll 1
     for (uint32_t wi = 0; wi < Nw && one == 0xffffffffu; ++wi) {
       bool mine = (ntmask[wi] >> lane) & 1u;
