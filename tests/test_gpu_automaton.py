@@ -404,3 +404,40 @@ def test_advance_wherever_the_tables_are(tables, batch):
     if tables == "all in global memory":  # (automata have items of their own)
         assert want[1] == seq.total_items
     assert want[0] == seq.num_sets
+
+
+@pytest.mark.parametrize("n", [64, 65, 1024, 1025, 2047, 2048, 5000])
+def test_lists_of_edges_and_of_tokens(n):
+    """Where strings end inside n tokens, one kernel item has n edges (grouped by item from 65 on, behind several edges from 1,025 on),
+    and where one string ends and the next begins inside n more, an edge has n tokens (several edges from 2,048 on, and more lists of
+    tokens in a round than there is room for)."""
+    w = workloads.build(2, V=300, batch=1, steps=1)
+    words = [bytes([97 + i // 676, 97 + i // 26 % 26, 97 + i % 26]) for i in range(n)]
+    vocab = [bytes([b]) for b in range(256)] + [x + b'",' for x in words] + [b'","' + x for x in words] + [x + b'":[]' for x in words[::2]] + [x + b'"]' for x in words[::3]] + [b""]
+    _run(w.ebnf, w.start, vocab, [list(p) for p in (b'["x', b'{"k":"x', b'{"', b'[["x"', b'[')])
+
+
+@pytest.mark.parametrize("depth", [20, 56, 73, 74, 75, 76, 112, 150, 190, 260])
+def test_charts_around_an_item_to_a_thread(depth):
+    """The contexts of a chart of up to 224 items are made by a thread for each; larger ones, and charts of more than 768 words, have
+    them made as they are asked for."""
+    vocab = [bytes([b]) for b in range(256)] + [b"]" * k for k in range(2, 33)] + [b"]}", b'],"', b"}]", b"1]", b"]]}", b'"]]', b"1,[[", b"]," * 8, b""]
+    w = workloads.build(2, V=300, batch=1, steps=1)
+    _run(w.ebnf, w.start, vocab, [list(p) for p in (b"[" * depth, b"[1," * depth + b'"', b'{"a":[' * (depth // 2) + b"1")])
+
+
+@pytest.mark.parametrize("n", [2, 12, 29, 31, 33, 70])
+@pytest.mark.parametrize("dfa", [True, False])
+def test_chains_completed_in_one_set(n, dfa):
+    """What is completed with a completed item in the set where both began: chains of n rules of one symbol, with something nullable
+    behind it, in sets below and above 32 items."""
+    text = "s ::= n0 | s \",\" n0\n" + "".join('n%d ::= n%d z | n%d "+" n%d\n' % (i, i + 1, i, i + 1) for i in range(n))
+    text += 'n%d ::= "x" | "(" s ")"\nz ::= "!" | ""' % n
+    data = b"x,(x+x!,(x)),x"
+    a, b, _ = _feed(text, "s", data, dict(chart_words=1 << 16), dfa)
+    assert a.tolist() == b.tolist()
+    seq = oracle.Sequence_(oracle.Grammar(text, "s"), pruned=True)
+    assert seq.advance(data)
+    assert int(a[0]) == seq.num_sets
+    if not dfa:  # (automata have items of their own)
+        assert int(a[1]) == seq.total_items
