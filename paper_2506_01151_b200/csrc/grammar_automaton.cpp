@@ -47,7 +47,8 @@ constexpr size_t GA_MAX_ITEMS = 1024;     // items of one set, predicted ones in
 
 // Where the chart has to be asked at many places a fill by the automaton is the slower one: its threads walk the trie one by one, and
 // each exit starts a thread for every item that completing the rule yields.  Two counts over the walk tell such grammars; they go without.
-// Fills of 64 rows of 128,256 tokens by the automaton and by the sweep, us (share of nodes with an exit; starts a node):
+// Fills of 64 rows of 128,256 tokens by a walk of the trie with the automaton and by the sweep, us (share of nodes with an exit; starts a
+// node); by edges, as fills are made now, JSON takes 41, the union of 20 65, and the line lies well on the safe side:
 //   JSON 94 and 239 (0.09; 0.6)   ambiguous JSON 400 and 1,000 (0.12; 1.4)   SQL 231 and 667 (0.03; 1.1)   JSON schema 77 and 263 (0.02; 0.04)
 //   HTML 923 and 457 (0.75; 69)   braces 1,758 and 753 (0.72; 1.4)   XML 14,000 and 1,280 (0.75; 4.6)   two like texts 1,750 and 603 (0.51; 3.3)
 //   a union of 60 variants 2,607 and 430 (0.05; 5.1)   a C-like language 1,883 and 669 (0.17; 36)   a union of 20 485 and 411 (0.05; 1.7)
