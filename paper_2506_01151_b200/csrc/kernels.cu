@@ -847,9 +847,9 @@ __device__ __forceinline__ void publish_row(const StateDev& S, uint32_t row) {
   if (sid >= 0) S.st_mask[sid] = (!(S.row_flags[row] & ROW_BROKEN) && !aborted && mrow >= (int32_t)S.B) ? mrow : -1;
   if (aborted && !S.af.on && row == S.jobs[0]) stat_add(S, CNT_STAT_ABORTS, 1u);
 }
-// (one thread of that kernel) The automaton's fill counts from zero again.
+// (one thread of that kernel) The automaton's fill counts from zero again, and the rows that it gives up have the whole item pool.
 __device__ __forceinline__ void fill_is_through(const StateDev& S) {
-  if (S.af.on) S.counters[CNT_AF_TICKET] = S.counters[CNT_AF_GIVEN] = S.counters[CNT_AF_GIVEN_TAKEN] = 0u;
+  if (S.af.on) S.counters[CNT_AF_TICKET] = S.counters[CNT_AF_GIVEN] = S.counters[CNT_AF_GIVEN_TAKEN] = S.counters[CNT_AUTO_ITEMS] = 0u;
 }
 
 // mask_out[row][w] for every row

@@ -171,6 +171,35 @@ def test_rows_that_outgrow_the_storage_of_contexts(n, batch):
     assert s["rows_swept_again"] <= batch and (n == 20 or s["rows_swept_again"] > 0)
 
 
+def test_rows_given_up_in_one_fill_after_the_other():
+    """The Earley sets of rows that are given up come from one pool (64 Mi words, some 50,000 a row here): every fill begins with all of
+    it, however many rows were swept before."""
+    import torch
+
+    import paper_2506_01151_b200 as fmt
+
+    text, vocab = _endings(340)
+    prefixes = [b"(" * 20, b"(" * 20 + b"x", b"(" * 20 + b"x)a"]
+    g, batch = fmt.Grammar(text, "s", vocab, len(vocab) - 1), 255
+    st = fmt.State(g, batch, cache=False)
+    for i in range(max(map(len, prefixes))):
+        t = [prefixes[b % 3][i] if i < len(prefixes[b % 3]) else -1 for b in range(batch)]
+        st.advance(torch.tensor(t, dtype=torch.int32, device="cuda"))
+    og, ov = oracle.Grammar(text, "s"), oracle.Vocab(vocab, len(vocab) - 1)
+    want = []
+    for p in prefixes:
+        s = oracle.Sequence_(og)
+        assert s.advance(p)
+        want.append(s.mask(ov))
+    want = np.tile(np.stack(want), (batch // 3, 1))
+    mask = torch.zeros((batch, g.mask_words), dtype=torch.int32, device="cuda")
+    for _ in range(9):
+        st.fill_mask(mask)
+        assert np.array_equal(mask.cpu().numpy().view(np.uint32), want)
+    s = st.stats()
+    assert s["capacity_errors"] == 0 and s["rows_swept_again"] > 1500
+
+
 @pytest.mark.parametrize("text, start, prefixes", [
     ('content ::= node*\nnode ::= char | entity | "<p>" content "</p>" | "<b>" content "</b>"\nchar ::= [^<&]\nentity ::= "&" [a-z]+ ";"\n', "content",
      [b"<p>some <b>bold", b"text &am", b"", b"<p><b>x</"]),
