@@ -143,9 +143,7 @@ static cudaError_t next_generations(fmt_state* s, cudaStream_t st) {
   StateDev& d = s->dev;
   cudaError_t e = cudaSuccess;
   if (s->next_gen + 1u > 65534u) {
-    if (d.af.on) e = cudaMemsetAsync(d.af.given, 0, (size_t)d.B * 4, st);
-    if (e == cudaSuccess && d.af.on) e = cudaMemsetAsync(d.counters + CNT_BAR_ERR, 0, 4, st);
-    if (e == cudaSuccess && !d.af.on) e = cudaMemsetAsync(d.au.hash, 0, (size_t)d.B * (d.au.hash_mask + 1u) * 4, st);
+    if (!d.af.on) e = cudaMemsetAsync(d.au.hash, 0, (size_t)d.B * (d.au.hash_mask + 1u) * 4, st);
     if (e == cudaSuccess && !d.af.on) e = cudaMemsetAsync(d.au.req, 0, (size_t)d.au.req_cap * 8, st);
     if (e == cudaSuccess && d.rt.on) e = cudaMemsetAsync(d.cx.ctab, 0, (size_t)d.B * CT_SLOTS * 8, st);
     if (e == cudaSuccess && d.rt.on) e = cudaMemsetAsync(d.cx.req2, 0, (size_t)d.cx.req2_cap * 16, st);

@@ -731,7 +731,12 @@ __global__ void __launch_bounds__(AF_THREADS, 2) automaton_fill_kernel(const __g
   };
   uint32_t looked_up = 0, contexts = 0;
   bool gave_up = false, filled = false;
-  if (blockIdx.x == 0 && tid == 0) stat_add(S, CNT_STAT_FILLS, S.B);
+  auto fill_tag = [&]() -> uint32_t { return S.counters[CNT_AF_NO] << 1 | 1u; };  // what this fill's blocks leave when one of them gives up
+  if (blockIdx.x == 0 && tid == 0) {
+    stat_add(S, CNT_STAT_FILLS, S.B);
+    const uint32_t e = vload(&S.counters[CNT_BAR_ERR]);  // (an earlier fill's; a block of this one that gives up writes this one's)
+    if (e && e != fill_tag()) atomicCAS(&S.counters[CNT_BAR_ERR], e, 0u);
+  }
   #pragma unroll 1
   for (uint32_t row = blockIdx.x; row < S.B;) {
     // ---- where the row's mask comes from: the state cache, another row of this call with the same chart, or from here
@@ -1047,7 +1052,7 @@ __global__ void __launch_bounds__(AF_THREADS, 2) automaton_fill_kernel(const __g
           if (ctl[AC_FULL]) ctl[AC_FAIL] = 1u + DIAG_QUEUE_FULL;
           if (++rounds > poll_limit(S, 22)) {
             diag(S, DIAG_WAIT_QUEUE);
-            if (atomicExch(&S.counters[CNT_BAR_ERR], S.gen) != S.gen) stat_add(S, CNT_STAT_ABORTS, 1u);
+            if (atomicExch(&S.counters[CNT_BAR_ERR], fill_tag()) != fill_tag()) stat_add(S, CNT_STAT_ABORTS, 1u);
             ctl[AC_FAIL] = AF_GIVEN_UP;
           }
         }
@@ -1097,7 +1102,7 @@ __global__ void __launch_bounds__(AF_THREADS, 2) automaton_fill_kernel(const __g
         __threadfence();
         if (tid == 0) {
           if (ctl[AC_FAIL] != AF_LATE) diag(S, ctl[AC_FAIL] - 1u);
-          *reinterpret_cast<volatile uint32_t*>(A.given + atomicAdd(&S.counters[CNT_AF_GIVEN], 1u)) = S.gen << 16 | row;
+          *reinterpret_cast<volatile uint32_t*>(A.given + atomicAdd(&S.counters[CNT_AF_GIVEN], 1u)) = row + 1u;
         }
       }
     }
@@ -1140,18 +1145,18 @@ __global__ void __launch_bounds__(AF_THREADS, 2) automaton_fill_kernel(const __g
         uint32_t k = blockIdx.x % A.sweep_slots, v = 0u;
         #pragma unroll 1
         for (uint32_t polls = 0; slot == 0xFFFFFFFFu; ++polls, k = (k + 1u) % A.sweep_slots) {
-          if ((v >> 16) != S.gen) v = vload(A.given + got);  // (written right after its number was drawn)
-          if ((v >> 16) == S.gen && atomicCAS(A.sweep_lock + k, 0u, 1u) == 0u) slot = k;
-          else if (fill_aborted(S, ld_acquire(&S.counters[CNT_BAR_ERR]))) break;
+          if (v == 0u) v = vload(A.given + got);  // (written right after its number was drawn)
+          if (v && atomicCAS(A.sweep_lock + k, 0u, 1u) == 0u) slot = k;
+          else if (ld_acquire(&S.counters[CNT_BAR_ERR]) == fill_tag()) break;
           else if (polls > poll_limit(S, 22)) {
             diag(S, DIAG_WAIT_VALUE);
-            if (atomicExch(&S.counters[CNT_BAR_ERR], S.gen) != S.gen) stat_add(S, CNT_STAT_ABORTS, 1u);
+            if (atomicExch(&S.counters[CNT_BAR_ERR], fill_tag()) != fill_tag()) stat_add(S, CNT_STAT_ABORTS, 1u);
             break;
           } else {
             __nanosleep(400);
           }
         }
-        ctl[AC_SLOT] = v & 0xFFFFu;
+        ctl[AC_SLOT] = v - 1u;
         __threadfence();
       }
       ctl[AC_ROW] = slot;

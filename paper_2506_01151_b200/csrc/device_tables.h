@@ -85,7 +85,7 @@ enum : uint32_t {
   CNT_STAT_TRANS = 26,  // transitions computed by the trie sweep (Earley steps)
   CNT_STAT_LOCAL = 28,  // local states created by the trie sweep
   CNT_BAR = 30,         // grid barrier of the trie sweep: arrivals
-  CNT_BAR_ERR = 31,     // a block gave up waiting: 1, or, where rows are filled by the automaton, the generation of the fill in which one did
+  CNT_BAR_ERR = 31,     // a block gave up waiting: 1, or, where rows are filled by the automaton, the mark of the fill in which one did (CNT_AF_NO)
   CNT_LEVEL_ALIVE = 32, // [MAX_TOKEN_BYTES + 2] per trie depth: some node of some job was alive
   CNT_LEVEL_REQ = 68,   // [MAX_TOKEN_BYTES + 2] per trie depth: transitions queued for computation
   CNT_HASH_GEN = 104,   // (the depth counters that every fill clears end here; the fills' generations are handed out by the host)
@@ -109,6 +109,7 @@ enum : uint32_t {
   CNT_AF_GIVEN = 194,          // rows given up in this fill
   CNT_AF_GIVEN_TAKEN = 195,    // how many of them a block has taken
   CNT_AF_TICKET = 196,         // rows handed out to blocks of the automaton's fill that have filled their first
+  CNT_AF_NO = 197,             // the fills so far, counted on the device: a captured fill that is replayed is one more (its mark: << 1 | 1)
   CNT_TOTAL = 200
 };
 
@@ -261,7 +262,7 @@ struct AutoFillDev {
   uint32_t* scratch;         // [grid][scratch_words]
   uint32_t scratch_words;
   uint32_t ctx_cap, pool_cap, big_cap;  // contexts per row, words for their lists, items of the largest expansion (powers of two)
-  uint32_t* given;           // [rows] the rows given up, generation of the fill (StateDev::gen) << 16 | row
+  uint32_t* given;           // [rows] the rows given up, + 1; 0 between fills
   uint32_t* sweep_lock;      // [sweep_slots] 1: a block sweeps a row in these tables (StateDev::au); 0 between launches
   uint32_t sweep_slots;
   uint32_t ahead;            // words that may be read from where a chart begins, however long it is

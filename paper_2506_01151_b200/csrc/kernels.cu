@@ -829,7 +829,7 @@ __global__ void __launch_bounds__(SWEEP_WARPS * 32, 1) sweep_kernel(GrammarDev G
 // the rows themselves are fine and the next fill computes them afresh.
 __device__ __forceinline__ int32_t resolve_mask_row(const StateDev& S, uint32_t row) {
   int32_t r = S.row_mask[row];
-  const bool aborted = fill_aborted(S, S.counters[CNT_BAR_ERR]);
+  const bool aborted = S.counters[CNT_BAR_ERR] != 0u;
   if ((S.row_flags[row] & ROW_BROKEN) || (aborted && S.row_job[row])) return MASK_ZERO;
   if (r <= MASK_ALIAS0) {  // the mask another row of this call computed: not to be used if that row broke
     const uint32_t other = (uint32_t)(MASK_ALIAS0 - r);
@@ -841,15 +841,18 @@ __device__ __forceinline__ int32_t resolve_mask_row(const StateDev& S, uint32_t 
 // (one thread per row, in the kernel that reads the masks) A mask computed in this call becomes the cache's, or its claim is
 // released: when the row had no cache row, or broke, or the fill was given up.
 __device__ __forceinline__ void publish_row(const StateDev& S, uint32_t row) {
+  if (S.af.on) S.af.given[row] = 0u;
   if (!S.row_job[row]) return;
-  const bool aborted = fill_aborted(S, S.counters[CNT_BAR_ERR]);
+  const bool aborted = S.counters[CNT_BAR_ERR] != 0u;
   const int32_t sid = S.row_state[row], mrow = S.row_mask[row];
   if (sid >= 0) S.st_mask[sid] = (!(S.row_flags[row] & ROW_BROKEN) && !aborted && mrow >= (int32_t)S.B) ? mrow : -1;
   if (aborted && !S.af.on && row == S.jobs[0]) stat_add(S, CNT_STAT_ABORTS, 1u);
 }
 // (one thread of that kernel) The automaton's fill counts from zero again, and the rows that it gives up have the whole item pool.
 __device__ __forceinline__ void fill_is_through(const StateDev& S) {
-  if (S.af.on) S.counters[CNT_AF_TICKET] = S.counters[CNT_AF_GIVEN] = S.counters[CNT_AF_GIVEN_TAKEN] = S.counters[CNT_AUTO_ITEMS] = 0u;
+  if (!S.af.on) return;
+  S.counters[CNT_AF_TICKET] = S.counters[CNT_AF_GIVEN] = S.counters[CNT_AF_GIVEN_TAKEN] = S.counters[CNT_AUTO_ITEMS] = 0u;
+  ++S.counters[CNT_AF_NO];
 }
 
 // mask_out[row][w] for every row

@@ -368,9 +368,6 @@ struct SweepWarp {
   }
 };
 
-// Has a bounded wait of this fill run out?  (Where rows are filled by the automaton the word keeps the generation of the fill that did.)
-__device__ __forceinline__ bool fill_aborted(const StateDev& S, uint32_t word) { return S.af.on ? word == S.gen : word != 0u; }
-
 // How often a bounded wait polls before it gives up: 2^dflt times, or 2^poll_limit_shift when the state
 // was created with a limit of its own (tests use a tiny one to take the give-up path).
 __device__ __forceinline__ uint32_t poll_limit(const StateDev& S, uint32_t dflt) {

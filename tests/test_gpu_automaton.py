@@ -470,3 +470,72 @@ def test_chains_completed_in_one_set(n, dfa):
     assert int(a[0]) == seq.num_sets
     if not dfa:  # (automata have items of their own)
         assert int(a[1]) == seq.total_items
+
+
+def test_a_captured_fill_that_gave_up_starts_afresh():
+    """A fill whose rounds run out hands out empty masks, and the next one is a fill like any, also where both are replays of one
+    captured call: "[[[[[[" with tokens of closing brackets takes a round for each, a string without tokens that end it takes one."""
+    import torch
+
+    import paper_2506_01151_b200 as fmt
+
+    w = workloads.build(2, V=300, batch=1, steps=1)
+    vocab = [bytes([b]) for b in range(256)] + [b"]" * k for k in range(2, 7)] + [b"xy", b""]
+    g = fmt.Grammar(w.ebnf, w.start, vocab, len(vocab) - 1)
+    st = fmt.State(g, 2, cache=False, wait_limit_log2=1)
+    seq, ov = oracle.Sequence_(oracle.Grammar(w.ebnf, w.start)), oracle.Vocab(vocab, len(vocab) - 1)
+    mask = torch.full((2, g.mask_words), -1, dtype=torch.int32, device="cuda")
+    graph = torch.cuda.CUDAGraph()
+    torch.cuda.synchronize()
+    with torch.cuda.graph(graph):
+        st.fill_mask(mask, stream=torch.cuda.current_stream().cuda_stream)
+
+    def feed(data):
+        for b in data:
+            st.advance(torch.full((2,), b, dtype=torch.int32, device="cuda"))
+        assert seq.advance(data)
+        torch.cuda.synchronize()
+        graph.replay()
+        torch.cuda.synchronize()
+        return mask.cpu().numpy().view(np.uint32)
+
+    assert not feed(b"[[[[[[").any() and st.stats()["fills_aborted"] == 1
+    for data in (b'"x', b"y"):
+        got = feed(data)
+        assert np.array_equal(got[0], seq.mask(ov)) and np.array_equal(got[1], seq.mask(ov))
+    assert not feed(b'",[[').any()
+    assert st.stats()["fills_aborted"] == 2 and st.stats()["capacity_errors"] == 0
+
+
+def test_captured_fills_with_rows_given_up():
+    """Rows that a replayed fill gives up are swept, those of this replay and not of the one before."""
+    import torch
+
+    import paper_2506_01151_b200 as fmt
+
+    text, vocab = _endings(340)
+    g, og, ov = fmt.Grammar(text, "s", vocab, len(vocab) - 1), oracle.Grammar(text, "s"), oracle.Vocab(vocab, len(vocab) - 1)
+    st = fmt.State(g, 24, cache=False)
+    mask = torch.full((24, g.mask_words), -1, dtype=torch.int32, device="cuda")
+    graph = torch.cuda.CUDAGraph()
+    torch.cuda.synchronize()
+    with torch.cuda.graph(graph):
+        st.fill_mask(mask, stream=torch.cuda.current_stream().cuda_stream)
+    deep, flat = b"(" * 20, b"((x)"
+    for replay in range(3):
+        texts = [deep + b"x" * (b % 2) if (b + replay) % 3 else flat for b in range(24)]
+        st.reset()
+        for i in range(max(map(len, texts))):
+            st.advance(torch.tensor([t[i] if i < len(t) else -1 for t in texts], dtype=torch.int32, device="cuda"))
+        torch.cuda.synchronize()
+        graph.replay()
+        torch.cuda.synchronize()
+        got, want = mask.cpu().numpy().view(np.uint32), {}
+        for t in set(texts):
+            s = oracle.Sequence_(og)
+            assert s.advance(t)
+            want[t] = s.mask(ov)
+        for b in range(24):
+            assert np.array_equal(got[b], want[texts[b]]), (replay, b)
+    s = st.stats()
+    assert s["rows_swept_again"] >= 3 * 12 and s["capacity_errors"] == 0 and s["fills_aborted"] == 0
