@@ -794,8 +794,8 @@ __global__ void __launch_bounds__(AF_THREADS, 2) automaton_fill_kernel(const __g
       filled = true;
       __syncthreads();
       const uint32_t n_items = J.off[J.m];
-      const bool few = staged && n_items <= AF_ITEMS;
-      const uint32_t most = min(AF_NODE, AF_NODES / n_items), own_item = lane * (AF_WARPS - 1u) + warp - 1u;  // (neighbouring items to different warps)
+      const bool few = staged && n_items <= AF_ITEMS;  // (a chart can have no item: a finite grammar's text, read to its end)
+      const uint32_t most = min(AF_NODE, AF_NODES / max(n_items, 1u)), own_item = lane * (AF_WARPS - 1u) + warp - 1u;  // (neighbouring items to different warps)
       uint2* const recs = reinterpret_cast<uint2*>(smem + SM_RECS);
       if (tid == 0) {  // a row for the mask, of the cache if one is left
         int32_t mrow = (int32_t)row;

@@ -539,3 +539,10 @@ def test_captured_fills_with_rows_given_up():
             assert np.array_equal(got[b], want[texts[b]]), (replay, b)
     s = st.stats()
     assert s["rows_swept_again"] >= 3 * 12 and s["capacity_errors"] == 0 and s["fills_aborted"] == 0
+
+
+def test_text_read_to_its_end():
+    """Nothing is left in the chart of a finite text that has been read to its end: EOS alone is valid."""
+    text = 's ::= "[" t "]" | "(" t ")"\nt ::= "ab" | "[" "x" "]"'
+    vocab = [bytes([b]) for b in range(256)] + [b"ab]", b"[x]", b"[x])", b"]]", b""]
+    _run(text, "s", vocab, [list(p) for p in (b"[ab]", b"([x])", b"[ab", b"(")])

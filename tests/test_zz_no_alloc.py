@@ -189,3 +189,22 @@ def test_noalloc_rows_that_outgrow_the_storage_of_contexts():
         seq = oracle.Sequence_(og)
         assert seq.advance(texts[b % 3])
         assert np.array_equal(got[b], seq.mask(ov)), b
+
+
+@pytest.mark.parametrize("accepting", [False, True])
+def test_noalloc_chart_without_items(accepting):
+    """One set and no item in it is a chart: nothing follows it but EOS, if it is accepting.  The chart beside it gets its mask."""
+    import torch
+
+    import paper_2506_01151_b200 as fmt
+
+    g = fmt.Grammar('s ::= "(" s ")" | "b"', "s", [b"(", b")", b"b", b"b)", b"(b)", b""], 5)
+    good = fmt.State(g, 1).chart_words(0)
+    empty = np.array([1, 0, int(accepting), 0, 0, 10, 0, 0, 0, 0], dtype=np.uint32)  # (the layout fmt_state_copy_chart documents)
+    offs = np.cumsum([0, len(empty), len(good), len(empty)]).astype(np.uint64)
+    charts = torch.from_numpy(np.concatenate([empty, good, empty]).view(np.int32)).cuda()
+    mask = torch.full((3, g.mask_words), -1, dtype=torch.int32, device="cuda")
+    status = torch.full((3,), -1, dtype=torch.int32, device="cuda")
+    fmt.fill_mask_noalloc(g, charts, offs, mask, status)
+    assert status.tolist() == [fmt.FMT_OK] * 3
+    assert mask[:, 0].tolist() == [int(accepting) << 5, 0b010101, int(accepting) << 5]
