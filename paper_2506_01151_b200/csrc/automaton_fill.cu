@@ -54,7 +54,7 @@ constexpr uint32_t CTX_NEW = 0xFFFFFFFFu;
 constexpr uint32_t AF_FOUND = 1u << 31;        // an entry whose edges are all of one item, with that item's context
 
 enum : uint32_t {
-  AC_OVF = 0, AC_FAIL = 2, AC_NCTX = 3, AC_POOL = 4, AC_NWORK = 5, AC_NBUF = 6, AC_OVER = 7, AC_SPILLED = 8, AC_WANT = 9,
+  AC_OVF = 0, AC_LATER = 1, AC_FAIL = 2, AC_NCTX = 3, AC_POOL = 4, AC_NWORK = 5, AC_NBUF = 6, AC_OVER = 7, AC_SPILLED = 8, AC_WANT = 9,
   AC_NWIDE = 10, AC_LIST = 11, AC_LIST_END = 12, AC_LOOKED = 13, AC_BEGAN = 14, AC_SLOT = 15,
   AC_EDGES = 16,   // [2] counters of the entries (see Deal)
   AC_TOKENS = 24,  // [2] and of the lists of tokens
@@ -639,12 +639,15 @@ __device__ __forceinline__ void expand_items(uint32_t m, uint32_t n, uint32_t mo
   C.exp[k] = make_uint2(n + most * k, cnt);
 }
 
-// More items of a last set than a warp's lanes hold.
-__device__ __noinline__ bool group_many(const GrammarDev& G, const AutoFillDev& A, uint32_t* ctl, uint32_t* buf, uint32_t n, uint2& out) {
+// More items of a last set than a warp's lanes hold.  False: their contexts do not fit shared memory (buf is in order then).
+__device__ __noinline__ bool group_many(const GrammarDev& G, uint32_t* ctl, uint32_t* buf, uint32_t n, uint2& out) {
+  return group_items(G, shared_contexts(), ctl, buf, n, out);
+}
+// The same when that was so.  Nobody else may be at the contexts: they are copied.
+__device__ __noinline__ bool group_spilled(const GrammarDev& G, const AutoFillDev& A, uint32_t* ctl, uint32_t* buf, uint32_t n, uint2& out) {
   Contexts C = shared_contexts();
-  if (group_items(G, C, ctl, buf, n, out)) return true;
   spill_contexts(C, ctl, A);
-  return group_items(G, C, ctl, buf, n, out);  // (sorted and without repeats already)
+  return group_items(G, C, ctl, buf, n, out);
 }
 
 // Wherever the chart and the contexts are, and however large the expansion is.
@@ -729,6 +732,8 @@ __global__ void __launch_bounds__(AF_THREADS, 2) automaton_fill_kernel(const __g
   auto token_deal = [&](uint32_t side) {
     return Deal{ctl + AC_TOKENS + 4u * side, lists, pre + 2u * AF_BATCH, owner + 2u * (AF_EDGES / 32u), AF_LISTS, AF_TOKENS};
   };
+  // where the kernel of a last set of so many items is put together
+  auto kernel_items = [&](uint32_t items) -> uint32_t* { return items <= AF_BUF ? buf : big_area(A) + A.big_cap / 4u + A.big_cap / 2u; };
   uint32_t looked_up = 0, contexts = 0;
   bool gave_up = false, filled = false;
   auto fill_tag = [&]() -> uint32_t { return S.counters[CNT_AF_NO] << 1 | 1u; };  // what this fill's blocks leave when one of them gives up
@@ -822,7 +827,7 @@ __global__ void __launch_bounds__(AF_THREADS, 2) automaton_fill_kernel(const __g
       __syncthreads();
       if (warp == 0) {  // the kernel of the chart's last set
         const uint32_t lo = J.off[J.m - 1u], hi = J.off[J.m], self = J.m - 1u;
-        uint32_t* b = hi - lo <= AF_BUF ? buf : big_area(A) + A.big_cap / 4u + A.big_cap / 2u;
+        uint32_t* const b = kernel_items(hi - lo);
         uint32_t n = 0;
         bool ok = hi - lo <= A.big_cap;
         if (ok)
@@ -842,9 +847,10 @@ __global__ void __launch_bounds__(AF_THREADS, 2) automaton_fill_kernel(const __g
           }
         __syncwarp();
         uint2 list = make_uint2(0u, 0u);
-        if (n > 32u || !group_shared(G.ga_item, lane < n ? b[lane] : 0xFFFFFFFFu, n, list)) ok = ok && group_many(G, A, ctl, b, n, list);
+        const bool later = ok && (n > 32u || !group_shared(G.ga_item, lane < n ? b[lane] : 0xFFFFFFFFu, n, list)) && !group_many(G, ctl, b, n, list);
         if (lane == 0) {
           ctl[AC_LIST] = list.x, ctl[AC_LIST_END] = list.y;
+          if (later) ctl[AC_LATER] = n;
           if (!ok) ctl[AC_FAIL] = 1u + DIAG_SET_SCRATCH;
         }
       } else {
@@ -852,6 +858,17 @@ __global__ void __launch_bounds__(AF_THREADS, 2) automaton_fill_kernel(const __g
         if (tid == AF_THREADS - 1) ctl[AC_BEGAN] = (uint32_t)(clock64() >> 10);
       }
       __syncthreads();
+      if (ctl[AC_LATER]) {  // (contexts leave shared memory when the other warps have made theirs)
+        if (warp == 0) {
+          uint2 list = make_uint2(0u, 0u);
+          const bool ok = group_spilled(G, A, ctl, kernel_items(J.off[J.m] - J.off[J.m - 1u]), ctl[AC_LATER], list);
+          if (lane == 0) {
+            ctl[AC_LIST] = list.x, ctl[AC_LIST_END] = list.y;
+            if (!ok) ctl[AC_FAIL] = 1u + DIAG_SET_SCRATCH;
+          }
+        }
+        __syncthreads();
+      }
 
       uint32_t* const mask = S.mask_rows + (size_t)ctl[AC_MASK] * G.Wm;
       bool spilled = false;

@@ -546,3 +546,17 @@ def test_text_read_to_its_end():
     text = 's ::= "[" t "]" | "(" t ")"\nt ::= "ab" | "[" "x" "]"'
     vocab = [bytes([b]) for b in range(256)] + [b"ab]", b"[x]", b"[x])", b"]]", b""]
     _run(text, "s", vocab, [list(p) for p in (b"[ab]", b"([x])", b"[ab", b"(")])
+
+
+@pytest.mark.parametrize("pairs", [98, 101, 102, 104])
+def test_contexts_that_leave_shared_memory_with_the_last_set(pairs):
+    """The items of the chart have contexts of their own; those of the last set's kernel, each begun in two of fifteen sets, come on
+    top, and from 102 pairs on all of them together are more than the 320 that shared memory holds."""
+    letters = b"abcdefghijklmno"
+    two = [(a, b) for a in range(15) for b in range(a + 1, 15)][:pairs]
+    end = lambda k: "%c%c" % (65 + k // 26, 65 + k % 26)
+    text = "s ::= p m \"!\"\np ::= [a-o]*\nm ::= " + " | ".join('x%d "%s"' % (k, end(k)) for k in range(pairs)) + ' | "(" m ")"\n'
+    text += "".join('x%d ::= "%sz" | "%sz"\n' % (k, letters[a:].decode(), letters[b:].decode()) for k, (a, b) in enumerate(two))
+    vocab = [bytes([b]) for b in range(256)] + [(end(k) + ("!" if k % 2 else "?")).encode() for k in range(pairs)] + [b""]
+    s = _run(text, "s", vocab, [list(letters + b"z")])
+    assert s["rows_swept_again"] == 0 and (s["walk_states"] > 320) == (pairs >= 102)
