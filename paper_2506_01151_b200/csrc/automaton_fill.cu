@@ -58,7 +58,9 @@ enum : uint32_t {
   AC_NWIDE = 10, AC_LIST = 11, AC_LIST_END = 12, AC_LOOKED = 13, AC_BEGAN = 14, AC_SLOT = 15,
   AC_EDGES = 16,   // [2] counters of the entries (see Deal)
   AC_TOKENS = 24,  // [2] and of the lists of tokens
-  AC_FULL = 32, AC_CLEARED = 33, AC_ROW = 33, AC_MASK = 34, AC_WORDS = 36
+  AC_FULL = 32, AC_CLEARED = 33, AC_ROW = 33, AC_MASK = 34,
+  AC_CROWDED = 35, AC_CUT = 36,  // rounds of all the block's rows: those that took one entry at a time, and those that put edges back
+  AC_WORDS = 40
 };
 static_assert(AC_WORDS % 4 == 0 && AC_WORDS <= AF_THREADS, "what follows in shared memory is cleared in 16-byte pieces; a thread clears a word");
 
@@ -796,6 +798,7 @@ __global__ void __launch_bounds__(AF_THREADS, 2) automaton_fill_kernel(const __g
       if (!filled)
         #pragma unroll 1
         for (uint32_t i = tid; i < AF_HSET; i += AF_THREADS) hset[i] = EMPTY_SLOT;
+      if (!filled && tid == 0) ctl[AC_CROWDED] = ctl[AC_CUT] = 0u;
       filled = true;
       __syncthreads();
       const uint32_t n_items = J.off[J.m];
@@ -974,7 +977,10 @@ __global__ void __launch_bounds__(AF_THREADS, 2) automaton_fill_kernel(const __g
               if (end > total) overflow(w.x + (max(from, total) - from), end - max(from, total), w.y);
             }
           // ---- the edges; those of a warp's next 32 are under way while these are looked at
-          if (tid == 0) looked_up += total;
+          if (tid == 0) {
+            looked_up += total;
+            if (total < all) ++ctl[AC_CUT];
+          }
           auto edge_of = [&](uint32_t base, uint2& w) -> uint4 {
             const uint32_t e = whose(E, n, base);
             if (base + lane >= total) return make_uint4(0u, 0u, 0u, 0u);
@@ -1040,7 +1046,10 @@ __global__ void __launch_bounds__(AF_THREADS, 2) automaton_fill_kernel(const __g
           const uint32_t k = dealt_lists(N), t = dealt_things(N);
           const bool tight = gtop + A.reserve + AF_TIGHT > A.stack_cap;
           __syncthreads();
-          if (tid == 0) ctl[AC_OVF] = 0u;
+          if (tid == 0) {
+            ctl[AC_OVF] = 0u;
+            if (tight) ++ctl[AC_CROWDED];
+          }
           if (tight) {
             #pragma unroll 1
             for (uint32_t i = tid; i < k; i += AF_THREADS) stack[gtop + i] = make_uint4(N.what[i].x, (i + 1u < k ? N.pre[i + 1u] : t) - N.pre[i], N.what[i].y, 0u);
@@ -1141,6 +1150,8 @@ __global__ void __launch_bounds__(AF_THREADS, 2) automaton_fill_kernel(const __g
   if (tid == 0) {
     stat_add(S, CNT_STAT_TRANS, ctl[AC_LOOKED]);
     stat_add(S, CNT_STAT_LOCAL, contexts);
+    if (ctl[AC_CROWDED]) stat_add(S, CNT_STAT_CROWDED, ctl[AC_CROWDED]);
+    if (ctl[AC_CUT]) stat_add(S, CNT_STAT_CUT, ctl[AC_CUT]);
   }
   // ---- rows that were given up, swept by the blocks that gave them up when they have no row left.  Only blocks that look for tables
   // wait, and who has tables waits for nobody.
@@ -1208,9 +1219,11 @@ static_assert(SM_CTL % 4 == 0 && SM_HSET % 4 == 0 && SM_SEEN % 4 == 0 && SM_RECS
 constexpr uint32_t AF_SWEEP_SMEM = block_sweep_words(AF_WARPS, MAX_NONTERMINALS / 32u) * 4u;  // a row that is given up is swept in the same shared memory
 constexpr uint32_t AF_SMEM_ASKED = AF_SMEM > AF_SWEEP_SMEM ? AF_SMEM : AF_SWEEP_SMEM;
 
-// Places of a block's stack that only its depth-first rounds use - what is left of an entry and what its edges start, along the longest
-// path of the trie - and the entries of a round that are put back.
-uint32_t automaton_fill_reserve() { return (MAX_TOKEN_BYTES + 2u) * (2u * AF_TIGHT_EDGES + 2u) + 3u * AF_BATCH; }
+// Places of a block's stack that only its depth-first rounds use, along the longest path of the trie - for every byte the edges to the
+// groups of a long list, then a group's, each edge's list and the rest of that, and what is left of both entries - and the entries of a
+// round that are put back.
+uint32_t automaton_fill_reserve() { return (MAX_TOKEN_BYTES + 2u) * (3u * AF_TIGHT_EDGES + 2u) + 3u * AF_BATCH; }
+static_assert(GA_EDGE_GROUP <= AF_CHUNK && AF_TIGHT_EDGES * AF_CHUNK <= AF_EDGES, "a group is one entry, and a depth-first round's lists find room");
 uint32_t automaton_fill_warps() { return AF_WARPS; }
 uint32_t automaton_fill_least_stack() { return automaton_fill_reserve() + AF_TIGHT + AF_SLICE; }
 

@@ -110,7 +110,9 @@ enum : uint32_t {
   CNT_AF_GIVEN_TAKEN = 195,    // how many of them a block has taken
   CNT_AF_TICKET = 196,         // rows handed out to blocks of the automaton's fill that have filled their first
   CNT_AF_NO = 197,             // the fills so far, counted on the device: a captured fill that is replayed is one more (its mark: << 1 | 1)
-  CNT_TOTAL = 200
+  CNT_STAT_CROWDED = 198,      // 64-bit: rounds of the automaton's fill that took one entry at a time, their stack being nearly full
+  CNT_STAT_CUT = 200,          // 64-bit: and those that put edges back on it, having no room for all that may follow
+  CNT_TOTAL = 204
 };
 
 enum : uint32_t {

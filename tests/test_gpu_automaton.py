@@ -35,7 +35,7 @@ def _run(text, start, vocab, prefixes, batch=None, check=None, **options):
         want.append(s.mask(ov))
     for b in range(batch) if check is None else check:
         assert np.array_equal(got[b], want[b % len(want)]), b
-    stats = st.stats()
+    stats = dict(st.stats(), counters=st.counters())
     assert stats["capacity_errors"] == 0 and stats["fills_aborted"] == 0
     return stats
 
@@ -140,12 +140,30 @@ def _braces():
 
 
 @pytest.mark.parametrize("batch", [1, 64, 149, 300])
-def test_rounds_that_push_more_than_the_stack_holds(batch):
-    """Threads and expansions that find no room in a round go to the block's stack, which is never pushed more than it holds: a row
-    has its mask, however many rows share the grid and however many children its nodes have."""
+def test_text_whose_every_byte_ends_a_rule(batch):
+    """Twenty thousand places at which the chart is asked: a row has its mask, however many rows share the grid."""
     text, vocab = _braces()
     s = _run(text, "doc", vocab, [list(p) for p in (b"x {a{b{c", b"{" * 30, b"a{}b{{", b"")], batch=batch, check=range(min(batch, 4)))
     assert s["walk_transitions"] > 20000 * batch  # (look-ups)
+
+
+CNT_CROWDED, CNT_CUT = 198, 200  # (device_tables.h)
+
+
+@pytest.mark.parametrize("batch", [1, 150, 300])
+def test_rounds_that_push_more_than_the_stack_holds(batch):
+    """A token of text for every two bytes it can begin with: each of 48,000 edges lists a further one, all at once, and a block's stack
+    has 32,768 places.  Rounds put back what may not find room, and take one entry at a time while little is left."""
+    kw = " | ".join('"\\x%02x!"' % b for b in range(256) if chr(b) not in "{}")
+    text = 'doc ::= piece*\npiece ::= char | "{" doc "}" | "}}" kw\nchar ::= [^{}\\x00-\\x20]\nkw ::= "!" | ' + kw + "\n"
+    rng = np.random.default_rng(12)
+    chars = np.array([b for b in range(33, 256) if chr(b) not in "{}"], np.uint8)
+    vocab = [bytes([b]) for b in range(256)]
+    vocab += [bytes([a, b]) + bytes(chars[rng.integers(0, len(chars), 2 if rng.random() < 0.9 else 6)]) for a in chars for b in chars]
+    vocab += sorted({bytes(rng.integers(0, 33, 7).astype(np.uint8)) for _ in range(80000)}) + [b""]  # (no text: see _braces)
+    s = _run(text, "doc", vocab, [list(p) for p in (b"x{a{b", b"")], batch=batch, check=range(min(batch, 2)))
+    assert s["rows_swept_again"] == 0 and s["walk_transitions"] > 80000 * batch
+    assert s["counters"][CNT_CROWDED] > 500 * batch and s["counters"][CNT_CUT] >= batch / 2  # (the second row has no braces to end)
 
 
 def _endings(n):
