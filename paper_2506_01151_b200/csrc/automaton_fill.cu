@@ -44,6 +44,7 @@ constexpr uint32_t AF_STAGE = 768;        // a chart up to this many words is re
 constexpr uint32_t AF_ITEMS = AF_THREADS - 32;  // items of a chart whose contexts are made and expanded beforehand, an item to a thread
 constexpr uint32_t AF_NODE = 24, AF_NODES = 1344;  // items of such an expansion, and of all of them, at most
 constexpr uint32_t AF_QUEUE = 13;         // completions that such an expansion makes at most
+constexpr uint32_t AF_SCAN = 256, AF_LANES = 4;  // items that a lane looks at to expand a context by itself, and contexts from which on lanes do
 constexpr uint32_t AF_CTX = AF_ITEMS + 96, AF_CTX_HASH = 1024, AF_POOL = 3072;  // contexts in shared memory, words of their lists
 constexpr uint32_t AF_BUF = 512, AF_WORK = 256, AF_HSET = 512;      // an expansion in shared memory (larger ones: global memory)
 constexpr uint32_t AF_KCYCLES = 1u << 14;      // a row that takes longer (2^24 cycles, 8.5 ms) is given up for a sweep by Earley steps
@@ -60,6 +61,7 @@ enum : uint32_t {
   AC_TOKENS = 24,  // [2] and of the lists of tokens
   AC_FULL = 32, AC_CLEARED = 33, AC_ROW = 33, AC_MASK = 34,
   AC_CROWDED = 35, AC_CUT = 36,  // rounds of all the block's rows: those that took one entry at a time, and those that put edges back
+  AC_ONE_BY_ONE = 37,            // the row's contexts are not for lanes
   AC_WORDS = 40
 };
 static_assert(AC_WORDS % 4 == 0 && AC_WORDS <= AF_THREADS, "what follows in shared memory is cleared in 16-byte pieces; a thread clears a word");
@@ -266,16 +268,15 @@ __device__ __noinline__ void spill_contexts(Contexts& C, uint32_t* ctl, const Au
   for (uint32_t i = lane; i <= D.hash_mask; i += 32) D.hash[i] = 0u;
   __syncwarp();
   #pragma unroll 1
-  for (uint32_t c = 0; c < n; ++c) {
+  for (uint32_t c = lane; c < n; c += 32) {  // (none is compared: a repeat, of a chart of few items, does as well)
     const uint2 o = D.org[c];
-    uint32_t slot = context_hash(D.lhs[c], D.pool + o.x, o.y) & D.hash_mask;
-    if (lane == 0) {
-      #pragma unroll 1
-      while (D.hash[slot]) slot = (slot + 1u) & D.hash_mask;
-      D.hash[slot] = c + 1u;
-    }
-    __syncwarp();
+    uint32_t h = 0;
+    #pragma unroll 1
+    for (uint32_t i = 0; i < o.y; ++i) h += mix32(D.pool[o.x + i] + 1u);
+    #pragma unroll 1
+    for (uint32_t slot = mix32(h + D.lhs[c] * 0x9E3779B9u + o.y) & D.hash_mask; atomicCAS(&D.hash[slot], 0u, c + 1u) != 0u;) slot = (slot + 1u) & D.hash_mask;  // (as context_hash has it)
   }
+  __syncwarp();
   C = D;
   if (lane == 0) ctl[AC_SPILLED] = 1u;
   __syncwarp();
@@ -544,6 +545,68 @@ __device__ __noinline__ bool expand_shared(const uint32_t* ga_item, uint32_t m, 
   if (lane == 0) C.exp[c] = list;
   __syncwarp();
   return true;
+}
+
+// Contexts of one origin, a lane for each (CTX_NEW: none): the lanes look through the sets that their completions lead to, then the warp enters
+// what each has found.  Those that have more than AF_NODE items or AF_QUEUE completions, or items of one rule begun in several
+// sets, and those for which there is no room stay as they were.  One after the other, by the whole warp, the contexts of 64 charts
+// of 20 kinds of brackets, 20 deep (some 800 items, 240 contexts), took 1,500 us a fill, now 820; below four at a time the warp is as fast.
+__device__ __noinline__ void expand_by_lanes(const uint32_t* ga_item, const Contexts& C, const AfChart& J, bool staged, uint32_t* ctl, uint32_t c) {
+  const uint32_t lane = lane_id();
+  const uint2* recs = reinterpret_cast<const uint2*>(smem + SM_RECS);
+  uint32_t* const found = smem + SM_BUF;  // [AF_NODE][32] rule << 16 | origin
+  static_assert(32u * AF_NODE <= AF_BUF + AF_WORK, "what the lanes have found");
+  uint32_t queue[AF_QUEUE], nq = 0, cnt = 0, left = AF_SCAN;  // what has been completed, non-terminal << 16 | origin
+  bool fits = c != CTX_NEW;
+  if (fits) queue[nq++] = C.lhs[c] << 16 | C.pool[C.org[c].x];
+#pragma unroll 1
+  for (uint32_t head = 0; fits && head < nq; ++head) {
+    const uint32_t a = queue[head] >> 16, o = queue[head] & 0xFFFFu, lo = J.off[o], hi = J.off[o + 1u];
+    fits = hi - lo <= left;
+    left -= hi - lo;
+#pragma unroll 1
+    for (uint32_t j = lo; fits && j < hi; ++j) {
+      const uint32_t it = J.items[j];
+      const uint2 rec = staged ? recs[j] : __ldg(reinterpret_cast<const uint2*>(ga_item) + (it & 0xFFFFu));
+      if (rec.x >> 16 != a) continue;
+      if (rec.y & GA_GOES_ON) {
+        const uint32_t v = ((it & 0xFFFFu) + 1u) << 16 | it >> 16;
+        uint32_t same = 0xFFFFFFFFu;
+#pragma unroll 1
+        for (uint32_t x = 0; x < cnt; ++x) {
+          const uint32_t u = found[32u * x + lane];
+          if (u >> 16 == v >> 16) same = u;
+        }
+        if (same != 0xFFFFFFFFu) fits = same == v;
+        else if (cnt == AF_NODE) fits = false;
+        else found[32u * cnt++ + lane] = v;
+      }
+      if ((rec.y & 0xFFFFu) != 0xFFFFu) {
+        const uint32_t up = rec.y << 16 | it >> 16;
+        uint32_t x = 0;
+#pragma unroll 1
+        while (x < nq && queue[x] != up) ++x;
+        if (x == AF_QUEUE) fits = false;
+        else if (x == nq) queue[nq++] = up;
+      }
+    }
+  }
+  __syncwarp();
+  uint32_t m = __ballot_sync(FULL, fits);
+  if (m == 0u && lane == 0) ctl[AC_ONE_BY_ONE] = 1u;  // (what one of them lacks others will: lists of a hundred rules, sets of hundreds of items)
+#pragma unroll 1
+  for (; m; m &= m - 1u) {
+    const uint32_t src = (uint32_t)__ffs(m) - 1u, n = __shfl_sync(FULL, cnt, src), x = lane < n ? found[32u * lane + src] : 0u;
+    const uint32_t to = intern_singles(C, ctl, lane < n, lane < n ? __ldg(&ga_item[2u * (x >> 16)]) & 0xFFFFu : 0u, x & 0xFFFFu);
+    const uint32_t at = ctl[AC_POOL];
+    if (__any_sync(FULL, lane < n && to == CTX_NEW) || n > C.pool_cap - at) break;
+    if (lane < n) C.pool[at + lane] = (x & 0xFFFF0000u) | to;
+    if (lane == src) C.exp[c] = make_uint2(at, n);
+    __syncwarp();
+    if (lane == 0) ctl[AC_POOL] = at + n;
+    __syncwarp();
+  }
+  __syncwarp();
 }
 
 // ---- contexts of one origin that a chart of few items can ask for, all at once
@@ -818,6 +881,7 @@ __global__ void __launch_bounds__(AF_THREADS, 2) automaton_fill_kernel(const __g
       }
       if (warp == 0) {
         if (lane < 4u) deal_clear(lane < 2u ? edge_deal(lane) : token_deal(lane - 2u));
+        if (lane == 30u) ctl[AC_ONE_BY_ONE] = 0u;
         if (few && lane == 31u) ctl[AC_NCTX] = n_items, ctl[AC_POOL] = n_items * (1u + most);
       } else if (staged) {  // what the expansions need to know about the chart's items
 #pragma unroll 1
@@ -1091,6 +1155,11 @@ __global__ void __launch_bounds__(AF_THREADS, 2) automaton_fill_kernel(const __g
 #pragma unroll 1
           for (uint32_t base = 0; base < k; base += 32) {
             const uint32_t c = base + lane < k ? N.what[base + lane].y : AF_FOUND;
+            const uint32_t many = __ballot_sync(FULL, !(c & AF_FOUND) && C.exp[c & ~AF_FOUND].y == CTX_NEW);
+            if (__popc(many) >= AF_LANES && !ctl[AC_ONE_BY_ONE]) {
+              const bool first = (uint32_t)__ffs(__match_any_sync(FULL, c)) == lane + 1u, mine = (many >> lane & 1u) && first && C.org[c & ~AF_FOUND].y == 1u;
+              if (__popc(__ballot_sync(FULL, mine)) >= AF_LANES) expand_by_lanes(G.ga_item, C, J, staged, ctl, mine ? c : CTX_NEW);
+            }
 #pragma unroll 1
             for (uint32_t todo = __ballot_sync(FULL, !(c & AF_FOUND) && C.exp[c & ~AF_FOUND].y == CTX_NEW); todo;) {
               const uint32_t x = __shfl_sync(FULL, c, __ffs(todo) - 1);

@@ -173,7 +173,7 @@ def _endings(n):
     text = "s ::= t\nt ::= \"x\" | " + " | ".join("t%d" % i for i in range(n)) + "\n"
     text += "".join('t%d ::= "(" t ")" "%s"\n' % (i, k) for i, k in enumerate(kinds))
     rng = np.random.default_rng(n)
-    chains = [b"".join(b")" + kinds[int(i)].encode() for i in rng.integers(0, n if k % 2 else 20, 16))[:32] for k in range(60)]
+    chains = [b"".join(b")" + kinds[int(i)].encode() for i in rng.integers(0, n if k % 2 else min(n, 20), 16))[:32] for k in range(60)]
     vocab = [bytes([b]) for b in range(256)] + [b"x" + c[:3 * k + 1] for k, c in enumerate(chains[:10])] + chains + [b")(", b"(("]
     letters = np.frombuffer(b"abcdefghijklmnopqrstuvwxyz", np.uint8)
     return text, vocab + sorted({bytes(letters[rng.integers(0, 26, 6)]) for _ in range(100000)}) + [b""]
@@ -187,6 +187,15 @@ def test_rows_that_outgrow_the_storage_of_contexts(n, batch):
     prefixes = [list(p) for p in (b"(" * 20, b"(" * 20 + b"x", b"(" * 20 + b"x)a", b"((x)a")]
     s = _run(text, "s", vocab, prefixes, batch=batch, check=range(min(batch, 4)))
     assert s["rows_swept_again"] <= batch and (n == 20 or s["rows_swept_again"] > 0)
+
+
+@pytest.mark.parametrize("kinds, depth", [(2, 60), (3, 60), (4, 60), (5, 40), (23, 12), (24, 12), (25, 12), (20, 24), (64, 5), (65, 5), (130, 4)])
+def test_contexts_asked_for_many_at_once(kinds, depth):
+    """A closing bracket asks for a context of every kind.  Charts of more items than threads: from four contexts on lanes expand them,
+    up to 24 items each, having looked at 256 (two sets of two items a kind); the others are left to the warp."""
+    text, vocab = _endings(kinds)
+    s = _run(text, "s", vocab, [list(p) for p in (b"(" * depth, b"(" * depth + b"x", b"(" * depth + b"x)a", b"((x)a")])
+    assert s["rows_swept_again"] == 0
 
 
 def test_rows_given_up_in_one_fill_after_the_other():
