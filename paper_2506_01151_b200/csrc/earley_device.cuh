@@ -534,6 +534,8 @@ __device__ __forceinline__ void scannable_bytes(const GrammarDev& G, const uint3
 }
 
 // Ascending bitonic sort of a[0..n), n > 32; the array must have room for the next power of two >= n, which must not exceed cap_pow2.
+// (A pair to a lane.  With an element to a lane, of which every other had nothing to do, an advance among sets of hundreds of items spent more here
+// than anywhere else once the loop was rolled: 64 rows of 180 like variants 29.7 us, now 21.8.)
 static __device__ __noinline__ void sort_large(uint32_t* a, uint32_t n, uint32_t cap_pow2) {
   const uint32_t lane = lane_id();
   uint32_t P = 32;
@@ -549,15 +551,12 @@ static __device__ __noinline__ void sort_large(uint32_t* a, uint32_t n, uint32_t
 #pragma unroll 1
     for (uint32_t j = k >> 1; j > 0; j >>= 1) {
 #pragma unroll 1
-      for (uint32_t i = lane; i < P; i += 32) {
-        uint32_t l = i ^ j;
-        if (l > i) {
-          uint32_t x = a[i], y = a[l];
-          bool up = (i & k) == 0;
-          if ((x > y) == up) {
-            a[i] = y;
-            a[l] = x;
-          }
+      for (uint32_t t = lane; t < P / 2u; t += 32) {
+        const uint32_t i = 2u * t - (t & (j - 1u)), l = i + j, x = a[i], y = a[l];
+        const bool up = (i & k) == 0;
+        if ((x > y) == up) {
+          a[i] = y;
+          a[l] = x;
         }
       }
       __syncwarp();
