@@ -548,7 +548,7 @@ fmt_status fmt_state_create(const fmt_grammar* g, uint32_t batch, const fmt_stat
     AL(af.scratch, (size_t)af.grid * af.scratch_words, 0);
     af.sweep_slots = std::min(batch, 16u);
     AL(af.given, batch + af.sweep_slots, 0);
-    af.sweep_lock = af.given + batch;
+    af.sweep_lock = reinterpret_cast<uint32_t*>(af.given + batch);
     if (e == cudaSuccess) e = alloc_row_sweeps(s);
   } else if (e == cudaSuccess) {
     e = alloc_sweep(s);

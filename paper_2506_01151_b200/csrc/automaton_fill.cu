@@ -802,11 +802,7 @@ __global__ void __launch_bounds__(AF_THREADS, 2) automaton_fill_kernel(const __g
   uint32_t looked_up = 0, contexts = 0;
   bool gave_up = false, filled = false;
   auto fill_tag = [&]() -> uint32_t { return S.counters[CNT_AF_NO] << 1 | 1u; };  // what this fill's blocks leave when one of them gives up
-  if (blockIdx.x == 0 && tid == 0) {
-    stat_add(S, CNT_STAT_FILLS, S.B);
-    const uint32_t e = vload(&S.counters[CNT_BAR_ERR]);  // (an earlier fill's; a block of this one that gives up writes this one's)
-    if (e && e != fill_tag()) atomicCAS(&S.counters[CNT_BAR_ERR], e, 0u);
-  }
+  if (blockIdx.x == 0 && tid == 0) stat_add(S, CNT_STAT_FILLS, S.B);
   #pragma unroll 1
   for (uint32_t row = blockIdx.x; row < S.B;) {
     // ---- where the row's mask comes from: the state cache, another row of this call with the same chart, or from here
@@ -816,6 +812,8 @@ __global__ void __launch_bounds__(AF_THREADS, 2) automaton_fill_kernel(const __g
     const int32_t sid = S.row_state ? S.row_state[row] : -1;
     const uint32_t taken = tid == 0 && S.cache_on ? vload(&S.counters[CNT_N_MASK_ROWS]) : 0u;
     const uint32_t ahead = tid < A.ahead ? chart[tid] : 0u;  // (asked for together with the header)
+    // an earlier fill's mark goes (by a thread that nobody waits for, when what it asks for is long there)
+    const uint32_t mark = row == 0u && tid == AF_THREADS - 1 ? vload(&S.counters[CNT_BAR_ERR]) : 0u;
     AfChart J;
     J.m = chart[CH_SETS];
     const uint32_t chart_words = chart[CH_WORDS], chart_flags = chart[CH_FLAGS];
@@ -842,6 +840,7 @@ __global__ void __launch_bounds__(AF_THREADS, 2) automaton_fill_kernel(const __g
       if (S.row_job) S.row_job[row] = here ? 1u : 0u;
       ctl[AC_ROW] = here ? 1u : 0u;
     }
+    if (mark && mark != fill_tag()) atomicCAS(&S.counters[CNT_BAR_ERR], mark, 0u);
     __syncthreads();
     if (ctl[AC_ROW]) {
       const bool accepting = (chart_flags & CHART_ACCEPTING) != 0u, staged = chart_words <= AF_STAGE;
@@ -1197,7 +1196,7 @@ __global__ void __launch_bounds__(AF_THREADS, 2) automaton_fill_kernel(const __g
         __threadfence();
         if (tid == 0) {
           if (ctl[AC_FAIL] != AF_LATE) diag(S, ctl[AC_FAIL] - 1u);
-          *reinterpret_cast<volatile uint32_t*>(A.given + atomicAdd(&S.counters[CNT_AF_GIVEN], 1u)) = row + 1u;
+          *reinterpret_cast<volatile unsigned long long*>(A.given + atomicAdd(&S.counters[CNT_AF_GIVEN], 1u)) = (unsigned long long)fill_tag() << 32 | row;
         }
       }
     }
@@ -1239,11 +1238,12 @@ __global__ void __launch_bounds__(AF_THREADS, 2) automaton_fill_kernel(const __g
         at = was;
       }
       if (got != 0xFFFFFFFFu) {
-        uint32_t k = blockIdx.x % A.sweep_slots, v = 0u;
+        uint32_t k = blockIdx.x % A.sweep_slots;
+        unsigned long long v = 0u;
         #pragma unroll 1
         for (uint32_t polls = 0; slot == 0xFFFFFFFFu; ++polls, k = (k + 1u) % A.sweep_slots) {
-          if (v == 0u) v = vload(A.given + got);  // (written right after its number was drawn)
-          if (v && atomicCAS(A.sweep_lock + k, 0u, 1u) == 0u) slot = k;
+          if (v >> 32 != fill_tag()) v = *reinterpret_cast<const volatile unsigned long long*>(A.given + got);  // (written right after its number was drawn)
+          if (v >> 32 == fill_tag() && atomicCAS(A.sweep_lock + k, 0u, 1u) == 0u) slot = k;
           else if (ld_acquire(&S.counters[CNT_BAR_ERR]) == fill_tag()) break;
           else if (polls > poll_limit(S, 22)) {
             diag(S, DIAG_WAIT_VALUE);
@@ -1253,7 +1253,7 @@ __global__ void __launch_bounds__(AF_THREADS, 2) automaton_fill_kernel(const __g
             __nanosleep(400);
           }
         }
-        ctl[AC_SLOT] = v - 1u;
+        ctl[AC_SLOT] = (uint32_t)v;
         __threadfence();
       }
       ctl[AC_ROW] = slot;

@@ -264,7 +264,7 @@ struct AutoFillDev {
   uint32_t* scratch;         // [grid][scratch_words]
   uint32_t scratch_words;
   uint32_t ctx_cap, pool_cap, big_cap;  // contexts per row, words for their lists, items of the largest expansion (powers of two)
-  uint32_t* given;           // [rows] the rows given up, + 1; 0 between fills
+  unsigned long long* given; // [rows] the rows given up, mark of the fill (CNT_AF_NO) << 32 | row
   uint32_t* sweep_lock;      // [sweep_slots] 1: a block sweeps a row in these tables (StateDev::au); 0 between launches
   uint32_t sweep_slots;
   uint32_t ahead;            // words that may be read from where a chart begins, however long it is

@@ -841,7 +841,6 @@ __device__ __forceinline__ int32_t resolve_mask_row(const StateDev& S, uint32_t 
 // (one thread per row, in the kernel that reads the masks) A mask computed in this call becomes the cache's, or its claim is
 // released: when the row had no cache row, or broke, or the fill was given up.
 __device__ __forceinline__ void publish_row(const StateDev& S, uint32_t row) {
-  if (S.af.on) S.af.given[row] = 0u;
   if (!S.row_job[row]) return;
   const bool aborted = S.counters[CNT_BAR_ERR] != 0u;
   const int32_t sid = S.row_state[row], mrow = S.row_mask[row];
@@ -852,7 +851,7 @@ __device__ __forceinline__ void publish_row(const StateDev& S, uint32_t row) {
 __device__ __forceinline__ void fill_is_through(const StateDev& S) {
   if (!S.af.on) return;
   S.counters[CNT_AF_TICKET] = S.counters[CNT_AF_GIVEN] = S.counters[CNT_AF_GIVEN_TAKEN] = S.counters[CNT_AUTO_ITEMS] = 0u;
-  ++S.counters[CNT_AF_NO];
+  atomicAdd(&S.counters[CNT_AF_NO], 1u);  // (nothing waits for it)
 }
 
 // mask_out[row][w] for every row

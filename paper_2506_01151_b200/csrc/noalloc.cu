@@ -54,7 +54,7 @@ constexpr uint32_t NA_CTX = 1024, NA_POOL = 8u << 10, NA_LARGE = 4u << 10;
 constexpr uint32_t NA_FILL_SCRATCH = 7u * NA_CTX + NA_POOL + NA_LARGE / 4u + NA_LARGE / 2u + NA_LARGE;
 constexpr size_t NA_OFF_FILL = NA_HEADER_WORDS + 4 * (size_t)NA_FILL_BLOCKS * NA_STACK;
 constexpr size_t NA_OFF_ROW_FLAGS = NA_OFF_FILL + (size_t)NA_FILL_BLOCKS * NA_FILL_SCRATCH;
-static_assert(NA_OFF_ROW_FLAGS + NA_MAX <= NA_SWEEP_WORDS, "the fill's tables do not fit");
+static_assert(NA_OFF_ROW_FLAGS + 2 * NA_MAX <= NA_SWEEP_WORDS && NA_OFF_ROW_FLAGS % 2 == 0, "the fill's tables do not fit");
 // behind both: tables of Earley sets for the charts that this fill gives up, one chart at a time
 constexpr uint32_t NA_BLOCK_WARPS = 8;
 constexpr size_t NA_ROW_ST_ENTRIES = 2u << 20;
@@ -103,7 +103,7 @@ __global__ void noalloc_prepare_kernel(GrammarDev G, StateDev S, uint32_t* scrat
   }
   for (size_t i = tid; i < (size_t)n * G.Wm; i += nth) mask[i] = 0u;
   if (S.af.on) {
-    if (tid < NA_MAX) S.af.given[tid] = 0u;
+    if (tid < NA_MAX) S.af.given[tid] = 0ull;
     if (tid == 0) *S.af.sweep_lock = 0u;
     return;
   }
@@ -245,7 +245,7 @@ extern "C" fmt_status fmt_fill_mask_noalloc(const fmt_grammar* g, const uint32_t
     A.scratch = scratch + NA_OFF_FILL;
     A.ctx_cap = NA_CTX, A.pool_cap = NA_POOL, A.big_cap = NA_LARGE;
     A.ahead = CH_HDR;  // (the caller's memory may end with its last chart)
-    A.given = scratch + NA_OFF_ROW_FLAGS;
+    A.given = reinterpret_cast<unsigned long long*>(scratch + NA_OFF_ROW_FLAGS);
     A.sweep_slots = 1, A.sweep_lock = scratch + NA_OFF_ROW_LOCK;
     S.big_scratch = scratch + NA_OFF_ROW_BIG;
     S.au.recs = scratch + NA_OFF_ROW_RECS;
