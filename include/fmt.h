@@ -179,7 +179,7 @@ typedef struct {
  * Along with the tables goes the grammar's automaton over the vocabulary: what a token's bytes do to one unfinished
  * Earley item, whatever the chart holds, worked out on the host (0.04 to 0.25 s for a 128 K vocabulary in the
  * measured workloads) and used by every fill.  A grammar for which it grows too large (sets of more than 1024 items,
- * 2^18 sets, half a second of work), or whose rules end inside tokens so often that its fills would be slower
+ * 2^18 sets, a second of work), or whose rules end inside tokens so often that its fills would be slower
  * with it (text character by character, unions of dozens of variants), goes without; its rows are then swept by Earley steps.
  * The grammar is immutable and may be shared by any number of states.
  */

@@ -33,12 +33,15 @@ using u64 = uint64_t;
 // limits; a grammar beyond them has no automaton and its fills run the Earley steps themselves
 constexpr u32 GA_MAX_SETS = 1u << 18;
 constexpr u64 GA_MAX_TRANS = 32u << 20;   // table entries (4 bytes each)
-// Look-ups of the walk over the trie, items scanned and every eighth comparison for a new transition; as many again for the wide items.
-// Together half a second at most (10 to 15 ns each: HTML with 90 tags, 44 million 0.69 s; JSON, SQL and JSON schemas over 128 K tokens have
-// 0.5 to 4 million, 0.04 to 0.2 s).
+// Look-ups of the walk over the trie, items scanned and every eighth comparison for a new transition: a quarter of a second at most (10 to
+// 15 ns each: HTML with 90 tags, 44 million 0.69 s; JSON, SQL and JSON schemas over 128 K tokens have 0.5 to 4 million, 0.04 to 0.2 s).
 constexpr u64 GA_MAX_WORK = 16u << 20;
-// Look-ups for the starts: those of JSON, SQL, JSON schemas and tagged unions over 128 K tokens take 0.3 to 1.6 times as many as that walk.
-constexpr u64 GA_MAX_START_WORK = 64u << 20;
+// The same for the starts, every eighth token of theirs and GA_LINK_WORK for each edge, which takes as long as that: three quarters of a
+// second at most.  Those of JSON, SQL, JSON schemas and tagged unions over 128 K tokens take 0.3 to 1.6 times as many look-ups as that
+// walk and have up to 200,000 edges; words of letters whose every byte may end a word, 12,000 of 32 bytes, have 6.6 million and took
+// 1.65 s while only look-ups counted.
+constexpr u64 GA_MAX_START_WORK = 48u << 20;
+constexpr u64 GA_LINK_WORK = 16;
 constexpr size_t GA_MAX_WORDS = 64u << 20;  // of masks, tokens and edges
 constexpr size_t GA_MASK_TOKENS = 1024;   // a kernel's item from which so many tokens follow has a mask in the place of a list
 constexpr size_t GA_LONG_LIST = 64;       // edges of a start from which on it has one for each item and the others behind it
@@ -432,6 +435,7 @@ class Builder {
         }
       }
       st[i].n_tok = (u32)toks.size();
+      work_ += toks.size() / 8u;
       if (i < roots && toks.size() >= GA_MASK_TOKENS) {
         const u32 words = (h_.Wm + 3u) & ~3u;
         mask_of[i] = (u32)(h_.ga_mask.size() / words);
@@ -449,7 +453,7 @@ class Builder {
       st[i].link = (u32)links.size();
       for (u32 c : exits)
         for (u32 d : f)
-          if (root_[d] != GA_DEAD && goes_on(c, root_[d])) links.push_back({d, start(c, root_[d])});
+          if (root_[d] != GA_DEAD && goes_on(c, root_[d])) links.push_back({d, start(c, root_[d])}), work_ += GA_LINK_WORK;
       st[i].n_link = (u32)links.size() - st[i].link;
     }
     // edges: deeper nodes have larger numbers, so what a start's edges lead to is there before it

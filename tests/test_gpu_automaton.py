@@ -240,22 +240,42 @@ def test_text_whose_rules_end_everywhere(text, start, prefixes, batch):
     assert s["walk_transitions"] < 2000 * batch and s["rows_swept_again"] == 0
 
 
-def test_compiling_takes_a_bounded_time():
-    """The automaton's tables take half a second at most, whether the grammar gets them or not (300 kinds of elements around text)."""
+def _compile_seconds(text, start, vocab, eos):
+    """Processor time of the automaton's tables (and of the upload)."""
     import time
 
     import paper_2506_01151_b200 as fmt
 
+    took = []
+    for host_only in (True, True, False):  # (the first call builds or loads the library)
+        t = time.process_time()
+        fmt.Grammar(text, start, vocab, eos, host_only=host_only)
+        took.append(time.process_time() - t)
+    return took[2] - took[1]
+
+
+def test_compiling_takes_a_bounded_time():
+    """The walk over the trie takes a quarter of a second at most, whether the grammar gets the tables or not (300 kinds of elements around
+    text, refused in the walk)."""
     w = workloads.build(2, V=128256, batch=1, steps=1)
     tags = _words(np.random.default_rng(1), 300, 4)
     text = "content ::= node*\nnode ::= char | entity | " + " | ".join('"<%s>" content "</%s>"' % (x, x) for x in tags)
     text += '\nchar ::= [^<&]\nentity ::= "&" [a-z]+ ";"\n'
-    took = []
-    for host_only in (True, True, False):  # (the first call builds or loads the library)
-        t = time.process_time()
-        fmt.Grammar(text, "content", w.vocab, w.eos, host_only=host_only)
-        took.append(time.process_time() - t)
-    assert took[2] - took[1] < 0.7, took  # (half a second, and the upload)
+    took = _compile_seconds(text, "content", w.vocab, w.eos)
+    assert took < 0.7, took
+
+
+def test_starts_and_edges_take_a_bounded_time():
+    """Words of letters whose every byte may end a word, one after the other: 24,000 tokens of 32 bytes would have 13 million edges.  The walk
+    and the starts' allowance, a second together, and the trie of 3 million nodes."""
+    rng = np.random.default_rng(1)
+    kw = " | ".join('"%s!"' % c for c in "abcdefghijklmnopqrstuvwxyz0123456789")
+    text = 's ::= "(" p ")"\np ::= (w | "(" p ")" | "=" kw)*\nkw ::= %s\nw ::= [a-z]+ "0"?\n' % kw
+    letters, others = np.frombuffer(b"abcdefghijklmnopqrstuvwxyz", np.uint8), np.frombuffer(b"0123456789!", np.uint8)
+    vocab = [bytes([b]) for b in range(256)] + [bytes(letters[rng.integers(0, 26, 32)]) for _ in range(24000)]
+    vocab += [b"!" + bytes(others[rng.integers(0, 11, 31)]) for _ in range(88800)] + [b""]  # (no text: see _braces)
+    took = _compile_seconds(text, "s", vocab, len(vocab) - 1)
+    assert took < 2.0, took  # (3.3 s while only look-ups counted, 0.95 now)
 
 
 def test_grammar_without_an_automaton():
