@@ -202,7 +202,8 @@ class Driver:
         self.state.advance(self.tokens[i], self.status, stream=s)
         lg = self.ring[i % self.n_ring] if logits is None else logits
         self.state.fill_and_apply(lg, self.fmt.BF16, stream=s)
-        # advance; [plan, entry look-up (2), sweep of new entries, its collection, job set-up,] fill, mask+apply
+        # advance; [plan, entry look-up (2), sweep of new entries, its collection, job set-up,] fill, mask+apply (a sweep without these
+        # entries has its plan, too: added where the step's kernels are known)
         self.launches += 9 if self.roots else 3
 
     def restart(self, warmup: int, clear_caches: bool):
@@ -412,7 +413,7 @@ def run_ours(args):
                        "what": "per decoding step (advance + fill + masking of B rows), CUDA events around every step of the median repeat"},
         "kernel_latency_ms": {name: ({"p50": percentile(xs, 0.5), "p99": percentile(xs, 0.99), "max": max(xs), "launches": len(xs)} if xs else None)
                               for name, xs in med["series"].items()},
-        "clocks": clocks, "e2e": e2e, "gpu_launches": med["launches"], "roofline": roofline,
+        "clocks": clocks, "e2e": e2e, "gpu_launches": med["launches"] + (0 if drv.roots or by_tables else K), "roofline": roofline,
         "cache": {"fills": st["fills"], "computed": jobs, "from_state_cache": st["fills_from_cache"], "shared_within_fill": st["fills_shared"],
                   "hit_rate": 1.0 - jobs / fills,
                   "computed_by": {"context_independent_row_only": st["rows_mask_only"], "sweep_in_frames": st["rows_from_root"],
