@@ -13,12 +13,15 @@
 // What bounds it: latency, 35,000 cycles for a row of JSON.  About 2,500 until the chart is there, 5,000 for the contexts of its items, 5,000 for
 // the starts and their masks, and a few rounds (as many as rules end one after the other inside a token) of 2,500 to 3,500 each: a
 // read of edges, a search, the sums that deal lists out to the lanes, and two barriers.  Fills on a B200 by a walk of the trie over byte
-// classes, a byte a round; by edges with eight blocks to a row, each with its own contexts; and now, us:
-//   37 rows of JSON, 50,001 tokens                      139     65     42
-//   256 rows of ambiguous JSON, 128,256 tokens        1,010    790    275
-//   24 charts of JSON, 32,000 tokens, no allocations    123     71     47
-// and with all that goes with it, 12 decoding steps of 128 rows of SQL, 152,064 tokens, 4.93, 2.33 and 2.13 ms, 16 of 64 rows of a JSON
-// schema, 128,256 tokens, 2.44, 1.52 and 1.40 ms, 24 of 8 rows of JSON 3.58, 2.14 and 1.67 ms.
+// classes, a byte a round; by edges with eight blocks to a row, each with its own contexts; and now, us (the last: 254 to 282 on one B200 and
+// another):
+//   37 rows of JSON, 50,001 tokens                      139     65     33
+//   24 charts of JSON, 32,000 tokens, no allocations    123     71     39
+//   256 rows of ambiguous JSON, 128,256 tokens        1,010    790    265
+// and with all that goes with it, 12 decoding steps of 128 rows of SQL, 152,064 tokens, 4.93, 2.33 and 2.10 ms, 16 of 64 rows of a JSON
+// schema, 128,256 tokens, 2.44, 1.52 and 1.37 ms, 24 of 8 rows of JSON 3.58, 2.14 and 1.62 ms.
+// Slower than by the walk of the trie, where up to eight blocks shared a row: text of braces whose every byte ends a rule (20,000
+// lists of an edge or two go through a block's rounds), 1 and 4 rows 268 and 196 us then, 286 now; 64 and 256 rows 306 and 689 then, 290 and 313.
 #include <cuda_runtime.h>
 
 #include <algorithm>

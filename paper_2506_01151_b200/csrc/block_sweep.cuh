@@ -12,7 +12,7 @@ __host__ __device__ constexpr uint32_t block_sweep_words(uint32_t warps, uint32_
   return BS_HDR + warps * (SWEEP_CUR + SWEEP_HSET + ((2u * Nw + 7u) & ~7u) + W_CTRS + 8u);
 }
 
-// The row's mask row is written (other blocks may still be setting bits in it that are right).  `slot`: whose tables (S.au) are used.
+// The row's mask row is written (all of it, whatever the fill has set in it before it gave the row up).  `slot`: whose tables (S.au) are used.
 // False: a capacity was exceeded.  By all threads of a block; smem: block_sweep_words, 16-byte aligned.
 __device__ __noinline__ bool sweep_row_by_block(const GrammarDev& G, const StateDev& S, uint32_t row, uint32_t slot, uint32_t* smem) {
   const AutoDev& A = S.au;

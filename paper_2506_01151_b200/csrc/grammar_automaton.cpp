@@ -48,13 +48,25 @@ constexpr size_t GA_LONG_LIST = 64;       // edges of a start from which on it h
 constexpr size_t GA_MAX_ITEMS = 1024;     // items of one set, predicted ones included: alternations of thousands of literals
                                           // would be scanned again for every set that predicts them
 
-// Where the chart has to be asked at many places a fill by the automaton is the slower one: its threads walk the trie one by one, and
-// each exit starts a thread for every item that completing the rule yields.  Two counts over the walk tell such grammars; they go without.
-// Fills of 64 rows of 128,256 tokens by a walk of the trie with the automaton and by the sweep, us (share of nodes with an exit; starts a
-// node); by edges, as fills are made now, JSON takes 41, the union of 20 65, and the line lies well on the safe side:
-//   JSON 94 and 239 (0.09; 0.6)   ambiguous JSON 400 and 1,000 (0.12; 1.4)   SQL 231 and 667 (0.03; 1.1)   JSON schema 77 and 263 (0.02; 0.04)
-//   HTML 923 and 457 (0.75; 69)   braces 1,758 and 753 (0.72; 1.4)   XML 14,000 and 1,280 (0.75; 4.6)   two like texts 1,750 and 603 (0.51; 3.3)
-//   a union of 60 variants 2,607 and 430 (0.05; 5.1)   a C-like language 1,883 and 669 (0.17; 36)   a union of 20 485 and 411 (0.05; 1.7)
+// Where the chart has to be asked at many places a fill by the automaton can be the slower one: each exit has an edge for every item that
+// completing the rule yields, and a block follows those of its row where the whole grid sweeps the trie.  Two counts over the walk tell such
+// grammars; they go without.  Fills of 4 and of 64 rows of 128,256 tokens (SQL 152,064, braces 60,000) on a B200, us, by edges / by the sweep:
+//                                       4 rows           64 rows
+//   JSON                              40 /    276       40 /    614
+//   ambiguous JSON                   396 /  1,342      405 /  4,255
+//   SQL                               45 /    326       45 /    966
+//   text of one kind of character     44 /    111       45 /    303
+//   two like texts                    45 /    203       46 /    466
+//   a union of 20 variants            63 /    154       64 /    378     (starts a node 1.7)
+//   braces                           286 /    163      290 /    375
+//   those without, with both limits lifted:
+//   a union of 40, of 60             110, 143 / 172    111, 147 / 404   (60: 5.1)
+//   a union of 100, of 180           218, 367 / 181    221, 375 / 411, 435
+//   HTML with 2 tags, with 20        455, 1,260 / 146  465, 1,275 / 397, 420  (exits at 0.75 of the nodes)
+//   XML                           13,100 /  1,018   18,000 /  1,504     (0.75)
+// HTML and XML are on the right side of the line, unions of a hundred variants gain in large batches and lose in small ones, and
+// those of 40 and 60 would be faster by edges: the line was drawn for fills that walked the trie, and a higher one for them has not
+// been looked for.  The texts of one kind have few nodes (GA_EXITS).
 constexpr u32 GA_EXIT_SHARE = 4;          // no automaton if more than one in so many nodes has an exit
 constexpr u32 GA_EXITS = 1024;            // (and more than so many nodes: a small trie is walked in no time)
 constexpr u32 GA_STARTS = 2;              // nor if there are more starts than so many a node

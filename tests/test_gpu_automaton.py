@@ -45,7 +45,7 @@ JSON_PREFIXES = [list(x) for x in (b"", b'{"a": "x', b"[1, 2", b'{"k": tr', b"[[
 
 @pytest.mark.parametrize("batch", [1, 2, 19, 37, 74, 75, 148, 297, 700])
 def test_rows_of_every_share_of_the_grid(batch):
-    """One row may be shared by up to eight thread blocks, or a block may take several rows in turn."""
+    """A block takes a row, or several rows in turn where there are more of them than blocks."""
     w = workloads.build(2, V=3000, batch=1, steps=1)
     _run(w.ebnf, w.start, w.vocab, JSON_PREFIXES, batch=batch)
 
@@ -99,7 +99,7 @@ def _union(variants):
 @pytest.mark.parametrize("variants", [59, 60, 61, 100, 180])
 @pytest.mark.parametrize("batch", [1, 4, 75, 300])
 def test_more_wide_items_than_there_is_room_for(variants, batch):
-    """Up to 60 items of a row's last set are answered by the masks made for them; the others are walked like any item."""
+    """A union's last set has an item of every variant, each with a mask of its own or a list of tokens: 59 to 180 of them are joined."""
     rng = np.random.default_rng(variants)
     some = np.frombuffer(b"0123456789kid[]{}:,", np.uint8)
     vocab = workloads.build(2, V=32000, batch=1, steps=1).vocab[:-1] + sorted({bytes(some[rng.integers(0, 19, 6)]) for _ in range(70000)}) + [b""]
@@ -111,7 +111,7 @@ def test_more_wide_items_than_there_is_room_for(variants, batch):
 @pytest.mark.parametrize("n", [511, 512, 513, 600, 1000])
 @pytest.mark.parametrize("batch", [1, 5, 300])
 def test_more_items_than_a_round_takes(n, batch):
-    """After the byte that all literals of an alternation begin with, the last set has an item for each: a round takes 512 threads."""
+    """After the byte that all literals of an alternation begin with, the last set has an item for each: their starts are taken 256 at a time."""
     rng = np.random.default_rng(n)
     names = _words(rng, n, 15, "k")
     text = 's ::= "[" v ("," v)* "]"\nv ::= "\\"" name "\\"" | "[" v "]"\nname ::= ' + " | ".join('"%s"' % x for x in names)
@@ -181,8 +181,8 @@ def _endings(n):
 
 @pytest.mark.parametrize("n, batch", [(20, 3), (100, 3), (340, 1), (340, 9), (340, 80)])
 def test_rows_that_outgrow_the_storage_of_contexts(n, batch):
-    """Contexts begin in shared memory (64) and go on in storage of the block's own (4,096).  A row that needs more is swept by
-    Earley steps in the same call, by one of its blocks; the rows beside it are not touched by that."""
+    """Contexts begin in shared memory (320) and go on in storage of the block's own (1,024).  A row that needs more is swept by
+    Earley steps in the same call, by a block that has no row left; the rows beside it are not touched by that."""
     text, vocab = _endings(n)
     prefixes = [list(p) for p in (b"(" * 20, b"(" * 20 + b"x", b"(" * 20 + b"x)a", b"((x)a")]
     s = _run(text, "s", vocab, prefixes, batch=batch, check=range(min(batch, 4)))
