@@ -815,8 +815,6 @@ __global__ void __launch_bounds__(AF_THREADS, 2) automaton_fill_kernel(const __g
     const int32_t sid = S.row_state ? S.row_state[row] : -1;
     const uint32_t taken = tid == 0 && S.cache_on ? vload(&S.counters[CNT_N_MASK_ROWS]) : 0u;
     const uint32_t ahead = tid < A.ahead ? chart[tid] : 0u;  // (asked for together with the header)
-    // an earlier fill's mark goes (by a thread that nobody waits for, when what it asks for is long there)
-    const uint32_t mark = row == 0u && tid == AF_THREADS - 1 ? vload(&S.counters[CNT_BAR_ERR]) : 0u;
     AfChart J;
     J.m = chart[CH_SETS];
     const uint32_t chart_words = chart[CH_WORDS], chart_flags = chart[CH_FLAGS];
@@ -843,7 +841,6 @@ __global__ void __launch_bounds__(AF_THREADS, 2) automaton_fill_kernel(const __g
       if (S.row_job) S.row_job[row] = here ? 1u : 0u;
       ctl[AC_ROW] = here ? 1u : 0u;
     }
-    if (mark && mark != fill_tag()) atomicCAS(&S.counters[CNT_BAR_ERR], mark, 0u);
     __syncthreads();
     if (ctl[AC_ROW]) {
       const bool accepting = (chart_flags & CHART_ACCEPTING) != 0u, staged = chart_words <= AF_STAGE;
@@ -1210,6 +1207,10 @@ __global__ void __launch_bounds__(AF_THREADS, 2) automaton_fill_kernel(const __g
     __syncthreads();
     row = ctl[AC_ROW];
     __syncthreads();
+  }
+  if (blockIdx.x == 0 && tid == AF_THREADS - 1) {  // an earlier fill's mark goes (a block of this one that gives up sets this one's)
+    const uint32_t mark = vload(&S.counters[CNT_BAR_ERR]);
+    if (mark && mark != fill_tag()) atomicCAS(&S.counters[CNT_BAR_ERR], mark, 0u);
   }
   if (!filled) return;
   looked_up = __reduce_add_sync(FULL, looked_up);
