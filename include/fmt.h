@@ -290,7 +290,9 @@ fmt_status fmt_state_forced_bytes(fmt_state* s, uint8_t* bytes_dev, size_t strid
 /*
  * Write the mask of every row (Sections 3.3, 4.1): mask_dev[row * stride_words + w].
  * stride_words >= ceil(V/32).  Rows whose pruned chart is in the state cache copy the cached
- * mask; the others sweep the vocabulary trie.
+ * mask; the others follow the grammar's automaton, or sweep the vocabulary trie where it has none.
+ * A fill by the automaton may be captured into a graph and replayed.  A sweep may not: its tables of Earley sets are
+ * told apart from the last fill's by a number that goes into the launch.
  */
 fmt_status fmt_fill_mask(fmt_state* s, uint32_t* mask_dev, size_t stride_words, void* stream);
 
